@@ -245,21 +245,24 @@ doa_status doa_model_order(const double *evals, int M, int N, int *mdl, int *aic
  * iteration stops after the first sweep that rotates nothing. Then X = U S V^H, and the eigenvalues of R are
  * S_k^2 / N with eigenvectors the columns of U. Small singular values keep their relative
  * accuracy (R's eigenvalues below ~1e-16 of the largest do not).
- * GPU form: the rows live in an FP64 copy Y of X in ws; each sweep is one pass over Y on all SMs
- * that applies the previous sweep's rotations and forms the Gram matrix Y Y^H in FP64, then the
- * sweep's rotations run on that Gram matrix in one CTA (its pair entries are the rotated Gram
- * entries, formed afresh from the rows once per sweep).
+ * GPU form: one cooperative kernel (its CTAs, one per SM at most, wait for one another). The rows
+ * live in an FP64 copy Y of X in ws; a pass over Y on all SMs applies the rotations found so far and
+ * forms the Gram matrix Y Y^H in FP64, and the sweep's rotations run on that Gram matrix in one CTA
+ * (its pair entries are the rotated Gram entries). While off-diagonal entries above 1e-4
+ * sqrt(alpha beta) are met and the diagonal spans less than 1e4, the next sweep continues on the
+ * rotated Gram matrix; every other sweep, and always the deciding one, starts from one formed afresh
+ * from the rows.
  *   X          : M x N snapshots, row-major with row stride ldx (>= N) elements: complex64
  *                (x_c128 = 0, 8-byte aligned) or complex128 (x_c128 = 1, 16-byte aligned).
  *   tol        : rotation threshold (> 0; 1e-15 is the usual choice). max_sweeps: 1..1000.
  *   evals      : M device doubles, descending (equal values in index order).
  *   U          : M x M complex128, column-major (ld M): column k is the singular vector of evals[k].
  *   info       : one device int32: the sweep count, or -DOA_ENOCONV when max_sweeps sweeps still
- *                rotated (outputs then hold the last sweep's Gram diagonal and rotations).
+ *                rotated (outputs then hold the last sweep's Gram diagonal and rotations), or
+ *                -DOA_ETIMEOUT if a bounded wait of the grid ran out (outputs undefined).
  *   ws         : device scratch of doa_svd_data_ws_bytes(M, N) bytes, 16-byte aligned (about
  *                16 M N bytes: the FP64 rows, plus the partial Gram matrices); DOA_ENOMEM if
- *                ws_bytes is smaller. The call enqueues 2 * max_sweeps kernels; those after
- *                convergence return at once.
+ *                ws_bytes is smaller.
  * Errors: DOA_EINVAL for M outside [2, 64], N < 1, ldx < N, a NULL or misaligned pointer, or a
  * bad tol / max_sweeps.
  */

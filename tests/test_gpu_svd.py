@@ -130,3 +130,43 @@ def test_svd_rank_one_and_sweep_cap(env):
     assert np.all(np.isfinite(ev)) and np.all(np.isfinite(U))
     A = np.abs(U)                                        # the cap left U a permutation (sorted by the
     assert np.all((A == 0.0) | (A == 1.0)) and np.all(A.sum(0) == 1.0) and np.all(A.sum(1) == 1.0)   # Gram diagonal)
+
+
+@pytest.mark.parametrize("M,N,cap", [(3, 50, 60), (17, 300, 60), (33, 1000, 60), (63, 500, 60), (64, 64, 60), (17, 300, 3),
+                                     (64, 2048, 4)])
+def test_svd_levels_at_odd_sizes_and_inside_the_cap(env, M, N, cap):
+    """The simultaneous rotations of a level at odd and full sizes, and a cap that ends the iteration
+    while sweeps run on the rotated Gram matrix: U holds every rotation taken (unitary), and the values
+    are the diagonal of U^H X X^H U / N to FP64 rounding of its largest entry (M N products)."""
+    torch, doa = env
+    rng = np.random.default_rng(100 * M + cap)
+    X = (rng.standard_normal((M, N)) + 1j * rng.standard_normal((M, N))).astype(np.complex64)
+    ev, U, info = _svd(torch, doa, X, max_sweeps=cap)
+    assert (info == -doa.ENOCONV) if cap < 10 else info > 0
+    assert np.abs(U.conj().T @ U - np.eye(M)).max() <= 1e-12
+    Y = U.conj().T @ X.astype(np.complex128)
+    diag = np.einsum("it,it->i", Y, Y.conj()).real / N
+    np.testing.assert_allclose(ev, diag, rtol=0, atol=1e-12 * diag.max())
+    assert np.all(np.diff(ev) <= 0)
+    if cap >= 10:
+        _check_unitary_and_diagonal(X, ev, U)
+
+
+def test_svd_under_stream_capture(env):
+    """The cooperative launch is captured into a graph and replays on new snapshots."""
+    torch, doa = env
+    inst = [synth.custom(12, 3, 500, None, 10.0, 0.1, seed=950 + k) for k in range(2)]
+    X = torch.from_numpy(inst[0].X).cuda()
+    ev = torch.empty(12, dtype=torch.float64, device="cuda")
+    U = torch.empty((12, 12), dtype=torch.complex128, device="cuda")
+    info = torch.zeros(1, dtype=torch.int32, device="cuda")
+    ws = doa.doa_svd_data(X, ev, U, info)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        doa.doa_svd_data(X, ev, U, info, ws=ws)
+    X.copy_(torch.from_numpy(inst[1].X))
+    graph.replay()
+    torch.cuda.synchronize()
+    evo, _, _ = oracle.svd_data(inst[1].X)
+    assert np.abs(ev.cpu().numpy() - evo).max() <= 1e-13 * evo[0]
