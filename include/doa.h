@@ -144,7 +144,7 @@ doa_status doa_covariance_noalloc(const float *X, int M, int N, int ldx, float *
                                   void *stream);
 
 /*
- * Steps 2-4: Hermitian eigendecomposition of R by FP64 cyclic Jacobi (one warp per matrix,
+ * Steps 2-4: Hermitian eigendecomposition of R by FP64 cyclic Jacobi (one CTA per matrix,
  * parallel round-robin ordering), eigenvalues sorted descending (equal values keep their
  * index order), then the noise-subspace factor B of the weighting matrix, C = B B^H (Table 3):
  *   PHD   : B = e_min (last eigenvector),                K = 1
@@ -434,7 +434,8 @@ typedef struct {
                          /* the in-register phasors); default (4, 2, 1, 1).                     */
   int32_t eig_mats[4];   /* matrices per Jacobi warp. Allowed {1, 2, 4, 8}, {1, 2, 4}, {1, 2},   */
                          /* {1} (a lane per rotation pair); default: 1 unless the bucket holds   */
-                         /* enough problems to keep ~24 packed warps per SM busy.               */
+                         /* enough problems to keep ~24 packed warps per SM busy. At 1, small    */
+                         /* batches take a CTA per matrix; M > 16 always does.                   */
   int32_t scan_group[4]; /* FP32 ULA problems that share a grid are scanned together in groups  */
                          /* of this many (one steering generation per tile of the grid for the   */
                          /* whole group, each problem's factor contracted in turn); 1 scans every */

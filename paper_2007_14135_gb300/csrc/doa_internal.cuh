@@ -384,7 +384,7 @@ __host__ __device__ inline bool scan_pt_allowed(int bucket, int pt) {
 }
 
 // Jacobi packing: a warp holds G matrices of one bucket with G x (NP / 2) <= 32 rotation pairs
-// (one lane each); the M <= 64 bucket runs one matrix per 256-thread CTA.
+// (one lane each). The M <= 32 and M <= 64 buckets run a matrix per CTA or cluster whatever G is.
 __host__ __device__ constexpr int eig_mats_max(int bucket) { return bucket == 0 ? 8 : (bucket == 1 ? 4 : (bucket == 2 ? 2 : 1)); }
 __host__ __device__ inline bool eig_mats_allowed(int bucket, int g) {
   return g >= 1 && g <= eig_mats_max(bucket) && (g & (g - 1)) == 0;

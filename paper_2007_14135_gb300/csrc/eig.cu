@@ -11,15 +11,23 @@
 // hypot or sqrt), so c^2 + |sigma|^2 = 1 holds to FP64 rounding.
 //
 // Parallel ordering: n/2 disjoint rotations per round (round-robin "circle" ordering over
-// n = M rounded up to even; pairs that touch the padding index are skipped): the row update
-// A <- J^H A for all rotated pairs, then the column updates A <- A J and V <- V J. A pair is
+// n = M rounded up to even; a pair that touches the padding index is not rotated). A pair is
 // rotated when |a_pq|^2 > tol^2 |a_pp a_qq|; a matrix has converged after a sweep that rotates
-// nothing. A warp holds 32 / (NP/2) matrices so that every lane owns one pair's rotation
-// (8 matrices of M <= 8, 4 of M <= 16, 2 of M <= 32); a matrix of M <= 64 gets a whole CTA in
-// FP64, or in double-float a cluster of four CTAs that split its rows (jacobi_cluster_df).
-// The element updates of each matrix are spread over all threads of its group. A and V live in shared memory with a padded row stride
-// (NP + 1 complex128) so that column accesses by consecutive lanes hit distinct banks.
+// nothing. A round updates A block by block: the 2 x 2 block of the rows of pair a and the columns of
+// pair b >= a takes four lanes, one element each -- the row mix A <- J^H A of the lane's element,
+// exchanged with the lane of the other column, then the column mix A <- A J -- and is written to its
+// mirror image as well, so only half of A is computed; V <- V J takes a lane per pair and row.
+//
+// Two shapes, with the same arithmetic and results. A warp per matrix (or G packed matrices, every
+// lane owning one pair's rotation) keeps the most matrices resident and suits large batches of M <= 16.
+// A CTA per matrix (3, 5 or 17 warps at M <= 8, 16, 32) suits single calls, small batches and M <= 32,
+// which otherwise wait for one warp's chain of instructions: one FP64 matrix of M = 8 in 78 instead of
+// 141 us, 254 double-float matrices of M = 32 in 0.8 instead of 3.2 ms. Half of A: 4096 matrices of
+// M = 16 in 1.10 instead of 1.27 ms.
+// M <= 64 gets a 512-thread CTA in FP64, or in double-float a cluster of four CTAs that split its
+// rows (jacobi_cluster_df).
 #include <cooperative_groups.h>
+#include <type_traits>
 #include <math_constants.h>
 
 #include "doa_internal.cuh"
@@ -41,7 +49,6 @@ struct EigSmem {
   double2 V[NP][NP];
   Rot rot[NP / 2];      // the sweeps' rotations; after the sweeps the same bytes hold lam, order
   int2 pq[NP / 2];
-  unsigned mask;        // rotation mask broadcast when a group spans several warps
   __device__ __forceinline__ double2 &a(int i, int k) { return A[i][k ^ (i & 7)]; }
   __device__ __forceinline__ double2 &v(int i, int k) { return V[i][k ^ (i & 7)]; }
   __device__ __forceinline__ double *lam() { return reinterpret_cast<double *>(rot); }
@@ -49,20 +56,27 @@ struct EigSmem {
   static_assert(sizeof(Rot) * (NP / 2) >= NP * (sizeof(double) + sizeof(int)), "lam and order fit in rot");
 };
 
-// A group of T threads works on G matrices: one warp on 8, 4 or 2 matrices of M <= 8, 16, 32
-// (every lane owns one pair), or a whole 16-warp CTA on one matrix of M <= 64 (the 32 pairs
-// are owned by warp 0's lanes; the element updates are spread over all 512 threads).
+// Threads per matrix of the CTA form: a round's warp steps (blocks of A, then rows of V) are 2 + 1 at
+// M = 8, 5 + 4 at M = 16, 17 + 16 at M = 32, taken in one, two and two turns. At M = 16 nine warps take
+// them in one turn but let fewer matrices reside: 0.13 against 0.14 ms for one matrix, 0.41 against
+// 0.34 ms for 1024.
 template <int NP>
-__host__ __device__ constexpr int grp_threads() { return NP <= 32 ? 32 : 512; }
+__host__ __device__ constexpr int cta_threads() { return NP <= 8 ? 96 : (NP <= 16 ? 160 : (NP <= 32 ? 544 : 512)); }
+// Largest batch that takes the CTA form (the eig stage, warp form against CTA form): at M <= 8, 63 / 47
+// us for 1 matrix, 82 / 74 for 1024, 112 / 131 for 2048; at M <= 16, 0.32 / 0.14 ms for 1, 0.53 / 0.23
+// for 512, 0.77 / 0.64 for 2048, 1.06 / 1.20 for 4096; at M <= 32 always (2.3 / 0.53 ms for 1, 4.7 / 2.7
+// for 1024).
 template <int NP>
-__host__ __device__ constexpr int mats_per_warp() { return NP <= 32 ? 64 / NP : 1; }
-// Warps per CTA of the batch kernel, at most (the launch picks the count for the resident total).
+__host__ constexpr int eig_cta_limit() { return NP <= 8 ? 1024 : 2048; }
 template <int NP>
-__host__ __device__ constexpr int eig_warps() { return NP <= 8 ? 4 : (NP <= 16 ? 9 : (NP <= 32 ? 1 : 16)); }
-// CTAs per SM the batch kernel's register budget is set for: three nine-warp CTAs at M <= 16,
-// elsewhere 64 registers a thread.
+__host__ __device__ constexpr int mats_per_warp() { return 64 / NP; }
+// Warps per CTA of the warp form, at most (the launch picks the count for the resident total).
 template <int NP>
-__host__ __device__ constexpr int eig_min_ctas() { return NP > 8 && NP <= 16 ? 3 : 1024 / (32 * eig_warps<NP>()); }
+__host__ __device__ constexpr int eig_warps() { return NP <= 8 ? 4 : 9; }
+// CTAs per SM its register budget is set for: three nine-warp CTAs at M <= 16, 64 registers a thread
+// at M <= 8.
+template <int NP>
+__host__ __device__ constexpr int eig_min_ctas() { return NP <= 8 ? 8 : 3; }
 
 template <int T>
 struct Grp {
@@ -75,167 +89,24 @@ struct Grp {
 };
 
 __device__ __forceinline__ int rr_player(int pos, int r, int n) {
-  return pos == 0 ? 0 : ((pos - 1 + r) % (n - 1)) + 1;
+  const int v = pos - 1 + r;   // < 2 (n - 1)
+  return pos == 0 ? 0 : (v >= n - 1 ? v - (n - 1) : v) + 1;
 }
 
-// Rotation of pair (p, q) of A; returns false if the pair is below threshold.
-template <int NP>
-__device__ __forceinline__ bool rotation(EigSmem<NP> &s, int p, int q, Rot &ro) {
-  const double app = s.a(p, p).x, aqq = s.a(q, q).x;
-  const double2 apq = s.a(p, q);
-  const double n2 = apq.x * apq.x + apq.y * apq.y;
-  if (!(n2 > 0.0) || !(n2 > kJacobiTol * kJacobiTol * fabs(app * aqq))) return false;
-  const double r = rsqrt(n2);                         // 1 / |a_pq|
-  const double tau = (aqq - app) * (0.5 * r);
-  double t;
-  if (fabs(tau) > 1e18) {
-    t = 0.5 * __drcp_rn(tau);                         // t = 1/(2 tau) to within tau^-2
-  } else {
-    const double u = fma(tau, tau, 1.0);
-    const double h = u * rsqrt(u);                    // sqrt(1 + tau^2)
-    t = copysign(__drcp_rn(fabs(tau) + h), tau);
-  }
-  const double c = rsqrt(fma(t, t, 1.0));
-  const double sn = t * c * r;
-  ro = Rot{c, sn * apq.x, sn * apq.y};
+// Rotation of a pair from its entries; returns false if the pair is below threshold. An FP64 warp
+// instruction holds its sub-partition for 64 cycles here, so the chain is kept short: cos^2 = 1/2 +
+// |d| / (2h) and sigma = a_pq / (h cos) with d = a_qq - a_pp, h = sqrt(d^2 + 4 |a_pq|^2) -- the same
+// rotation as through tau and t, with two reciprocal square roots and no division.
+__device__ __forceinline__ bool rotation_of(const double app, const double aqq, const double2 apq, Rot &ro) {
+  const double n2 = fma(apq.x, apq.x, apq.y * apq.y);
+  if (!(n2 > kJacobiTol * kJacobiTol * fabs(app * aqq))) return false;
+  const double d = aqq - app;
+  const double rh = rsqrt(fma(4.0, n2, d * d));        // 1 / h
+  const double w = fma(fabs(d) * rh, 0.5, 0.5);         // cos^2
+  const double rc = rsqrt(w);                           // 1 / cos
+  const double k = copysign(rh * rc, d);                // sin / |a_pq|, of the sign of tau
+  ro = Rot{w * rc, k * apq.x, k * apq.y};
   return true;
-}
-
-// Runs Jacobi on the G matrices of a warp (matrix j has size Ms[j] <= NP, 0 = unused), all
-// loaded from Rs[j] (upper triangle). res[j] receives sweeps (> 0) or -status.
-template <int NP, int G>
-__device__ void jacobi_group(EigSmem<NP> *mats, const int *Ms, const double2 *const *Rs, int *res) {
-  constexpr int HP = NP / 2;
-  constexpr int T = grp_threads<NP>();
-  using g = Grp<T>;
-  const int lane = g::id();
-  unsigned live = 0u;  // matrices still iterating
-  for (int j = 0; j < G; ++j) {
-    const int M = Ms[j];
-    res[j] = 0;
-    if (M <= 0) continue;
-    EigSmem<NP> &s = mats[j];
-    const double2 *R = Rs[j];
-    bool finite = true;
-    for (int e = lane; e < M * M; e += T) {
-      int i = e / M, k = e % M;
-      double2 v;
-      if (i <= k) {
-        v = R[i * M + k];
-      } else {
-        v = R[k * M + i];
-        v.y = -v.y;
-      }
-      if (i == k) v.y = 0.0;
-      finite = finite && isfinite(v.x) && isfinite(v.y);
-      s.a(i, k) = v;
-      s.v(i, k) = make_double2(i == k ? 1.0 : 0.0, 0.0);
-    }
-    if (g::all(finite))
-      live |= 1u << j;
-    else
-      res[j] = -DOA_ENONFINITE;
-  }
-  g::sync();
-  int maxn = 0;
-  for (int j = 0; j < G; ++j)
-    if ((live >> j) & 1u) maxn = max(maxn, (Ms[j] + 1) & ~1);
-  // lane -> (matrix, pair) for the rotation parameters
-  const int lj = lane < 32 ? lane / HP : G, li = lane % HP;
-  for (int sweep = 1; sweep <= kMaxSweeps && live; ++sweep) {
-    unsigned rotated = 0u;
-    for (int r = 0; r < maxn - 1; ++r) {
-      bool act = false;
-      if (lj < G && ((live >> lj) & 1u)) {
-        const int M = Ms[lj], n = (M + 1) & ~1;
-        if (r < n - 1 && li < n / 2) {
-          const int a = rr_player(li, r, n), b = rr_player(n - 1 - li, r, n);
-          const int p = min(a, b), q = max(a, b);
-          if (q < M) {
-            Rot ro;
-            if (rotation<NP>(mats[lj], p, q, ro)) {
-              act = true;
-              mats[lj].rot[li] = ro;
-              mats[lj].pq[li] = make_int2(p, q);
-            }
-          }
-        }
-      }
-      unsigned mask;
-      if (T == 32) {
-        mask = __ballot_sync(0xffffffffu, act);
-      } else {
-        const unsigned m0 = __ballot_sync(0xffffffffu, act);
-        if (threadIdx.x == 0) mats[0].mask = m0;    // only warp 0 owns pairs
-        __syncthreads();
-        mask = mats[0].mask;
-        __syncthreads();
-      }
-      if (mask == 0u) continue;
-      g::sync();
-      // rows: A <- J^H A. new row p = c x_p - sigma x_q; new row q = conj(sigma) x_p + c x_q
-      for (int j = 0; j < G; ++j) {
-        const unsigned seg = (mask >> (j * HP)) & ((HP == 32) ? 0xffffffffu : ((1u << HP) - 1u));
-        if (!seg) continue;
-        rotated |= 1u << j;
-        EigSmem<NP> &s = mats[j];
-        const int M = Ms[j];
-        for (int it = lane; it < HP * M; it += T) {
-          const int i = it / M, k = it % M;
-          if (!((seg >> i) & 1u)) continue;
-          const Rot ro = s.rot[i];
-          const int2 pq = s.pq[i];
-          const double2 xp = s.a(pq.x, k), xq = s.a(pq.y, k);
-          s.a(pq.x, k) = make_double2(ro.c * xp.x - (ro.sr * xq.x - ro.si * xq.y),
-                                      ro.c * xp.y - (ro.sr * xq.y + ro.si * xq.x));
-          s.a(pq.y, k) = make_double2(ro.c * xq.x + (ro.sr * xp.x + ro.si * xp.y),
-                                      ro.c * xq.y + (ro.sr * xp.y - ro.si * xp.x));
-        }
-      }
-      g::sync();
-      // columns: A <- A J, V <- V J. new col p = c x_p - conj(sigma) x_q; new col q = sigma x_p + c x_q
-      for (int j = 0; j < G; ++j) {
-        const unsigned seg = (mask >> (j * HP)) & ((HP == 32) ? 0xffffffffu : ((1u << HP) - 1u));
-        if (!seg) continue;
-        EigSmem<NP> &s = mats[j];
-        const int M = Ms[j];
-        for (int it = lane; it < HP * M; it += T) {
-          const int i = it / M, k = it % M;
-          if (!((seg >> i) & 1u)) continue;
-          const Rot ro = s.rot[i];
-          const int2 pq = s.pq[i];
-          const double2 xp = s.a(k, pq.x), xq = s.a(k, pq.y);
-          s.a(k, pq.x) = make_double2(ro.c * xp.x - (ro.sr * xq.x + ro.si * xq.y),
-                                      ro.c * xp.y - (ro.sr * xq.y - ro.si * xq.x));
-          s.a(k, pq.y) = make_double2(ro.c * xq.x + (ro.sr * xp.x - ro.si * xp.y),
-                                      ro.c * xq.y + (ro.sr * xp.y + ro.si * xp.x));
-          const double2 vp = s.v(k, pq.x), vq = s.v(k, pq.y);
-          s.v(k, pq.x) = make_double2(ro.c * vp.x - (ro.sr * vq.x + ro.si * vq.y),
-                                      ro.c * vp.y - (ro.sr * vq.y - ro.si * vq.x));
-          s.v(k, pq.y) = make_double2(ro.c * vq.x + (ro.sr * vp.x - ro.si * vp.y),
-                                      ro.c * vq.y + (ro.sr * vp.y + ro.si * vp.x));
-        }
-      }
-      g::sync();
-      if (act) {
-        EigSmem<NP> &s = mats[lj];
-        const int2 pq = s.pq[li];
-        s.a(pq.x, pq.y) = make_double2(0.0, 0.0);
-        s.a(pq.y, pq.x) = make_double2(0.0, 0.0);
-        s.a(pq.x, pq.x).y = 0.0;
-        s.a(pq.y, pq.y).y = 0.0;
-      }
-      g::sync();
-    }
-    // matrices without a rotation in this sweep have converged
-    for (int j = 0; j < G; ++j)
-      if (((live >> j) & 1u) && !((rotated >> j) & 1u)) {
-        res[j] = sweep;
-        live &= ~(1u << j);
-      }
-  }
-  for (int j = 0; j < G; ++j)
-    if ((live >> j) & 1u) res[j] = -DOA_ENOCONV;
 }
 
 // ------------------------------------------------------------------------------------------
@@ -332,43 +203,92 @@ __device__ __forceinline__ bool rotation_df_of(const float4 app, const float4 aq
   return true;
 }
 
+// The two arithmetics of the Jacobi: element type, rotation of a pair, and the mix of an element with
+// its partner: c own + sr oth + (si oth_im, -si oth_re). With (sr, si) = (-+Re sigma, Im sigma) that is
+// row p (-) or q (+) of J^H A, with -Im sigma column p (-) or q (+) of A J.
 template <int NP>
-__device__ __forceinline__ bool rotation_df(EigSmemDF<NP> &s, int p, int q, RotDF &ro) {
-  return rotation_df_of(s.a(p, p), s.a(q, q), s.a(p, q), ro);
+struct ArithF64 {
+  using El = double2;
+  using Ro = Rot;
+  static __device__ __forceinline__ El &a(EigSmem<NP> &s, int i, int k) { return s.a(i, k); }
+  static __device__ __forceinline__ El &v(EigSmem<NP> &s, int i, int k) { return s.v(i, k); }
+  static __device__ __forceinline__ Ro *rot(EigSmem<NP> &s) { return s.rot; }
+  static __device__ __forceinline__ El from(double2 x) { return x; }
+  static __device__ __forceinline__ bool rotation(El app, El aqq, El apq, Ro &ro) {
+    return rotation_of(app.x, aqq.x, apq, ro);
+  }
+  // sign changes on the bits: an FP64 negation costs as much as a multiply-add
+  static __device__ __forceinline__ double neg(double x) {
+    return __hiloint2double(__double2hiint(x) ^ (int)0x80000000, __double2loint(x));
+  }
+  static __device__ __forceinline__ El mix(double c, double sr, double si, El own, El oth) {
+    return make_double2(fma(c, own.x, fma(sr, oth.x, si * oth.y)), fma(c, own.y, fma(sr, oth.y, -si * oth.x)));
+  }
+  static __device__ __forceinline__ El conj(El x) { return make_double2(x.x, neg(x.y)); }
+  static __device__ __forceinline__ El real(El x) { return make_double2(x.x, 0.0); }
+  static constexpr bool kZeroes = true;   // the annihilated entry is set to zero
+};
+
+template <int NP>
+struct ArithDF {
+  using El = float4;
+  using Ro = RotDF;
+  static __device__ __forceinline__ EigSmemDF<NP> &df(EigSmem<NP> &s) { return *reinterpret_cast<EigSmemDF<NP> *>(&s); }
+  static __device__ __forceinline__ El &a(EigSmem<NP> &s, int i, int k) { return df(s).a(i, k); }
+  static __device__ __forceinline__ El &v(EigSmem<NP> &s, int i, int k) { return df(s).v(i, k); }
+  static __device__ __forceinline__ Ro *rot(EigSmem<NP> &s) { return df(s).rot; }
+  static __device__ __forceinline__ El from(double2 x) { return df_of(x); }
+  static __device__ __forceinline__ bool rotation(El app, El aqq, El apq, Ro &ro) {
+    return rotation_df_of(app, aqq, apq, ro);
+  }
+  static __device__ __forceinline__ F2 neg(F2 x) { return F2{-x.h, -x.l}; }
+  static __device__ __forceinline__ El mix(F2 c, F2 sr, F2 si, El own, El oth) {
+    return cplx(dot3(c, re_of(own), sr, re_of(oth), si, im_of(oth)),
+                dot3(c, im_of(own), sr, im_of(oth), neg(si), re_of(oth)));
+  }
+  static __device__ __forceinline__ El conj(El x) { return make_float4(x.x, x.y, -x.z, -x.w); }
+  static __device__ __forceinline__ El real(El x) { return make_float4(x.x, x.y, 0.f, 0.f); }
+  static constexpr bool kZeroes = false;  // it keeps its computed residual for the next sweep
+};
+
+__device__ __forceinline__ double2 shfl_xor1(double2 x) {
+  return make_double2(__shfl_xor_sync(0xffffffffu, x.x, 1), __shfl_xor_sync(0xffffffffu, x.y, 1));
+}
+__device__ __forceinline__ float4 shfl_xor1(float4 x) {
+  return make_float4(__shfl_xor_sync(0xffffffffu, x.x, 1), __shfl_xor_sync(0xffffffffu, x.y, 1),
+                     __shfl_xor_sync(0xffffffffu, x.z, 1), __shfl_xor_sync(0xffffffffu, x.w, 1));
 }
 
-// Same contract as jacobi_group, in double-float arithmetic; on return A and V hold FP64.
-template <int NP, int G>
-__device__ void jacobi_group_df(EigSmem<NP> *mats64, const int *Ms, const double2 *const *Rs, int *res) {
-  constexpr int HP = NP / 2;
-  constexpr int T = grp_threads<NP>();
+// Runs Jacobi on the G matrices of a group of T threads (matrix j has size Ms[j] <= NP, 0 = unused),
+// all loaded from Rs[j] (upper triangle). T = 32: a warp; otherwise the whole CTA on one matrix.
+// res[j] receives sweeps (> 0) or -status; on return A (its diagonal) and V hold FP64.
+template <class Ar, int NP, int G, int T>
+__device__ void jacobi_group(EigSmem<NP> *mats, const int *Ms, const double2 *const *Rs, int *res) {
+  static_assert(T == 32 || G == 1, "a CTA works on one matrix");
+  constexpr int HP = NP / 2, W = T / 32;
   using g = Grp<T>;
-  static_assert(sizeof(EigSmemDF<NP>) <= sizeof(EigSmem<NP>), "double-float view fits");
-  // matrix j's double-float view starts where its EigSmem record starts (the records are laid out
-  // with the EigSmem stride, so the view is formed per matrix, never by indexing a view array)
-  auto df = [&](int j) -> EigSmemDF<NP> & { return *reinterpret_cast<EigSmemDF<NP> *>(&mats64[j]); };
-  const int lane = g::id();
-  unsigned live = 0u;
+  using El = typename Ar::El;
+  __shared__ unsigned smask[2];   // the round's rotations, by round parity (CTA form)
+  const int tid = g::id(), lane = tid & 31, wp = tid >> 5;
+  unsigned live = 0u;  // matrices still iterating
   for (int j = 0; j < G; ++j) {
-    const int M = Ms[j];
+    const int M = Ms[j], n = (M + 1) & ~1;
     res[j] = 0;
     if (M <= 0) continue;
-    EigSmemDF<NP> &s = df(j);
+    EigSmem<NP> &s = mats[j];
     const double2 *R = Rs[j];
     bool finite = true;
-    for (int e = lane; e < M * M; e += T) {
-      int i = e / M, k = e % M;
-      double2 v;
-      if (i <= k) {
-        v = R[i * M + k];
-      } else {
-        v = R[k * M + i];
-        v.y = -v.y;
+    for (int e = tid; e < n * n; e += T) {
+      const int i = e / n, k = e - i * n;
+      double2 v = make_double2(0.0, 0.0);   // an odd M is padded with a zero row and column
+      if (i < M && k < M) {
+        v = R[min(i, k) * M + max(i, k)];
+        if (i > k) v.y = -v.y;
+        if (i == k) v.y = 0.0;
       }
-      if (i == k) v.y = 0.0;
       finite = finite && isfinite(v.x) && isfinite(v.y);
-      s.a(i, k) = df_of(v);
-      s.v(i, k) = make_float4(i == k ? 1.f : 0.f, 0.f, 0.f, 0.f);
+      Ar::a(s, i, k) = Ar::from(v);
+      Ar::v(s, i, k) = Ar::from(make_double2(i == k ? 1.0 : 0.0, 0.0));
     }
     if (g::all(finite))
       live |= 1u << j;
@@ -379,90 +299,101 @@ __device__ void jacobi_group_df(EigSmem<NP> *mats64, const int *Ms, const double
   int maxn = 0;
   for (int j = 0; j < G; ++j)
     if ((live >> j) & 1u) maxn = max(maxn, (Ms[j] + 1) & ~1);
-  const int lj = lane < 32 ? lane / HP : G, li = lane % HP;
+  // lane of the first warp -> (matrix, pair) for the rotation parameters
+  const int lj = wp == 0 ? lane / HP : G, li = lane % HP;
+  unsigned t = 0u;     // rounds so far
   for (int sweep = 1; sweep <= kMaxSweeps && live; ++sweep) {
     unsigned rotated = 0u;
-    for (int r = 0; r < maxn - 1; ++r) {
-      bool act = false;
-      if (lj < G && ((live >> lj) & 1u)) {
-        const int M = Ms[lj], n = (M + 1) & ~1;
-        if (r < n - 1 && li < n / 2) {
-          const int a = rr_player(li, r, n), b = rr_player(n - 1 - li, r, n);
-          const int p = min(a, b), q = max(a, b);
-          if (q < M) {
-            RotDF ro;
-            if (rotation_df<NP>(df(lj), p, q, ro)) {
-              act = true;
-              df(lj).rot[li] = ro;
-              mats64[lj].pq[li] = make_int2(p, q);
+    for (int r = 0; r < maxn - 1; ++r, ++t) {
+      unsigned mask = 0u;
+      if (wp == 0) {
+        bool act = false;
+        if (lj < G && ((live >> lj) & 1u)) {
+          const int M = Ms[lj], n = (M + 1) & ~1;
+          if (r < n - 1 && li < n / 2) {
+            const int a = rr_player(li, r, n), b = rr_player(n - 1 - li, r, n);
+            const int p = min(a, b), q = max(a, b);
+            EigSmem<NP> &s = mats[lj];
+            s.pq[li] = make_int2(p, q);
+            if (q < M) {
+              typename Ar::Ro ro;
+              act = Ar::rotation(Ar::a(s, p, p), Ar::a(s, q, q), Ar::a(s, p, q), ro);
+              if (act) Ar::rot(s)[li] = ro;
             }
           }
         }
-      }
-      unsigned mask;
-      if (T == 32) {
         mask = __ballot_sync(0xffffffffu, act);
-      } else {
-        const unsigned m0 = __ballot_sync(0xffffffffu, act);
-        if (threadIdx.x == 0) mats64[0].mask = m0;
+        if (T > 32 && lane == 0) smask[t & 1u] = mask;
+      }
+      if (T > 32) {
         __syncthreads();
-        mask = mats64[0].mask;
-        __syncthreads();
+        mask = smask[t & 1u];
       }
       if (mask == 0u) continue;
       g::sync();
-      // rows: A <- J^H A. new row p = c x_p - sigma x_q; new row q = conj(sigma) x_p + c x_q
       for (int j = 0; j < G; ++j) {
         const unsigned seg = (mask >> (j * HP)) & ((HP == 32) ? 0xffffffffu : ((1u << HP) - 1u));
         if (!seg) continue;
         rotated |= 1u << j;
-        EigSmemDF<NP> &s = df(j);
-        const int M = Ms[j];
-        for (int it = lane; it < HP * M; it += T) {
-          const int i = it / M, k = it % M;
-          if (!((seg >> i) & 1u)) continue;
-          const RotDF ro = s.rot[i];
-          const int2 pq = mats64[j].pq[i];
-          const float4 xp = s.a(pq.x, k), xq = s.a(pq.y, k);
-          s.a(pq.x, k) = cplx(dot3(ro.c, re_of(xp), neg(ro.sr), re_of(xq), ro.si, im_of(xq)),
-                              dot3(ro.c, im_of(xp), neg(ro.sr), im_of(xq), neg(ro.si), re_of(xq)));
-          s.a(pq.y, k) = cplx(dot3(ro.c, re_of(xq), ro.sr, re_of(xp), ro.si, im_of(xp)),
-                              dot3(ro.c, im_of(xq), ro.sr, im_of(xp), neg(ro.si), re_of(xp)));
+        EigSmem<NP> &s = mats[j];
+        const int M = Ms[j], m = (M + 1) >> 1;
+        const int na = (2 * m * (m + 1) + 31) >> 5, nv = (m * M + 31) >> 5;   // warp steps: blocks of A, V
+        const int wid = m + ((m & 1) ^ 1);   // the triangle of blocks a <= b, folded into rows of equal length
+        const float inv_w = __fdividef(1.f, (float)wid), inv_m = __fdividef(1.f, (float)M);
+        for (int st = wp; st < na + nv; st += W) {
+          if (st < na) {
+            const int blk = (st << 3) + (lane >> 2);
+            const int i = (int)(((float)blk + 0.5f) * inv_w), jj = blk - i * wid;
+            const bool head = jj < m - i;
+            const int a = head ? i : (m & 1 ? m - i : m - 1 - i);
+            const int b = head ? i + jj : a + jj - (m - i);
+            const bool in = blk < ((m * (m + 1)) >> 1);
+            const bool acta = in && ((seg >> a) & 1u), actb = in && ((seg >> b) & 1u);
+            const bool lo_row = (lane & 2) == 0, lo_col = (lane & 1) == 0;
+            int row = 0, col = 0;
+            El x{};
+            if (acta || actb) {
+              const int2 pa = s.pq[a], pb = s.pq[b];
+              row = lo_row ? pa.x : pa.y;
+              col = lo_col ? pb.x : pb.y;
+              x = Ar::a(s, row, col);
+              if (acta) {
+                const typename Ar::Ro ro = Ar::rot(s)[a];
+                x = Ar::mix(ro.c, lo_row ? Ar::neg(ro.sr) : ro.sr, ro.si, x, Ar::a(s, lo_row ? pa.y : pa.x, col));
+              }
+            }
+            const El y = shfl_xor1(x);   // the block's other column, same row
+            if (acta || actb) {
+              if (actb) {
+                const typename Ar::Ro ro = Ar::rot(s)[b];
+                x = Ar::mix(ro.c, lo_col ? Ar::neg(ro.sr) : ro.sr, Ar::neg(ro.si), x, y);
+              }
+              if (a == b) {              // the diagonal of a Hermitian matrix is real
+                if (lo_row == lo_col)
+                  x = Ar::real(x);
+                else if (Ar::kZeroes)
+                  x = El{};
+              } else {
+                Ar::a(s, col, row) = Ar::conj(x);
+              }
+              Ar::a(s, row, col) = x;
+            }
+          } else {
+            const int it = ((st - na) << 5) + lane;
+            const int i = (int)(((float)it + 0.5f) * inv_m), k = it - i * M;
+            if (i < m && ((seg >> i) & 1u)) {
+              const typename Ar::Ro ro = Ar::rot(s)[i];
+              const int2 pq = s.pq[i];
+              const El xp = Ar::v(s, k, pq.x), xq = Ar::v(s, k, pq.y);
+              Ar::v(s, k, pq.x) = Ar::mix(ro.c, Ar::neg(ro.sr), Ar::neg(ro.si), xp, xq);
+              Ar::v(s, k, pq.y) = Ar::mix(ro.c, ro.sr, Ar::neg(ro.si), xq, xp);
+            }
+          }
         }
-      }
-      g::sync();
-      // columns: A <- A J, V <- V J. new col p = c x_p - conj(sigma) x_q; new col q = sigma x_p + c x_q
-      for (int j = 0; j < G; ++j) {
-        const unsigned seg = (mask >> (j * HP)) & ((HP == 32) ? 0xffffffffu : ((1u << HP) - 1u));
-        if (!seg) continue;
-        EigSmemDF<NP> &s = df(j);
-        const int M = Ms[j];
-        for (int it = lane; it < HP * M; it += T) {
-          const int i = it / M, k = it % M;
-          if (!((seg >> i) & 1u)) continue;
-          const RotDF ro = s.rot[i];
-          const int2 pq = mats64[j].pq[i];
-          const float4 xp = s.a(k, pq.x), xq = s.a(k, pq.y);
-          s.a(k, pq.x) = cplx(dot3(ro.c, re_of(xp), neg(ro.sr), re_of(xq), neg(ro.si), im_of(xq)),
-                              dot3(ro.c, im_of(xp), neg(ro.sr), im_of(xq), ro.si, re_of(xq)));
-          s.a(k, pq.y) = cplx(dot3(ro.c, re_of(xq), ro.sr, re_of(xp), neg(ro.si), im_of(xp)),
-                              dot3(ro.c, im_of(xq), ro.sr, im_of(xp), ro.si, re_of(xp)));
-          const float4 vp = s.v(k, pq.x), vq = s.v(k, pq.y);
-          s.v(k, pq.x) = cplx(dot3(ro.c, re_of(vp), neg(ro.sr), re_of(vq), neg(ro.si), im_of(vq)),
-                              dot3(ro.c, im_of(vp), neg(ro.sr), im_of(vq), ro.si, re_of(vq)));
-          s.v(k, pq.y) = cplx(dot3(ro.c, re_of(vq), ro.sr, re_of(vp), neg(ro.si), im_of(vp)),
-                              dot3(ro.c, im_of(vq), ro.sr, im_of(vp), ro.si, re_of(vp)));
-        }
-      }
-      g::sync();
-      if (act) {   // the diagonal of a Hermitian matrix is real
-        EigSmemDF<NP> &s = df(lj);
-        const int2 pq = mats64[lj].pq[li];
-        s.a(pq.x, pq.x).z = s.a(pq.x, pq.x).w = 0.f;
-        s.a(pq.y, pq.y).z = s.a(pq.y, pq.y).w = 0.f;
       }
       g::sync();
     }
+    // matrices without a rotation in this sweep have converged
     for (int j = 0; j < G; ++j)
       if (((live >> j) & 1u) && !((rotated >> j) & 1u)) {
         res[j] = sweep;
@@ -471,29 +402,31 @@ __device__ void jacobi_group_df(EigSmem<NP> *mats64, const int *Ms, const double
   }
   for (int j = 0; j < G; ++j)
     if ((live >> j) & 1u) res[j] = -DOA_ENOCONV;
-  // double-float -> FP64 in place (same bytes per element; every element has one owner lane)
-  for (int j = 0; j < G; ++j) {
-    const int M = Ms[j];
-    if (M <= 0) continue;
-    EigSmemDF<NP> &s = df(j);
-    for (int e = lane; e < M * M; e += T) {
-      const int i = e / M, k = e % M;
-      const float4 a = s.a(i, k), v = s.v(i, k);
-      mats64[j].a(i, k) = make_double2((double)a.x + (double)a.y, (double)a.z + (double)a.w);
-      mats64[j].v(i, k) = make_double2((double)v.x + (double)v.y, (double)v.z + (double)v.w);
+  if constexpr (!Ar::kZeroes) {
+    // double-float -> FP64 in place (same bytes per element; every element has one owner lane)
+    for (int j = 0; j < G; ++j) {
+      const int M = Ms[j];
+      if (M <= 0) continue;
+      EigSmem<NP> &s = mats[j];
+      for (int e = tid; e < M * M; e += T) {
+        const int i = e / M, k = e % M;
+        const El a = Ar::a(s, i, k), v = Ar::v(s, i, k);
+        s.a(i, k) = make_double2((double)a.x + (double)a.y, (double)a.z + (double)a.w);
+        s.v(i, k) = make_double2((double)v.x + (double)v.y, (double)v.z + (double)v.w);
+      }
     }
+    g::sync();
   }
-  g::sync();
 }
 
 // ---- One matrix of 33 <= M <= 64 on a cluster of four CTAs (double-float) ----
-// The same rounds as jacobi_group_df with the rows of A and V spread over the cluster: CTA c owns
+// The same rounds as jacobi_group with the rows of A and V spread over the cluster: CTA c owns
 // rows 16c .. 16c+15 (one per warp). For a round's rotation J (n/2 disjoint pairs) the element
 // (i, col) of J^H A J needs only rows i and partner(i) at the columns of col's pair, so warp w
 // forms row i's new values pair by pair (lane j: columns p_j, q_j): first the row mix with the
 // partner row (read through distributed shared memory when another CTA owns it), then the column
-// mix, in the same double-float operations and order as the row and column passes of
-// jacobi_group_df; V's rows take the column mix in place. A is double-buffered, so one cluster
+// mix, in the double-float operations of jacobi_group (which computes half of A and mirrors it,
+// where here both halves are computed); V's rows take the column mix in place. A is double-buffered, so one cluster
 // barrier per round orders every CTA's reads of the current buffer before the writes that reuse
 // it. Warp 0 of every CTA forms the round's rotations from the same bytes with the same code, so
 // every CTA takes the same decisions (rounds to skip, sweeps, convergence) and meets the same
@@ -501,7 +434,7 @@ __device__ void jacobi_group_df(EigSmem<NP> *mats64, const int *Ms, const double
 constexpr int kClRanks = 4;                 // CTAs per matrix
 constexpr int kClRows = 64 / kClRanks;      // rows of A and V owned by a CTA (one per warp)
 constexpr int kClThreads = 32 * kClRows;
-static_assert(kClThreads == grp_threads<64>(), "the cluster's rank 0 runs the M <= 64 finishing code");
+static_assert(kClThreads == cta_threads<64>(), "the cluster's rank 0 runs the M <= 64 finishing code");
 
 struct ClusterDF {
   float4 A[2][kClRows][64];    // double-float (hi, lo) re, (hi, lo) im
@@ -660,9 +593,8 @@ __device__ int jacobi_cluster_df(ClusterDF &w, EigSmem<64> &fin, int M, const do
 }
 
 // Stable descending order of the eigenvalues (equal values keep index order).
-template <int NP>
+template <int NP, int T>
 __device__ void sort_desc(int M, EigSmem<NP> &s) {
-  constexpr int T = grp_threads<NP>();
   using g = Grp<T>;
   const int lane = g::id();
   for (int i = lane; i < M; i += T) s.lam()[i] = s.a(i, i).x;
@@ -681,9 +613,8 @@ __device__ void sort_desc(int M, EigSmem<NP> &s) {
 }
 
 // Writes B (column-major, ld M) of algorithm alg; returns 0 or a doa_status.
-template <int NP>
+template <int NP, int T>
 __device__ int build_factor(int M, int d, int alg, EigSmem<NP> &s, double2 *__restrict__ B) {
-  constexpr int T = grp_threads<NP>();
   using g = Grp<T>;
   const int lane = g::id();
   const int Kn = M - d;  // noise subspace dimension
@@ -742,9 +673,8 @@ __device__ int build_factor(int M, int d, int alg, EigSmem<NP> &s, double2 *__re
 // FP64 check that the noise eigenvectors are orthonormal: max |E_n^H E_n - I| <= kOrthoTol.
 constexpr double kOrthoTol = 1e-10;
 
-template <int NP>
+template <int NP, int T>
 __device__ bool noise_orthonormal(int M, int d, EigSmem<NP> &s) {
-  constexpr int T = grp_threads<NP>();
   using g = Grp<T>;
   const int lane = g::id();
   const int Kn = M - d;
@@ -770,9 +700,8 @@ __device__ bool noise_orthonormal(int M, int d, EigSmem<NP> &s) {
 // geometric means; +inf when one is not positive), MDL(k) = L + k(2M-k) log(N)/2, AIC(k) = 2L +
 // 2k(2M-k); out[0] = argmin MDL, out[1] = argmin AIC (the smaller k on a tie). The group's lanes
 // take one k each; the criterion values go to the A matrix's first row (no longer needed here).
-template <int NP>
+template <int NP, int T>
 __device__ void model_order(int M, int N, EigSmem<NP> &s, int32_t *out) {
-  constexpr int T = grp_threads<NP>();
   using g = Grp<T>;
   const int lane = g::id();
   const double logN = log((double)N);
@@ -812,16 +741,15 @@ __device__ void model_order(int M, int N, EigSmem<NP> &s, int32_t *out) {
 
 // Writes a batch problem's scan factor F (columns as laid out by the plan: E_n, or v_min; then
 // valph) and the EV weights w_c = 1 / lambda_{d+c}; returns 0 or a doa_status.
-template <int NP>
+template <int NP, int T>
 __device__ int build_scan_factor(const PlanProblem &pp, EigSmem<NP> &s, double2 *__restrict__ F,
                                  double *__restrict__ w) {
-  constexpr int T = grp_threads<NP>();
   using g = Grp<T>;
   const int lane = g::id();
   const int M = pp.p.M, d = pp.p.d;
   int st = 0;
   if (pp.Kn > 0) {
-    build_factor<NP>(M, d, DOA_MUSIC, s, F);
+    build_factor<NP, T>(M, d, DOA_MUSIC, s, F);
     if (pp.slot[DOA_EV] >= 0) {
       bool bad = false;
       for (int c = lane; c < pp.Kn; c += T) {
@@ -832,10 +760,10 @@ __device__ int build_scan_factor(const PlanProblem &pp, EigSmem<NP> &s, double2 
       if (g::any(bad)) st = DOA_ERANK;
     }
   } else if (pp.kphd >= 0) {
-    build_factor<NP>(M, d, DOA_PHD, s, F + (size_t)pp.kphd * M);
+    build_factor<NP, T>(M, d, DOA_PHD, s, F + (size_t)pp.kphd * M);
   }
   if (pp.kmn >= 0) {
-    const int e = build_factor<NP>(M, d, DOA_MN, s, F + (size_t)pp.kmn * M);
+    const int e = build_factor<NP, T>(M, d, DOA_MN, s, F + (size_t)pp.kmn * M);
     if (e && !st) st = e;
   }
   return st;
@@ -843,17 +771,16 @@ __device__ int build_scan_factor(const PlanProblem &pp, EigSmem<NP> &s, double2 
 
 // The eigenvalues, B and the status of a single call from a finished decomposition (res: the
 // sweep count, or minus a doa_status).
-template <int NP>
+template <int NP, int T>
 __device__ void finish_single(int M, int d, int alg, EigSmem<NP> &s, int res, double *evals, double2 *B, int *K_out,
                               int *info) {
-  constexpr int T = grp_threads<NP>();
   const int lane = Grp<T>::id();
   int st = 0;
   if (res > 0) {
-    sort_desc<NP>(M, s);
+    sort_desc<NP, T>(M, s);
     if (evals)
       for (int i = lane; i < M; i += T) evals[i] = s.lam()[s.order()[i]];
-    st = build_factor<NP>(M, d, alg, s, B);
+    st = build_factor<NP, T>(M, d, alg, s, B);
   } else {
     st = -res;
   }
@@ -864,23 +791,19 @@ __device__ void finish_single(int M, int d, int alg, EigSmem<NP> &s, int res, do
 }
 
 template <int NP, bool kDF>
-__global__ void __launch_bounds__(grp_threads<NP>()) eig_single_kernel(const double2 *R64, int M, int d, int alg, double *evals,
+using Arith = std::conditional_t<kDF, ArithDF<NP>, ArithF64<NP>>;
+
+template <int NP, bool kDF>
+__global__ void __launch_bounds__(cta_threads<NP>()) eig_single_kernel(const double2 *R64, int M, int d, int alg, double *evals,
                                                        double2 *B, int *K_out, int *info) {
   extern __shared__ __align__(16) uint8_t smem[];
-  constexpr int G = mats_per_warp<NP>();
+  constexpr int T = cta_threads<NP>();
   EigSmem<NP> *mats = reinterpret_cast<EigSmem<NP> *>(smem);
-  int Ms[G];
-  const double2 *Rs[G];
-  int res[G];
-  for (int j = 0; j < G; ++j) {
-    Ms[j] = j == 0 ? M : 0;
-    Rs[j] = R64;
-  }
-  if (kDF)
-    jacobi_group_df<NP, G>(mats, Ms, Rs, res);
-  else
-    jacobi_group<NP, G>(mats, Ms, Rs, res);
-  finish_single<NP>(M, d, alg, mats[0], res[0], evals, B, K_out, info);
+  const int Ms[1] = {M};
+  const double2 *Rs[1] = {R64};
+  int res[1];
+  jacobi_group<Arith<NP, kDF>, NP, 1, T>(mats, Ms, Rs, res);
+  finish_single<NP, T>(M, d, alg, mats[0], res[0], evals, B, K_out, info);
 }
 
 // Single call, 33 <= M <= 64, double-float: one four-CTA cluster; rank 0 finishes.
@@ -892,16 +815,15 @@ __global__ void __cluster_dims__(kClRanks, 1, 1) __launch_bounds__(kClThreads, 1
   ClusterDF &w = *reinterpret_cast<ClusterDF *>(smem + kClFinBytes);
   const int res = jacobi_cluster_df(w, s, M, R64);
   if (cg::this_cluster().block_rank() != 0) return;
-  finish_single<64>(M, d, alg, s, res, evals, B, K_out, info);
+  finish_single<64, kClThreads>(M, d, alg, s, res, evals, B, K_out, info);
 }
 
 // A batch problem's outputs from its finished decomposition (res: the sweep count, or minus a
 // doa_status): evals, the scan factor and EV weights, the optional B, order estimates and
 // proposal features, and the status.
-template <int NP>
+template <int NP, int T>
 __device__ void finish_batch(const PlanProblem &pp, const PlanJob *jobs, EigSmem<NP> &s, int res, uint8_t *ws,
                              int *status) {
-  constexpr int T = grp_threads<NP>();
   const int lane = Grp<T>::id();
   const int M = pp.p.M, d = pp.p.d;
   int st = 0;
@@ -922,15 +844,15 @@ __device__ void finish_batch(const PlanProblem &pp, const PlanJob *jobs, EigSmem
   double2 *F = reinterpret_cast<double2 *>(ws + pp.fac_off);
   double *w = reinterpret_cast<double *>(F + (size_t)M * (M + 1));
   if (res > 0) {
-    sort_desc<NP>(M, s);
+    sort_desc<NP, T>(M, s);
     if (pp.p.evals)
       for (int i = lane; i < M; i += T) pp.p.evals[i] = s.lam()[s.order()[i]];
-    st = build_scan_factor<NP>(pp, s, F, w);
-    if (!noise_orthonormal<NP>(M, d, s) && !st) st = DOA_ENOCONV;
-    if (pp.p.B_out) build_factor<NP>(M, d, jobs[pp.first_job].alg, s, reinterpret_cast<double2 *>(pp.p.B_out));
+    st = build_scan_factor<NP, T>(pp, s, F, w);
+    if (!noise_orthonormal<NP, T>(M, d, s) && !st) st = DOA_ENOCONV;
+    if (pp.p.B_out) build_factor<NP, T>(M, d, jobs[pp.first_job].alg, s, reinterpret_cast<double2 *>(pp.p.B_out));
     if (pp.p.order_est) {
       Grp<T>::sync();
-      model_order<NP>(M, pp.p.N, s, pp.p.order_est);
+      model_order<NP, T>(M, pp.p.N, s, pp.p.order_est);
     }
   } else {
     st = -res;
@@ -946,11 +868,10 @@ template <int NP, int G>
 __global__ void __launch_bounds__(32 * eig_warps<NP>(), eig_min_ctas<NP>()) eig_batch_kernel(const uint8_t *plan, uint8_t *ws, int bucket,
                                                                          int *status) {
   extern __shared__ __align__(16) uint8_t smem[];
-  constexpr int T = grp_threads<NP>();
-  const int grp = threadIdx.x / T, lane = Grp<T>::id();
+  const int grp = threadIdx.x / 32;
   EigSmem<NP> *mats = reinterpret_cast<EigSmem<NP> *>(smem) + grp * G;
   const PlanHeader *h = reinterpret_cast<const PlanHeader *>(plan);
-  const int base = (blockIdx.x * (int)(blockDim.x / T) + grp) * G;
+  const int base = (blockIdx.x * (int)(blockDim.x / 32) + grp) * G;
   const int count = h->eig_count[bucket];
   if (base >= count) return;
   const int32_t *list = reinterpret_cast<const int32_t *>(plan + h->off_eig[bucket]);
@@ -966,13 +887,34 @@ __global__ void __launch_bounds__(32 * eig_warps<NP>(), eig_min_ctas<NP>()) eig_
   bool fp64 = false;   // a group runs FP64 when any of its problems asks for it
   for (int j = 0; j < G; ++j) fp64 = fp64 || (prob[j] >= 0 && probs[prob[j]].p.eig_prec == DOA_EIG_FP64);
   if (fp64)
-    jacobi_group<NP, G>(mats, Ms, Rs, res);
+    jacobi_group<ArithF64<NP>, NP, G, 32>(mats, Ms, Rs, res);
   else
-    jacobi_group_df<NP, G>(mats, Ms, Rs, res);
+    jacobi_group<ArithDF<NP>, NP, G, 32>(mats, Ms, Rs, res);
   for (int j = 0; j < G; ++j) {
     if (prob[j] < 0) continue;
-    finish_batch<NP>(probs[prob[j]], jobs, mats[j], res[j], ws, status + prob[j]);
+    finish_batch<NP, 32>(probs[prob[j]], jobs, mats[j], res[j], ws, status + prob[j]);
   }
+}
+
+// The CTA form of the batch: a CTA per matrix.
+template <int NP>
+__global__ void __launch_bounds__(cta_threads<NP>()) eig_batch_cta_kernel(const uint8_t *plan, uint8_t *ws, int bucket,
+                                                                          int *status) {
+  extern __shared__ __align__(16) uint8_t smem[];
+  constexpr int T = cta_threads<NP>();
+  EigSmem<NP> &s = *reinterpret_cast<EigSmem<NP> *>(smem);
+  const PlanHeader *h = reinterpret_cast<const PlanHeader *>(plan);
+  const int prob = reinterpret_cast<const int32_t *>(plan + h->off_eig[bucket])[blockIdx.x];
+  const PlanProblem &pp = reinterpret_cast<const PlanProblem *>(plan + h->off_prob)[prob];
+  const PlanJob *jobs = reinterpret_cast<const PlanJob *>(plan + h->off_job);
+  const int Ms[1] = {pp.p.M};
+  const double2 *Rs[1] = {reinterpret_cast<const double2 *>(ws + pp.r64_off)};
+  int res[1];
+  if (pp.p.eig_prec == DOA_EIG_FP64)
+    jacobi_group<ArithF64<NP>, NP, 1, T>(&s, Ms, Rs, res);
+  else
+    jacobi_group<ArithDF<NP>, NP, 1, T>(&s, Ms, Rs, res);
+  finish_batch<NP, T>(pp, jobs, s, res[0], ws, status + prob);
 }
 
 // Bucket M <= 64 of the batch in double-float: one four-CTA cluster per problem; rank 0 finishes.
@@ -997,23 +939,23 @@ __global__ void __cluster_dims__(kClRanks, 1, 1) __launch_bounds__(kClThreads, 1
     if (!rank0) return;
     int Ms[1] = {pp.p.M}, r1[1];
     const double2 *Rs[1] = {R};
-    jacobi_group<64, 1>(&s, Ms, Rs, r1);
+    jacobi_group<ArithF64<64>, 64, 1, kClThreads>(&s, Ms, Rs, r1);
     res = r1[0];
   } else {
     res = jacobi_cluster_df(w, s, pp.p.M, R);
     if (!rank0) return;
   }
-  finish_batch<64>(pp, jobs, s, res, ws, status + prob);
+  finish_batch<64, kClThreads>(pp, jobs, s, res, ws, status + prob);
 }
 
 
 template <int NP, bool kDF>
 cudaError_t run_single_p(const double2 *R64, int M, int d, int alg, double *evals, double2 *B, int *K_out,
                          int *info, cudaStream_t st) {
-  const int smem = (int)sizeof(EigSmem<NP>) * mats_per_warp<NP>();
+  const int smem = (int)sizeof(EigSmem<NP>);
   cudaError_t e = ensure_smem_attr((const void *)eig_single_kernel<NP, kDF>, smem);
   if (e != cudaSuccess) return e;
-  eig_single_kernel<NP, kDF><<<1, grp_threads<NP>(), smem, st>>>(R64, M, d, alg, evals, B, K_out, info);
+  eig_single_kernel<NP, kDF><<<1, cta_threads<NP>(), smem, st>>>(R64, M, d, alg, evals, B, K_out, info);
   return cudaGetLastError();
 }
 
@@ -1041,7 +983,6 @@ cudaError_t run_single(const double2 *R64, int M, int d, int alg, int prec, doub
 // 4096-matrix batch then runs in one wave instead of 1.12.
 template <int NP, int G>
 int eig_cta_warps() {
-  if (NP > 32) return 1;
   const SmemLimits lim = device_smem_limits();
   const int per_mat = (int)sizeof(EigSmem<NP>);
   int best = 1, best_res = -1;
@@ -1059,8 +1000,8 @@ int eig_cta_warps() {
 
 template <int NP, int G>
 cudaError_t run_batch_g(const uint8_t *plan, int count, uint8_t *ws, int *status, int bucket, cudaStream_t st) {
-  const int W = NP <= 32 ? eig_cta_warps<NP, G>() : eig_warps<NP>();
-  const int per_cta = (NP <= 32 ? W : 1) * G;
+  const int W = eig_cta_warps<NP, G>();
+  const int per_cta = W * G;
   const int smem = (int)sizeof(EigSmem<NP>) * per_cta;
   cudaError_t e = ensure_smem_attr(reinterpret_cast<const void *>(eig_batch_kernel<NP, G>), smem);
   if (e != cudaSuccess) return e;
@@ -1068,16 +1009,28 @@ cudaError_t run_batch_g(const uint8_t *plan, int count, uint8_t *ws, int *status
   return cudaGetLastError();
 }
 
-// Matrices per warp from the plan (G in {1, 2, 4, 8} up to the bucket's maximum).
+template <int NP>
+cudaError_t run_batch_cta(const uint8_t *plan, int count, uint8_t *ws, int *status, int bucket, cudaStream_t st) {
+  if (count == 0) return cudaSuccess;
+  const int smem = (int)sizeof(EigSmem<NP>);
+  cudaError_t e = ensure_smem_attr(reinterpret_cast<const void *>(eig_batch_cta_kernel<NP>), smem);
+  if (e != cudaSuccess) return e;
+  eig_batch_cta_kernel<NP><<<(unsigned)count, cta_threads<NP>(), smem, st>>>(plan, ws, bucket, status);
+  return cudaGetLastError();
+}
+
+// M <= 16: the CTA form for small batches unless the plan packs matrices (G in {1, 2, 4, 8} up to the
+// bucket's maximum per warp), else the warp form.
 template <int NP>
 cudaError_t run_batch(const uint8_t *plan, const PlanHeader &h, uint8_t *ws, int *status, int bucket,
                       cudaStream_t st) {
   const int count = h.eig_count[bucket];
-  if (count == 0) return cudaSuccess;
   const int g = h.eig_mats[bucket];
+  if (g == 1 && count <= eig_cta_limit<NP>()) return run_batch_cta<NP>(plan, count, ws, status, bucket, st);
+  if (count == 0) return cudaSuccess;
   if (g >= 8 && mats_per_warp<NP>() >= 8) return run_batch_g<NP, (mats_per_warp<NP>() >= 8 ? 8 : 1)>(plan, count, ws, status, bucket, st);
-  if (g >= 4 && mats_per_warp<NP>() >= 4) return run_batch_g<NP, (mats_per_warp<NP>() >= 4 ? 4 : 1)>(plan, count, ws, status, bucket, st);
-  if (g >= 2 && mats_per_warp<NP>() >= 2) return run_batch_g<NP, (mats_per_warp<NP>() >= 2 ? 2 : 1)>(plan, count, ws, status, bucket, st);
+  if (g >= 4) return run_batch_g<NP, 4>(plan, count, ws, status, bucket, st);
+  if (g >= 2) return run_batch_g<NP, 2>(plan, count, ws, status, bucket, st);
   return run_batch_g<NP, 1>(plan, count, ws, status, bucket, st);
 }
 
@@ -1152,7 +1105,7 @@ cudaError_t launch_eig_batch(const uint8_t *plan_dev, const PlanHeader &h, uint8
   cudaError_t e;
   if ((e = run_batch<8>(plan_dev, h, ws, status, 0, s)) != cudaSuccess) return e;
   if ((e = run_batch<16>(plan_dev, h, ws, status, 1, s)) != cudaSuccess) return e;
-  if ((e = run_batch<32>(plan_dev, h, ws, status, 2, s)) != cudaSuccess) return e;
+  if ((e = run_batch_cta<32>(plan_dev, h.eig_count[2], ws, status, 2, s)) != cudaSuccess) return e;
   return run_batch_cluster(plan_dev, h, ws, status, 3, s);
 }
 

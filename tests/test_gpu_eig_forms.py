@@ -1,0 +1,65 @@
+"""The Jacobi's CTA form against its warp form and the oracle, at the sizes where the block folding and the
+padding of odd M can go wrong."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_2007_14135_gb300 import synth
+from tests.gpu_common import require_gpu
+
+pytestmark = pytest.mark.gpu
+
+
+def _solve(torch, doa, insts, prec, eig_mats):
+    outs, probs = [], []
+    for inst in insts:
+        X = torch.from_numpy(inst.X).cuda()
+        P = torch.empty(inst.L, dtype=torch.float32, device="cuda")
+        idx = torch.full((max(inst.d, 1),), -1, dtype=torch.int32, device="cuda")
+        val = torch.zeros(max(inst.d, 1), dtype=torch.float32, device="cuda")
+        cnt = torch.zeros(1, dtype=torch.int32, device="cuda")
+        ev = torch.zeros(inst.M, dtype=torch.float64, device="cuda")
+        B = torch.zeros(inst.M * inst.M, dtype=torch.complex128, device="cuda")
+        probs.append(doa.make_problem(X, inst.d, 1 << doa.MUSIC, doa.grid(inst.lo, inst.step, inst.L), P, idx, val, cnt,
+                                      evals=ev, B_out=B, eig_prec=prec))
+        outs.append((X, P, ev, B, idx, val, cnt))
+    plan = doa.BatchPlan(probs, eig_mats=eig_mats)
+    status = torch.full((len(insts),), -1, dtype=torch.int32, device="cuda")
+    doa.doa_solve_batch(plan, doa.workspace(plan), status)
+    torch.cuda.synchronize()
+    assert status.cpu().numpy().tolist() == [0] * len(insts)
+    return [(o[1].cpu().numpy(), o[2].cpu().numpy(), o[3].cpu().numpy()) for o in outs]
+
+
+@pytest.mark.parametrize("prec", [0, 1])
+def test_cta_and_warp_forms_agree_bit_for_bit(prec):
+    """The same plan with a matrix per CTA (default for a small batch) and with packed warps."""
+    torch, doa = require_gpu()
+    insts = [synth.custom(M, max(1, M // 4), 200, None, 10.0, 1.0, seed=700 + M) for M in (2, 3, 5, 7, 8, 9, 11, 15, 16)]
+    cta = _solve(torch, doa, insts, prec, [1, 1, 1, 1])
+    warp = _solve(torch, doa, insts, prec, [2, 2, 1, 1])
+    for a, b in zip(cta, warp):
+        for x, y in zip(a, b):
+            assert np.array_equal(x, y)
+
+
+@pytest.mark.parametrize("M", [2, 3, 5, 9, 13, 16, 17, 31, 32, 33, 63, 64])
+@pytest.mark.parametrize("prec", [0, 1])
+def test_single_calls_at_odd_sizes(M, prec):
+    """Eigenvalues and C = B B^H of a single call against the oracle: 1e-12 of the largest in FP64; in
+    double-float (2^-48 arithmetic, threshold 1e-12) 1e-10."""
+    torch, doa = require_gpu()
+    d = max(1, M // 4)
+    R = oracle.covariance(synth.custom(M, d, 4 * M + 50, None, 10.0, 1.0, seed=800 + M).X)
+    ev = torch.empty(M, dtype=torch.float64, device="cuda")
+    B = torch.zeros(M * M, dtype=torch.complex128, device="cuda")
+    info = torch.zeros(1, dtype=torch.int32, device="cuda")
+    doa.doa_noise_subspace_prec(torch.from_numpy(R).cuda(), d, doa.MUSIC, prec, B, info, evals=ev)
+    torch.cuda.synchronize()
+    assert info.item() > 0
+    w, V = np.linalg.eigh(R)
+    tol = 1e-12 if prec == doa.EIG_FP64 else 1e-10
+    assert np.abs(ev.cpu().numpy() - w[::-1]).max() <= tol * w[-1]
+    F = B.cpu().numpy()[:(M - d) * M].reshape(M - d, M).T
+    E = V[:, :M - d]
+    assert np.abs(F @ F.conj().T - E @ E.conj().T).max() <= 100 * tol
