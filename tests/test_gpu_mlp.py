@@ -121,3 +121,48 @@ def test_training_reduces_loss_and_checkpoint_roundtrip(env, tmp_path):
     net2.forward(Xd[:B], net2.workspace(B), probs=p2)
     torch.cuda.synchronize()
     assert torch.equal(p1, p2) and net2.t == net.t
+
+
+@pytest.mark.parametrize("B", [8, 120, 128, 136, 19464])
+def test_forward_tiles_and_alignment(env, B):
+    """Ragged last tiles, more tiles than SMs, and features and outputs off the 16-byte boundary (one float):
+    the same results bit for bit as aligned ones, and within the oracle test's bounds."""
+    torch, doa = env
+    net = doa.Mlp(seed=15)
+    rng = np.random.default_rng(B)
+    X, _ = _batch(rng, B)
+    ws = net.workspace(B)
+    got = []
+    for off in (0, 1):
+        buf = torch.zeros(B * 272 + 1, dtype=torch.float32, device="cuda")
+        x = buf[off:off + B * 272].view(B, 272)
+        x.copy_(torch.from_numpy(X))
+        outs = [torch.full((B * 181 + 1,), -7.0, dtype=torch.float32, device="cuda") for _ in range(2)]
+        views = [o[off:off + B * 181].view(B, 181) for o in outs]
+        net.forward(x, ws, probs=views[0], logits=views[1])
+        torch.cuda.synchronize()
+        for o in outs:      # the float beside the output is untouched
+            assert o[B * 181 if off == 0 else 0].item() == -7.0
+        got.append([v.cpu().numpy() for v in views])
+    assert np.array_equal(got[0][0], got[1][0]) and np.array_equal(got[0][1], got[1][1])
+    z_ref, _ = mlp_oracle.forward(_rounded_params(torch, net), _bf16(torch, X))
+    cos, rel = _cos_rel(got[0][1], z_ref)
+    assert cos > 0.9999 and rel < 2e-2, (cos, rel)
+
+
+@pytest.mark.parametrize("B", [8, 136, 5632, 5640, 19592])
+def test_gradients_split_and_tiles(env, B):
+    """Both sides of the batch split of the weight gradients, ragged tiles, more tiles than SMs."""
+    torch, doa = env
+    net = doa.Mlp(seed=16)
+    rng = np.random.default_rng(B + 1)
+    X, Y = _batch(rng, B)
+    loss = torch.zeros(1, dtype=torch.float32, device="cuda")
+    net.backward(torch.from_numpy(X).cuda(), torch.from_numpy(Y).cuda(), net.workspace(B), loss=loss)
+    torch.cuda.synchronize()
+    l_ref, g_ref = mlp_oracle.loss_and_grads(_rounded_params(torch, net), _bf16(torch, X), Y.astype(np.float64))
+    assert abs(loss.item() - l_ref) < 1e-2 * abs(l_ref)
+    for l in range(4):
+        for key, ref in (("gW", g_ref[l][0]), ("gb", g_ref[l][1])):
+            cos, rel = _cos_rel(net.buf[key][l].cpu().numpy(), ref)
+            assert cos > 0.999 and rel < 5e-2, (key, l, cos, rel)
