@@ -16,7 +16,10 @@
 // nothing. A round updates A block by block: the 2 x 2 block of the rows of pair a and the columns of
 // pair b >= a takes four lanes, one element each -- the row mix A <- J^H A of the lane's element,
 // exchanged with the lane of the other column, then the column mix A <- A J -- and is written to its
-// mirror image as well, so only half of A is computed; V <- V J takes a lane per pair and row.
+// mirror image as well, so only half of A is computed; V <- V J takes a lane per pair and row. Matrices
+// of M <= 8 (where half the blocks take as many warp steps as all of them) and those whose eigenvectors
+// go into a 2-D refinement compute both halves: where a minimum of the planar array's spectrum meets its
+// mirror image at the array plane, the refined angle moves by the square root of a rounding error.
 //
 // Two shapes, with the same arithmetic and results. A warp per matrix (or G packed matrices, every
 // lane owning one pair's rotation) keeps the most matrices resident and suits large batches of M <= 16.
@@ -261,9 +264,9 @@ __device__ __forceinline__ float4 shfl_xor1(float4 x) {
 
 // Runs Jacobi on the G matrices of a group of T threads (matrix j has size Ms[j] <= NP, 0 = unused),
 // all loaded from Rs[j] (upper triangle). T = 32: a warp; otherwise the whole CTA on one matrix.
-// res[j] receives sweeps (> 0) or -status; on return A (its diagonal) and V hold FP64.
+// both[j]: compute both halves of A (always at M <= 8). res[j] receives sweeps (> 0) or -status; on return A (its diagonal) and V hold FP64.
 template <class Ar, int NP, int G, int T>
-__device__ void jacobi_group(EigSmem<NP> *mats, const int *Ms, const double2 *const *Rs, int *res) {
+__device__ void jacobi_group(EigSmem<NP> *mats, const int *Ms, const double2 *const *Rs, const bool *both, int *res) {
   static_assert(T == 32 || G == 1, "a CTA works on one matrix");
   constexpr int HP = NP / 2, W = T / 32;
   using g = Grp<T>;
@@ -337,17 +340,18 @@ __device__ void jacobi_group(EigSmem<NP> *mats, const int *Ms, const double2 *co
         rotated |= 1u << j;
         EigSmem<NP> &s = mats[j];
         const int M = Ms[j], m = (M + 1) >> 1;
-        const int na = (2 * m * (m + 1) + 31) >> 5, nv = (m * M + 31) >> 5;   // warp steps: blocks of A, V
-        const int wid = m + ((m & 1) ^ 1);   // the triangle of blocks a <= b, folded into rows of equal length
+        const bool full = NP <= 8 || both[j];
+        const int na = ((full ? 4 * m * m : 2 * m * (m + 1)) + 31) >> 5, nv = (m * M + 31) >> 5;   // warp steps: blocks of A, V
+        const int wid = full ? m : m + ((m & 1) ^ 1);   // the square of blocks, or the triangle of blocks a <= b, folded into rows of equal length
         const float inv_w = __fdividef(1.f, (float)wid), inv_m = __fdividef(1.f, (float)M);
         for (int st = wp; st < na + nv; st += W) {
           if (st < na) {
             const int blk = (st << 3) + (lane >> 2);
             const int i = (int)(((float)blk + 0.5f) * inv_w), jj = blk - i * wid;
-            const bool head = jj < m - i;
+            const bool head = full || jj < m - i;
             const int a = head ? i : (m & 1 ? m - i : m - 1 - i);
-            const int b = head ? i + jj : a + jj - (m - i);
-            const bool in = blk < ((m * (m + 1)) >> 1);
+            const int b = full ? jj : (head ? i + jj : a + jj - (m - i));
+            const bool in = blk < (full ? m * m : (m * (m + 1)) >> 1);
             const bool acta = in && ((seg >> a) & 1u), actb = in && ((seg >> b) & 1u);
             const bool lo_row = (lane & 2) == 0, lo_col = (lane & 1) == 0;
             int row = 0, col = 0;
@@ -373,7 +377,7 @@ __device__ void jacobi_group(EigSmem<NP> *mats, const int *Ms, const double2 *co
                   x = Ar::real(x);
                 else if (Ar::kZeroes)
                   x = El{};
-              } else {
+              } else if (!full) {
                 Ar::a(s, col, row) = Ar::conj(x);
               }
               Ar::a(s, row, col) = x;
@@ -801,8 +805,9 @@ __global__ void __launch_bounds__(cta_threads<NP>()) eig_single_kernel(const dou
   EigSmem<NP> *mats = reinterpret_cast<EigSmem<NP> *>(smem);
   const int Ms[1] = {M};
   const double2 *Rs[1] = {R64};
+  const bool both[1] = {false};
   int res[1];
-  jacobi_group<Arith<NP, kDF>, NP, 1, T>(mats, Ms, Rs, res);
+  jacobi_group<Arith<NP, kDF>, NP, 1, T>(mats, Ms, Rs, both, res);
   finish_single<NP, T>(M, d, alg, mats[0], res[0], evals, B, K_out, info);
 }
 
@@ -864,6 +869,8 @@ __device__ void finish_batch(const PlanProblem &pp, const PlanJob *jobs, EigSmem
   Grp<T>::sync();
 }
 
+__device__ __forceinline__ bool refines_2d(const doa_problem &p) { return p.geom.pos && p.peak_angle; }
+
 template <int NP, int G>
 __global__ void __launch_bounds__(32 * eig_warps<NP>(), eig_min_ctas<NP>()) eig_batch_kernel(const uint8_t *plan, uint8_t *ws, int bucket,
                                                                          int *status) {
@@ -885,11 +892,13 @@ __global__ void __launch_bounds__(32 * eig_warps<NP>(), eig_min_ctas<NP>()) eig_
     Rs[j] = prob[j] >= 0 ? reinterpret_cast<const double2 *>(ws + probs[prob[j]].r64_off) : nullptr;
   }
   bool fp64 = false;   // a group runs FP64 when any of its problems asks for it
+  bool both[G];
+  for (int j = 0; j < G; ++j) both[j] = prob[j] >= 0 && refines_2d(probs[prob[j]].p);
   for (int j = 0; j < G; ++j) fp64 = fp64 || (prob[j] >= 0 && probs[prob[j]].p.eig_prec == DOA_EIG_FP64);
   if (fp64)
-    jacobi_group<ArithF64<NP>, NP, G, 32>(mats, Ms, Rs, res);
+    jacobi_group<ArithF64<NP>, NP, G, 32>(mats, Ms, Rs, both, res);
   else
-    jacobi_group<ArithDF<NP>, NP, G, 32>(mats, Ms, Rs, res);
+    jacobi_group<ArithDF<NP>, NP, G, 32>(mats, Ms, Rs, both, res);
   for (int j = 0; j < G; ++j) {
     if (prob[j] < 0) continue;
     finish_batch<NP, 32>(probs[prob[j]], jobs, mats[j], res[j], ws, status + prob[j]);
@@ -909,11 +918,12 @@ __global__ void __launch_bounds__(cta_threads<NP>()) eig_batch_cta_kernel(const 
   const PlanJob *jobs = reinterpret_cast<const PlanJob *>(plan + h->off_job);
   const int Ms[1] = {pp.p.M};
   const double2 *Rs[1] = {reinterpret_cast<const double2 *>(ws + pp.r64_off)};
+  const bool both[1] = {refines_2d(pp.p)};
   int res[1];
   if (pp.p.eig_prec == DOA_EIG_FP64)
-    jacobi_group<ArithF64<NP>, NP, 1, T>(&s, Ms, Rs, res);
+    jacobi_group<ArithF64<NP>, NP, 1, T>(&s, Ms, Rs, both, res);
   else
-    jacobi_group<ArithDF<NP>, NP, 1, T>(&s, Ms, Rs, res);
+    jacobi_group<ArithDF<NP>, NP, 1, T>(&s, Ms, Rs, both, res);
   finish_batch<NP, T>(pp, jobs, s, res[0], ws, status + prob);
 }
 
@@ -939,7 +949,8 @@ __global__ void __cluster_dims__(kClRanks, 1, 1) __launch_bounds__(kClThreads, 1
     if (!rank0) return;
     int Ms[1] = {pp.p.M}, r1[1];
     const double2 *Rs[1] = {R};
-    jacobi_group<ArithF64<64>, 64, 1, kClThreads>(&s, Ms, Rs, r1);
+    const bool both[1] = {refines_2d(pp.p)};
+    jacobi_group<ArithF64<64>, 64, 1, kClThreads>(&s, Ms, Rs, both, r1);
     res = r1[0];
   } else {
     res = jacobi_cluster_df(w, s, pp.p.M, R);
