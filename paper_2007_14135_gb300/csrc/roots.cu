@@ -14,8 +14,16 @@
 // Horner evaluation,
 // 8 n eps sum_t |a_t| |z|^t (clustered roots -- the pairs z, 1/conj(z) near the circle -- cannot be
 // resolved further). A converged root keeps its value and takes no further correction; the
-// iteration ends when all have converged, 400 iterations at most (else DOA_ENOCONV). One warp per
-// (problem, algorithm) job: lanes own coefficients, then roots; the selection runs on lane 0.
+// iteration ends when all have converged, 400 iterations at most (else DOA_ENOCONV). Outside the unit
+// circle p is evaluated as z^n q(1/z) with the reversed coefficients, so powers never overflow: with
+// plain Horner a root beyond 20 or so (a small leading coefficient) put infinities into the FP32 phase,
+// which then ran to its cap and left the FP64 phase to start from the circle.
+// One warp per (problem, algorithm) job: lanes own coefficients, then roots, then selected roots.
+//
+// Bound by FP64 issue (an FP64 warp instruction holds its sub-partition for 64 cycles), so the FP64
+// iteration keeps only the two Horner recurrences in FP64 -- the repulsion sum and the rounding bound
+// steer the step and its stop, and FP32 serves them -- and the selection works in parallel lanes.
+// Measured (2048 jobs of degree 30): 5.1 -> 0.58 ms.
 #include <math_constants.h>
 
 #include "doa_internal.cuh"
@@ -25,21 +33,21 @@ namespace {
 
 constexpr int kRootWarps = 4;
 constexpr int kMaxDeg = 2 * kMaxM - 2;
+constexpr int kRootsPerLane = (kMaxDeg + 31) / 32;
 constexpr int kRootMaxIter = 400;
+constexpr int kRootMaxIterF = 64;    // FP32 phase
 
 struct RootShared {
   float2 af[kMaxDeg + 1];   // the coefficients rounded to FP32 (first phase)
-  float amf[kMaxDeg + 1];
-  float2 zf[kMaxDeg];
-  float2 wf[kMaxDeg];
+  float amf[kMaxDeg + 1];   // |a_t| (for the rounding bound of the Horner evaluation)
+  float2 zf[kMaxDeg];       // FP32 roots; in the second phase the FP64 roots' leading parts
+  float2 wf[kMaxDeg];       // FP32 corrections; in the second phase the FP64 roots' remainders
   double2 a[kMaxDeg + 1];   // polynomial coefficients, a[t] multiplies z^t
-  double am[kMaxDeg + 1];   // |a_t| (for the rounding bound of the Horner evaluation)
   double2 z[kMaxDeg];       // current roots
   double2 w[kMaxDeg];       // corrections of this iteration
   int conv[kMaxDeg];        // root converged (its correction is no longer computed)
 };
 
-__device__ __forceinline__ double2 cadd(double2 a, double2 b) { return make_double2(a.x + b.x, a.y + b.y); }
 __device__ __forceinline__ float2 fcmul(float2 a, float2 b) {
   return make_float2(fmaf(a.x, b.x, -a.y * b.y), fmaf(a.x, b.y, a.y * b.x));
 }
@@ -79,16 +87,17 @@ __device__ __forceinline__ double root_weight(const RootJob &j, int c) {
 __device__ int root_music_warp(const RootJob &j, RootShared &sh, double *out) {
   const int lane = threadIdx.x & 31;
   const int M = j.M, n = 2 * M - 2;
-  // coefficients: a[t] = c_{t - (M-1)}
-  for (int t = lane; t <= n; t += 32) {
-    const int l = t - (M - 1);
+  // coefficients: a[t] = c_{t - (M-1)}, c_{-l} = conj(c_l); lanes pair up on an l >= 0, each taking every
+  // other column
+  for (int l0 = 0; l0 < M; l0 += 16) {
+    const int l = l0 + (lane >> 1);
     double cr = 0.0, ci = 0.0;
-    for (int c = 0; c < j.Kf; ++c) {
+    for (int c = lane & 1; c < j.Kf && l < M; c += 2) {
       const double wc = root_weight(j, c);
       if (wc == 0.0) continue;
       const double2 *f = j.F + (size_t)c * M;
       double sr = 0.0, si = 0.0;
-      for (int q = max(0, -l); q < M && q + l < M; ++q) {   // f_q conj(f_{q+l})
+      for (int q = 0; q + l < M; ++q) {   // f_q conj(f_{q+l})
         const double2 x = f[q], y = f[q + l];
         sr = fma(x.x, y.x, fma(x.y, y.y, sr));
         si = fma(x.y, y.x, fma(-x.x, y.y, si));
@@ -96,10 +105,15 @@ __device__ int root_music_warp(const RootJob &j, RootShared &sh, double *out) {
       cr = fma(wc, sr, cr);
       ci = fma(wc, si, ci);
     }
-    sh.a[t] = make_double2(cr, ci);
-    sh.am[t] = sqrt(cr * cr + ci * ci);
-    sh.af[t] = make_float2((float)cr, (float)ci);
-    sh.amf[t] = (float)sh.am[t];
+    cr += __shfl_xor_sync(0xffffffffu, cr, 1);
+    ci += __shfl_xor_sync(0xffffffffu, ci, 1);
+    if (l < M && (l > 0 || (lane & 1) == 0)) {   // the even lane writes c_l, the odd one c_{-l}
+      const int t = (lane & 1) ? M - 1 - l : M - 1 + l;
+      const double im = (lane & 1) ? -ci : (l == 0 ? 0.0 : ci);
+      sh.a[t] = make_double2(cr, im);
+      sh.af[t] = make_float2((float)cr, (float)im);
+      sh.amf[t] = (float)sqrt(cr * cr + ci * ci);
+    }
   }
   for (int i = lane; i < n; i += 32) {
     float s, c;
@@ -115,24 +129,32 @@ __device__ int root_music_warp(const RootJob &j, RootShared &sh, double *out) {
   // first phase, FP32 (the FP64 rate is 1/73 of FP32 here): corrections down to 1e-6 |z| or the
   // FP32 rounding bound of p(z); the FP64 phase then polishes the same roots
   if (usable) {
-    for (int it = 0; it < kRootMaxIter; ++it) {
+    for (int it = 0; it < kRootMaxIterF; ++it) {
       bool small = true;
       for (int i = lane; i < n; i += 32) {
         if (sh.conv[i]) continue;
         const float2 zi = sh.zf[i];
-        const float zm = sqrtf(fmaf(zi.x, zi.x, zi.y * zi.y));
-        float2 p = sh.af[n], dp = make_float2(0.f, 0.f);
-        float pe = sh.amf[n];
-        for (int t = n - 1; t >= 0; --t) {
-          dp = fcadd(fcmul(dp, zi), p);
-          p = fcadd(fcmul(p, zi), sh.af[t]);
-          pe = fmaf(pe, zm, sh.amf[t]);
+        const float zm2 = fmaf(zi.x, zi.x, zi.y * zi.y), zm = sqrtf(zm2);
+        const bool outer = zm2 > 1.f;               // evaluate q(x) = x^n p(1/x) at x = 1/z
+        const float2 x = outer ? fcdiv(make_float2(1.f, 0.f), zi) : zi;
+        const float xm = outer ? 1.f / zm : zm;
+        int t = outer ? 0 : n;
+        const int dt = outer ? 1 : -1;
+        float2 p = sh.af[t], dp = make_float2(0.f, 0.f);
+        float pe = sh.amf[t];
+        for (int k = 0; k < n; ++k) {
+          t += dt;
+          dp = fcadd(fcmul(dp, x), p);
+          p = fcadd(fcmul(p, x), sh.af[t]);
+          pe = fmaf(pe, xm, sh.amf[t]);
         }
         float2 rep = make_float2(0.f, 0.f);
         for (int k = 0; k < n; ++k) {
           if (k == i) continue;
           rep = fcadd(rep, fcdiv(make_float2(1.f, 0.f), fcsub(zi, sh.zf[k])));
         }
+        // Newton ratio p / p': outside it is q / (x (n q - x q'))
+        if (outer) dp = fcmul(x, fcsub(make_float2(n * p.x, n * p.y), fcmul(x, dp)));
         const float2 ratio = fcdiv(p, dp);
         const float2 wi = fcdiv(ratio, fcsub(make_float2(1.f, 0.f), fcmul(ratio, rep)));
         sh.wf[i] = wi;
@@ -160,7 +182,9 @@ __device__ int root_music_warp(const RootJob &j, RootShared &sh, double *out) {
       double s, c;
       sincos(2.0 * CUDART_PI * (double)i / (double)n + 0.4, &s, &c);
       sh.z[i] = make_double2(c, s);
+      sh.zf[i] = make_float2((float)c, (float)s);
     }
+    sh.wf[i] = make_float2((float)(sh.z[i].x - (double)sh.zf[i].x), (float)(sh.z[i].y - (double)sh.zf[i].y));
     sh.w[i] = make_double2(0.0, 0.0);
     sh.conv[i] = 0;
   }
@@ -171,32 +195,46 @@ __device__ int root_music_warp(const RootJob &j, RootShared &sh, double *out) {
       for (int i = lane; i < n; i += 32) {
         if (sh.conv[i]) continue;                    // converged: no more correction
         const double2 zi = sh.z[i];
-        const double zm = sqrt(zi.x * zi.x + zi.y * zi.y);
-        double2 p = sh.a[n], dp = make_double2(0.0, 0.0);
-        double pe = sh.am[n];
-        for (int t = n - 1; t >= 0; --t) {          // Horner for p, p' and the bound sum |a_t| |z|^t
-          dp = cadd(cmul(dp, zi), p);
-          p = cadd(cmul(p, zi), sh.a[t]);
-          pe = fma(pe, zm, sh.am[t]);
+        const float2 zh = sh.zf[i], zl = sh.wf[i];
+        const float zm = hypotf(zh.x, zh.y);
+        const bool outer = zm > 1.f;
+        const double2 x = outer ? crcp(zi) : zi;
+        const float xm = outer ? 1.f / zm : zm;
+        int t = outer ? 0 : n;
+        const int dt = outer ? 1 : -1;
+        double2 p = sh.a[t], dp = make_double2(0.0, 0.0);
+        float pe = sh.amf[t];
+        for (int k = 0; k < n; ++k) {                // Horner for p, p' and the bound sum |a_t| |x|^t
+          t += dt;
+          const double2 at = sh.a[t];
+          dp = make_double2(fma(dp.x, x.x, fma(-dp.y, x.y, p.x)), fma(dp.x, x.y, fma(dp.y, x.x, p.y)));
+          p = make_double2(fma(p.x, x.x, fma(-p.y, x.y, at.x)), fma(p.x, x.y, fma(p.y, x.x, at.y)));
+          pe = fmaf(pe, xm, sh.amf[t]);
         }
-        double2 rep = make_double2(0.0, 0.0);       // sum_{k != i} 1 / (z_i - z_k)
+        float2 rep = make_float2(0.f, 0.f);          // sum_{k != i} 1 / (z_i - z_k)
         for (int k = 0; k < n; ++k) {
           if (k == i) continue;
-          rep = cadd(rep, crcp(csub(zi, sh.z[k])));
+          const float2 kh = sh.zf[k], kl = sh.wf[k];
+          const float2 d = make_float2((zh.x - kh.x) + (zl.x - kl.x), (zh.y - kh.y) + (zl.y - kl.y));
+          rep = fcadd(rep, fcdiv(make_float2(1.f, 0.f), d));
         }
+        if (outer) dp = cmul(x, csub(make_double2(n * p.x, n * p.y), cmul(x, dp)));
         const double2 ratio = cdiv(p, dp);
-        const double2 den = csub(make_double2(1.0, 0.0), cmul(ratio, rep));
+        const double2 den = csub(make_double2(1.0, 0.0), cmul(ratio, make_double2((double)rep.x, (double)rep.y)));
         const double2 wi = cdiv(ratio, den);
         sh.w[i] = wi;
         const double mag = sqrt(wi.x * wi.x + wi.y * wi.y);
         const double res = sqrt(p.x * p.x + p.y * p.y);
-        const bool ok = isfinite(mag) && (mag <= 1e-14 * fmax(1.0, zm) || res <= 8.0 * n * 1.1102230246251565e-16 * pe);
+        const bool ok = isfinite(mag) && (mag <= 1e-14 * (double)fmaxf(1.f, zm) || res <= 8.0 * n * 1.1102230246251565e-16 * (double)pe);
         small = small && ok;
         if (ok) sh.conv[i] = 1;
       }
       __syncwarp();
       for (int i = lane; i < n; i += 32) {
-        sh.z[i] = csub(sh.z[i], sh.w[i]);
+        const double2 z = csub(sh.z[i], sh.w[i]);
+        sh.z[i] = z;
+        sh.zf[i] = make_float2((float)z.x, (float)z.y);
+        sh.wf[i] = make_float2((float)(z.x - (double)sh.zf[i].x), (float)(z.y - (double)sh.zf[i].y));
         sh.w[i] = make_double2(0.0, 0.0);
       }
       __syncwarp();
@@ -206,44 +244,63 @@ __device__ int root_music_warp(const RootJob &j, RootShared &sh, double *out) {
       }
     }
   }
-  if (lane == 0) {
-    // the d roots with |z| <= 1 of largest modulus (lower index on a tie), then angles ascending
-    double sel[kMaxM];
-    int ns = 0;
-    if (st == 0) {
-      int taken[kMaxM];
-      for (int q = 0; q < j.d; ++q) {
-        int best = -1;
-        double bm = -1.0;
-        for (int i = 0; i < n; ++i) {
-          const double2 zi = sh.z[i];
-          const double m = sqrt(zi.x * zi.x + zi.y * zi.y);
-          if (!(m <= 1.0) || !(m > bm)) continue;
-          bool used = false;
-          for (int r = 0; r < ns; ++r) used = used || taken[r] == i;
-          if (used) continue;
-          best = i;
-          bm = m;
-        }
-        if (best < 0) break;
-        taken[ns] = best;
-        const double2 zb = sh.z[best];
-        const double sx = fmin(fmax(atan2(zb.y, zb.x) / CUDART_PI, -1.0), 1.0);
-        sel[ns++] = asin(sx) * (180.0 / CUDART_PI);
-      }
-      for (int a = 1; a < ns; ++a) {
-        const double v = sel[a];
-        int b = a - 1;
-        while (b >= 0 && sel[b] > v) {
-          sel[b + 1] = sel[b];
-          --b;
-        }
-        sel[b + 1] = v;
-      }
-      if (ns < j.d) st = DOA_ENOCONV;
+  // the d roots with |z| <= 1 of largest modulus (lower index on a tie): d rounds of an arg-max over the
+  // lanes' roots, moduli compared by their bits (all are >= 0)
+  long long m[kRootsPerLane];
+#pragma unroll
+  for (int k = 0; k < kRootsPerLane; ++k) {
+    const int i = lane + 32 * k;
+    m[k] = -1;
+    if (i < n) {
+      const double2 zi = sh.z[i];
+      const double r = sqrt(zi.x * zi.x + zi.y * zi.y);
+      if (r <= 1.0) m[k] = __double_as_longlong(r);
     }
-    for (int q = 0; q < j.d; ++q) out[q] = q < ns ? sel[q] : CUDART_NAN;
   }
+  int ns = 0;
+  int *taken = sh.conv;                     // root indices of the selection (the flags are done with)
+  __syncwarp();
+  for (int q = 0; q < j.d && st == 0; ++q) {
+    long long best = -1;
+    int bi = 1 << 30;
+#pragma unroll
+    for (int k = 0; k < kRootsPerLane; ++k)
+      if (m[k] > best) {
+        best = m[k];
+        bi = lane + 32 * k;
+      }
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) {
+      const long long ob = __shfl_xor_sync(0xffffffffu, best, off);
+      const int oi = __shfl_xor_sync(0xffffffffu, bi, off);
+      if (ob > best || (ob == best && oi < bi)) {
+        best = ob;
+        bi = oi;
+      }
+    }
+    if (best < 0) break;
+#pragma unroll
+    for (int k = 0; k < kRootsPerLane; ++k)
+      if (bi == lane + 32 * k) m[k] = -1;
+    if (lane == 0) taken[q] = bi;
+    ns = q + 1;
+  }
+  __syncwarp();
+  double *sel = reinterpret_cast<double *>(sh.w);
+  for (int q = lane; q < ns; q += 32) {
+    const double2 zb = sh.z[taken[q]];
+    const double sx = fmin(fmax(atan2(zb.y, zb.x) / CUDART_PI, -1.0), 1.0);
+    sel[q] = asin(sx) * (180.0 / CUDART_PI);
+  }
+  __syncwarp();
+  for (int q = lane; q < ns; q += 32) {     // ascending: every angle goes to its rank
+    const double v = sel[q];
+    int rank = 0;
+    for (int k = 0; k < ns; ++k) rank += sel[k] < v || (sel[k] == v && k < q);
+    out[rank] = v;
+  }
+  for (int q = ns + lane; q < j.d; q += 32) out[q] = CUDART_NAN;
+  if (ns < j.d) st = DOA_ENOCONV;
   __syncwarp();
   return st;
 }

@@ -77,3 +77,23 @@ def test_root_music_one_noise_vector(env, M, d):
     assert info.item() == 0
     want, _ = oracle.root_music(Bf @ Bf.conj().T, d)
     np.testing.assert_allclose(th.cpu().numpy(), want, rtol=0, atol=1e-6)
+
+
+@pytest.mark.parametrize("lead", [1e-2, 1e-6, 1e-10])
+def test_root_music_with_far_roots(env, lead):
+    """A factor whose last element is tiny: the polynomial's leading coefficient is small and its outer
+    roots are far outside the circle, where powers of z overflow FP32. Angles within 1e-6 degree of the
+    oracle, as in the tests above."""
+    torch, doa = env
+    M, d = 16, 2
+    inst = synth.custom(M - 1, d, 4096, None, 15.0, 1.0, seed=990)
+    ev, V, _ = oracle.eigh(oracle.covariance(inst.X))
+    v = factor_from_decomposition(ev, V, d, MN)[:, 0]
+    b = np.concatenate([v, [lead * abs(v[0])]]).astype(np.complex128)
+    th = torch.full((d,), -99.0, dtype=torch.float64, device="cuda")
+    info = torch.full((1,), 7, dtype=torch.int32, device="cuda")
+    doa.doa_root_music(torch.from_numpy(b).cuda(), M, 1, d, th, info)
+    torch.cuda.synchronize()
+    assert info.item() == 0
+    want, _ = oracle.root_music(np.outer(b, b.conj()), d)
+    np.testing.assert_allclose(th.cpu().numpy(), want, rtol=0, atol=1e-6)
