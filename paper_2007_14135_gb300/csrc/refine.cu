@@ -21,14 +21,25 @@
 // half-width, halved up to 40 times until den does not increase; stop below a 1e-13 rad move, when
 // no halving decreases den, or after 60 steps.
 //
-// One warp per (problem, algorithm) job: lanes own elements for the steering vector and its
-// derivatives (shared memory), then factor columns for the contractions, and a shuffle reduction
-// gives every lane the same den, gradient and Hessian, so all lanes take the same decisions.
+// One warp per peak, the warps of a CTA on one job's peaks (its factor staged in shared memory). Bound by
+// FP64 issue: an FP64 warp instruction holds its sub-partition for 64 cycles whatever the number of active
+// lanes, so what counts is the number of instructions, not of lanes. Lanes own elements for the steering
+// vector and its derivatives (shared memory), then one real recurrence each for the contractions (a
+// column's real or imaginary part of one derivative: 2 M multiply-adds instead of a column's 12 M), then
+// columns; sums run over as many lanes as there are columns, several quantities side by side, and every
+// lane gets the same den, gradient and Hessian, so all lanes take the same decisions. A line search
+// evaluates 32 / W step lengths at once (W = 8 or 16 lanes each, or the whole warp for larger arrays) and
+// takes the first that does not increase den. All of it adds in the order of a column per lane and a
+// butterfly over the lanes.
 // In the batch the iteration starts from the vertex of the parabola through the FP32 spectrum's
 // 1/P at the peak and its neighbours (per axis in 2-D), which leaves Newton one or two steps; the
 // local minimiser it converges to does not depend on the start.
+// Measured (2048 ULA jobs of four peaks and 512 circular-array jobs of two): 7.5 -> 2.3 ms, of which about
+// 2 ms is one peak's 60 steps with some twenty halvings each; the 2-D jobs therefore start first.
 #include <float.h>
 #include <math_constants.h>
+
+#include <algorithm>
 
 #include "doa_internal.cuh"
 
@@ -64,9 +75,12 @@ __device__ __forceinline__ double vertex_offset(float pa, float pb, float pc) {
   return fmin(fmax(0.5 * (da - dc) / curv, -0.9), 0.9);
 }
 
+constexpr int kChainCols = 32;   // columns up to which a lane takes one real recurrence
 struct RefShared {
   double2 v[6][kMaxM];   // a and its derivatives (1-D: a, a', a''; 2-D: a, a_t, a_p, a_tt, a_tp, a_pp)
+  double y[12][kChainCols + 1];   // F^H v: real and imaginary parts per column
 };
+constexpr int kStageM = 16;      // factors up to this M are staged in shared memory
 
 __device__ __forceinline__ double2 cmul_j(double s, double2 a) {   // (j s) a
   return make_double2(-s * a.y, s * a.x);
@@ -82,10 +96,57 @@ __device__ __forceinline__ double col_weight(const RefineJob &j, int c) {
   }
 }
 
-__device__ __forceinline__ double warp_sum(double v) {
+// Sum over groups of W lanes (a butterfly; W = 32: the warp).
+template <int W>
+__device__ __forceinline__ double group_sum(double v) {
 #pragma unroll
-  for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+  for (int off = W / 2; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
   return v;
+}
+// Three sums over the lanes of columns (zero in the other lanes): side by side in lane groups when the
+// columns fit in 8 or 16 lanes.
+__device__ __forceinline__ void sum3(int Kf, double &a, double &b, double &c) {
+  const int lane = threadIdx.x & 31;
+  if (Kf <= 8) {
+    const double tb = __shfl_sync(0xffffffffu, b, lane & 7), tc = __shfl_sync(0xffffffffu, c, lane & 7);
+    const double s = group_sum<8>(lane < 8 ? a : (lane < 16 ? tb : tc));
+    a = __shfl_sync(0xffffffffu, s, 0);
+    b = __shfl_sync(0xffffffffu, s, 8);
+    c = __shfl_sync(0xffffffffu, s, 16);
+  } else if (Kf <= 16) {
+    const double tb = __shfl_sync(0xffffffffu, b, lane & 15);
+    const double s = group_sum<16>(lane < 16 ? a : tb);
+    a = __shfl_sync(0xffffffffu, s, 0);
+    b = __shfl_sync(0xffffffffu, s, 16);
+    c = __shfl_sync(0xffffffffu, group_sum<16>(c), 0);
+  } else {
+    a = group_sum<32>(a);
+    b = group_sum<32>(b);
+    c = group_sum<32>(c);
+  }
+}
+__device__ __forceinline__ double flip(bool f, double x) {
+  return __hiloint2double(__double2hiint(x) ^ (f ? (int)0x80000000 : 0), __double2loint(x));
+}
+// Real (im = 0) or imaginary (im = 1) part of conj(f)^T v.
+__device__ __forceinline__ double chain(const double2 *f, const double2 *v, int M, bool im) {
+  double r = 0.0;
+#pragma unroll 4
+  for (int m = 0; m < M; ++m) {
+    const double2 b = f[m], a = v[m];
+    r = fma(b.x, im ? a.y : a.x, fma(flip(im, b.y), im ? a.x : a.y, r));
+  }
+  return r;
+}
+// y[2 k + im][c] = part im of conj(f_c)^T v[k] for nv vectors, a recurrence per lane.
+__device__ __forceinline__ void contract(const RefineJob &j, int nv, RefShared &sh) {
+  const int n = 2 * nv * j.Kf;
+  const float inv = __fdividef(1.f, (float)j.Kf);
+  for (int e = threadIdx.x & 31; e < n; e += 32) {
+    const int k = (int)(((float)e + 0.5f) * inv), c = e - k * j.Kf;
+    sh.y[k][c] = chain(j.F + (size_t)c * j.M, sh.v[k >> 1], j.M, (k & 1) != 0);
+  }
+  __syncwarp();
 }
 
 // conj(f_c)^T v for lane-owned column c (v in shared memory).
@@ -118,18 +179,30 @@ __device__ void ula_eval(const RefineJob &j, double th, RefShared &sh, double &f
   }
   __syncwarp();
   double pf = 0.0, p1 = 0.0, p2 = 0.0;
+  const bool chains = j.Kf <= kChainCols;
+  if (chains) contract(j, 3, sh);
   for (int col = lane; col < j.Kf; col += 32) {
     const double wc = col_weight(j, col);
     if (wc == 0.0) continue;
-    const double2 y = col_dot(j, col, sh.v[0]), y1 = col_dot(j, col, sh.v[1]), y2 = col_dot(j, col, sh.v[2]);
+    double2 y, y1, y2;
+    if (chains) {
+      y = make_double2(sh.y[0][col], sh.y[1][col]);
+      y1 = make_double2(sh.y[2][col], sh.y[3][col]);
+      y2 = make_double2(sh.y[4][col], sh.y[5][col]);
+    } else {
+      y = col_dot(j, col, sh.v[0]);
+      y1 = col_dot(j, col, sh.v[1]);
+      y2 = col_dot(j, col, sh.v[2]);
+    }
     pf += wc * (y.x * y.x + y.y * y.y);
     p1 += 2.0 * wc * (y.x * y1.x + y.y * y1.y);
     p2 += 2.0 * wc * ((y.x * y2.x + y.y * y2.y) + (y1.x * y1.x + y1.y * y1.y));
   }
   __syncwarp();
-  f = warp_sum(pf);
-  f1 = warp_sum(p1);
-  f2 = warp_sum(p2);
+  f = pf;
+  f1 = p1;
+  f2 = p2;
+  sum3(j.Kf, f, f1, f2);
 }
 
 __device__ double refine_ula_warp(const RefineJob &j, int k, RefShared &sh) {
@@ -156,69 +229,150 @@ __device__ double refine_ula_warp(const RefineJob &j, int k, RefShared &sh) {
 }
 
 // ---- geometry -------------------------------------------------------------------------------
-// den and (when deriv) its gradient and Hessian (H[0] = tt, H[1] = tp, H[2] = pp) at (th, ph).
-__device__ double geo_eval(const RefineJob &j, double th, double ph, bool deriv, RefShared &sh, double *g,
-                           double *H) {
-  const int lane = threadIdx.x & 31;
+// sin and cos of both angles at once: even lanes take th, odd lanes ph.
+struct Trig {
   double st, ct, sp, cp;
-  sincos(th, &st, &ct);
-  sincos(ph, &sp, &cp);
-  const double u0 = st * sp, u1 = ct * sp, u2 = cp;
-  const double tp2 = 2.0 * kPi;
-  for (int m = lane; m < j.M; m += 32) {
+};
+__device__ __forceinline__ Trig trig(double th, double ph) {
+  const int lane = threadIdx.x & 31;
+  double s, c;
+  sincos((lane & 1) ? ph : th, &s, &c);
+  const double so = __shfl_xor_sync(0xffffffffu, s, 1), co = __shfl_xor_sync(0xffffffffu, c, 1);
+  return (lane & 1) ? Trig{so, co, s, c} : Trig{s, c, so, co};
+}
+__device__ __forceinline__ double2 geo_phasor(double t) {
+  const double fr = t - rint(t);
+  return phasor_q64((uint64_t)__double2ll_rn(fr * 4611686018427387904.0) << 2);
+}
+
+// den at one point per group of W lanes (every lane of a group passes the same point; Kf <= W or W = 32).
+template <int W>
+__device__ double geo_den(const RefineJob &j, double th, double ph, RefShared &sh) {
+  const int lane = threadIdx.x & 31, gl = lane & (W - 1);
+  const Trig g = trig(th, ph);
+  const double u0 = g.st * g.sp, u1 = g.ct * g.sp, u2 = g.cp;
+  double2 *a = sh.v[0] + (W == 32 ? 0 : (lane & ~(W - 1)));
+  for (int m = gl; m < j.M; m += W) {
     const double px = j.pos[3 * m] - j.cx, py = j.pos[3 * m + 1] - j.cy, pz = j.pos[3 * m + 2] - j.cz;
-    const double t = px * u0 + py * u1 + pz * u2;
-    const double fr = t - rint(t);
-    const double2 a = phasor_q64((uint64_t)__double2ll_rn(fr * 4611686018427387904.0) << 2);
-    sh.v[0][m] = a;
-    if (deriv) {
-      const double t_t = px * (ct * sp) + py * (-st * sp);
-      const double t_p = px * (st * cp) + py * (ct * cp) + pz * (-sp);
-      const double t_tt = px * (-st * sp) + py * (-ct * sp);
-      const double t_tp = px * (ct * cp) + py * (-st * cp);
-      const double t_pp = px * (-st * sp) + py * (-ct * sp) + pz * (-cp);
-      sh.v[1][m] = cmul_j(tp2 * t_t, a);
-      sh.v[2][m] = cmul_j(tp2 * t_p, a);
-      double2 q = cmul_j(tp2 * t_tt, a);
-      double r = tp2 * tp2 * t_t * t_t;
-      sh.v[3][m] = make_double2(q.x - r * a.x, q.y - r * a.y);
-      q = cmul_j(tp2 * t_tp, a);
-      r = tp2 * tp2 * t_t * t_p;
-      sh.v[4][m] = make_double2(q.x - r * a.x, q.y - r * a.y);
-      q = cmul_j(tp2 * t_pp, a);
-      r = tp2 * tp2 * t_p * t_p;
-      sh.v[5][m] = make_double2(q.x - r * a.x, q.y - r * a.y);
+    a[m] = geo_phasor(px * u0 + py * u1 + pz * u2);
+  }
+  __syncwarp();
+  double pf = 0.0;
+  if (W < 32) {
+    // the group's recurrences: column gl's real part, then its imaginary part on the lanes left over
+    double *y = sh.y[0] + (lane / W) * 2 * W;   // rows of y taken as one array: 32 / W x 2 W <= 64 values
+    for (int e = gl; e < 2 * j.Kf; e += W) {
+      const bool im = e >= j.Kf;
+      const int c = im ? e - j.Kf : e;
+      y[(im ? W : 0) + c] = chain(j.F + (size_t)c * j.M, a, j.M, im);
+    }
+    __syncwarp();
+    if (gl < j.Kf) {
+      const double wc = col_weight(j, gl);
+      if (wc != 0.0) {
+        const double2 z = make_double2(y[gl], y[W + gl]);
+        pf += wc * (z.x * z.x + z.y * z.y);
+      }
+    }
+  } else {
+    for (int col = lane; col < j.Kf; col += 32) {
+      const double wc = col_weight(j, col);
+      if (wc == 0.0) continue;
+      const double2 y = col_dot(j, col, a);
+      pf += wc * (y.x * y.x + y.y * y.y);
     }
   }
   __syncwarp();
+  return group_sum<W>(pf);
+}
+
+// den, its gradient and Hessian (H[0] = tt, H[1] = tp, H[2] = pp) at (th, ph). With M, Kf <= W the lane
+// groups share the element derivatives (each group takes every 32 / W-th of them).
+template <int W>
+__device__ double geo_eval(const RefineJob &j, double th, double ph, RefShared &sh, double *g, double *H) {
+  const int lane = threadIdx.x & 31, gl = lane & (W - 1), grp = lane / W;
+  constexpr int G = 32 / W;
+  const Trig tr = trig(th, ph);
+  const double st = tr.st, ct = tr.ct, sp = tr.sp, cp = tr.cp;
+  const double u0 = st * sp, u1 = ct * sp, u2 = cp;
+  const double tp2 = 2.0 * kPi;
+  for (int m = gl; m < j.M; m += W) {
+    const double px = j.pos[3 * m] - j.cx, py = j.pos[3 * m + 1] - j.cy, pz = j.pos[3 * m + 2] - j.cz;
+    const double2 a = geo_phasor(px * u0 + py * u1 + pz * u2);
+    if (grp == 0) sh.v[0][m] = a;
+    const double t_t = px * (ct * sp) + py * (-st * sp);
+    const double t_p = px * (st * cp) + py * (ct * cp) + pz * (-sp);
+    for (int k = grp; k < 2; k += G) sh.v[1 + k][m] = cmul_j(tp2 * (k == 0 ? t_t : t_p), a);
+    for (int k = grp; k < 3; k += G) {   // tt, tp, pp
+      const double A = k == 1 ? ct * cp : -st * sp, B = k == 1 ? -st * cp : -ct * sp, C = k == 2 ? -cp : 0.0;
+      const double2 q = cmul_j(tp2 * (px * A + py * B + pz * C), a);
+      const double r = tp2 * tp2 * (k == 2 ? t_p : t_t) * (k == 0 ? t_t : t_p);
+      sh.v[3 + k][m] = make_double2(q.x - r * a.x, q.y - r * a.y);
+    }
+  }
+  __syncwarp();
+  if (W < 32) {   // Kf <= W: groups take every G-th of the first- and second-order sums
+    contract(j, 6, sh);
+    const double wc = gl < j.Kf ? col_weight(j, gl) : 0.0;
+    const bool on = gl < j.Kf && wc != 0.0;
+    const double2 y = on ? make_double2(sh.y[0][gl], sh.y[1][gl]) : make_double2(0.0, 0.0);
+    double r1[3], r2[3];
+    for (int k = grp; k < 3; k += G) {
+      // k = 0, 1, 2: den, g_t, g_p and H_tt, H_tp, H_pp
+      double s1 = 0.0, s2 = 0.0;
+      if (on) {
+        const double2 z = k == 0 ? y : make_double2(sh.y[2 * k][gl], sh.y[2 * k + 1][gl]);
+        s1 = (k == 0 ? wc : 2.0 * wc) * (y.x * z.x + y.y * z.y);
+        const double2 z2 = make_double2(sh.y[6 + 2 * k][gl], sh.y[7 + 2 * k][gl]);
+        const int ia = k == 2 ? 4 : 2, ib = k == 0 ? 2 : 4;
+        const double2 za = make_double2(sh.y[ia][gl], sh.y[ia + 1][gl]), zb = make_double2(sh.y[ib][gl], sh.y[ib + 1][gl]);
+        s2 = 2.0 * wc * ((y.x * z2.x + y.y * z2.y) + (za.x * zb.x + za.y * zb.y));
+      }
+      r1[k / G] = s1;
+      r2[k / G] = s2;
+    }
+    double o1[3], o2[3];
+#pragma unroll
+    for (int k = 0; k < 3; k += G) {
+      const double s1 = group_sum<W>(k + grp < 3 ? r1[k / G] : 0.0), s2 = group_sum<W>(k + grp < 3 ? r2[k / G] : 0.0);
+#pragma unroll
+      for (int i = 0; i < G && k + i < 3; ++i) {
+        o1[k + i] = __shfl_sync(0xffffffffu, s1, i * W);
+        o2[k + i] = __shfl_sync(0xffffffffu, s2, i * W);
+      }
+    }
+    g[0] = o1[1];
+    g[1] = o1[2];
+    H[0] = o2[0];
+    H[1] = o2[1];
+    H[2] = o2[2];
+    __syncwarp();
+    return o1[0];
+  }
   double pf = 0.0, pg0 = 0.0, pg1 = 0.0, ph0 = 0.0, ph1 = 0.0, ph2 = 0.0;
   for (int col = lane; col < j.Kf; col += 32) {
     const double wc = col_weight(j, col);
     if (wc == 0.0) continue;
     const double2 y = col_dot(j, col, sh.v[0]);
     pf += wc * (y.x * y.x + y.y * y.y);
-    if (deriv) {
-      const double2 yt = col_dot(j, col, sh.v[1]), yp = col_dot(j, col, sh.v[2]);
-      const double2 ytt = col_dot(j, col, sh.v[3]), ytp = col_dot(j, col, sh.v[4]), ypp = col_dot(j, col, sh.v[5]);
-      pg0 += 2.0 * wc * (y.x * yt.x + y.y * yt.y);
-      pg1 += 2.0 * wc * (y.x * yp.x + y.y * yp.y);
-      ph0 += 2.0 * wc * ((y.x * ytt.x + y.y * ytt.y) + (yt.x * yt.x + yt.y * yt.y));
-      ph1 += 2.0 * wc * ((y.x * ytp.x + y.y * ytp.y) + (yt.x * yp.x + yt.y * yp.y));
-      ph2 += 2.0 * wc * ((y.x * ypp.x + y.y * ypp.y) + (yp.x * yp.x + yp.y * yp.y));
-    }
+    const double2 yt = col_dot(j, col, sh.v[1]), yp = col_dot(j, col, sh.v[2]);
+    const double2 ytt = col_dot(j, col, sh.v[3]), ytp = col_dot(j, col, sh.v[4]), ypp = col_dot(j, col, sh.v[5]);
+    pg0 += 2.0 * wc * (y.x * yt.x + y.y * yt.y);
+    pg1 += 2.0 * wc * (y.x * yp.x + y.y * yp.y);
+    ph0 += 2.0 * wc * ((y.x * ytt.x + y.y * ytt.y) + (yt.x * yt.x + yt.y * yt.y));
+    ph1 += 2.0 * wc * ((y.x * ytp.x + y.y * ytp.y) + (yt.x * yp.x + yt.y * yp.y));
+    ph2 += 2.0 * wc * ((y.x * ypp.x + y.y * ypp.y) + (yp.x * yp.x + yp.y * yp.y));
   }
   __syncwarp();
-  const double f = warp_sum(pf);
-  if (deriv) {
-    g[0] = warp_sum(pg0);
-    g[1] = warp_sum(pg1);
-    H[0] = warp_sum(ph0);
-    H[1] = warp_sum(ph1);
-    H[2] = warp_sum(ph2);
-  }
-  return f;
+  g[0] = group_sum<32>(pg0);
+  g[1] = group_sum<32>(pg1);
+  H[0] = group_sum<32>(ph0);
+  H[1] = group_sum<32>(ph1);
+  H[2] = group_sum<32>(ph2);
+  return group_sum<32>(pf);
 }
 
+template <int W>
 __device__ void refine_geo_warp(const RefineJob &j, int flat, RefShared &sh, double *out) {
   const int l = flat / j.La, k = flat - l * j.La;
   double x0 = __dmul_rn(__dadd_rn(j.az_lo, __dmul_rn((double)k, j.az_step)), kD2R);
@@ -233,12 +387,15 @@ __device__ void refine_geo_warp(const RefineJob &j, int flat, RefShared &sh, dou
     if (l > 0 && l + 1 < j.Le)
       x1 += vertex_offset(j.P[(size_t)(l - 1) * j.La + k], pc, j.P[(size_t)(l + 1) * j.La + k]) * j.el_step * kD2R;
   }
+  double g[2], H[3], f = 0.0;
+  bool have = false;   // f, g, H belong to (x0, x1) already
   for (int it = 0; it < kRefMaxIter; ++it) {
-    double g[2], H[3];
-    const double f = geo_eval(j, x0, x1, true, sh, g, H);
+    if (!have) f = geo_eval<W>(j, x0, x1, sh, g, H);
+    have = false;
     const double det = H[0] * H[2] - H[1] * H[1];
+    const bool newton = H[0] > 0.0 && det > 0.0;
     double d0, d1;
-    if (H[0] > 0.0 && det > 0.0) {
+    if (newton) {
       d0 = -(H[2] * g[0] - H[1] * g[1]) / det;
       d1 = -(H[0] * g[1] - H[1] * g[0]) / det;
       if (fmax(fabs(d0), fabs(d1)) < 1e-6) {
@@ -255,16 +412,36 @@ __device__ void refine_geo_warp(const RefineJob &j, int flat, RefShared &sh, dou
       d0 = gn > 0.0 ? -g[0] / gn * wdt : 0.0;
       d1 = gn > 0.0 ? -g[1] / gn * wdt : 0.0;
     }
-    double t = 1.0, n0 = x0, n1 = x1;
+    double n0 = x0, n1 = x1;
     bool accepted = false;
-    for (int h = 0; h <= 40; ++h) {
-      n0 = fmin(fmax(x0 + t * d0, bl0), bh0);
-      n1 = fmin(fmax(x1 + t * d1, bl1), bh1);
-      if (geo_eval(j, n0, n1, false, sh, nullptr, nullptr) <= f) {
-        accepted = true;
-        break;
+    if (newton) {   // the whole step is usually taken: its derivatives come with it
+      n0 = fmin(fmax(x0 + d0, bl0), bh0);
+      n1 = fmin(fmax(x1 + d1, bl1), bh1);
+      double gn[2], Hn[3];
+      const double fn = geo_eval<W>(j, n0, n1, sh, gn, Hn);
+      if (fn <= f) {
+        accepted = have = true;
+        f = fn;
+        g[0] = gn[0];
+        g[1] = gn[1];
+        H[0] = Hn[0];
+        H[1] = Hn[1];
+        H[2] = Hn[2];
       }
-      t *= 0.5;
+    }
+    // step lengths 1, 1/2, ... 2^-40: each group of lanes evaluates one, the first accepted is taken
+    for (int h0 = newton ? 1 : 0; h0 <= 40 && !accepted; h0 += 32 / W) {
+      const int h = h0 + (int)(threadIdx.x & 31) / W;
+      const double t = __hiloint2double((1023 - h) << 20, 0);   // 2^-h
+      const double c0 = fmin(fmax(x0 + t * d0, bl0), bh0), c1 = fmin(fmax(x1 + t * d1, bl1), bh1);
+      const bool le = geo_den<W>(j, c0, c1, sh) <= f && h <= 40;
+      const unsigned hit = __ballot_sync(0xffffffffu, le);
+      if (hit) {
+        const int src = __ffs(hit) - 1;
+        n0 = __shfl_sync(0xffffffffu, c0, src);
+        n1 = __shfl_sync(0xffffffffu, c1, src);
+        accepted = true;
+      }
     }
     if (!accepted) break;
     const double mv = fmax(fabs(n0 - x0), fabs(n1 - x1));
@@ -276,14 +453,22 @@ __device__ void refine_geo_warp(const RefineJob &j, int flat, RefShared &sh, dou
   out[1] = x1 / kD2R;
 }
 
-// Refines peaks idx[0..n) of one job; out: n angles (ULA) or n (azimuth, elevation) pairs.
-__device__ void refine_job_warp(const RefineJob &j, const int *idx, int n, double *out, RefShared &sh) {
+// Refines peaks idx[q], q = first, first + step, ... < n of one job; out: n angles (ULA) or n (azimuth,
+// elevation) pairs.
+__device__ void refine_job_warp(const RefineJob &j, const int *idx, int first, int step, int n, double *out,
+                                RefShared &sh) {
   const int lane = threadIdx.x & 31;
-  for (int q = 0; q < n; ++q) {
+  const int w = max(j.M, j.Kf);
+  for (int q = first; q < n; q += step) {
     const int k = idx[q];
     if (j.pos) {
       double r[2];
-      refine_geo_warp(j, k, sh, r);
+      if (w <= 8)
+        refine_geo_warp<8>(j, k, sh, r);
+      else if (w <= 16)
+        refine_geo_warp<16>(j, k, sh, r);
+      else
+        refine_geo_warp<32>(j, k, sh, r);
       if (lane == 0) {
         out[2 * q] = r[0];
         out[2 * q + 1] = r[1];
@@ -294,6 +479,15 @@ __device__ void refine_job_warp(const RefineJob &j, const int *idx, int n, doubl
     }
     __syncwarp();
   }
+}
+
+// Copies a small factor to shared memory and points the job at it; the whole CTA calls it.
+__device__ void stage_factor(RefineJob &j, double2 *Fs) {
+  if (j.M <= kStageM && j.Kf <= kStageM + 1) {
+    for (int e = threadIdx.x; e < j.M * j.Kf; e += blockDim.x) Fs[e] = j.F[e];
+    j.F = Fs;
+  }
+  __syncthreads();
 }
 
 __device__ void set_centroid(RefineJob &j) {
@@ -310,13 +504,15 @@ __device__ void set_centroid(RefineJob &j) {
 
 __global__ void __launch_bounds__(32 * kRefWarps) refine_batch_kernel(const uint8_t *plan, uint8_t *ws) {
   __shared__ RefShared sh[kRefWarps];
+  __shared__ double2 Fs[kStageM * (kStageM + 1)];
   const PlanHeader *h = reinterpret_cast<const PlanHeader *>(plan);
   const int warp = threadIdx.x >> 5;
-  const int job = blockIdx.x * kRefWarps + warp;
-  if (job >= h->njobs) return;
+  // the first half of the CTAs takes the 2-D jobs, whose longest searches are the kernel's tail
+  const bool geo = blockIdx.x < h->njobs;
+  const int job = geo ? blockIdx.x : blockIdx.x - h->njobs;
   const PlanJob &jb = reinterpret_cast<const PlanJob *>(plan + h->off_job)[job];
   const PlanProblem &pp = reinterpret_cast<const PlanProblem *>(plan + h->off_prob)[jb.prob];
-  if (!pp.p.peak_angle || pp.p.d < 1) return;
+  if (!pp.p.peak_angle || pp.p.d < 1 || (pp.p.geom.pos != nullptr) != geo) return;
   RefineJob j{};
   j.F = reinterpret_cast<const double2 *>(ws + pp.fac_off);
   j.w = pp.Kn > 0 && pp.slot[DOA_EV] >= 0
@@ -345,22 +541,25 @@ __global__ void __launch_bounds__(32 * kRefWarps) refine_batch_kernel(const uint
   const int d = pp.p.d;
   const int n = min(pp.p.peak_count[jb.slot], d);
   const int per = j.pos ? 2 : 1;
-  refine_job_warp(j, pp.p.peak_idx + (size_t)jb.slot * d, n, pp.p.peak_angle + (size_t)jb.slot * d * per, sh[warp]);
+  stage_factor(j, Fs);
+  refine_job_warp(j, pp.p.peak_idx + (size_t)jb.slot * d, warp, kRefWarps, n, pp.p.peak_angle + (size_t)jb.slot * d * per, sh[warp]);
 }
 
-__global__ void __launch_bounds__(32) refine_single_kernel(RefineJob j, const int *idx, const int *count, int cap,
-                                                           double *out) {
-  __shared__ RefShared sh;
+__global__ void __launch_bounds__(32 * kRefWarps) refine_single_kernel(RefineJob j, const int *idx, const int *count,
+                                                                       int cap, double *out) {
+  __shared__ RefShared sh[kRefWarps];
+  __shared__ double2 Fs[kStageM * (kStageM + 1)];
   if (j.pos) set_centroid(j);
-  const int n = min(*count, cap);
-  refine_job_warp(j, idx, n, out, sh);
+  const int n = min(*count, cap), warp = threadIdx.x >> 5;
+  stage_factor(j, Fs);
+  refine_job_warp(j, idx, blockIdx.x * kRefWarps + warp, gridDim.x * kRefWarps, n, out, sh[warp]);
 }
 
 }  // namespace
 
 cudaError_t launch_refine_batch(const uint8_t *plan_dev, const PlanHeader &h, uint8_t *ws, cudaStream_t s) {
   if (h.nrefine == 0 || h.njobs == 0) return cudaSuccess;
-  refine_batch_kernel<<<(h.njobs + kRefWarps - 1) / kRefWarps, 32 * kRefWarps, 0, s>>>(plan_dev, ws);
+  refine_batch_kernel<<<2 * h.njobs, 32 * kRefWarps, 0, s>>>(plan_dev, ws);
   return cudaGetLastError();
 }
 
@@ -382,7 +581,8 @@ cudaError_t launch_refine_single(const double2 *B, int M, int K, double lo, doub
   j.el_lo = el_lo;
   j.el_step = el_step;
   j.La = La;
-  refine_single_kernel<<<1, 32, 0, s>>>(j, idx, count, cap, out);
+  const int ctas = std::max(1, std::min((cap + kRefWarps - 1) / kRefWarps, 16));
+  refine_single_kernel<<<ctas, 32 * kRefWarps, 0, s>>>(j, idx, count, cap, out);
   return cudaGetLastError();
 }
 

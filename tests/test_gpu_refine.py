@@ -246,3 +246,47 @@ def test_all_outputs_together(env):
                 continue
             a, b = t_all[key].cpu().numpy(), t_one[key].cpu().numpy()
             assert np.array_equal(a, b, equal_nan=True), (maker, key)
+
+
+@pytest.mark.parametrize("M,d", [(3, 1), (8, 2), (9, 2), (16, 3), (17, 2), (33, 4)])
+def test_refine_single_at_lane_group_sizes(env, M, d):
+    """Factors around the lane-group widths (8, 16, whole warp), more peaks than the warps of a CTA: ULA
+    angles within 1e-9 degree and 2-D ones within 1e-8 of the oracle on the same factor, as in the
+    single-call tests above."""
+    torch, doa = env
+    inst = synth.custom(M, d, 2000, None, 15.0, 0.5, seed=1200 + M)
+    ev, V, _ = oracle.eigh(oracle.covariance(inst.X))
+    Bf = factor_from_decomposition(ev, V, d, MUSIC)
+    C = Bf @ Bf.conj().T
+    B = torch.from_numpy(np.ascontiguousarray(Bf.T).reshape(-1)).cuda()
+    P = oracle.scan(C, inst.lo, inst.step, inst.L)[0]
+    peaks = [k for k in range(1, inst.L - 1) if P[k] > P[k - 1] and P[k] > P[k + 1]]
+    idx = torch.tensor(peaks, dtype=torch.int32, device="cuda")
+    cnt = torch.tensor([len(peaks)], dtype=torch.int32, device="cuda")
+    th = torch.full((len(peaks) + 1,), -7.0, dtype=torch.float64, device="cuda")
+    doa.doa_refine_peaks(B, M, M - d, doa.grid(inst.lo, inst.step, inst.L), idx, cnt, th)
+    torch.cuda.synchronize()
+    got = th.cpu().numpy()
+    assert got[-1] == -7.0
+    for q, k in enumerate(peaks):
+        want, _ = oracle.refine_peak(C, inst.lo, inst.step, k)
+        assert abs(got[q] - want) <= 1e-9 * max(1.0, abs(want)), (k, got[q], want)
+    rng = np.random.default_rng(M)
+    pos = rng.uniform(-0.6, 0.6, size=(M, 3))
+    g = synth.geometry_custom(pos, d, 2000, 20.0, 0.0, 2.0, 180, 10.0, 2.0, 36, True, seed=1300 + M)
+    ev, V, _ = oracle.eigh(oracle.covariance(g.X))
+    Bf = factor_from_decomposition(ev, V, d, MUSIC)
+    C = Bf @ Bf.conj().T
+    ref = oracle.solve_geometry(g.X, d, MUSIC, pos, 0.0, 2.0, 180, 10.0, 2.0, 36, True)
+    inner = [int(k) for k in ref["idx"] if 0 < k // 180 < 35]      # minima inside the grid: well conditioned
+    idx = torch.tensor(inner or [0], dtype=torch.int32, device="cuda")
+    cnt = torch.tensor([len(inner)], dtype=torch.int32, device="cuda")
+    out = torch.zeros(2 * max(1, len(inner)), dtype=torch.float64, device="cuda")
+    posd = torch.from_numpy(np.ascontiguousarray(pos)).cuda()
+    B = torch.from_numpy(np.ascontiguousarray(Bf.T).reshape(-1)).cuda()
+    doa.doa_refine_peaks2d(B, M, M - d, doa.grid(0.0, 2.0, 180), doa.geometry(posd, 10.0, 2.0, 36, True), idx, cnt, out)
+    torch.cuda.synchronize()
+    got = out.cpu().numpy().reshape(-1, 2)
+    for q, k in enumerate(inner):
+        (wt, wp), _ = oracle.refine_peak2d(C, pos, 0.0, 2.0, 180, 10.0, 2.0, k)
+        assert abs(got[q, 0] - wt) <= 1e-8 and abs(got[q, 1] - wp) <= 1e-8, (k, got[q], wt, wp)
