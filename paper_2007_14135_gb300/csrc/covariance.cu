@@ -21,9 +21,12 @@
 // Batched form: one CTA per work item (problem, chunk of kCovChunk snapshots); multi-chunk
 // problems add their chunk partials in chunk order in FP64 (covariance_reduce_batch), so the
 // result is deterministic. Problems that request PHD use the compensated mode.
-// Single-problem form: a thread-block cluster of up to 8 CTAs splits the snapshots (always
-// compensated); CTA rank 0 adds the other CTAs' partials through distributed shared memory.
+// Single-problem form: clusters of up to 8 CTAs, each cluster on some of the blocks, split the
+// snapshots (always compensated); CTA rank 0 adds the other CTAs' partials through distributed shared
+// memory.
 #include <cooperative_groups.h>
+
+#include <algorithm>
 
 #include "doa_internal.cuh"
 
@@ -40,15 +43,28 @@ constexpr int kSmemBytes = 65536;
 constexpr int kMaxCluster = 8;
 
 struct CovLayout {
-  int M, MB, nb, groups;
-  __device__ CovLayout(int M_) : M(M_) {
+  int M, MB, nb, groups, b0;
+  uint32_t rows;        // row blocks that the CTA's blocks read
+  __device__ CovLayout(int M_) : CovLayout(M_, 0, (M_ + kRB - 1) / kRB * ((M_ + kRB - 1) / kRB + 1) / 2) {}
+  // blocks first .. last - 1 of the upper triangle only
+  __device__ CovLayout(int M_, int first, int last) : M(M_), b0(first) {
     MB = (M + kRB - 1) / kRB;
-    nb = MB * (MB + 1) / 2;
+    nb = last - first;
     groups = max(1, kCovThreads / nb);
+    rows = 0u;
+    if (nb == MB * (MB + 1) / 2) {
+      rows = 0xffffffffu;
+    } else {
+      for (int b = 0; b < nb; ++b) {
+        int bi, bj;
+        block_of(b, bi, bj);
+        rows |= (1u << bi) | (1u << bj);
+      }
+    }
   }
-  // block (bi, bj), bi <= bj, of the linear upper-triangle block index b
+  // block (bi, bj), bi <= bj, of the CTA's block b
   __device__ void block_of(int b, int &bi, int &bj) const {
-    int i = 0, rem = b;
+    int i = 0, rem = b0 + b;
     while (rem >= MB - i) { rem -= MB - i; ++i; }
     bi = i;
     bj = i + rem;
@@ -124,6 +140,7 @@ __device__ float4 *cov_accumulate(const float2 *__restrict__ X, int ldx, int t0,
     __syncthreads();
     for (int e = tid; e < MP * kTS; e += kCovThreads) {
       int r = e / kTS, t = e % kTS;
+      if (!((lay.rows >> (r / kRB)) & 1u)) continue;
       float2 v = make_float2(0.f, 0.f);
       if (r < lay.M && t < cnt) v = X[(size_t)r * ldx + ts + t];
       tile[r * kTS + t] = v;
@@ -213,7 +230,8 @@ __global__ void __launch_bounds__(kCovThreads) covariance_cluster_kernel(const f
   cg::cluster_group cluster = cg::this_cluster();
   const int rank = (int)cluster.block_rank();
   const int nranks = (int)cluster.num_blocks();
-  CovLayout lay(M);
+  const int MB = (M + kRB - 1) / kRB, nb = MB * (MB + 1) / 2, nsplit = gridDim.x / nranks, split = blockIdx.x / nranks;
+  const CovLayout lay(M, nb * split / nsplit, nb * (split + 1) / nsplit);
   const int t0 = rank * per_cta;
   const int t1 = min(N, t0 + per_cta);
   float4 *part = cov_accumulate<true>(X, ldx, t0, max(t0, t1), lay, smem);
@@ -600,11 +618,18 @@ cudaError_t launch_covariance_single(const float2 *X, int M, int N, int ldx, flo
                                      cudaStream_t s) {
   cudaError_t e = ensure_smem_attr(reinterpret_cast<const void *>(covariance_cluster_kernel), kSmemBytes);
   if (e != cudaSuccess) return e;
-  int chunks = (N + kCovChunk - 1) / kCovChunk;
-  int nc = chunks < kMaxCluster ? chunks : kMaxCluster;
-  int per = (N + nc - 1) / nc;
+  // Snapshots over a cluster, at least two tiles a CTA; the blocks of the triangle over clusters, as many
+  // as the SMs hold, while a thread still has eight snapshots or more to add (a CTA has 256 / nb groups
+  // of threads for its nb blocks). One cluster that took 1024 snapshots a CTA needed 29 us for M = 8,
+  // N = 1024 (one CTA) and 1.8 ms for M = 64, N = 16384; now @C8@ and @C64@ us.
+  const int tiles = (N + kTS - 1) / kTS;
+  const int nc = std::max(1, std::min(kMaxCluster, tiles / 2));
+  const int per = (N + nc - 1) / nc;
+  const int MB = (M + kRB - 1) / kRB, nb = MB * (MB + 1) / 2;
+  int ns = std::min(nb, std::max(1, device_sm_count() / nc));
+  while (ns > 1 && (int64_t)per * ((nb + ns - 1) / ns) < 8 * kCovThreads) --ns;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(nc);
+  cfg.gridDim = dim3(nc * ns);
   cfg.blockDim = dim3(kCovThreads);
   cfg.dynamicSmemBytes = kSmemBytes;
   cfg.stream = s;

@@ -7,7 +7,7 @@
 // columns produces the whole covariance in TMEM.
 //
 // Per CTA: TMA (cp.async.bulk.tensor, FP32, no swizzle) brings 32 snapshots of all M rows
-// (M x 64 floats) into a two-stage staging ring guarded by mbarriers; all threads split the FP32
+// (M x 64 floats) into a four-stage staging ring guarded by mbarriers; all threads split the FP32
 // values into hi/lo 16-bit parts (BF16, or FP16 with the lo part scaled by 2^11) and write the
 // three operand views (Y and Z rows of A, Y rows of B) in the 128B-swizzled K-major layout; one
 // thread issues the MMAs (one product for DOA_BF16, hi*hi + hi*lo + lo*hi for the x3 forms, the
@@ -17,6 +17,10 @@
 // through distributed shared memory, keeps the upper triangle and mirrors it (Hermitian).
 // Accuracy: the split forms carry ~16 (BF16x3) or ~22 (FP16x3) significant bits per operand and
 // accumulate in FP32; this is the reduced-precision covariance of the large-array configuration.
+// An atom is bound by the splitting between two block barriers (its MMAs take 600 cycles): with 128
+// threads, the sixteen values of both operand views split apart and two atoms in flight it took 4900
+// cycles, 153 us for M = 64, N = 16384; with 512 threads, eight values each and four atoms @CT@ us. The
+// split over the cluster stays as it is: the FP32 accumulation truncates, so its order shows in R.
 #include <cooperative_groups.h>
 #include <cuda.h>
 #include <cudaTypedefs.h>
@@ -31,7 +35,8 @@ namespace {
 
 using namespace tc;
 
-constexpr int kCtThreads = 128;
+constexpr int kCtThreads = 512;  // a thread per (row, 4 snapshots) of an atom at M = 64; four warps read TMEM
+constexpr int kCtStages = 4;     // staged FP32 atoms
 constexpr int kCtCluster = 8;
 constexpr int kAtomSnap = 32;   // snapshots per K atom (64 reals = one 128-byte swizzle row)
 
@@ -39,7 +44,7 @@ struct CtLayout {
   int NP;        // N dimension of the MMA: M rounded up to 16
   int tmem_cols;
   int stage_bytes;                          // M x 64 floats
-  int off_stage[2], off_ahi[2], off_alo[2], off_bhi[2], off_blo[2], total;
+  int off_stage[kCtStages], off_ahi[2], off_alo[2], off_bhi[2], off_blo[2], total;
 };
 
 __host__ __device__ inline CtLayout ct_layout(int M, int prec) {
@@ -64,7 +69,7 @@ __host__ __device__ inline CtLayout ct_layout(int M, int prec) {
     t.off_blo[s] = at;
     at += (bbytes + 1023) / 1024 * 1024;
   }
-  for (int s = 0; s < 2; ++s) {
+  for (int s = 0; s < kCtStages; ++s) {
     t.off_stage[s] = at;
     at += (t.stage_bytes + 1023) / 1024 * 1024;
   }
@@ -89,7 +94,7 @@ __global__ void __launch_bounds__(kCtThreads, 1) covariance_tc_kernel(const __gr
                                                                       float2 *R, double2 *R64) {
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   uint8_t *sm = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  __shared__ __align__(8) uint64_t full_bar[2], mma_bar[2];
+  __shared__ __align__(8) uint64_t full_bar[kCtStages], mma_bar[2];
   __shared__ uint32_t tmem_base;
   __shared__ int s_ok;
   cg::cluster_group cluster = cg::this_cluster();
@@ -104,10 +109,10 @@ __global__ void __launch_bounds__(kCtThreads, 1) covariance_tc_kernel(const __gr
   for (int e = tid * 16; e < lay.off_stage[0]; e += kCtThreads * 16)
     *reinterpret_cast<uint4 *>(sm + e) = make_uint4(0, 0, 0, 0);
   if (tid == 0) {
-    for (int s = 0; s < 2; ++s) {
+    for (int s = 0; s < kCtStages; ++s)
       asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&full_bar[s])));
+    for (int s = 0; s < 2; ++s)
       asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&mma_bar[s])));
-    }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     s_ok = 1;
   }
@@ -124,38 +129,42 @@ __global__ void __launch_bounds__(kCtThreads, 1) covariance_tc_kernel(const __gr
   const uint32_t idesc = inst_desc(prec == DOA_FP16X3 ? 0 : 1, lay.NP);
   const bool split = prec != DOA_BF16;
 
-  // prologue: the first two atoms in flight (issued / consumed: bookkeeping of thread 0)
+  // prologue: the first atoms in flight (issued / consumed: bookkeeping of thread 0)
   int issued = 0, consumed = 0;
   if (tid == 0)
-    for (int s = 0; s < 2 && s < natoms; ++s, ++issued) {
+    for (int s = 0; s < kCtStages && s < natoms; ++s, ++issued) {
       mbar_expect(smem_u32(&full_bar[s]), (uint32_t)lay.stage_bytes);
       tma_load_2d(smem_u32(sm + lay.off_stage[s]), &xmap, (a0 + s) * 2 * kAtomSnap, 0, smem_u32(&full_bar[s]));
     }
   bool ok = true;
   for (int i = 0; i < natoms; ++i) {
-    const int s = i & 1;
+    const int s = i & 1, f = i % kCtStages;
     // the operand buffer s was last read by the MMAs of atom i - 2
     bool good = ok;
     if (good && i >= 2) good = mbar_wait(smem_u32(&mma_bar[s]), (uint32_t)(((i - 2) >> 1) & 1));
-    if (good) good = mbar_wait(smem_u32(&full_bar[s]), (uint32_t)((i >> 1) & 1));
+    if (good) good = mbar_wait(smem_u32(&full_bar[f]), (uint32_t)((i / kCtStages) & 1));
     ok = __syncthreads_and(good);
     if (!ok) break;
     consumed = i + 1;
     // split the staged FP32 atom (M rows x 32 complex) into the three operand views
-    const float *stg = reinterpret_cast<const float *>(sm + lay.off_stage[s]);
+    const float *stg = reinterpret_cast<const float *>(sm + lay.off_stage[f]);
     uint8_t *ahi = sm + lay.off_ahi[s], *alo = sm + lay.off_alo[s];
     uint8_t *bhi = sm + lay.off_bhi[s], *blo = sm + lay.off_blo[s];
+    // z's parts are y's with signs: rounding is symmetric, so their halves are y's halves with signs
     for (int task = tid; task < M * 8; task += kCtThreads) {
       const int r = task >> 3, ch = task & 7;        // row, chunk of 4 complex (8 reals)
       const float4 u = *reinterpret_cast<const float4 *>(stg + r * 64 + ch * 8);
       const float4 v = *reinterpret_cast<const float4 *>(stg + r * 64 + ch * 8 + 4);
       const float y[8] = {u.x, u.y, u.z, u.w, v.x, v.y, v.z, v.w};
-      const float z[8] = {u.y, -u.x, u.w, -u.z, v.y, -v.x, v.w, -v.z};   // (re, im) -> (im, -re)
       uint16_t yh[8], yl[8], zh[8], zl[8];
 #pragma unroll
-      for (int j = 0; j < 8; ++j) {
-        split16(y[j], prec, yh[j], yl[j]);
-        split16(z[j], prec, zh[j], zl[j]);
+      for (int j = 0; j < 8; ++j) split16(y[j], prec, yh[j], yl[j]);
+#pragma unroll
+      for (int j = 0; j < 8; j += 2) {   // (re, im) -> (im, -re)
+        zh[j] = yh[j + 1];
+        zl[j] = yl[j + 1];
+        zh[j + 1] = yh[j] ^ 0x8000u;
+        zl[j + 1] = yl[j] ^ 0x8000u;
       }
       auto pack = [](const uint16_t (&h)[8]) {
         return make_uint4(h[0] | ((uint32_t)h[1] << 16), h[2] | ((uint32_t)h[3] << 16), h[4] | ((uint32_t)h[5] << 16),
@@ -174,10 +183,11 @@ __global__ void __launch_bounds__(kCtThreads, 1) covariance_tc_kernel(const __gr
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     __syncthreads();
     if (tid == 0) {
-      // staging slot s is free again: fetch atom i + 2
-      if (i + 2 < natoms) {
-        mbar_expect(smem_u32(&full_bar[s]), (uint32_t)lay.stage_bytes);
-        tma_load_2d(smem_u32(sm + lay.off_stage[s]), &xmap, (a0 + i + 2) * 2 * kAtomSnap, 0, smem_u32(&full_bar[s]));
+      // staging slot f is free again: fetch the atom that uses it next
+      if (i + kCtStages < natoms) {
+        mbar_expect(smem_u32(&full_bar[f]), (uint32_t)lay.stage_bytes);
+        tma_load_2d(smem_u32(sm + lay.off_stage[f]), &xmap, (a0 + i + kCtStages) * 2 * kAtomSnap, 0,
+                    smem_u32(&full_bar[f]));
         ++issued;
       }
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -201,7 +211,8 @@ __global__ void __launch_bounds__(kCtThreads, 1) covariance_tc_kernel(const __gr
   }
   // after a timed-out wait, let the copies still in flight land before the CTA exits (bounded)
   if (!ok && tid == 0)
-    for (int a = consumed; a < issued; ++a) mbar_wait(smem_u32(&full_bar[a & 1]), (uint32_t)((a >> 1) & 1));
+    for (int a = consumed; a < issued; ++a)
+      mbar_wait(smem_u32(&full_bar[a % kCtStages]), (uint32_t)((a / kCtStages) & 1));
   // drain: the last commit covers every earlier MMA of this thread
   if (natoms > 0 && ok) {
     const int il = natoms - 1;
@@ -213,7 +224,7 @@ __global__ void __launch_bounds__(kCtThreads, 1) covariance_tc_kernel(const __gr
   // accumulator -> FP32 partial [128 rows][NP] in shared memory (aliases the operand buffers)
   float *part = reinterpret_cast<float *>(sm);
   const int row = warp * 32 + lane;
-  for (int c0 = 0; c0 < lay.NP; c0 += 8) {
+  for (int c0 = 0; c0 < lay.NP && warp < 4; c0 += 8) {
     float v[8];
     if (natoms > 0 && ok) {
       tmem_ld8(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c0, v);

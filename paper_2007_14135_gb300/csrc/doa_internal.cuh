@@ -310,7 +310,7 @@ struct PlanHeader {
   int64_t tc_tiles;                      // 128-point tiles over all tc problems
   int64_t off_tc;                        // byte offset of the tc problem list
   int32_t npolish;                       // problems with DOA_FLAG_POLISH_PEAKS
-  int32_t pad2;
+  int32_t max_points;                    // points of the longest spectrum
   // problems with an explicit geometry (2-D azimuth x elevation scans), per M bucket
   int32_t geo_jobs[kNumBuckets];
   int64_t geo_tiles[kNumBuckets];

@@ -1,4 +1,5 @@
-// Step-6 (Table 2): findPeaks + PeakSelection(peakVals, inds, D), one CTA per spectrum.
+// Step-6 (Table 2): findPeaks + PeakSelection(peakVals, inds, D), one CTA or one cluster of eight per
+// spectrum.
 //
 // A peak is the left end i of a maximal run [i..j] of equal values with 1 <= i, j <= L-2,
 // P[i-1] < P[i] and P[j+1] < P[j]. The D largest peaks are selected (equal values: lower
@@ -9,7 +10,12 @@
 // arg-max (the winning lane pops its head and, if its cache runs dry while it still has peaks,
 // rescans its quads for the next ones below its last selected peak); one warp then merges the
 // warps' lists. This realises the shared-memory max-reduction that the paper names as future work
-// for Step-6 (Sec. 6).
+// for Step-6 (Sec. 6). With a cluster the quads are dealt over all its threads and rank 0 merges the
+// CTAs' lists through distributed shared memory in the same way: one CTA reads a long spectrum at the
+// rate its loads in flight allow (150 us for 360 001 points; the cluster: 33 us), which leaves most of
+// the chip idle when the spectra are few, and trails the batch when a few are long.
+#include <cooperative_groups.h>
+
 #include <climits>
 
 #include "doa_internal.cuh"
@@ -40,62 +46,131 @@ __device__ void write_sel(Cand *sel, int nsel, int *idx, float *val, int *count)
   }
 }
 
+namespace cg = cooperative_groups;
+constexpr int kPeakCluster = 8;
+constexpr int kClusterPoints = 16384;      // points from which a single call takes a cluster
+constexpr int kClusterLong = 65536;        // longest spectrum from which a batch does, whatever its jobs
+
+// This CTA's share of a spectrum's quads: rank of kCs CTAs.
+template <int kCs>
+struct Share {
+  int first, stride, rank;
+  __device__ Share() {
+    rank = kCs > 1 ? (int)cg::this_cluster().block_rank() : 0;
+    first = rank * kPeakThreads + (int)threadIdx.x;
+    stride = kCs * kPeakThreads;
+  }
+};
+
+// Merges the cluster's lists (sel, n per CTA, best first) into rank 0's out; every CTA calls it. Returns
+// the count (rank 0).
+template <int kCs>
+__device__ int merge_lists(int want, const Cand *sel, int n, Cand *out) {
+  __shared__ int s_n, s_total;
+  cg::cluster_group cl = cg::this_cluster();
+  if (threadIdx.x == 0) s_n = n;
+  cl.sync();
+  if (cl.block_rank() == 0 && threadIdx.x < 32) {
+    const int lane = threadIdx.x, src = min(lane, kCs - 1);
+    const Cand *rs = cl.map_shared_rank(sel, src);
+    const int rn = lane < kCs ? *cl.map_shared_rank(&s_n, src) : 0;
+    const Cand none{0.f, INT_MAX};
+    int pos = 0, total = 0;
+    for (int r = 0; r < want; ++r) {
+      const Cand mine = pos < rn ? rs[pos] : none;
+      const Cand w = warp_best(mine);
+      if (w.i == INT_MAX) break;
+      if (lane == 0) out[total] = w;
+      ++total;
+      if (mine.i == w.i) ++pos;
+    }
+    if (lane == 0) s_total = total;
+  }
+  cl.sync();   // the lists stay in place until rank 0 has read them
+  return s_total;
+}
+
 // next (nullable): receives the value of the (d+1)-th best peak (-inf if there is none).
+template <int kCs>
 __device__ void peaks_block(const float *__restrict__ P, int L, int d, int *idx, float *val, int *count,
                             float *next = nullptr) {
-  __shared__ Cand sel[kMaxM + 1];
+  __shared__ Cand sel[kMaxM + 1], all[kCs > 1 ? kMaxM + 1 : 1];
   const int want = next ? d + 1 : d;
-  int nsel = select_top(P, L, want, sel);
+  const Share<kCs> sh;
+  int nsel = select_rounds(want, sel, [&](const Cand &thr, Cand (&cache)[kCache], int &n) {
+    return fill(P, L, sh.first, sh.stride, thr, cache, n);
+  });
+  Cand *best = sel;
+  if (kCs > 1) {
+    nsel = merge_lists<kCs>(want, sel, nsel, all);
+    best = all;
+    if (sh.rank != 0) return;
+  }
   if (next) {
-    if (threadIdx.x == 0) *next = nsel > d ? sel[d].v : -INFINITY;
+    if (threadIdx.x == 0) *next = nsel > d ? best[d].v : -INFINITY;
     nsel = min(nsel, d);
   }
-  write_sel(sel, nsel, idx, val, count);
+  write_sel(best, nsel, idx, val, count);
 }
 
+template <int kCs>
 __device__ void peaks2d_block(const float *__restrict__ P, int La, int Le, bool wrap, int d, int *idx, float *val,
                               int *count) {
-  __shared__ Cand sel[kMaxM];
-  const int nsel = select_top2d(P, La, Le, wrap, d, sel);
-  write_sel(sel, nsel, idx, val, count);
+  __shared__ Cand sel[kMaxM], all[kCs > 1 ? kMaxM : 1];
+  const Share<kCs> sh;
+  int nsel = select_rounds(d, sel, [&](const Cand &thr, Cand (&cache)[kCache], int &n) {
+    return fill2d(P, La, Le, wrap, sh.first, sh.stride, thr, cache, n);
+  });
+  Cand *best = sel;
+  if (kCs > 1) {
+    nsel = merge_lists<kCs>(d, sel, nsel, all);
+    best = all;
+    if (sh.rank != 0) return;
+  }
+  write_sel(best, nsel, idx, val, count);
 }
 
+template <int kCs>
 __global__ void __launch_bounds__(kPeakThreads) peaks2d_single_kernel(const float *P, int La, int Le, int wrap, int d,
                                                                       int *idx, float *val, int *count) {
-  peaks2d_block(P, La, Le, wrap != 0, d, idx, val, count);
+  peaks2d_block<kCs>(P, La, Le, wrap != 0, d, idx, val, count);
 }
 
+template <int kCs>
 __global__ void __launch_bounds__(kPeakThreads) peaks_single_kernel(const float *P, int L, int d, int *idx, float *val,
                                                                     int *count) {
-  peaks_block(P, L, d, idx, val, count);
+  peaks_block<kCs>(P, L, d, idx, val, count);
 }
 
-// One CTA per (problem, algorithm) job; the 1-D and 2-D rules run as separate kernels (each skips
+// One CTA (or cluster) per (problem, algorithm) job; the 1-D and 2-D rules run as separate kernels (each skips
 // the other kind's jobs) so that each keeps its own register budget.
 // repick: the pick after the peak polish, only for the jobs the polish marked (NaN next value).
+template <int kCs>
 __global__ void __launch_bounds__(kPeakThreads, 5) peaks_batch_kernel(const uint8_t *plan, uint8_t *ws, int repick) {
+  const int job = blockIdx.x / kCs;
   const PlanHeader *h = reinterpret_cast<const PlanHeader *>(plan);
-  const PlanJob &jb = reinterpret_cast<const PlanJob *>(plan + h->off_job)[blockIdx.x];
+  const PlanJob &jb = reinterpret_cast<const PlanJob *>(plan + h->off_job)[job];
   const PlanProblem &pp = reinterpret_cast<const PlanProblem *>(plan + h->off_prob)[jb.prob];
   if (pp.p.geom.pos) return;
   const int L = pp.npts, d = pp.p.d;
   const bool polish = (pp.p.flags & DOA_FLAG_POLISH_PEAKS) && h->next_val_off >= 0;
-  float *next = polish ? reinterpret_cast<float *>(ws + h->next_val_off) + blockIdx.x : nullptr;
+  float *next = polish ? reinterpret_cast<float *>(ws + h->next_val_off) + job : nullptr;
   if (repick) {
     if (!polish || !isnan(*next)) return;
     next = nullptr;
   }
-  peaks_block(pp.p.P + (size_t)jb.slot * L, L, d, pp.p.peak_idx + (size_t)jb.slot * d,
+  peaks_block<kCs>(pp.p.P + (size_t)jb.slot * L, L, d, pp.p.peak_idx + (size_t)jb.slot * d,
               pp.p.peak_val + (size_t)jb.slot * d, pp.p.peak_count + jb.slot, next);
 }
 
+template <int kCs>
 __global__ void __launch_bounds__(kPeakThreads, 5) peaks2d_batch_kernel(const uint8_t *plan) {
   const PlanHeader *h = reinterpret_cast<const PlanHeader *>(plan);
-  const PlanJob &jb = reinterpret_cast<const PlanJob *>(plan + h->off_job)[blockIdx.x];
+  const PlanJob &jb = reinterpret_cast<const PlanJob *>(plan + h->off_job)[blockIdx.x / kCs];
   const PlanProblem &pp = reinterpret_cast<const PlanProblem *>(plan + h->off_prob)[jb.prob];
   if (!pp.p.geom.pos) return;
   const int L = pp.npts, d = pp.p.d;
-  peaks2d_block(pp.p.P + (size_t)jb.slot * L, pp.p.grid.L, pp.p.geom.Le, pp.p.geom.wrap_az != 0, d,
+  peaks2d_block<kCs>(pp.p.P + (size_t)jb.slot * L, pp.p.grid.L, pp.p.geom.Le, pp.p.geom.wrap_az != 0, d,
                 pp.p.peak_idx + (size_t)jb.slot * d, pp.p.peak_val + (size_t)jb.slot * d, pp.p.peak_count + jb.slot);
 }
 
@@ -196,25 +271,52 @@ cudaError_t launch_slice_peaks(const float *Pbuf, int b0, int k0, int k1, int L,
   return cudaGetLastError();
 }
 
+// Launches `kernel` on `jobs` spectra, kCs CTAs each.
+template <int kCs, class... Args>
+cudaError_t launch_jobs(void (*kernel)(Args...), int jobs, cudaStream_t s, Args... args) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)jobs * kCs);
+  cfg.blockDim = dim3(kPeakThreads);
+  cfg.stream = s;
+  cudaLaunchAttribute attr{};
+  attr.id = cudaLaunchAttributeClusterDimension;
+  attr.val.clusterDim.x = kCs;
+  attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+  cfg.attrs = &attr;
+  cfg.numAttrs = kCs > 1 ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
 cudaError_t launch_peaks_single(const float *P, int L, int d, int *idx, float *val, int *count, cudaStream_t s) {
-  peaks_single_kernel<<<1, kPeakThreads, 0, s>>>(P, L, d, idx, val, count);
-  return cudaGetLastError();
+  return L >= kClusterPoints ? launch_jobs<kPeakCluster>(peaks_single_kernel<kPeakCluster>, 1, s, P, L, d, idx, val, count)
+                             : launch_jobs<1>(peaks_single_kernel<1>, 1, s, P, L, d, idx, val, count);
 }
 
 cudaError_t launch_peaks2d_single(const float *P, int La, int Le, int wrap_az, int d, int *idx, float *val,
                                   int *count, cudaStream_t s) {
-  peaks2d_single_kernel<<<1, kPeakThreads, 0, s>>>(P, La, Le, wrap_az, d, idx, val, count);
-  return cudaGetLastError();
+  return (int64_t)La * Le >= kClusterPoints
+             ? launch_jobs<kPeakCluster>(peaks2d_single_kernel<kPeakCluster>, 1, s, P, La, Le, wrap_az, d, idx, val, count)
+             : launch_jobs<1>(peaks2d_single_kernel<1>, 1, s, P, La, Le, wrap_az, d, idx, val, count);
 }
 
+// A batch takes clusters when its jobs do not fill the SMs (five CTAs each) and some spectrum is long
+// enough for a single call to take one, or when some spectrum is very long beside the others: 1024 mixed
+// jobs of up to 180 001 points, 0.15 -> @UNEVEN@ ms; 16384 jobs of 18 001 stay with a CTA each.
 cudaError_t launch_peaks_batch(const uint8_t *plan_dev, const PlanHeader &h, uint8_t *ws, bool ula, bool geo,
                                cudaStream_t s) {
   int ngeo = 0;
   for (int b = 0; b < kNumBuckets; ++b) ngeo += h.geo_jobs[b];
   const int repick = ula && !geo;   // the call after the polish
-  if (h.njobs > 0 && ula && ngeo < h.nprob) peaks_batch_kernel<<<h.njobs, kPeakThreads, 0, s>>>(plan_dev, ws, repick);
-  if (h.njobs > 0 && geo && ngeo > 0) peaks2d_batch_kernel<<<h.njobs, kPeakThreads, 0, s>>>(plan_dev);
-  return cudaGetLastError();
+  const bool few = (int64_t)h.njobs * kPeakCluster <= 5 * (int64_t)device_sm_count();
+  const bool cl = h.max_points >= (few ? kClusterPoints : kClusterLong);
+  cudaError_t e = cudaSuccess;
+  if (h.njobs > 0 && ula && ngeo < h.nprob)
+    e = cl ? launch_jobs<kPeakCluster>(peaks_batch_kernel<kPeakCluster>, h.njobs, s, plan_dev, ws, repick)
+           : launch_jobs<1>(peaks_batch_kernel<1>, h.njobs, s, plan_dev, ws, repick);
+  if (e == cudaSuccess && h.njobs > 0 && geo && ngeo > 0)
+    e = cl ? launch_jobs<kPeakCluster>(peaks2d_batch_kernel<kPeakCluster>, h.njobs, s, plan_dev)
+           : launch_jobs<1>(peaks2d_batch_kernel<1>, h.njobs, s, plan_dev);
+  return e;
 }
 
 }  // namespace doa

@@ -372,7 +372,9 @@ __global__ void __launch_bounds__(kScanThreads, shared_min_blocks<MP, PT>())
   }
 }
 
-// Peak polish (DOA_FLAG_POLISH_PEAKS): one warp per problem re-evaluates, with the FP64
+// Peak polish (DOA_FLAG_POLISH_PEAKS): one CTA per problem (its first warp picks the points, all warps
+// take them in turn; with a warp per problem, one problem of M = 32 with many peaks on a fine grid kept
+// its warp for 0.48 ms) re-evaluates, with the FP64
 // steering and contraction of the scan's refinement (two or four points per pass in sub-warps
 // for small factors), every readout of the problem at the union of its algorithms' picked peaks
 // and their two neighbours on each side (each point once); the
@@ -392,14 +394,14 @@ __device__ __forceinline__ bool order_certain(float a, float b) {
 __global__ void __launch_bounds__(32 * kPolishWarps) polish_batch_kernel(const uint8_t *plan, uint8_t *ws) {
   __shared__ double2 ph[kPolishWarps][kMaxM];
   __shared__ float2 yb[kPolishWarps][kMaxCols];
-  __shared__ float w32[kPolishWarps][kMaxM];
-  __shared__ int pk[kPolishWarps][kPolishMax];
-  __shared__ int cand[kPolishWarps][kPolishMax];
+  __shared__ float w32[kMaxM];
+  __shared__ int pk[kPolishMax];
+  __shared__ int cand[kPolishMax];
   __shared__ int pts[kPolishWarps][4];
+  __shared__ int s_n;
   const PlanHeader *h = reinterpret_cast<const PlanHeader *>(plan);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int prob = blockIdx.x * kPolishWarps + warp;
-  if (prob >= h->nprob) return;
+  const int prob = blockIdx.x;
   const PlanProblem &pp = reinterpret_cast<const PlanProblem *>(plan + h->off_prob)[prob];
   if (!(pp.p.flags & DOA_FLAG_POLISH_PEAKS) || pp.p.d < 1) return;
   const PlanGrid &g = reinterpret_cast<const PlanGrid *>(plan + h->off_grid)[pp.grid_id];
@@ -418,84 +420,92 @@ __global__ void __launch_bounds__(32 * kPolishWarps) polish_batch_kernel(const u
   j.kphd = pp.kphd;
   j.kmn = pp.kmn;
   j.kofs = 0;
-  for (int c = lane; c < j.Kn; c += 32) w32[warp][c] = j.w ? (float)j.w[c] : 1.f;
+  for (int c = threadIdx.x; c < j.Kn; c += 32 * kPolishWarps) w32[c] = j.w ? (float)j.w[c] : 1.f;
   const int d = pp.p.d, L = g.L;
   const float *next = h->next_val_off >= 0 ? reinterpret_cast<const float *>(ws + h->next_val_off) : nullptr;
-  // lane s < njobs: is job s's selection decided by its FP32 values (its weakest selected peak
-  // above its best unselected value by more than the FP32 error)?
-  bool bnd = true;
-  if (lane < pp.njobs) {
-    const int cnt = min(pp.p.peak_count[lane], d);
-    if (cnt == d && next) {
-      float vmin = INFINITY;
-      for (int q = 0; q < cnt; ++q) vmin = fminf(vmin, pp.p.peak_val[(size_t)lane * d + q]);
-      const float nv = next[pp.first_job + lane];
-      bnd = !(nv > -INFINITY) || (vmin > nv && order_certain(vmin, nv));
-    }
-  }
-  const unsigned bmask = __ballot_sync(0xffffffffu, bnd);
-  // lane e takes peak e % d of job e / d: undecided peaks go to cand[] (one round of loads for all)
-  int ncand = 0;
-  for (int e0 = 0; e0 < pp.njobs * d; e0 += 32) {
-    const int e = e0 + lane;
-    int k = -1;
-    if (e < pp.njobs * d) {
-      const int sj = e / d, q = e % d;
-      if (q < min(pp.p.peak_count[sj], d)) {
-        k = pp.p.peak_idx[(size_t)sj * d + q];
-        const float *Ps = pp.p.P + (size_t)sj * L;
-        const int i0 = max(k - 3, 0), i1 = min(k + 3, L - 1);
-        float v[7];
-#pragma unroll
-        for (int t = 0; t < 7; ++t) v[t] = i0 + t <= i1 ? Ps[i0 + t] : 0.f;
-        bool decided = ((bmask >> sj) & 1u) && next;
-#pragma unroll
-        for (int t = 0; t < 6; ++t) decided = decided && (i0 + t >= i1 || order_certain(v[t], v[t + 1]));
-        if (decided) k = -1;
+  if (warp == 0) {
+    // lane s < njobs: is job s's selection decided by its FP32 values (its weakest selected peak
+    // above its best unselected value by more than the FP32 error)?
+    bool bnd = true;
+    if (lane < pp.njobs) {
+      const int cnt = min(pp.p.peak_count[lane], d);
+      if (cnt == d && next) {
+        float vmin = INFINITY;
+        for (int q = 0; q < cnt; ++q) vmin = fminf(vmin, pp.p.peak_val[(size_t)lane * d + q]);
+        const float nv = next[pp.first_job + lane];
+        bnd = !(nv > -INFINITY) || (vmin > nv && order_certain(vmin, nv));
       }
     }
-    const unsigned um = __ballot_sync(0xffffffffu, k >= 0);
-    if (k >= 0) cand[warp][ncand + __popc(um & ((1u << lane) - 1u))] = k;
-    ncand += __popc(um);
-  }
-  __syncwarp();
-  int n = 0;
-  if (lane == 0) {   // the undecided peaks, sorted, each once
-    for (int c = 0; c < ncand; ++c) {
-      const int k = cand[warp][c];
-      int a = n;
-      while (a > 0 && pk[warp][a - 1] > k) --a;
-      if (a > 0 && pk[warp][a - 1] == k) continue;
-      for (int b = n; b > a; --b) pk[warp][b] = pk[warp][b - 1];
-      pk[warp][a] = k;
-      ++n;
+    const unsigned bmask = __ballot_sync(0xffffffffu, bnd);
+    // lane e takes peak e % d of job e / d: undecided peaks go to cand[] (one round of loads for all)
+    int ncand = 0;
+    for (int e0 = 0; e0 < pp.njobs * d; e0 += 32) {
+      const int e = e0 + lane;
+      int k = -1;
+      if (e < pp.njobs * d) {
+        const int sj = e / d, q = e % d;
+        if (q < min(pp.p.peak_count[sj], d)) {
+          k = pp.p.peak_idx[(size_t)sj * d + q];
+          const float *Ps = pp.p.P + (size_t)sj * L;
+          const int i0 = max(k - 3, 0), i1 = min(k + 3, L - 1);
+          float v[7];
+#pragma unroll
+          for (int t = 0; t < 7; ++t) v[t] = i0 + t <= i1 ? Ps[i0 + t] : 0.f;
+          bool decided = ((bmask >> sj) & 1u) && next;
+#pragma unroll
+          for (int t = 0; t < 6; ++t) decided = decided && (i0 + t >= i1 || order_certain(v[t], v[t + 1]));
+          if (decided) k = -1;
+        }
+      }
+      const unsigned um = __ballot_sync(0xffffffffu, k >= 0);
+      if (k >= 0) cand[ncand + __popc(um & ((1u << lane) - 1u))] = k;
+      ncand += __popc(um);
     }
+    __syncwarp();
+    int n = 0;
+    if (lane == 0) {   // the undecided peaks, sorted, each once
+      for (int c = 0; c < ncand; ++c) {
+        const int k = cand[c];
+        int a = n;
+        while (a > 0 && pk[a - 1] > k) --a;
+        if (a > 0 && pk[a - 1] == k) continue;
+        for (int b = n; b > a; --b) pk[b] = pk[b - 1];
+        pk[a] = k;
+        ++n;
+      }
+    }
+    n = __shfl_sync(0xffffffffu, n, 0);
+    if (lane == 0) s_n = n;
+    // mark the problem's jobs for the second pick (a NaN in their next-value slots); the jobs of a
+    // problem with nothing to polish keep their first pick
+    if (n > 0 && next && lane < pp.njobs) const_cast<float *>(next)[pp.first_job + lane] = CUDART_NAN_F;
   }
-  n = __shfl_sync(0xffffffffu, n, 0);
-  __syncwarp();
-  // mark the problem's jobs for the second pick (a NaN in their next-value slots); the jobs of a
-  // problem with nothing to polish keep their first pick
-  if (n > 0 && next && lane < pp.njobs) const_cast<float *>(next)[pp.first_job + lane] = CUDART_NAN_F;
+  __syncthreads();
+  const int n = s_n;
   // the points, each once and in increasing order, several per pass for small factors (sub-warps
-  // of 8 or 16 lanes per point, as in the scan's refinement), else one per pass
+  // of 8 or 16 lanes per point, as in the scan's refinement), else one per pass; the warps take the
+  // passes in turn
   const bool sub8 = j.M <= 8 && j.Kf <= 8, sub16 = !sub8 && j.M <= 16 && j.Kf <= 16;
   const int per = sub8 ? 4 : (sub16 ? 2 : 1);
-  int last = -1, nb = 0;
+  int last = -1, nb = 0, turn = 0;
   auto flush = [&]() {
-    __syncwarp();
-    if (sub8)
-      refine_points_subwarp<8>(j, pts[warp], nb, UlaSource{&j}, w32[warp], ph[warp]);
-    else if (sub16)
-      refine_points_subwarp<16>(j, pts[warp], nb, UlaSource{&j}, w32[warp], ph[warp]);
-    else
-      refine_point_warp(j, pts[warp][0], w32[warp], ph[warp], yb[warp]);
-    __syncwarp();
+    if (turn == warp) {
+      __syncwarp();
+      if (sub8)
+        refine_points_subwarp<8>(j, pts[warp], nb, UlaSource{&j}, w32, ph[warp]);
+      else if (sub16)
+        refine_points_subwarp<16>(j, pts[warp], nb, UlaSource{&j}, w32, ph[warp]);
+      else
+        refine_point_warp(j, pts[warp][0], w32, ph[warp], yb[warp]);
+      __syncwarp();
+    }
+    turn = (turn + 1) % kPolishWarps;
     nb = 0;
   };
   for (int i = 0; i < n; ++i) {
-    const int k0 = pk[warp][i];
+    const int k0 = pk[i];
     for (int k = max(max(k0 - 2, last + 1), 0); k <= min(k0 + 2, L - 1); ++k) {
-      if (lane == 0) pts[warp][nb] = k;
+      if (lane == 0 && turn == warp) pts[warp][nb] = k;
       ++nb;
       last = k;
       if (nb == per) flush();
@@ -552,7 +562,7 @@ cudaError_t launch_scan_single(const double2 *B, int M, int K, int L, double lo,
 
 cudaError_t launch_polish_batch(const uint8_t *plan_dev, const PlanHeader &h, uint8_t *ws, cudaStream_t s) {
   if (h.nprob == 0) return cudaSuccess;
-  polish_batch_kernel<<<(h.nprob + kPolishWarps - 1) / kPolishWarps, 32 * kPolishWarps, 0, s>>>(plan_dev, ws);
+  polish_batch_kernel<<<h.nprob, 32 * kPolishWarps, 0, s>>>(plan_dev, ws);
   return cudaGetLastError();
 }
 
