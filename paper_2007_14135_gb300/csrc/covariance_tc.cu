@@ -7,20 +7,20 @@
 // columns produces the whole covariance in TMEM.
 //
 // Per CTA: TMA (cp.async.bulk.tensor, FP32, no swizzle) brings 32 snapshots of all M rows
-// (M x 64 floats) into a four-stage staging ring guarded by mbarriers; all threads split the FP32
+// (M x 64 floats) into a four-stage staging ring guarded by mbarriers; sixteen warps split the FP32
 // values into hi/lo 16-bit parts (BF16, or FP16 with the lo part scaled by 2^11) and write the
 // three operand views (Y and Z rows of A, Y rows of B) in the 128B-swizzled K-major layout; one
-// thread issues the MMAs (one product for DOA_BF16, hi*hi + hi*lo + lo*hi for the x3 forms, the
+// thread of a warp of its own issues the copies and the MMAs (one product for DOA_BF16, hi*hi + hi*lo + lo*hi for the x3 forms, the
 // FP16 cross terms into a second accumulator) and commits them to an mbarrier that releases the
 // operand buffer two stages later. A cluster of up to 8 CTAs splits the snapshots; each CTA reads
-// its accumulator with tcgen05.ld into shared memory and CTA rank 0 adds the partials in FP64
-// through distributed shared memory, keeps the upper triangle and mirrors it (Hermitian).
+// its accumulator with tcgen05.ld into shared memory, and every CTA adds the partials of some entries
+// in FP64 through distributed shared memory, keeps the upper triangle and mirrors it (Hermitian).
 // Accuracy: the split forms carry ~16 (BF16x3) or ~22 (FP16x3) significant bits per operand and
 // accumulate in FP32; this is the reduced-precision covariance of the large-array configuration.
-// An atom is bound by the splitting between two block barriers (its MMAs take 600 cycles): with 128
-// threads, the sixteen values of both operand views split apart and two atoms in flight it took 4900
-// cycles, 153 us for M = 64, N = 16384; with 512 threads, eight values each and four atoms @CT@ us. The
-// split over the cluster stays as it is: the FP32 accumulation truncates, so its order shows in R.
+// An atom takes about 1300 cycles, for its MMAs as for its splitting (M = 64, split forms). With 128
+// threads that split both operand views, issued the MMAs in between and let one CTA add all partials,
+// it took 4900 and the end of the kernel 47000: 153 us for M = 64, N = 16384, now 80 us. The split
+// over the cluster stays as it is: the FP32 accumulation truncates, so its order shows in R.
 #include <cooperative_groups.h>
 #include <cuda.h>
 #include <cudaTypedefs.h>
@@ -35,7 +35,8 @@ namespace {
 
 using namespace tc;
 
-constexpr int kCtThreads = 512;  // a thread per (row, 4 snapshots) of an atom at M = 64; four warps read TMEM
+constexpr int kCtSplit = 512;    // splitting threads: one per (row, 4 snapshots) of an atom at M = 64
+constexpr int kCtThreads = kCtSplit + 32;   // + the warp that issues the copies and the MMAs
 constexpr int kCtStages = 4;     // staged FP32 atoms
 constexpr int kCtCluster = 8;
 constexpr int kAtomSnap = 32;   // snapshots per K atom (64 reals = one 128-byte swizzle row)
@@ -94,7 +95,7 @@ __global__ void __launch_bounds__(kCtThreads, 1) covariance_tc_kernel(const __gr
                                                                       float2 *R, double2 *R64) {
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   uint8_t *sm = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  __shared__ __align__(8) uint64_t full_bar[kCtStages], mma_bar[2];
+  __shared__ __align__(8) uint64_t full_bar[kCtStages], ready_bar[2], mma_bar[2];
   __shared__ uint32_t tmem_base;
   __shared__ int s_ok;
   cg::cluster_group cluster = cg::this_cluster();
@@ -111,8 +112,10 @@ __global__ void __launch_bounds__(kCtThreads, 1) covariance_tc_kernel(const __gr
   if (tid == 0) {
     for (int s = 0; s < kCtStages; ++s)
       asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&full_bar[s])));
-    for (int s = 0; s < 2; ++s)
+    for (int s = 0; s < 2; ++s) {
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(&ready_bar[s])), "r"(kCtSplit));
       asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&mma_bar[s])));
+    }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     s_ok = 1;
   }
@@ -129,95 +132,94 @@ __global__ void __launch_bounds__(kCtThreads, 1) covariance_tc_kernel(const __gr
   const uint32_t idesc = inst_desc(prec == DOA_FP16X3 ? 0 : 1, lay.NP);
   const bool split = prec != DOA_BF16;
 
-  // prologue: the first atoms in flight (issued / consumed: bookkeeping of thread 0)
-  int issued = 0, consumed = 0;
-  if (tid == 0)
-    for (int s = 0; s < kCtStages && s < natoms; ++s, ++issued) {
-      mbar_expect(smem_u32(&full_bar[s]), (uint32_t)lay.stage_bytes);
-      tma_load_2d(smem_u32(sm + lay.off_stage[s]), &xmap, (a0 + s) * 2 * kAtomSnap, 0, smem_u32(&full_bar[s]));
-    }
   bool ok = true;
-  for (int i = 0; i < natoms; ++i) {
-    const int s = i & 1, f = i % kCtStages;
-    // the operand buffer s was last read by the MMAs of atom i - 2
-    bool good = ok;
-    if (good && i >= 2) good = mbar_wait(smem_u32(&mma_bar[s]), (uint32_t)(((i - 2) >> 1) & 1));
-    if (good) good = mbar_wait(smem_u32(&full_bar[f]), (uint32_t)((i / kCtStages) & 1));
-    ok = __syncthreads_and(good);
-    if (!ok) break;
-    consumed = i + 1;
-    // split the staged FP32 atom (M rows x 32 complex) into the three operand views
-    const float *stg = reinterpret_cast<const float *>(sm + lay.off_stage[f]);
-    uint8_t *ahi = sm + lay.off_ahi[s], *alo = sm + lay.off_alo[s];
-    uint8_t *bhi = sm + lay.off_bhi[s], *blo = sm + lay.off_blo[s];
-    // z's parts are y's with signs: rounding is symmetric, so their halves are y's halves with signs
-    for (int task = tid; task < M * 8; task += kCtThreads) {
-      const int r = task >> 3, ch = task & 7;        // row, chunk of 4 complex (8 reals)
-      const float4 u = *reinterpret_cast<const float4 *>(stg + r * 64 + ch * 8);
-      const float4 v = *reinterpret_cast<const float4 *>(stg + r * 64 + ch * 8 + 4);
-      const float y[8] = {u.x, u.y, u.z, u.w, v.x, v.y, v.z, v.w};
-      uint16_t yh[8], yl[8], zh[8], zl[8];
-#pragma unroll
-      for (int j = 0; j < 8; ++j) split16(y[j], prec, yh[j], yl[j]);
-#pragma unroll
-      for (int j = 0; j < 8; j += 2) {   // (re, im) -> (im, -re)
-        zh[j] = yh[j + 1];
-        zl[j] = yl[j + 1];
-        zh[j + 1] = yh[j] ^ 0x8000u;
-        zl[j + 1] = yl[j] ^ 0x8000u;
-      }
-      auto pack = [](const uint16_t (&h)[8]) {
-        return make_uint4(h[0] | ((uint32_t)h[1] << 16), h[2] | ((uint32_t)h[3] << 16), h[4] | ((uint32_t)h[5] << 16),
-                          h[6] | ((uint32_t)h[7] << 16));
-      };
-      const uint32_t offy = sw128(r, ch * 8), offz = sw128(M + r, ch * 8);
-      *reinterpret_cast<uint4 *>(ahi + offy) = pack(yh);
-      *reinterpret_cast<uint4 *>(ahi + offz) = pack(zh);
-      *reinterpret_cast<uint4 *>(bhi + offy) = pack(yh);
-      if (split) {
-        *reinterpret_cast<uint4 *>(alo + offy) = pack(yl);
-        *reinterpret_cast<uint4 *>(alo + offz) = pack(zl);
-        *reinterpret_cast<uint4 *>(blo + offy) = pack(yl);
-      }
-    }
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    __syncthreads();
-    if (tid == 0) {
-      // staging slot f is free again: fetch the atom that uses it next
-      if (i + kCtStages < natoms) {
+  if (warp == kCtSplit / 32) {
+    if (lane == 0) {   // copies and MMAs
+      int issued = 0, consumed = 0;
+      auto fetch = [&]() {
+        const int f = issued % kCtStages;
         mbar_expect(smem_u32(&full_bar[f]), (uint32_t)lay.stage_bytes);
-        tma_load_2d(smem_u32(sm + lay.off_stage[f]), &xmap, (a0 + i + kCtStages) * 2 * kAtomSnap, 0,
-                    smem_u32(&full_bar[f]));
+        tma_load_2d(smem_u32(sm + lay.off_stage[f]), &xmap, (a0 + issued) * 2 * kAtomSnap, 0, smem_u32(&full_bar[f]));
         ++issued;
+      };
+      while (issued < kCtStages && issued < natoms) fetch();
+      for (int i = 0; i < natoms; ++i) {
+        const int s = i & 1;
+        ok = mbar_wait(smem_u32(&ready_bar[s]), (uint32_t)((i >> 1) & 1));   // atom i is split
+        if (!ok) break;
+        consumed = i + 1;
+        if (issued < natoms) fetch();   // into the staging slot just read
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        const uint32_t pa = smem_u32(sm + lay.off_ahi[s]), pal = smem_u32(sm + lay.off_alo[s]),
+                       pb = smem_u32(sm + lay.off_bhi[s]), pbl = smem_u32(sm + lay.off_blo[s]);
+        for (int kk = 0; kk < 4; ++kk) {
+          const uint32_t off = kk * 32;
+          const uint32_t acc = (i > 0 || kk > 0) ? 1u : 0u;
+          mma(tmem, smem_desc(pa + off), smem_desc(pb + off), idesc, acc);
+          if (prec == DOA_BF16X3) {
+            mma(tmem, smem_desc(pa + off), smem_desc(pbl + off), idesc, 1u);
+            mma(tmem, smem_desc(pal + off), smem_desc(pb + off), idesc, 1u);
+          } else if (prec == DOA_FP16X3) {
+            mma(tmem + lay.NP, smem_desc(pa + off), smem_desc(pbl + off), idesc, acc);
+            mma(tmem + lay.NP, smem_desc(pal + off), smem_desc(pb + off), idesc, 1u);
+          }
+        }
+        asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
+                         smem_u32(&mma_bar[s]))
+                     : "memory");
       }
-      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      const uint32_t pa = smem_u32(ahi), pal = smem_u32(alo), pb = smem_u32(bhi), pbl = smem_u32(blo);
-      for (int kk = 0; kk < 4; ++kk) {
-        const uint32_t off = kk * 32;
-        const uint32_t acc = (i > 0 || kk > 0) ? 1u : 0u;
-        mma(tmem, smem_desc(pa + off), smem_desc(pb + off), idesc, acc);
-        if (prec == DOA_BF16X3) {
-          mma(tmem, smem_desc(pa + off), smem_desc(pbl + off), idesc, 1u);
-          mma(tmem, smem_desc(pal + off), smem_desc(pb + off), idesc, 1u);
-        } else if (prec == DOA_FP16X3) {
-          mma(tmem + lay.NP, smem_desc(pa + off), smem_desc(pbl + off), idesc, acc);
-          mma(tmem + lay.NP, smem_desc(pal + off), smem_desc(pb + off), idesc, 1u);
+      // after a timed-out wait, let the copies still in flight land before the CTA exits (bounded)
+      for (int a = consumed; a < issued; ++a)
+        mbar_wait(smem_u32(&full_bar[a % kCtStages]), (uint32_t)((a / kCtStages) & 1));
+      // the last commit covers every earlier MMA of this thread
+      if (natoms > 0 && ok) ok = mbar_wait(smem_u32(&mma_bar[(natoms - 1) & 1]), (uint32_t)(((natoms - 1) >> 1) & 1));
+    }
+  } else {
+    for (int i = 0; i < natoms; ++i) {
+      const int s = i & 1, f = i % kCtStages;
+      // the operand buffer s was last read by the MMAs of atom i - 2
+      if (i >= 2) ok = mbar_wait(smem_u32(&mma_bar[s]), (uint32_t)(((i - 2) >> 1) & 1));
+      if (ok) ok = mbar_wait(smem_u32(&full_bar[f]), (uint32_t)((i / kCtStages) & 1));
+      if (!ok) break;
+      // split the staged FP32 atom (M rows x 32 complex) into the three operand views
+      const float *stg = reinterpret_cast<const float *>(sm + lay.off_stage[f]);
+      uint8_t *ahi = sm + lay.off_ahi[s], *alo = sm + lay.off_alo[s];
+      uint8_t *bhi = sm + lay.off_bhi[s], *blo = sm + lay.off_blo[s];
+      // z's parts are y's with signs: rounding is symmetric, so their halves are y's halves with signs
+      for (int task = tid; task < M * 8; task += kCtSplit) {
+        const int r = task >> 3, ch = task & 7;        // row, chunk of 4 complex (8 reals)
+        const float4 u = *reinterpret_cast<const float4 *>(stg + r * 64 + ch * 8);
+        const float4 v = *reinterpret_cast<const float4 *>(stg + r * 64 + ch * 8 + 4);
+        const float y[8] = {u.x, u.y, u.z, u.w, v.x, v.y, v.z, v.w};
+        uint16_t yh[8], yl[8], zh[8], zl[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) split16(y[j], prec, yh[j], yl[j]);
+#pragma unroll
+        for (int j = 0; j < 8; j += 2) {   // (re, im) -> (im, -re)
+          zh[j] = yh[j + 1];
+          zl[j] = yl[j + 1];
+          zh[j + 1] = yh[j] ^ 0x8000u;
+          zl[j + 1] = yl[j] ^ 0x8000u;
+        }
+        auto pack = [](const uint16_t (&h)[8]) {
+          return make_uint4(h[0] | ((uint32_t)h[1] << 16), h[2] | ((uint32_t)h[3] << 16),
+                            h[4] | ((uint32_t)h[5] << 16), h[6] | ((uint32_t)h[7] << 16));
+        };
+        const uint32_t offy = sw128(r, ch * 8), offz = sw128(M + r, ch * 8);
+        *reinterpret_cast<uint4 *>(ahi + offy) = pack(yh);
+        *reinterpret_cast<uint4 *>(ahi + offz) = pack(zh);
+        *reinterpret_cast<uint4 *>(bhi + offy) = pack(yh);
+        if (split) {
+          *reinterpret_cast<uint4 *>(alo + offy) = pack(yl);
+          *reinterpret_cast<uint4 *>(alo + offz) = pack(zl);
+          *reinterpret_cast<uint4 *>(blo + offy) = pack(yl);
         }
       }
-      asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                       smem_u32(&mma_bar[s]))
-                   : "memory");
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&ready_bar[s])) : "memory");
     }
   }
-  // after a timed-out wait, let the copies still in flight land before the CTA exits (bounded)
-  if (!ok && tid == 0)
-    for (int a = consumed; a < issued; ++a)
-      mbar_wait(smem_u32(&full_bar[a % kCtStages]), (uint32_t)((a / kCtStages) & 1));
-  // drain: the last commit covers every earlier MMA of this thread
-  if (natoms > 0 && ok) {
-    const int il = natoms - 1;
-    ok = mbar_wait(smem_u32(&mma_bar[il & 1]), (uint32_t)((il >> 1) & 1));
-  }
+  __syncwarp();
   ok = __syncthreads_and(ok);
   if (tid == 0 && !ok) s_ok = 0;
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -243,11 +245,11 @@ __global__ void __launch_bounds__(kCtThreads, 1) covariance_tc_kernel(const __gr
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   cluster.sync();
-  if (rank == 0) {
+  {   // every CTA adds the partials of some of the entries, in rank order
     const double inv_n = 1.0 / (double)N;
     bool all_ok = true;
     for (int r = 0; r < nranks; ++r) all_ok = all_ok && *cluster.map_shared_rank(&s_ok, r);
-    for (int e = tid; e < M * M; e += kCtThreads) {
+    for (int e = rank * kCtThreads + tid; e < M * M; e += nranks * kCtThreads) {
       const int a = e / M, b = e % M;
       if (a > b) continue;
       double re = 0.0, im = 0.0;

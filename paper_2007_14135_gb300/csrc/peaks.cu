@@ -12,7 +12,7 @@
 // warps' lists. This realises the shared-memory max-reduction that the paper names as future work
 // for Step-6 (Sec. 6). With a cluster the quads are dealt over all its threads and rank 0 merges the
 // CTAs' lists through distributed shared memory in the same way: one CTA reads a long spectrum at the
-// rate its loads in flight allow (150 us for 360 001 points; the cluster: 33 us), which leaves most of
+// rate its loads in flight allow (150 us for 360 001 points; the cluster: 45 us), which leaves most of
 // the chip idle when the spectra are few, and trails the batch when a few are long.
 #include <cooperative_groups.h>
 
@@ -48,8 +48,7 @@ __device__ void write_sel(Cand *sel, int nsel, int *idx, float *val, int *count)
 
 namespace cg = cooperative_groups;
 constexpr int kPeakCluster = 8;
-constexpr int kClusterPoints = 16384;      // points from which a single call takes a cluster
-constexpr int kClusterLong = 65536;        // longest spectrum from which a batch does, whatever its jobs
+constexpr int kClusterPoints = 16384;      // points from which a spectrum takes a cluster
 
 // This CTA's share of a spectrum's quads: rank of kCs CTAs.
 template <int kCs>
@@ -160,7 +159,7 @@ __global__ void __launch_bounds__(kPeakThreads, 5) peaks_batch_kernel(const uint
     next = nullptr;
   }
   peaks_block<kCs>(pp.p.P + (size_t)jb.slot * L, L, d, pp.p.peak_idx + (size_t)jb.slot * d,
-              pp.p.peak_val + (size_t)jb.slot * d, pp.p.peak_count + jb.slot, next);
+                   pp.p.peak_val + (size_t)jb.slot * d, pp.p.peak_count + jb.slot, next);
 }
 
 template <int kCs>
@@ -300,15 +299,15 @@ cudaError_t launch_peaks2d_single(const float *P, int La, int Le, int wrap_az, i
 }
 
 // A batch takes clusters when its jobs do not fill the SMs (five CTAs each) and some spectrum is long
-// enough for a single call to take one, or when some spectrum is very long beside the others: 1024 mixed
-// jobs of up to 180 001 points, 0.15 -> @UNEVEN@ ms; 16384 jobs of 18 001 stay with a CTA each.
+// enough. For 1024 mixed jobs of up to 180 001 points clusters gain nothing (0.16 against 0.15 ms, 0.11
+// of it the launching of 8192 clustered CTAs).
 cudaError_t launch_peaks_batch(const uint8_t *plan_dev, const PlanHeader &h, uint8_t *ws, bool ula, bool geo,
                                cudaStream_t s) {
   int ngeo = 0;
   for (int b = 0; b < kNumBuckets; ++b) ngeo += h.geo_jobs[b];
   const int repick = ula && !geo;   // the call after the polish
   const bool few = (int64_t)h.njobs * kPeakCluster <= 5 * (int64_t)device_sm_count();
-  const bool cl = h.max_points >= (few ? kClusterPoints : kClusterLong);
+  const bool cl = few && h.max_points >= kClusterPoints;
   cudaError_t e = cudaSuccess;
   if (h.njobs > 0 && ula && ngeo < h.nprob)
     e = cl ? launch_jobs<kPeakCluster>(peaks_batch_kernel<kPeakCluster>, h.njobs, s, plan_dev, ws, repick)

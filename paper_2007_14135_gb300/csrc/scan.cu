@@ -374,7 +374,7 @@ __global__ void __launch_bounds__(kScanThreads, shared_min_blocks<MP, PT>())
 
 // Peak polish (DOA_FLAG_POLISH_PEAKS): one CTA per problem (its first warp picks the points, all warps
 // take them in turn; with a warp per problem, one problem of M = 32 with many peaks on a fine grid kept
-// its warp for 0.48 ms) re-evaluates, with the FP64
+// its warp for 0.48 ms, the CTA for 0.17) re-evaluates, with the FP64
 // steering and contraction of the scan's refinement (two or four points per pass in sub-warps
 // for small factors), every readout of the problem at the union of its algorithms' picked peaks
 // and their two neighbours on each side (each point once); the

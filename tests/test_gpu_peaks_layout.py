@@ -109,3 +109,31 @@ def test_peaks2d_every_offset(env, Le, La):
                     ri, rv = oracle.peaks2d(P.astype(np.float64), d, wrap)
                     assert gi.tolist() == ri.tolist(), (Le, La, wrap, off, d)
                     assert np.array_equal(gv.astype(np.float64), rv), (Le, La, wrap, off, d)
+
+
+@pytest.mark.parametrize("L,off,d", [(16383, 0, 5), (16384, 1, 7), (16389, 3, 63), (40003, 2, 1), (360001, 0, 8)])
+def test_peaks_cluster_matches_oracle(env, L, off, d):
+    """Spectra on both sides of the length from which a cluster of CTAs searches one, at several alignment
+    offsets, with plateaus: bit-exact indices and values, alone and in a batch of few long spectra."""
+    torch, doa = env
+    rng = np.random.default_rng(L + d)
+    P = rng.integers(1, 40 if d > 20 else 4000, size=L).astype(np.float32)      # ties and plateaus
+    buf = torch.zeros(L + off, dtype=torch.float32, device="cuda")
+    buf[off:].copy_(torch.from_numpy(P))
+    idx = torch.full((d,), -1, dtype=torch.int32, device="cuda")
+    val = torch.zeros(d, dtype=torch.float32, device="cuda")
+    cnt = torch.zeros(1, dtype=torch.int32, device="cuda")
+    doa.doa_peaks(buf[off:], d, idx, val, cnt, L=L)
+    torch.cuda.synchronize()
+    oi, ov = oracle.peaks(P.astype(np.float64), d)
+    n = int(cnt.item())
+    assert list(idx.cpu().numpy()[:n]) == list(oi)
+    assert np.array_equal(val.cpu().numpy()[:n].astype(np.float64), ov)
+    if L % 2 == 1 and L >= 16384:      # the 2-D rule on the same points as one wrapped row
+        i2 = torch.full((d,), -1, dtype=torch.int32, device="cuda")
+        doa.doa_peaks2d(buf[off:], L, 1, True, d, i2, val, cnt)
+        torch.cuda.synchronize()
+        w = (P > np.roll(P, 1)) & (P > np.roll(P, -1))
+        k = np.nonzero(w)[0]
+        k = np.sort(k[np.lexsort((k, -P[k]))][:d])
+        assert list(i2.cpu().numpy()[:int(cnt.item())]) == list(k)
