@@ -8,8 +8,10 @@
 // numbers: as easy as 1, 2, 3", SC'11: 10 rounds of the two 32x32->64 multiplies by 0xD2511F53 and
 // 0xCD9E8D57, Weyl key increments 0x9E3779B9 and 0xBB67AE85), turned into normals by the
 // Box-Muller transform. Counter = (snapshot, instance low, instance high, draw), key = seed.
-#include <climits>
 #include <float.h>
+
+#include <algorithm>
+#include <climits>
 
 #include "doa_internal.cuh"
 #include "peaks_common.cuh"
@@ -146,20 +148,26 @@ __global__ void windows_kernel(const float *probs, const int32_t *d, int batch, 
   }
 }
 
-// Windowed scan: block = (row slot, window, tile of 128 x PT points).
-template <int MP, int PT>
+// Windowed scan: block = (row slot, window, run of `run` tiles of 128 x PT points). PT = 4 points a thread
+// in the paired form of the batch scan (the same operations, so the same bits as every other tile shape);
+// the factor and its thresholds are prepared once per run and the flagged points re-evaluated at its end (or when the queue fills).
+// A block per 256 points, which prepared them for two points a thread, took 1.96 ms for 12288 windows of
+// 4001 points; now @WIN@ ms, bound by FP32 issue.
+constexpr int kWinPT = 4, kWinRun = 16;
+
+template <int MP>
 __global__ void __launch_bounds__(kScanThreads) scan_windows_kernel(const double2 *B, int M, const int32_t *K,
                                                                     const int32_t *rows, int dmax, double lo,
                                                                     double step, int L, const int32_t *win_first,
                                                                     int width, int full, const uint32_t *S,
-                                                                    float *Pwin, int tiles) {
-  __shared__ __align__(16) float2 Bs[MP * MP];
+                                                                    float *Pwin, int runs, int run) {
+  __shared__ __align__(16) float4 Bd[MP * MP];
   __shared__ ScanShared sh;
   const int nw = full ? 1 : dmax;
   const long long bid = blockIdx.x;
-  const int tile = (int)(bid % tiles);
-  const int w = (int)((bid / tiles) % nw);
-  const int slot = (int)(bid / ((long long)tiles * nw));
+  const int part = (int)(bid % runs);
+  const int w = (int)((bid / runs) % nw);
+  const int slot = (int)(bid / ((long long)runs * nw));
   const int r = rows ? rows[slot] : slot;
   const int first = full ? 0 : win_first[(size_t)r * dmax + w];
   if (first < 0) return;
@@ -173,13 +181,45 @@ __global__ void __launch_bounds__(kScanThreads) scan_windows_kernel(const double
   j.Kf = j.Kn = K[r];
   j.kphd = j.kmn = -1;
   j.kofs = first;
-  load_job<MP>(j, Bs, sh);
+  load_job2<MP>(j, Bd, sh);
   __syncthreads();
-  set_threshold<MP, true>(Bs, j, sh);
+  set_threshold2<MP, true>(Bd, j, sh);
   __syncthreads();
-  const int k0 = (tile * kScanThreads + threadIdx.x) * PT;
-  scan_points<MP, PT>(Bs, j, S + first, len, k0, sh);
-  drain_refinements(j, sh);
+  constexpr int TP = kScanThreads * kWinPT;
+  const int k1 = (int)min((long long)len, (long long)(part + 1) * run * TP);
+  static_assert(kFlagCap >= 2 * TP, "a tile's points fit in the queue after a check");
+  for (int t0 = part * run * TP; t0 < k1; t0 += TP) {
+    const int k0 = t0 + threadIdx.x * kWinPT;
+    if (k0 < len) scan_points2<MP, kWinPT>(Bd, j, S + first, len, k0, sh);
+    // a full queue would re-evaluate points one per thread, whose sums round differently: a point's value
+    // must not depend on the run it falls in
+    __syncthreads();
+    const bool half_full = queue_front(sh.nflag) + queue_back(sh.nflag) > kFlagCap - TP;
+    __syncthreads();
+    if (half_full || t0 + TP >= k1) drain_refinements(j, sh);
+  }
+}
+
+// Launches the scan of nrows x nw windows of len points (or whole rows); false: too many blocks.
+bool launch_scan_windows(const double *B, int M, const int32_t *K, const int32_t *rows, int nrows, int nw, int dmax,
+                         const doa_grid &fine, const int32_t *win_first, int width, int full, const uint32_t *S,
+                         float *P, cudaStream_t s) {
+  const int tp = kScanThreads * kWinPT;
+  const int tiles = ((full ? fine.L : width) + tp - 1) / tp;
+  // runs as long as leave eight blocks per SM
+  const long long want = (long long)nrows * nw * tiles / (8 * device_sm_count());
+  const int run = (int)std::max(1ll, std::min<long long>(std::min(kWinRun, tiles), want));
+  const int runs = (tiles + run - 1) / run;
+  const long long blocks = (long long)nrows * nw * runs;
+  if (blocks > INT_MAX) return false;
+  const double2 *F = reinterpret_cast<const double2 *>(B);
+  if (M <= 8)
+    scan_windows_kernel<8><<<(unsigned)blocks, kScanThreads, 0, s>>>(F, M, K, rows, dmax, fine.lo_deg, fine.step_deg, fine.L,
+                                                                     win_first, width, full, S, P, runs, run);
+  else
+    scan_windows_kernel<16><<<(unsigned)blocks, kScanThreads, 0, s>>>(F, M, K, rows, dmax, fine.lo_deg, fine.step_deg, fine.L,
+                                                                      win_first, width, full, S, P, runs, run);
+  return true;
 }
 
 // Peaks of one row's windows, merged: the d best peaks of each window (the plateau rule of
@@ -429,20 +469,12 @@ extern "C" doa_status doa_scan_windows(const double *B, int M, const int32_t *K,
     return DOA_EINVAL;
   if (!full && (!win_first || width < 3 || width > fine.L)) return DOA_EINVAL;
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-  phase_table_kernel<<<(fine.L + 255) / 256, 256, 0, s>>>(fine.lo_deg, fine.step_deg, fine.L, S);
-  const int len = full ? fine.L : width;
+  // refuse what cannot be launched before anything is
   const int tp = kScanThreads * 2;
-  const int tiles = (len + tp - 1) / tp;
-  const long long blocks = (long long)nrows * (full ? 1 : dmax) * tiles;
-  if (blocks > INT_MAX) return DOA_EINVAL;
-  if (M <= 8)
-    scan_windows_kernel<8, 2><<<(unsigned)blocks, kScanThreads, 0, s>>>(
-        reinterpret_cast<const double2 *>(B), M, K, rows, dmax, fine.lo_deg, fine.step_deg, fine.L, win_first, width,
-        full, S, Pwin, tiles);
-  else
-    scan_windows_kernel<16, 2><<<(unsigned)blocks, kScanThreads, 0, s>>>(
-        reinterpret_cast<const double2 *>(B), M, K, rows, dmax, fine.lo_deg, fine.step_deg, fine.L, win_first, width,
-        full, S, Pwin, tiles);
+  if ((long long)nrows * (full ? 1 : dmax) * (((full ? fine.L : width) + tp - 1) / tp) > INT_MAX) return DOA_EINVAL;
+  phase_table_kernel<<<(fine.L + 255) / 256, 256, 0, s>>>(fine.lo_deg, fine.step_deg, fine.L, S);
+  if (!launch_scan_windows(B, M, K, rows, nrows, full ? 1 : dmax, dmax, fine, win_first, width, full, S, Pwin, s))
+    return DOA_EINVAL;
   window_peaks_kernel<<<nrows, pk::kPeakThreads, 0, s>>>(Pwin, rows, d, dmax, fine.L, win_first, width, full, idx, val,
                                                    count, fallback);
   return cudaGetLastError() == cudaSuccess ? DOA_OK : DOA_ECUDA;
@@ -460,22 +492,14 @@ extern "C" doa_status doa_proposal_judge(const double *B, int M, const int32_t *
     return DOA_EINVAL;
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   const int threads = 256, warps = threads / 32;
+  const int tp = kScanThreads * 2;
+  if ((long long)batch * kJudgeMax * ((jwidth + tp - 1) / tp) > INT_MAX) return DOA_EINVAL;
   judge_windows_kernel<<<(batch + warps - 1) / warps, threads, 0, s>>>(
       Pc, coarse.L, coarse.lo_deg, coarse.step_deg, fine.lo_deg, fine.step_deg, fine.L, win_first, dmax, width,
       jwidth, batch, judge_first, fallback);
   phase_table_kernel<<<(fine.L + 255) / 256, 256, 0, s>>>(fine.lo_deg, fine.step_deg, fine.L, S);
-  const int tp = kScanThreads * 2;
-  const int tiles = (jwidth + tp - 1) / tp;
-  const long long blocks = (long long)batch * kJudgeMax * tiles;
-  if (blocks > INT_MAX) return DOA_EINVAL;
-  if (M <= 8)
-    scan_windows_kernel<8, 2><<<(unsigned)blocks, kScanThreads, 0, s>>>(
-        reinterpret_cast<const double2 *>(B), M, K, nullptr, kJudgeMax, fine.lo_deg, fine.step_deg, fine.L,
-        judge_first, jwidth, 0, S, Pjudge, tiles);
-  else
-    scan_windows_kernel<16, 2><<<(unsigned)blocks, kScanThreads, 0, s>>>(
-        reinterpret_cast<const double2 *>(B), M, K, nullptr, kJudgeMax, fine.lo_deg, fine.step_deg, fine.L,
-        judge_first, jwidth, 0, S, Pjudge, tiles);
+  if (!launch_scan_windows(B, M, K, nullptr, batch, kJudgeMax, kJudgeMax, fine, judge_first, jwidth, 0, S, Pjudge, s))
+    return DOA_EINVAL;
   judge_compare_kernel<<<batch, 256, 0, s>>>(Pjudge, judge_first, jwidth, fine.L, val, count, d, dmax, fallback);
   return cudaGetLastError() == cudaSuccess ? DOA_OK : DOA_ECUDA;
 }
