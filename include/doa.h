@@ -439,7 +439,9 @@ typedef struct {
   int32_t scan_group[4]; /* FP32 ULA problems that share a grid are scanned together in groups  */
                          /* of this many (one steering generation per tile of the grid for the   */
                          /* whole group, each problem's factor contracted in turn); 1 scans every */
-                         /* problem alone. Allowed powers of two 1..32; default 32.              */
+                         /* problem alone. Allowed powers of two 1..32; default 32. Geometry     */
+                         /* problems of M <= 16 that share positions and grid are grouped alike, */
+                         /* when there are enough of them (fewer are scanned alone).             */
 } doa_tuning;
 
 /*

@@ -246,7 +246,7 @@ bool count_plan(const doa_problem *probs, int nprob, PlanSizes &sz, std::vector<
 
 struct PlanOffsets {
   int64_t prob, job, grid, cov, reduce, eig[kNumBuckets], scan[kNumBuckets], tc, geo[kNumBuckets], geo_grid,
-      geo_steer, covtc[2], sg[kNumBuckets], sgl[kNumBuckets], tcg, tcc, tcgl, total;
+      geo_steer, covtc[2], sg[kNumBuckets], sgl[kNumBuckets], tcg, tcc, tcgl, gg[kNumBuckets], ggl[kNumBuckets], total;
 };
 
 PlanOffsets plan_offsets(const PlanSizes &sz) {
@@ -299,6 +299,13 @@ PlanOffsets plan_offsets(const PlanSizes &sz) {
   at = round_up(at + (int64_t)sz.tc * sizeof(PlanTcChunk), 16);
   o.tcgl = at;
   at = round_up(at + (int64_t)sz.tc * 4, 16);
+  // shared-steering geometry groups: room for every geometry problem of the bucket
+  for (int b = 0; b < kNumBuckets; ++b) {
+    o.gg[b] = at;
+    at = round_up(at + (int64_t)sz.geo[b] * sizeof(PlanScanGroup), 16);
+    o.ggl[b] = at;
+    at = round_up(at + (int64_t)sz.geo[b] * 4, 16);
+  }
   o.total = at;
   return o;
 }
@@ -640,6 +647,24 @@ doa_status doa_batch_plan(const doa_problem *probs, int nprob, const doa_tuning 
   auto tc_grouped = [&](int i) {
     return ula_tc(probs[i]) && sgsize[m_bucket(probs[i].M)] > 1 && tc_sharers[tc_key(i)].size() >= 2;
   };
+  // shared-steering geometry scan: the problems of one steering table in groups of at most sg_size[b],
+  // of fewer where the table's problems would not fill the chip with units otherwise (geo_gsize[t] = 0:
+  // scanned one by one)
+  std::vector<std::vector<int32_t>> steer_sharers((size_t)sz.ngeo_steer);
+  std::vector<int> geo_gsize((size_t)sz.ngeo_steer, 0);
+  for (int i = 0; i < nprob; ++i)
+    if (probs[i].geom.pos && steer_of[i] >= 0) steer_sharers[steer_of[i]].push_back(i);
+  auto geo_tiles_of = [&](int t) {
+    const int tp = kScanThreads * geo_group_pt(m_bucket(pst[t].M));
+    return (int64_t)(pst[t].npts + tp - 1) / tp;
+  };
+  for (int t = 0; t < sz.ngeo_steer; ++t) {
+    const int b = m_bucket(pst[t].M);
+    if (geo_group_pt(b) == 0) continue;
+    const int64_t units = geo_tiles_of(t) * (int64_t)steer_sharers[t].size();
+    const int64_t gs = std::min<int64_t>(sgsize[b], units / kGeoGroupMinUnits);
+    geo_gsize[t] = gs >= geo_group_min(b) ? (int)gs : 0;
+  }
   for (int i = 0; i < nprob; ++i) {
     const doa_problem &p = probs[i];
     PlanProblem &q = pp[i];
@@ -684,10 +709,14 @@ doa_status doa_batch_plan(const doa_problem *probs, int nprob, const doa_tuning 
     q.fac_off = ws;
     ws = round_up(ws + factor_bytes(M), 256);
     if (p.geom.pos) {
-      const int tp = kScanThreads * pt[b];
-      q.tile_start = h.geo_tiles[b];
-      h.geo_tiles[b] += (q.npts + tp - 1) / tp;
-      geo[b][h.geo_jobs[b]++] = i;
+      ++h.geo_jobs[b];
+      q.tile_start = 0;
+      if (q.geo_steer < 0 || geo_gsize[q.geo_steer] == 0) {
+        const int tp = kScanThreads * pt[b];
+        q.tile_start = h.geo_tiles[b];
+        h.geo_tiles[b] += (q.npts + tp - 1) / tp;
+        geo[b][h.geo_alone[b]++] = i;
+      }
     } else if (grouped(i) || tc_grouped(i)) {
       q.tile_start = 0;   // scanned by its group (grid-shared scan)
     } else if (p.prec == DOA_FP32) {
@@ -731,6 +760,30 @@ doa_status doa_batch_plan(const doa_problem *probs, int nprob, const doa_tuning 
         h.sg_units[b] += e.tiles;
         for (int q = 0; q < e.count; ++q) sgl[h.sg_probs[b]++] = v[f + q];
       }
+    }
+  }
+  // the geometry groups, table by table, of nearly equal sizes
+  for (int b = 0; b < kNumBuckets; ++b) {
+    h.off_gg[b] = o.gg[b];
+    h.off_ggl[b] = o.ggl[b];
+  }
+  for (int t = 0; t < sz.ngeo_steer; ++t) {
+    if (geo_gsize[t] == 0) continue;
+    const int b = m_bucket(pst[t].M);
+    PlanScanGroup *grp = reinterpret_cast<PlanScanGroup *>(base + o.gg[b]);
+    int32_t *ggl = reinterpret_cast<int32_t *>(base + o.ggl[b]);
+    const std::vector<int32_t> &v = steer_sharers[t];
+    const int64_t ng = ((int64_t)v.size() + geo_gsize[t] - 1) / geo_gsize[t];
+    for (int64_t k = 0; k < ng; ++k) {
+      const size_t f0 = v.size() * (size_t)k / (size_t)ng, f1 = v.size() * (size_t)(k + 1) / (size_t)ng;
+      PlanScanGroup &e = grp[h.gg_groups[b]++];
+      e.grid_id = t;
+      e.first = h.gg_probs[b];
+      e.count = (int32_t)(f1 - f0);
+      e.tiles = (int32_t)geo_tiles_of(t);
+      e.unit_start = h.gg_units[b];
+      h.gg_units[b] += e.tiles;
+      for (size_t q = f0; q < f1; ++q) ggl[h.gg_probs[b]++] = v[q];
     }
   }
   // tensor-core groups: each key's problems in order, packed while their columns (2 Kf rounded

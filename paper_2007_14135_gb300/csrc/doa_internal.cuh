@@ -235,7 +235,7 @@ constexpr int kSteerAlign = 1024;   // row stride multiple: every scan tile's po
 // generated once and contracted with each problem's factor in turn). Units are numbered group by
 // group from unit_start.
 struct PlanScanGroup {
-  int32_t grid_id;
+  int32_t grid_id;        // grid; of the shared-steering geometry scan, the steering table
   int32_t first;          // first entry of the group in the bucket's problem list
   int32_t count;          // problems in the group (<= kScanGroupMax)
   int32_t tiles;          // tiles of kScanThreads x scan_pt points covering the grid
@@ -281,6 +281,16 @@ constexpr int64_t kTcgRecBytes = 2 * kTcgWBytes + kTcgMaxProbs * (int64_t)sizeof
 
 constexpr int kScanGroupMax = 32;       // problems per group (their jobs are staged in shared memory)
 constexpr int kScanGroupDefault = 32;
+// Shared-steering geometry scan: points per thread of a bucket's unit (0: its problems are scanned
+// one by one; the phasors of two points of M > 16 elements no longer fit a thread's registers), the
+// units a table's problems are split into at least (with fewer, sharing the table's reads leaves SMs
+// without work), and the smallest group worth a preparation launch. Batches of one circular array,
+// 360 x 90 points, whole solves one by one / in groups: M = 8, 4096 problems 2387 / 2217 us, 1024
+// 725 / 695, 256 (groups of 13) 297 / 294, 64 (groups of 3) 174 / 188; M = 16, 1024 problems
+// 2400 / 2158, 64 (groups of 6) 506 / 426; M = 12, 64 (6) 346 / 326, 32 (3) 277 / 290.
+__host__ __device__ constexpr int geo_group_pt(int bucket) { return bucket == 0 ? 4 : bucket == 1 ? 2 : 0; }
+constexpr int64_t kGeoGroupMinUnits = 1216;
+__host__ __device__ constexpr int geo_group_min(int bucket) { return bucket == 0 ? 16 : 4; }
 __host__ __device__ inline bool scan_group_allowed(int g) { return g >= 1 && g <= kScanGroupMax && (g & (g - 1)) == 0; }
 
 struct PlanCovItem {
@@ -347,12 +357,21 @@ struct PlanHeader {
   int32_t tcg_pad;
   int64_t tcg_units;                     // (tile, chunk) units
   int64_t off_tcg, off_tcc, off_tcgl;    // PlanTcGroup, PlanTcChunk arrays and the problem list
+  // shared-steering geometry scan, per M bucket (the problems of these groups are counted in geo_jobs
+  // but are not in the per-problem lists, which hold geo_alone problems)
+  int32_t gg_groups[kNumBuckets];
+  int32_t gg_probs[kNumBuckets];         // problems in the groups
+  int32_t geo_alone[kNumBuckets];
+  int64_t gg_units[kNumBuckets];
+  int64_t off_gg[kNumBuckets];           // PlanScanGroup arrays (grid_id: the shared steering table)
+  int64_t off_ggl[kNumBuckets];          // their problem lists
 };
 
 // The Python binding reads these header fields by position (int32 index 22 = scan_pt, 58 = eig_mats,
 // 62 = cov_first, 67 = tc_jobs, 74 = npolish, 76 = geo_jobs, 96 = ngeo_grids, 100 = nrefine,
 // 101 = nroots, 104 = ngeo_steer, 108 = ncovtc, 114 = covtc_flag_off (int64), 116 = sg_size,
-// 120 = sg_groups, 124 = sg_units (int64), 148 = sg_probs, 152 = tcg_groups, 156 = tcg_units (int64)).
+// 120 = sg_groups, 124 = sg_units (int64), 148 = sg_probs, 152 = tcg_groups, 156 = tcg_units (int64),
+// 172 = geo_alone, 176 = gg_units (int64)).
 static_assert(offsetof(PlanHeader, scan_pt) == 88, "PlanHeader layout changed");
 static_assert(offsetof(PlanHeader, scan_tiles) == 56, "PlanHeader layout changed");
 static_assert(offsetof(PlanHeader, eig_mats) == 232, "PlanHeader layout changed");
@@ -370,8 +389,10 @@ static_assert(offsetof(PlanHeader, covtc_flag_off) == 456, "PlanHeader layout ch
 static_assert(offsetof(PlanHeader, sg_size) == 464 && offsetof(PlanHeader, sg_units) == 496 &&
                   offsetof(PlanHeader, sg_probs) == 592,
               "PlanHeader layout changed");
-static_assert(offsetof(PlanHeader, tcg_groups) == 608 && offsetof(PlanHeader, tcg_units) == 624 &&
-                  sizeof(PlanHeader) == 656,
+static_assert(offsetof(PlanHeader, tcg_groups) == 608 && offsetof(PlanHeader, tcg_units) == 624,
+              "PlanHeader layout changed");
+static_assert(offsetof(PlanHeader, geo_alone) == 688 && offsetof(PlanHeader, gg_units) == 704 &&
+                  sizeof(PlanHeader) == 800,
               "PlanHeader layout changed");
 
 // Scan tiles: kScanThreads threads, each evaluating PT consecutive grid points (tile shape
@@ -409,10 +430,10 @@ cudaError_t ensure_smem_attr(const void *func, int bytes);
 int device_sm_count();
 // The first bytes of a batch workspace hold per-solve counters (uint32, zeroed at the start of
 // every doa_solve_batch): the next unit of the grid-shared FP32 scan (slot bucket), the next run
-// of the per-problem FP32 scan (slot 4 + bucket) and the next unit of the grid-shared
-// tensor-core scan (slot 8).
+// of the per-problem FP32 scan (slot 4 + bucket), the next unit of the grid-shared
+// tensor-core scan (slot 8) and of the shared-steering geometry scan (slot 12 + bucket).
 constexpr int64_t kWsCounterBytes = 256;
-constexpr int kCtrShared = 0, kCtrBatch = 4, kCtrTcg = 8;
+constexpr int kCtrShared = 0, kCtrBatch = 4, kCtrTcg = 8, kCtrGeo = 12;
 // Shared memory of the current device: per SM, per block (opt-in maximum), reserved per block.
 struct SmemLimits {
   int per_sm, per_block, reserve;

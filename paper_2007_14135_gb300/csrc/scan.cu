@@ -210,15 +210,6 @@ __global__ void __launch_bounds__(kScanThreads) scan_prep_kernel(const uint8_t *
   if (lane < 4) w32[MP + lane] = thr[lane];
 }
 
-// 16-byte global -> shared copies that complete asynchronously (one group per problem).
-__device__ __forceinline__ void cp_async16(void *dst, const void *src) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"((uint32_t)__cvta_generic_to_shared(dst)),
-               "l"(src)
-               : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;\n" ::: "memory"); }
-
 // CTAs per SM the register budget of the grid-shared scan is set for: 4 where the steering of a
 // thread's points fits in 128 registers without spilling, else 3.
 template <int MP, int PT>
@@ -331,44 +322,7 @@ __global__ void __launch_bounds__(kScanThreads, shared_min_blocks<MP, PT>())
           contract_points<MP, PT, UlaSource, true>(Bs, j, a, L, k0, sh, UlaSource{&j}, Wsm[0], Wsm[0] + MP, tags, i);
       }
     }
-    // FP64 re-evaluation of the unit's flagged points, several per warp for small factors; the
-    // queue holds the points of each problem together (problems run one after the other)
-    __syncthreads();
-    const int n = queue_front(sh.nflag), nb = queue_back(sh.nflag);
-    for (int i0 = warp * 4; i0 < n; i0 += kScanWarps * 4) {
-      const int end = min(i0 + 4, n);
-      for (int c0 = i0; c0 < end;) {
-        const int tag = tags[c0];
-        int c1 = c0 + 1;
-        while (c1 < end && tags[c1] == tag) ++c1;
-        const ScanJob &j = jobs[tag];
-        const float *wg = reinterpret_cast<const float *>(reinterpret_cast<const uint8_t *>(j.F) + fac32_off(j.M) +
-                                                          (size_t)(j.M + 1) * MP * 16);
-        const UlaSource src{&j};
-        if (j.M <= 8 && j.Kf <= 8) {
-          refine_points_subwarp<8>(j, sh.flags + c0, c1 - c0, src, wg, sh.ph[warp]);
-        } else if (j.M <= 16 && j.Kf <= 16) {
-          for (int c = c0; c < c1; c += 2) refine_points_subwarp<16>(j, sh.flags + c, min(2, c1 - c), src, wg, sh.ph[warp]);
-        } else {
-          for (int c = c0; c < c1; ++c) refine_point_warp_src(j, sh.flags[c], src, wg, sh.ph[warp], sh.yb[warp]);
-        }
-        c0 = c1;
-      }
-    }
-    // points flagged for PHD / MN alone (the back of the queue): those columns only
-    for (int i0 = kFlagCap - nb + warp * 4; i0 < kFlagCap; i0 += kScanWarps * 4) {
-      const int end = min(i0 + 4, kFlagCap);
-      for (int c0 = i0; c0 < end;) {
-        const int tag = tags[c0];
-        int c1 = c0 + 1;
-        while (c1 < end && tags[c1] == tag) ++c1;
-        const ScanJob &j = jobs[tag];
-        refine_single_run(j, sh.flags + c0, sh.fmask + c0, c1 - c0, UlaSource{&j});
-        c0 = c1;
-      }
-    }
-    __syncthreads();
-    if (tid == 0) sh.nflag = 0;
+    drain_tagged<MP>(jobs, tags, sh, [](const ScanJob &j) { return UlaSource{&j}; });
   }
 }
 

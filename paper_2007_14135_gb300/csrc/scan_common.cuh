@@ -431,6 +431,65 @@ __device__ __forceinline__ void drain_refinements(const ScanJob &j, ScanShared &
   drain_refinements_src(j, UlaSource{&j}, sh);
 }
 
+// FP32 copy of a grouped problem's EV weights and thresholds, behind its factor copy (fac32_off).
+template <int MP>
+__device__ __forceinline__ const float *job_w32(const ScanJob &j) {
+  return reinterpret_cast<const float *>(reinterpret_cast<const uint8_t *>(j.F) + fac32_off(j.M) +
+                                         (size_t)(j.M + 1) * MP * 16);
+}
+
+// Drains the queue of a unit that holds the points of several problems (all threads of the CTA call
+// this): tags[] names each entry's job, src_of(job) its FP64 steering source. Several points per warp
+// for small factors; the entries of each problem are together (problems run one after the other).
+template <int MP, class SrcOf>
+__device__ __forceinline__ void drain_tagged(const ScanJob *jobs, const uint8_t *tags, ScanShared &sh, SrcOf src_of) {
+  const int warp = threadIdx.x >> 5;
+  __syncthreads();
+  const int n = queue_front(sh.nflag), nb = queue_back(sh.nflag);
+  for (int i0 = warp * 4; i0 < n; i0 += kScanWarps * 4) {
+    const int end = min(i0 + 4, n);
+    for (int c0 = i0; c0 < end;) {
+      const int tag = tags[c0];
+      int c1 = c0 + 1;
+      while (c1 < end && tags[c1] == tag) ++c1;
+      const ScanJob &j = jobs[tag];
+      const float *wg = job_w32<MP>(j);
+      const auto src = src_of(j);
+      if (j.M <= 8 && j.Kf <= 8) {
+        refine_points_subwarp<8>(j, sh.flags + c0, c1 - c0, src, wg, sh.ph[warp]);
+      } else if (j.M <= 16 && j.Kf <= 16) {
+        for (int c = c0; c < c1; c += 2) refine_points_subwarp<16>(j, sh.flags + c, min(2, c1 - c), src, wg, sh.ph[warp]);
+      } else {
+        for (int c = c0; c < c1; ++c) refine_point_warp_src(j, sh.flags[c], src, wg, sh.ph[warp], sh.yb[warp]);
+      }
+      c0 = c1;
+    }
+  }
+  // points flagged for PHD / MN alone (the back of the queue): those columns only
+  for (int i0 = kFlagCap - nb + warp * 4; i0 < kFlagCap; i0 += kScanWarps * 4) {
+    const int end = min(i0 + 4, kFlagCap);
+    for (int c0 = i0; c0 < end;) {
+      const int tag = tags[c0];
+      int c1 = c0 + 1;
+      while (c1 < end && tags[c1] == tag) ++c1;
+      const ScanJob &j = jobs[tag];
+      refine_single_run(j, sh.flags + c0, sh.fmask + c0, c1 - c0, src_of(j));
+      c0 = c1;
+    }
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) sh.nflag = 0;
+}
+
+// 16-byte global -> shared copies that complete asynchronously (one group per problem).
+__device__ __forceinline__ void cp_async16(void *dst, const void *src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"((uint32_t)__cvta_generic_to_shared(dst)),
+               "l"(src)
+               : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
+__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;\n" ::: "memory"); }
+
 template <int PT>
 __device__ __forceinline__ void store_row(float *P, int L, int k0, const float (&out)[PT]) {
   if (PT == 4 && k0 + 3 < L && ((reinterpret_cast<uintptr_t>(P + k0) & 15u) == 0)) {
@@ -448,8 +507,8 @@ __device__ __forceinline__ void store_row(float *P, int L, int k0, const float (
 // present readout, and every point where some readout's den is below its refinement threshold
 // queued for drain_refinements_src (or, on queue overflow, re-evaluated in place from src). With
 // kExt every queued point also records `tag` in tags[] (the grid-shared scan queues the points of
-// several problems).
-template <int PT, class Src, bool kExt>
+// several problems). kRoom: the caller keeps room in the queue for every point.
+template <int PT, class Src, bool kExt, bool kRoom = false>
 __device__ __forceinline__ void finish_points(const ScanJob &j, const float (&dp)[PT], const float (&dm)[PT],
                                               const float (&de)[PT], const float (&dn)[PT], int L, int k0,
                                               ScanShared &sh, const Src &src, const float *w32, const float *thr_,
@@ -472,6 +531,10 @@ __device__ __forceinline__ void finish_points(const ScanJob &j, const float (&dp
   DOA_READOUT(kRoEv, de)
   DOA_READOUT(kRoMn, dn)
 #undef DOA_READOUT
+  unsigned any = 0u;
+#pragma unroll
+  for (int q = 0; q < PT; ++q) any |= mk[q];
+  if (any == 0u) return;
   bool over[PT];
 #pragma unroll
   for (int q = 0; q < PT; ++q) {
@@ -483,7 +546,7 @@ __device__ __forceinline__ void finish_points(const ScanJob &j, const float (&dp
       const unsigned inc = whole ? 1u : 0x10000u;
       const unsigned old = atomicAdd(&sh.nflag, inc);
       const int f = queue_front(old), b = queue_back(old);
-      if (f + b < kFlagCap) {
+      if (kRoom || f + b < kFlagCap) {
         const int slot = whole ? f : kFlagCap - 1 - b;
         sh.flags[slot] = k0 + q;
         sh.fmask[slot] = (uint8_t)mk[q];
@@ -495,6 +558,7 @@ __device__ __forceinline__ void finish_points(const ScanJob &j, const float (&dp
     }
   }
   // queue overflow (more than kFlagCap small denominators before a drain): refine in place
+  if constexpr (kRoom) return;
 #pragma unroll
   for (int q = 0; q < PT; ++q)
     if (over[q]) refine_point_thread_src(j, k0 + q, src, w32);
@@ -605,8 +669,8 @@ __device__ __forceinline__ uint64_t f2sub(uint64_t a, uint64_t b) {
 // ay[p][m] holding Re / Im of a_m at points k0 + 2p and k0 + 2p + 1. Per element and pair, four
 // paired FMAs: yr += bx ax + by ay, yi_a += bx ay, yi_b += by ax (yi = yi_a - yi_b at the end of the
 // column), so every FMA of the contraction is half an instruction. Readouts, thresholds and the
-// refinement queue are those of contract_points.
-template <int MP, int PT, class Src, bool kExt = false>
+// refinement queue are those of contract_points (kRoom: of finish_points).
+template <int MP, int PT, class Src, bool kExt = false, bool kRoom = false>
 __device__ __forceinline__ void contract_points2(const float4 *Bd, const ScanJob &j, const uint64_t (&ax)[PT / 2][MP],
                                                  const uint64_t (&ay)[PT / 2][MP], int L, int k0, ScanShared &sh,
                                                  const Src &src, const float *w32x = nullptr,
@@ -674,7 +738,7 @@ __device__ __forceinline__ void contract_points2(const float4 *Bd, const ScanJob
     fe[2 * q] = f2lo(de[q]), fe[2 * q + 1] = f2hi(de[q]);
     fn[2 * q] = f2lo(dn[q]), fn[2 * q + 1] = f2hi(dn[q]);
   }
-  finish_points<PT, Src, kExt>(j, fp, fm, fe, fn, L, k0, sh, src, w32, thr_, tags, tag);
+  finish_points<PT, Src, kExt, kRoom>(j, fp, fm, fe, fn, L, k0, sh, src, w32, thr_, tags, tag);
 }
 
 // ---------------------------------------------------------------------------------------------

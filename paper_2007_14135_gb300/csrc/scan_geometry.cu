@@ -105,8 +105,9 @@ struct GeoSource {
   }
 };
 
-// Shared steering table t of the plan (blockIdx.y): tab[m * ldt + i] = a_m at flat point i, the
-// FP64 phasor of the refinement rounded to FP32; rows m >= M and points i >= npts are zero.
+// Shared steering table t of the plan (blockIdx.y): row m holds a_m of the flat points, two points
+// at a time as (Re, Re, Im, Im) (the operand pairs of the paired contraction), the FP64 phasor of the
+// refinement rounded to FP32; rows m >= M and points i >= npts are zero.
 __global__ void geo_steer_kernel(const uint8_t *plan, uint8_t *ws) {
   const PlanHeader *h = reinterpret_cast<const PlanHeader *>(plan);
   const PlanGeoSteer st = reinterpret_cast<const PlanGeoSteer *>(plan + h->off_geo_steer)[blockIdx.y];
@@ -142,26 +143,41 @@ __global__ void geo_steer_kernel(const uint8_t *plan, uint8_t *ws) {
         const double2 a = src.phasor(d, m);
         v = make_float2((float)a.x, (float)a.y);
       }
-      tab[(size_t)m * st.ldt + i] = v;
+      float *row = reinterpret_cast<float *>(tab + (size_t)m * st.ldt) + 4 * (i >> 1) + (i & 1);
+      row[0] = v.x;
+      row[2] = v.y;
     }
   }
+}
+
+// Centroid of the M positions (FP64, in order).
+__device__ __forceinline__ void geo_centroid(const double *pos, int M, double *cen) {
+  double cx = 0.0, cy = 0.0, cz = 0.0;
+  for (int m = 0; m < M; ++m) {
+    cx += pos[3 * m];
+    cy += pos[3 * m + 1];
+    cz += pos[3 * m + 2];
+  }
+  cen[0] = cx / M;
+  cen[1] = cy / M;
+  cen[2] = cz / M;
+}
+
+// ((eps_a + 3) / 4)^2, the factor of the refinement thresholds (see the top of the file).
+__device__ __forceinline__ double geo_threshold_scale(const double *pos, int M, const double *cen) {
+  double rho = 0.0;
+  for (int m = 0; m < M; ++m)
+    rho = fmax(rho, fabs(pos[3 * m] - cen[0]) + fabs(pos[3 * m + 1] - cen[1]) + fabs(pos[3 * m + 2] - cen[2]));
+  const double ea = 2.0 * 3.141592653589793 * rho * 7.0 + 3.0;
+  const double sc = (ea + 3.0) / 4.0;
+  return fmax(sc * sc, 1.0);
 }
 
 // Per-job constants: centroid, FP32 positions and the scaled thresholds. Every thread of the CTA
 // calls it after load_job; it ends with a barrier.
 template <int MP>
 __device__ void geo_setup(const float2 *Bs, const ScanJob &j, const GeoParams &g, GeoShared &gs, ScanShared &sh) {
-  if (threadIdx.x == 0) {
-    double cx = 0.0, cy = 0.0, cz = 0.0;
-    for (int m = 0; m < j.M; ++m) {
-      cx += g.pos[3 * m];
-      cy += g.pos[3 * m + 1];
-      cz += g.pos[3 * m + 2];
-    }
-    gs.cen[0] = cx / j.M;
-    gs.cen[1] = cy / j.M;
-    gs.cen[2] = cz / j.M;
-  }
+  if (threadIdx.x == 0) geo_centroid(g.pos, j.M, gs.cen);
   __syncthreads();
   for (int m = threadIdx.x; m < MP; m += blockDim.x) {
     float4 p = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -173,13 +189,7 @@ __device__ void geo_setup(const float2 *Bs, const ScanJob &j, const GeoParams &g
   set_threshold<MP>(Bs, j, sh);
   __syncthreads();
   if (threadIdx.x == 0) {
-    double rho = 0.0;
-    for (int m = 0; m < j.M; ++m)
-      rho = fmax(rho, fabs(g.pos[3 * m] - gs.cen[0]) + fabs(g.pos[3 * m + 1] - gs.cen[1]) +
-                          fabs(g.pos[3 * m + 2] - gs.cen[2]));
-    const double ea = 2.0 * 3.141592653589793 * rho * 7.0 + 3.0;
-    double sc = (ea + 3.0) / 4.0;
-    sc = fmax(sc * sc, 1.0);
+    const double sc = geo_threshold_scale(g.pos, j.M, gs.cen);
     for (int r = 0; r < 4; ++r) sh.thr[r] = (float)(sh.thr[r] * sc);
   }
   __syncthreads();
@@ -203,12 +213,16 @@ __device__ __forceinline__ void geo_points(const float2 *Bs, const ScanJob &j, c
 #pragma unroll
         for (int q2 = 0; q2 < PT / 2; ++q2) {
           const float4 v = __ldg(reinterpret_cast<const float4 *>(row) + q2);
-          a[2 * q2][m] = make_float2(v.x, v.y);
-          a[2 * q2 + 1][m] = make_float2(v.z, v.w);
+          a[2 * q2][m] = make_float2(v.x, v.z);
+          a[2 * q2 + 1][m] = make_float2(v.y, v.w);
         }
       } else {
+        static_assert(PT % 2 == 0 || PT == 1, "one point of a pair, or whole pairs");
 #pragma unroll
-        for (int q = 0; q < PT; ++q) a[q][m] = __ldg(row + q);
+        for (int q = 0; q < PT; ++q) {
+          const float *e = reinterpret_cast<const float *>(row - (i0 & 1)) + (i0 & 1) + q;
+          a[q][m] = make_float2(__ldg(e), __ldg(e + 2));
+        }
       }
     }
     contract_points<MP, PT>(Bs, j, a, npts, i0, sh, src);
@@ -272,6 +286,24 @@ __global__ void __launch_bounds__(kScanThreads) scan_geometry_single_kernel(cons
   geo_drain(j, src, sh);
 }
 
+// Scan job of a geometry problem of the batch (factor and EV weights in the workspace).
+__device__ __forceinline__ ScanJob geo_job(const PlanProblem &pp, const uint8_t *ws) {
+  ScanJob j{};
+  j.F = reinterpret_cast<const double2 *>(ws + pp.fac_off);
+  j.w = pp.Kn > 0 && pp.slot[DOA_EV] >= 0
+            ? reinterpret_cast<const double *>(ws + pp.fac_off) + 2 * pp.p.M * (pp.p.M + 1)
+            : nullptr;
+  j.S64 = nullptr;
+  for (int r = 0; r < 4; ++r) j.P[r] = pp.slot[r] >= 0 ? pp.p.P + (size_t)pp.slot[r] * pp.npts : nullptr;
+  j.M = pp.p.M;
+  j.Kf = pp.Kf;
+  j.Kn = pp.Kn;
+  j.kphd = pp.kphd;
+  j.kmn = pp.kmn;
+  j.kofs = 0;
+  return j;
+}
+
 // Batched: the tiles of the geometry problems of one M bucket, dealt in runs of kRun tiles like the
 // ULA batch scan (run r to CTA r mod gridDim). Flagged points accumulate over a run and are
 // re-evaluated when the run ends or its problem changes, so the warps share the FP64 work of
@@ -285,7 +317,7 @@ __global__ void __launch_bounds__(kScanThreads) scan_geometry_batch_kernel(const
   __shared__ ScanShared sh;
   __shared__ GeoShared gs;
   const PlanHeader *h = reinterpret_cast<const PlanHeader *>(plan);
-  const int nunits = h->geo_jobs[bucket];
+  const int nunits = h->geo_alone[bucket];
   const int64_t ntiles = h->geo_tiles[bucket];
   const int32_t *list = reinterpret_cast<const int32_t *>(plan + h->off_geo[bucket]);
   const PlanProblem *probs = reinterpret_cast<const PlanProblem *>(plan + h->off_prob);
@@ -313,19 +345,7 @@ __global__ void __launch_bounds__(kScanThreads) scan_geometry_batch_kernel(const
       if (u != cur) {
         if (cur >= 0) geo_drain(j, src, sh);
         pp = &probs[list[u]];
-        const int npts = pp->npts;
-        j.F = reinterpret_cast<const double2 *>(ws + pp->fac_off);
-        j.w = pp->Kn > 0 && pp->slot[DOA_EV] >= 0
-                  ? reinterpret_cast<const double *>(ws + pp->fac_off) + 2 * pp->p.M * (pp->p.M + 1)
-                  : nullptr;
-        j.S64 = nullptr;
-        for (int r = 0; r < 4; ++r) j.P[r] = pp->slot[r] >= 0 ? pp->p.P + (size_t)pp->slot[r] * npts : nullptr;
-        j.M = pp->p.M;
-        j.Kf = pp->Kf;
-        j.Kn = pp->Kn;
-        j.kphd = pp->kphd;
-        j.kmn = pp->kmn;
-        j.kofs = 0;
+        j = geo_job(*pp, ws);
         const PlanGeoGrid &gg = geo_grids[pp->geo_grid];
         g.pos = pp->p.geom.pos;
         g.t32 = reinterpret_cast<const float2 *>(ws + gg.t32_off);
@@ -353,6 +373,155 @@ __global__ void __launch_bounds__(kScanThreads) scan_geometry_batch_kernel(const
   }
 }
 
+
+// Shared-steering scan: the problems of one steering table in groups. A unit is one tile of the
+// table for every problem of a group: each thread reads its points' phasors into registers once and
+// contracts them with the factor of each problem in turn (the paired form, the next factor copied
+// asynchronously meanwhile), where the per-problem scan reads the table's 8 MP bytes per point again
+// for every problem: 8.5 GB of L2 reads for 4096 problems of 8 elements on 32400 points, and the
+// unpaired FMAs beside them: that batch 2.57 -> 2.26 ms in all, its scan 1.86 -> 1.55 ms. The FMA pipe is
+// half busy: three warps per scheduler wait on their own chains, on the barrier of each problem, and
+// (a tenth) on the FP64 re-evaluations at a unit's end.
+// Factors, EV weights and thresholds are prepared once per solve (the values geo_setup computes), so
+// a problem's spectrum is that of the per-problem scan bit for bit. The queue is drained at the end
+// of a unit, and before a problem whose points might no longer all fit (a point that finds it full is
+// re-evaluated by its own thread, which sums in another order).
+template <int MP>
+__global__ void __launch_bounds__(kScanThreads) geo_prep_kernel(const uint8_t *plan, uint8_t *ws, int bucket) {
+  const PlanHeader *h = reinterpret_cast<const PlanHeader *>(plan);
+  const int32_t *list = reinterpret_cast<const int32_t *>(plan + h->off_ggl[bucket]);
+  const PlanProblem *probs = reinterpret_cast<const PlanProblem *>(plan + h->off_prob);
+  const int i = blockIdx.x * kScanWarps + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  if (i >= h->gg_probs[bucket]) return;
+  const PlanProblem &pp = probs[list[i]];
+  const ScanJob j = geo_job(pp, ws);
+  float4 *F32 = reinterpret_cast<float4 *>(ws + pp.fac_off + fac32_off(j.M));
+  float *w32 = reinterpret_cast<float *>(F32 + (j.M + 1) * MP);
+  for (int e = lane; e < j.Kf * MP; e += 32) {
+    const int k = e / MP, m = e % MP;
+    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (m < j.M) {
+      const double2 b = j.F[(size_t)k * j.M + m];
+      const float bx = (float)b.x, by = (float)b.y;
+      v = make_float4(bx, bx, by, by);
+    }
+    F32[e] = v;
+  }
+  for (int k = lane; k < j.Kn; k += 32) w32[k] = j.w ? (float)j.w[k] : 1.f;
+  __syncwarp();
+  float thr[4] = {0.f, 0.f, 0.f, 0.f};
+  job_thresholds2<MP>(F32, w32, j.Kf, j.Kn, j.kphd, j.kmn, thr);
+  double cen[3];
+  geo_centroid(pp.p.geom.pos, j.M, cen);
+  const double sc = geo_threshold_scale(pp.p.geom.pos, j.M, cen);
+  if (lane < 4) w32[MP + lane] = (float)(thr[lane] * sc);
+}
+
+template <int MP, int PT>
+__global__ void __launch_bounds__(kScanThreads, 3) scan_geometry_shared_kernel(const uint8_t *plan, uint8_t *ws,
+                                                                               int bucket) {
+  constexpr int HP = PT / 2, TP = kScanThreads * PT;
+  static_assert(PT % 2 == 0 && kSteerAlign % TP == 0, "paired points; a tile lies inside one table row");
+  static_assert(kFlagCap >= TP, "the points of one problem's tile fit the queue");
+  __shared__ __align__(16) float Fsm[2][4 * (MP + 1) * MP];
+  __shared__ __align__(16) float Wsm[2][MP + 4];   // EV weights, then the 4 thresholds
+  __shared__ uint8_t tags[kFlagCap];
+  __shared__ ScanShared sh;
+  __shared__ ScanJob jobs[kScanGroupMax];   // the current group's jobs (read once per group)
+  __shared__ double cen[3];
+  __shared__ unsigned s_unit;
+  const PlanHeader *h = reinterpret_cast<const PlanHeader *>(plan);
+  const PlanScanGroup *groups = reinterpret_cast<const PlanScanGroup *>(plan + h->off_gg[bucket]);
+  const int ngroups = h->gg_groups[bucket];
+  const int64_t nunits = h->gg_units[bucket];
+  const int32_t *list = reinterpret_cast<const int32_t *>(plan + h->off_ggl[bucket]);
+  const PlanProblem *probs = reinterpret_cast<const PlanProblem *>(plan + h->off_prob);
+  const PlanGeoGrid *geo_grids = reinterpret_cast<const PlanGeoGrid *>(plan + h->off_geo_grid);
+  const PlanGeoSteer *steers = reinterpret_cast<const PlanGeoSteer *>(plan + h->off_geo_steer);
+  unsigned *next_unit = reinterpret_cast<unsigned *>(ws) + kCtrGeo + bucket;
+  const int tid = threadIdx.x;
+  if (tid == 0) sh.nflag = 0;
+  int cached = -1;   // group whose jobs are in shared memory (every thread holds the same value)
+  for (;;) {
+    if (tid == 0) s_unit = atomicAdd(next_unit, 1u);
+    __syncthreads();   // (s_unit was last read before the barriers of the previous unit)
+    const int64_t u = s_unit;
+    if (u >= nunits) break;
+    int gi = 0, hi = ngroups - 1;
+    while (gi < hi) {  // last group with unit_start <= u
+      const int mid = (gi + hi + 1) >> 1;
+      if (groups[mid].unit_start <= u) gi = mid; else hi = mid - 1;
+    }
+    const PlanScanGroup gr = groups[gi];
+    const PlanGeoSteer &st = steers[gr.grid_id];
+    const PlanGeoGrid &gg = geo_grids[st.geo_grid];
+    if (gi != cached) {   // the previous unit's drain has ended (barrier at its end)
+      for (int i = tid; i < gr.count; i += kScanThreads) jobs[i] = geo_job(probs[list[gr.first + i]], ws);
+      if (tid == 0) geo_centroid(st.pos, st.M, cen);
+      __syncthreads();
+      cached = gi;
+    }
+    GeoSource src;
+    src.pos = st.pos;
+    src.t64 = reinterpret_cast<const double2 *>(ws + gg.t64_off);
+    src.cx = cen[0];
+    src.cy = cen[1];
+    src.cz = cen[2];
+    src.La = gg.La;
+    // the copies of problem i of the group into buffer b: Kf columns of the factor, then the MP EV
+    // weights and 4 thresholds, all 16-byte multiples
+    auto issue = [&](int i, int b) {
+      const ScanJob &ji = jobs[i];
+      const float4 *fsrc = reinterpret_cast<const float4 *>(reinterpret_cast<const uint8_t *>(ji.F) + fac32_off(ji.M));
+      float4 *dst = reinterpret_cast<float4 *>(Fsm[b]);
+      for (int e = tid; e < ji.Kf * MP; e += kScanThreads) cp_async16(dst + e, fsrc + e);
+      const float4 *wsrc = reinterpret_cast<const float4 *>(job_w32<MP>(ji));
+      for (int e = tid; e < (MP + 4) / 4; e += kScanThreads) cp_async16(reinterpret_cast<float4 *>(Wsm[b]) + e, wsrc + e);
+      cp_async_commit();
+    };
+    issue(0, 0);
+    const int i0 = (int)(u - gr.unit_start) * TP + tid * PT;
+    uint64_t ax[HP][MP], ay[HP][MP];
+    const float2 *tab = reinterpret_cast<const float2 *>(ws + st.tab_off) + i0;
+#pragma unroll
+    for (int m = 0; m < MP; ++m) {
+#pragma unroll
+      for (int q = 0; q < HP; ++q) {
+        const ulonglong2 v = __ldg(reinterpret_cast<const ulonglong2 *>(tab + (size_t)m * st.ldt) + q);
+        ax[q][m] = v.x;
+        ay[q][m] = v.y;
+      }
+    }
+    for (int i = 0; i < gr.count; ++i) {
+      const int b = i & 1;
+      cp_async_wait_all();   // this thread's copies of problem i have landed
+      // everyone's have, and problem i - 1 is no longer read from buffer b ^ 1; each thread has seen its
+      // own additions to the queue, so some thread has seen them all
+      const unsigned nf = *reinterpret_cast<volatile unsigned *>(&sh.nflag);
+      if (__syncthreads_or(queue_front(nf) + queue_back(nf) > kFlagCap - TP)) {
+        drain_tagged<MP>(jobs, tags, sh, [&](const ScanJob &) { return src; });
+        __syncthreads();
+      }
+      if (i + 1 < gr.count) issue(i + 1, b ^ 1);
+      contract_points2<MP, PT, GeoSource, true, true>(reinterpret_cast<const float4 *>(Fsm[b]), jobs[i], ax, ay, st.npts, i0,
+                                                sh, src, Wsm[b], Wsm[b] + MP, tags, i);
+    }
+    drain_tagged<MP>(jobs, tags, sh, [&](const ScanJob &) { return src; });
+  }
+}
+
+template <int MP, int PT>
+cudaError_t run_geo_shared(const uint8_t *plan, const PlanHeader &h, uint8_t *ws, int bucket, cudaStream_t s) {
+  static_assert(PT == geo_group_pt(MP == 8 ? 0 : 1), "the tile the plan counted units with");
+  if (h.gg_units[bucket] == 0) return cudaSuccess;
+  geo_prep_kernel<MP><<<(h.gg_probs[bucket] + kScanWarps - 1) / kScanWarps, kScanThreads, 0, s>>>(plan, ws, bucket);
+  int per_sm = 0;
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, scan_geometry_shared_kernel<MP, PT>, kScanThreads, 0);
+  if (per_sm < 1) per_sm = 1;
+  const int64_t grid = std::min<int64_t>((int64_t)device_sm_count() * per_sm, h.gg_units[bucket]);
+  scan_geometry_shared_kernel<MP, PT><<<(unsigned)grid, kScanThreads, 0, s>>>(plan, ws, bucket);
+  return cudaGetLastError();
+}
 
 template <int MP, int PT>
 cudaError_t run_geo_batch(const uint8_t *plan, const PlanHeader &h, uint8_t *ws, int bucket, cudaStream_t s) {
@@ -402,7 +571,10 @@ cudaError_t launch_geo_tables(const uint8_t *plan_dev, const PlanHeader &h, uint
 }
 
 cudaError_t launch_scan_geometry_batch(const uint8_t *plan_dev, const PlanHeader &h, uint8_t *ws, cudaStream_t s) {
-  cudaError_t e;
+  cudaError_t e = run_geo_shared<8, geo_group_pt(0)>(plan_dev, h, ws, 0, s);
+  if (e != cudaSuccess) return e;
+  e = run_geo_shared<16, geo_group_pt(1)>(plan_dev, h, ws, 1, s);
+  if (e != cudaSuccess) return e;
   switch (h.scan_pt[0]) {
     case 1: e = run_geo_batch<8, 1>(plan_dev, h, ws, 0, s); break;
     case 2: e = run_geo_batch<8, 2>(plan_dev, h, ws, 0, s); break;

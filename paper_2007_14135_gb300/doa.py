@@ -403,7 +403,7 @@ class BatchPlan:
         cf = [int(v) for v in h[62:67]]                       # cov_first: classes MB = 2, 3, 4, other
         cov = sum(2 for c in range(3) if cf[c + 1] > cf[c]) + int(cf[4] > cf[3]) + int(h[5] > 0)
         eig_b = sum(int(c) > 0 for c in h[6:10])
-        scan_b = sum(int(c) > 0 for c in h[10:14]) + int(h[67] > 0) + sum(int(c) > 0 for c in h[76:80])
+        scan_b = sum(int(c) > 0 for c in h[10:14]) + int(h[67] > 0) + sum(int(c) > 0 for c in h[172:176])
         ngeo = sum(int(c) for c in h[76:80])
         peaks = int(ngeo < int(h[1])) + int(ngeo > 0) + (2 if int(h[74]) > 0 else 0)
         covtc = int(h[108] > 0) + int(h[109] > 0)
@@ -411,6 +411,7 @@ class BatchPlan:
         # grid-shared scan: a prep kernel and the scan kernel per M bucket that has groups
         shared = 2 * sum(int(u) > 0 for u in self.host[496:528].view(np.int64))
         shared += 2 * int(h[152] > 0)                          # tensor-core groups: prep + scan
+        shared += 2 * sum(int(u) > 0 for u in self.host[704:736].view(np.int64))   # geometry groups: the same
         return (int(h[3] > 0) + int(h[96] > 0) + int(h[104] > 0) + cov + covtc + eig_b + scan_b + shared + peaks
                 + int(h[100] > 0) + int(h[101] > 0))
 
