@@ -50,14 +50,14 @@ namespace cg = cooperative_groups;
 constexpr int kPeakCluster = 8;
 constexpr int kClusterPoints = 16384;      // points from which a spectrum takes a cluster
 
-// This CTA's share of a spectrum's quads: rank of kCs CTAs.
-template <int kCs>
+// This CTA's share of a spectrum's quads: rank of kCs CTAs of T threads.
+template <int kCs, int T>
 struct Share {
   int first, stride, rank;
   __device__ Share() {
     rank = kCs > 1 ? (int)cg::this_cluster().block_rank() : 0;
-    first = rank * kPeakThreads + (int)threadIdx.x;
-    stride = kCs * kPeakThreads;
+    first = rank * T + (int)threadIdx.x;
+    stride = kCs * T;
   }
 };
 
@@ -90,13 +90,13 @@ __device__ int merge_lists(int want, const Cand *sel, int n, Cand *out) {
 }
 
 // next (nullable): receives the value of the (d+1)-th best peak (-inf if there is none).
-template <int kCs>
+template <int kCs, int T>
 __device__ void peaks_block(const float *__restrict__ P, int L, int d, int *idx, float *val, int *count,
                             float *next = nullptr) {
   __shared__ Cand sel[kMaxM + 1], all[kCs > 1 ? kMaxM + 1 : 1];
   const int want = next ? d + 1 : d;
-  const Share<kCs> sh;
-  int nsel = select_rounds(want, sel, [&](const Cand &thr, Cand (&cache)[kCache], int &n) {
+  const Share<kCs, T> sh;
+  int nsel = select_rounds<T>(want, sel, [&](const Cand &thr, Cand (&cache)[kCache], int &n) {
     return fill(P, L, sh.first, sh.stride, thr, cache, n);
   });
   Cand *best = sel;
@@ -116,7 +116,7 @@ template <int kCs>
 __device__ void peaks2d_block(const float *__restrict__ P, int La, int Le, bool wrap, int d, int *idx, float *val,
                               int *count) {
   __shared__ Cand sel[kMaxM], all[kCs > 1 ? kMaxM : 1];
-  const Share<kCs> sh;
+  const Share<kCs, kPeakThreads> sh;
   int nsel = select_rounds(d, sel, [&](const Cand &thr, Cand (&cache)[kCache], int &n) {
     return fill2d(P, La, Le, wrap, sh.first, sh.stride, thr, cache, n);
   });
@@ -138,14 +138,24 @@ __global__ void __launch_bounds__(kPeakThreads) peaks2d_single_kernel(const floa
 template <int kCs>
 __global__ void __launch_bounds__(kPeakThreads) peaks_single_kernel(const float *P, int L, int d, int *idx, float *val,
                                                                     int *count) {
-  peaks_block<kCs>(P, L, d, idx, val, count);
+  peaks_block<kCs, kPeakThreads>(P, L, d, idx, val, count);
 }
+
+// Threads per SM of the 1-D batch kernel, and the threads of a job's CTA in a batch of spectra that are many
+// but not long (kSmallPoints): the barriers of a job and the merge of its lists by one warp leave a CTA
+// of 256 threads idle for a third of its time, while two warps per job wait little and 20 jobs per SM
+// overlap. 4096 x 4 spectra of 18 001 points: 32 threads 0.246, 64 0.227, 128 0.243, 256 0.303 ms. A long
+// spectrum keeps 256 threads, so that it does not outlast the batch.
+// (2-D: 256 threads measured best, 0.22 against 0.28 ms with 64, and four quads per thread in 64
+// registers, 0.18 ms against 0.21 with two in 48.)
+constexpr int kBatchThreads = 1280;
+constexpr int kSmallThreads = 64, kSmallPoints = 65536;
 
 // One CTA (or cluster) per (problem, algorithm) job; the 1-D and 2-D rules run as separate kernels (each skips
 // the other kind's jobs) so that each keeps its own register budget.
 // repick: the pick after the peak polish, only for the jobs the polish marked (NaN next value).
-template <int kCs>
-__global__ void __launch_bounds__(kPeakThreads, 5) peaks_batch_kernel(const uint8_t *plan, uint8_t *ws, int repick) {
+template <int kCs, int T>
+__global__ void __launch_bounds__(T, kBatchThreads / T) peaks_batch_kernel(const uint8_t *plan, uint8_t *ws, int repick) {
   const int job = blockIdx.x / kCs;
   const PlanHeader *h = reinterpret_cast<const PlanHeader *>(plan);
   const PlanJob &jb = reinterpret_cast<const PlanJob *>(plan + h->off_job)[job];
@@ -158,12 +168,12 @@ __global__ void __launch_bounds__(kPeakThreads, 5) peaks_batch_kernel(const uint
     if (!polish || !isnan(*next)) return;
     next = nullptr;
   }
-  peaks_block<kCs>(pp.p.P + (size_t)jb.slot * L, L, d, pp.p.peak_idx + (size_t)jb.slot * d,
+  peaks_block<kCs, T>(pp.p.P + (size_t)jb.slot * L, L, d, pp.p.peak_idx + (size_t)jb.slot * d,
                    pp.p.peak_val + (size_t)jb.slot * d, pp.p.peak_count + jb.slot, next);
 }
 
 template <int kCs>
-__global__ void __launch_bounds__(kPeakThreads, 5) peaks2d_batch_kernel(const uint8_t *plan) {
+__global__ void __launch_bounds__(kPeakThreads, 4) peaks2d_batch_kernel(const uint8_t *plan) {
   const PlanHeader *h = reinterpret_cast<const PlanHeader *>(plan);
   const PlanJob &jb = reinterpret_cast<const PlanJob *>(plan + h->off_job)[blockIdx.x / kCs];
   const PlanProblem &pp = reinterpret_cast<const PlanProblem *>(plan + h->off_prob)[jb.prob];
@@ -271,11 +281,11 @@ cudaError_t launch_slice_peaks(const float *Pbuf, int b0, int k0, int k1, int L,
 }
 
 // Launches `kernel` on `jobs` spectra, kCs CTAs each.
-template <int kCs, class... Args>
+template <int kCs, int T, class... Args>
 cudaError_t launch_jobs(void (*kernel)(Args...), int jobs, cudaStream_t s, Args... args) {
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3((unsigned)jobs * kCs);
-  cfg.blockDim = dim3(kPeakThreads);
+  cfg.blockDim = dim3(T);
   cfg.stream = s;
   cudaLaunchAttribute attr{};
   attr.id = cudaLaunchAttributeClusterDimension;
@@ -287,15 +297,15 @@ cudaError_t launch_jobs(void (*kernel)(Args...), int jobs, cudaStream_t s, Args.
 }
 
 cudaError_t launch_peaks_single(const float *P, int L, int d, int *idx, float *val, int *count, cudaStream_t s) {
-  return L >= kClusterPoints ? launch_jobs<kPeakCluster>(peaks_single_kernel<kPeakCluster>, 1, s, P, L, d, idx, val, count)
-                             : launch_jobs<1>(peaks_single_kernel<1>, 1, s, P, L, d, idx, val, count);
+  return L >= kClusterPoints ? launch_jobs<kPeakCluster, kPeakThreads>(peaks_single_kernel<kPeakCluster>, 1, s, P, L, d, idx, val, count)
+                             : launch_jobs<1, kPeakThreads>(peaks_single_kernel<1>, 1, s, P, L, d, idx, val, count);
 }
 
 cudaError_t launch_peaks2d_single(const float *P, int La, int Le, int wrap_az, int d, int *idx, float *val,
                                   int *count, cudaStream_t s) {
   return (int64_t)La * Le >= kClusterPoints
-             ? launch_jobs<kPeakCluster>(peaks2d_single_kernel<kPeakCluster>, 1, s, P, La, Le, wrap_az, d, idx, val, count)
-             : launch_jobs<1>(peaks2d_single_kernel<1>, 1, s, P, La, Le, wrap_az, d, idx, val, count);
+             ? launch_jobs<kPeakCluster, kPeakThreads>(peaks2d_single_kernel<kPeakCluster>, 1, s, P, La, Le, wrap_az, d, idx, val, count)
+             : launch_jobs<1, kPeakThreads>(peaks2d_single_kernel<1>, 1, s, P, La, Le, wrap_az, d, idx, val, count);
 }
 
 // A batch takes clusters when its jobs do not fill the SMs (five CTAs each) and some spectrum is long
@@ -308,13 +318,16 @@ cudaError_t launch_peaks_batch(const uint8_t *plan_dev, const PlanHeader &h, uin
   const int repick = ula && !geo;   // the call after the polish
   const bool few = (int64_t)h.njobs * kPeakCluster <= 5 * (int64_t)device_sm_count();
   const bool cl = few && h.max_points >= kClusterPoints;
+  const bool small = h.max_points <= kSmallPoints &&
+                     (int64_t)h.njobs * kSmallThreads >= kBatchThreads * (int64_t)device_sm_count();
   cudaError_t e = cudaSuccess;
   if (h.njobs > 0 && ula && ngeo < h.nprob)
-    e = cl ? launch_jobs<kPeakCluster>(peaks_batch_kernel<kPeakCluster>, h.njobs, s, plan_dev, ws, repick)
-           : launch_jobs<1>(peaks_batch_kernel<1>, h.njobs, s, plan_dev, ws, repick);
+    e = cl ? launch_jobs<kPeakCluster, kPeakThreads>(peaks_batch_kernel<kPeakCluster, kPeakThreads>, h.njobs, s, plan_dev, ws, repick)
+        : small ? launch_jobs<1, kSmallThreads>(peaks_batch_kernel<1, kSmallThreads>, h.njobs, s, plan_dev, ws, repick)
+                : launch_jobs<1, kPeakThreads>(peaks_batch_kernel<1, kPeakThreads>, h.njobs, s, plan_dev, ws, repick);
   if (e == cudaSuccess && h.njobs > 0 && geo && ngeo > 0)
-    e = cl ? launch_jobs<kPeakCluster>(peaks2d_batch_kernel<kPeakCluster>, h.njobs, s, plan_dev)
-           : launch_jobs<1>(peaks2d_batch_kernel<1>, h.njobs, s, plan_dev);
+    e = cl ? launch_jobs<kPeakCluster, kPeakThreads>(peaks2d_batch_kernel<kPeakCluster>, h.njobs, s, plan_dev)
+           : launch_jobs<1, kPeakThreads>(peaks2d_batch_kernel<1>, h.njobs, s, plan_dev);
   return e;
 }
 

@@ -137,3 +137,34 @@ def test_peaks_cluster_matches_oracle(env, L, off, d):
         k = np.nonzero(w)[0]
         k = np.sort(k[np.lexsort((k, -P[k]))][:d])
         assert list(i2.cpu().numpy()[:int(cnt.item())]) == list(k)
+
+
+@pytest.mark.parametrize("L,d", [(181, 1), (1801, 3), (1023, 0)])
+def test_many_spectra_match_the_single_picker(env, L, d):
+    """A batch of enough spectra takes a small CTA for each: the picks are those of doa_peaks on the
+    spectra the same solve wrote (3200 jobs, spectra starting at odd offsets)."""
+    torch, doa = env
+    B, M, N, mask = 800, 4, 64, 0xF
+    gen = torch.Generator(device="cuda").manual_seed(L)
+    X = torch.view_as_complex(torch.randn(B, M, N, 2, generator=gen, device="cuda"))
+    P = torch.zeros(B * 4 * L + 1, device="cuda")[1:].view(B, 4 * L)
+    dk = max(d, 1)
+    idx = torch.full((B, 4 * dk), -1, dtype=torch.int32, device="cuda")
+    val = torch.zeros((B, 4 * dk), device="cuda")
+    cnt = torch.full((B, 4), -1, dtype=torch.int32, device="cuda")
+    probs = [doa.make_problem(X[i], d, mask, doa.grid(-90.0, 180.0 / (L - 1), L), P[i], idx[i] if d else None,
+                              val[i] if d else None, cnt[i], None) for i in range(B)]
+    plan = doa.BatchPlan(probs)
+    status = torch.full((B,), -1, dtype=torch.int32, device="cuda")
+    doa.doa_solve_batch(plan, doa.workspace(plan), status)
+    torch.cuda.synchronize()
+    assert int(status.abs().max()) == 0
+    for i in range(0, B, 37):
+        for a in range(4):
+            i1 = torch.full((dk,), -1, dtype=torch.int32, device="cuda")
+            v1 = torch.zeros(dk, device="cuda")
+            c1 = torch.zeros(1, dtype=torch.int32, device="cuda")
+            doa.doa_peaks(P[i, a * L:(a + 1) * L], d, i1, v1, c1)
+            n = int(c1)
+            assert int(cnt[i, a]) == n
+            assert torch.equal(idx[i, a * d:a * d + n], i1[:n]) and torch.equal(val[i, a * d:a * d + n], v1[:n])
