@@ -34,8 +34,10 @@
 // In the batch the iteration starts from the vertex of the parabola through the FP32 spectrum's
 // 1/P at the peak and its neighbours (per axis in 2-D), which leaves Newton one or two steps; the
 // local minimiser it converges to does not depend on the start.
-// Measured (2048 ULA jobs of four peaks and 512 circular-array jobs of two): 7.5 -> 2.3 ms, of which about
-// 2 ms is one peak's 60 steps with some twenty halvings each; the 2-D jobs therefore start first.
+// Measured (2048 ULA jobs of four peaks and 512 circular-array jobs of two): 7.5 -> 1.4 ms. The kernel's
+// length is that of one peak's 60 steps with some twenty halvings each (2.4 ms on one warp), so the
+// 2-D jobs start first, and the four warps of a CTA share a search that does not end soon: the whole
+// solve of that batch 3.92 -> 2.93 ms with that search, 3.04 -> 2.72 without.
 #include <float.h>
 #include <math_constants.h>
 
@@ -48,6 +50,9 @@ namespace {
 
 constexpr int kRefWarps = 4;
 constexpr int kRefMaxIter = 60;
+// Steps of a 2-D search that its warp takes alone (most searches end within them). The batch above at 3, 6, 12
+// and 20: 2.77, 2.82, 2.78, 2.82 ms in the mean of three drawings, 2.89, 2.97, 2.98, 3.11 at the longest search.
+constexpr int kSoloSteps = 4;
 constexpr double kD2R = 3.14159265358979323846 / 180.0;
 constexpr double kPi = 3.14159265358979323846;
 
@@ -372,13 +377,32 @@ __device__ double geo_eval(const RefineJob &j, double th, double ph, RefShared &
   return group_sum<32>(pf);
 }
 
-template <int W>
-__device__ void refine_geo_warp(const RefineJob &j, int flat, RefShared &sh, double *out) {
+// A search on its way: the point, den and its derivatives there (when have), the steps taken.
+struct GeoState {
+  double x0, x1, f, g[2], H[3];
+  int it;
+  bool have;
+};
+// What the warps of a search tell each other at a barrier: den and its derivatives at one point (by the
+// first warp), and each warp's first accepted step length of a round.
+struct GeoSlot {
+  double ev[6];
+  double n[kRefWarps][2];
+  int hit[kRefWarps];
+};
+// Long searches of a CTA: the state each warp left open, and two slots per search, used in turn (so that
+// one barrier is enough: a slot is written again after the next barrier, when all have read it).
+struct GeoLong {
+  GeoState st[kRefWarps];
+  int open[kRefWarps];
+  GeoSlot slot[2][2];
+};
+
+// Start of the search at grid point flat: the vertex of the parabola per axis (batch) or the point.
+__device__ void geo_start(const RefineJob &j, int flat, GeoState &st) {
   const int l = flat / j.La, k = flat - l * j.La;
   double x0 = __dmul_rn(__dadd_rn(j.az_lo, __dmul_rn((double)k, j.az_step)), kD2R);
   double x1 = __dmul_rn(__dadd_rn(j.el_lo, __dmul_rn((double)l, j.el_step)), kD2R);
-  const double hw0 = fabs(j.az_step) * kD2R, hw1 = fabs(j.el_step) * kD2R;
-  const double bl0 = x0 - hw0, bh0 = x0 + hw0, bl1 = x1 - hw1, bh1 = x1 + hw1;
   if (j.P) {
     const float pc = j.P[flat];
     const int km = k > 0 ? k - 1 : (j.wrap ? j.La - 1 : -1), kp = k + 1 < j.La ? k + 1 : (j.wrap ? 0 : -1);
@@ -387,10 +411,66 @@ __device__ void refine_geo_warp(const RefineJob &j, int flat, RefShared &sh, dou
     if (l > 0 && l + 1 < j.Le)
       x1 += vertex_offset(j.P[(size_t)(l - 1) * j.La + k], pc, j.P[(size_t)(l + 1) * j.La + k]) * j.el_step * kD2R;
   }
-  double g[2], H[3], f = 0.0;
-  bool have = false;   // f, g, H belong to (x0, x1) already
-  for (int it = 0; it < kRefMaxIter; ++it) {
-    if (!have) f = geo_eval<W>(j, x0, x1, sh, g, H);
+  st.x0 = x0;
+  st.x1 = x1;
+  st.it = 0;
+  st.have = false;
+}
+
+// Takes steps of the search at grid point flat until it ends (true) or st.it reaches max_it, by this warp
+// alone (parts = 1) or as warp `part` of `parts` (all with the same state; search `group` of the CTA): then
+// the first warp computes the derivatives and the step lengths are dealt over the warps. While the
+// first warp evaluates a whole Newton step, the others already try the shorter ones.
+template <int W>
+__device__ bool geo_steps(const RefineJob &j, int flat, int max_it, int part, int parts, int group, RefShared &sh,
+                          GeoLong &co, GeoState &st) {
+  constexpr int G = 32 / W;   // step lengths a warp evaluates at once
+  const int lane = threadIdx.x & 31;
+  const int l = flat / j.La, k = flat - l * j.La;
+  const double c0 = __dmul_rn(__dadd_rn(j.az_lo, __dmul_rn((double)k, j.az_step)), kD2R);
+  const double c1 = __dmul_rn(__dadd_rn(j.el_lo, __dmul_rn((double)l, j.el_step)), kD2R);
+  const double hw0 = fabs(j.az_step) * kD2R, hw1 = fabs(j.el_step) * kD2R;
+  const double bl0 = c0 - hw0, bh0 = c0 + hw0, bl1 = c1 - hw1, bh1 = c1 + hw1;
+  double x0 = st.x0, x1 = st.x1, f = st.f;
+  double g[2] = {st.g[0], st.g[1]}, H[3] = {st.H[0], st.H[1], st.H[2]};
+  bool have = st.have;   // f, g, H belong to (x0, x1) already
+  bool done = false;
+  int it = st.it, set = 0;
+  auto meet = [&]() {   // the warps of this search
+    if (parts == kRefWarps)
+      __syncthreads();
+    else if (group == 0)
+      asm volatile("bar.sync 1, 64;" ::: "memory");
+    else
+      asm volatile("bar.sync 2, 64;" ::: "memory");
+  };
+  auto post_eval = [&](double fv, const double *gv, const double *Hv) {
+    double *e = co.slot[group][set].ev;
+    if (lane == 0) {
+      e[0] = fv;
+      e[1] = gv[0];
+      e[2] = gv[1];
+      e[3] = Hv[0];
+      e[4] = Hv[1];
+      e[5] = Hv[2];
+    }
+  };
+  for (; it < max_it; ++it) {
+    if (!have) {
+      if (part == 0) f = geo_eval<W>(j, x0, x1, sh, g, H);
+      if (parts > 1) {
+        if (part == 0) post_eval(f, g, H);
+        meet();
+        const double *e = co.slot[group][set].ev;
+        f = e[0];
+        g[0] = e[1];
+        g[1] = e[2];
+        H[0] = e[3];
+        H[1] = e[4];
+        H[2] = e[5];
+        set ^= 1;
+      }
+    }
     have = false;
     const double det = H[0] * H[2] - H[1] * H[1];
     const bool newton = H[0] > 0.0 && det > 0.0;
@@ -403,7 +483,10 @@ __device__ void refine_geo_warp(const RefineJob &j, int flat, RefShared &sh, dou
         const double mv = fmax(fabs(n0 - x0), fabs(n1 - x1));
         x0 = n0;
         x1 = n1;
-        if (mv < 1e-13) break;
+        if (mv < 1e-13) {
+          done = true;
+          break;
+        }
         continue;
       }
     } else {
@@ -414,69 +497,177 @@ __device__ void refine_geo_warp(const RefineJob &j, int flat, RefShared &sh, dou
     }
     double n0 = x0, n1 = x1;
     bool accepted = false;
+    // the first accepted of step lengths 2^-h, h = h0 .. h0 + G - 1 (each group of lanes evaluates one)
+    auto try_lengths = [&](int h0) {
+      const int h = h0 + lane / W;
+      const double t = __hiloint2double((1023 - h) << 20, 0);   // 2^-h
+      const double m0 = fmin(fmax(x0 + t * d0, bl0), bh0), m1 = fmin(fmax(x1 + t * d1, bl1), bh1);
+      const bool le = geo_den<W>(j, m0, m1, sh) <= f && h <= 40;
+      const unsigned hit = __ballot_sync(0xffffffffu, le);
+      const int src = hit ? __ffs(hit) - 1 : 0;
+      const double s0 = __shfl_sync(0xffffffffu, m0, src), s1 = __shfl_sync(0xffffffffu, m1, src);
+      if (hit) {
+        n0 = s0;
+        n1 = s1;
+      }
+      return hit != 0u;
+    };
+    auto post_hit = [&](bool hit) {
+      GeoSlot &sl = co.slot[group][set];
+      if (lane == 0) {
+        sl.hit[part] = hit;
+        sl.n[part][0] = n0;
+        sl.n[part][1] = n1;
+      }
+    };
+    auto first_hit = [&](int p0) {   // after the barrier: the lowest warp's hit has the longest step
+      const GeoSlot &sl = co.slot[group][set];
+      for (int p = p0; p < parts && !accepted; ++p)
+        if (sl.hit[p]) {
+          n0 = sl.n[p][0];
+          n1 = sl.n[p][1];
+          accepted = true;
+        }
+    };
+    int h0 = 0;
     if (newton) {   // the whole step is usually taken: its derivatives come with it
-      n0 = fmin(fmax(x0 + d0, bl0), bh0);
-      n1 = fmin(fmax(x1 + d1, bl1), bh1);
-      double gn[2], Hn[3];
-      const double fn = geo_eval<W>(j, n0, n1, sh, gn, Hn);
+      h0 = 1;
+      double fn = 0.0, gn[2] = {0.0, 0.0}, Hn[3] = {0.0, 0.0, 0.0};
+      const double w0 = fmin(fmax(x0 + d0, bl0), bh0), w1 = fmin(fmax(x1 + d1, bl1), bh1);
+      if (part == 0) {
+        fn = geo_eval<W>(j, w0, w1, sh, gn, Hn);
+      } else {
+        // 2 G lengths per warp, in order: two of these take as long as the derivatives
+        const int b = 1 + (part - 1) * 2 * G;
+        post_hit(try_lengths(b) || try_lengths(b + G));
+      }
+      if (parts > 1) {
+        if (part == 0) post_eval(fn, gn, Hn);
+        meet();
+        const double *e = co.slot[group][set].ev;
+        fn = e[0];
+        gn[0] = e[1];
+        gn[1] = e[2];
+        Hn[0] = e[3];
+        Hn[1] = e[4];
+        Hn[2] = e[5];
+      }
       if (fn <= f) {
         accepted = have = true;
+        n0 = w0;
+        n1 = w1;
         f = fn;
         g[0] = gn[0];
         g[1] = gn[1];
         H[0] = Hn[0];
         H[1] = Hn[1];
         H[2] = Hn[2];
+      } else if (parts > 1) {
+        first_hit(1);
+        h0 = 1 + (parts - 1) * 2 * G;
+      }
+      set ^= 1;
+    }
+    for (; h0 <= 40 && !accepted; h0 += parts * G) {
+      const bool hit = try_lengths(h0 + part * G);
+      if (parts == 1) {
+        accepted = hit;
+      } else {
+        post_hit(hit);
+        meet();
+        first_hit(0);
+        set ^= 1;
       }
     }
-    // step lengths 1, 1/2, ... 2^-40: each group of lanes evaluates one, the first accepted is taken
-    for (int h0 = newton ? 1 : 0; h0 <= 40 && !accepted; h0 += 32 / W) {
-      const int h = h0 + (int)(threadIdx.x & 31) / W;
-      const double t = __hiloint2double((1023 - h) << 20, 0);   // 2^-h
-      const double c0 = fmin(fmax(x0 + t * d0, bl0), bh0), c1 = fmin(fmax(x1 + t * d1, bl1), bh1);
-      const bool le = geo_den<W>(j, c0, c1, sh) <= f && h <= 40;
-      const unsigned hit = __ballot_sync(0xffffffffu, le);
-      if (hit) {
-        const int src = __ffs(hit) - 1;
-        n0 = __shfl_sync(0xffffffffu, c0, src);
-        n1 = __shfl_sync(0xffffffffu, c1, src);
-        accepted = true;
-      }
+    if (!accepted) {
+      done = true;
+      break;
     }
-    if (!accepted) break;
     const double mv = fmax(fabs(n0 - x0), fabs(n1 - x1));
     x0 = n0;
     x1 = n1;
-    if (mv < 1e-13) break;
+    if (mv < 1e-13) {
+      done = true;
+      break;
+    }
   }
-  out[0] = x0 / kD2R;
-  out[1] = x1 / kD2R;
+  st.x0 = x0;
+  st.x1 = x1;
+  st.f = f;
+  st.g[0] = g[0];
+  st.g[1] = g[1];
+  st.H[0] = H[0];
+  st.H[1] = H[1];
+  st.H[2] = H[2];
+  st.it = it;
+  st.have = have;
+  return done || it >= kRefMaxIter;
 }
 
-// Refines peaks idx[q], q = first, first + step, ... < n of one job; out: n angles (ULA) or n (azimuth,
-// elevation) pairs.
-__device__ void refine_job_warp(const RefineJob &j, const int *idx, int first, int step, int n, double *out,
-                                RefShared &sh) {
-  const int lane = threadIdx.x & 31;
-  const int w = max(j.M, j.Kf);
-  for (int q = first; q < n; q += step) {
-    const int k = idx[q];
-    if (j.pos) {
-      double r[2];
-      if (w <= 8)
-        refine_geo_warp<8>(j, k, sh, r);
-      else if (w <= 16)
-        refine_geo_warp<16>(j, k, sh, r);
-      else
-        refine_geo_warp<32>(j, k, sh, r);
-      if (lane == 0) {
-        out[2 * q] = r[0];
-        out[2 * q + 1] = r[1];
-      }
-    } else {
-      const double th = refine_ula_warp(j, k, sh);
-      if (lane == 0) out[q] = th;
+// The 2-D peaks first, first + step, ... of a job, kRefWarps at a time; every warp of the CTA calls it. A warp
+// takes a peak's first kSoloSteps steps alone; the searches that are not over then (a flat valley: tens of
+// steps of some twenty halvings each) are taken on by two warps each, a single one by all four.
+template <int W>
+__device__ void refine_geo_job(const RefineJob &j, const int *idx, int first, int step, int n, double *out,
+                               RefShared &sh, GeoLong &co) {
+  static_assert(kRefWarps == 4, "two searches of two warps, or one of four");
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  for (int q0 = first; q0 < n; q0 += step) {
+    const int q = q0 + warp;
+    GeoState st;
+    bool open = false;
+    if (q < n) {
+      geo_start(j, idx[q], st);
+      open = !geo_steps<W>(j, idx[q], kSoloSteps, 0, 1, 0, sh, co, st);
     }
+    if (lane == 0) {
+      co.open[warp] = open;
+      if (open) co.st[warp] = st;
+      if (q < n && !open) {
+        out[2 * q] = st.x0 / kD2R;
+        out[2 * q + 1] = st.x1 / kD2R;
+      }
+    }
+    __syncthreads();
+    int left = 0;   // open searches, a bit each
+    for (int w = 0; w < kRefWarps; ++w) left |= (co.open[w] ? 1 : 0) << w;
+    while (left) {
+      const int wa = __ffs(left) - 1;
+      left &= left - 1;
+      const bool two = left != 0;
+      const int wb = two ? __ffs(left) - 1 : wa;
+      left &= two ? left - 1 : 0;
+      const int group = two ? warp >> 1 : 0, w = group ? wb : wa, part = two ? warp & 1 : warp;
+      st = co.st[w];
+      geo_steps<W>(j, idx[q0 + w], kRefMaxIter, part, two ? 2 : 4, group, sh, co, st);
+      if (part == 0 && lane == 0) {
+        out[2 * (q0 + w)] = st.x0 / kD2R;
+        out[2 * (q0 + w) + 1] = st.x1 / kD2R;
+      }
+      __syncthreads();
+    }
+    __syncthreads();
+  }
+}
+
+// Refines peaks idx[q], q = first .. first + kRefWarps - 1, first + step, ... < n of one job; out: n angles (ULA) or
+// n (azimuth, elevation) pairs. Every warp of the CTA calls it.
+__device__ void refine_job(const RefineJob &j, const int *idx, int first, int step, int n, double *out, RefShared *sh,
+                           GeoLong &co) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int w = max(j.M, j.Kf);
+  if (j.pos) {
+    if (w <= 8)
+      refine_geo_job<8>(j, idx, first, step, n, out, sh[warp], co);
+    else if (w <= 16)
+      refine_geo_job<16>(j, idx, first, step, n, out, sh[warp], co);
+    else
+      refine_geo_job<32>(j, idx, first, step, n, out, sh[warp], co);
+    return;
+  }
+  for (int q = first + warp; q < n; q += step) {
+    const double th = refine_ula_warp(j, idx[q], sh[warp]);
+    if (lane == 0) out[q] = th;
     __syncwarp();
   }
 }
@@ -502,11 +693,11 @@ __device__ void set_centroid(RefineJob &j) {
   j.cz = cz / j.M;
 }
 
-__global__ void __launch_bounds__(32 * kRefWarps) refine_batch_kernel(const uint8_t *plan, uint8_t *ws) {
+__global__ void __launch_bounds__(32 * kRefWarps, 3) refine_batch_kernel(const uint8_t *plan, uint8_t *ws) {
   __shared__ RefShared sh[kRefWarps];
   __shared__ double2 Fs[kStageM * (kStageM + 1)];
   const PlanHeader *h = reinterpret_cast<const PlanHeader *>(plan);
-  const int warp = threadIdx.x >> 5;
+  __shared__ GeoLong co;
   // the first half of the CTAs takes the 2-D jobs, whose longest searches are the kernel's tail
   const bool geo = blockIdx.x < h->njobs;
   const int job = geo ? blockIdx.x : blockIdx.x - h->njobs;
@@ -542,7 +733,7 @@ __global__ void __launch_bounds__(32 * kRefWarps) refine_batch_kernel(const uint
   const int n = min(pp.p.peak_count[jb.slot], d);
   const int per = j.pos ? 2 : 1;
   stage_factor(j, Fs);
-  refine_job_warp(j, pp.p.peak_idx + (size_t)jb.slot * d, warp, kRefWarps, n, pp.p.peak_angle + (size_t)jb.slot * d * per, sh[warp]);
+  refine_job(j, pp.p.peak_idx + (size_t)jb.slot * d, 0, kRefWarps, n, pp.p.peak_angle + (size_t)jb.slot * d * per, sh, co);
 }
 
 __global__ void __launch_bounds__(32 * kRefWarps) refine_single_kernel(RefineJob j, const int *idx, const int *count,
@@ -550,9 +741,10 @@ __global__ void __launch_bounds__(32 * kRefWarps) refine_single_kernel(RefineJob
   __shared__ RefShared sh[kRefWarps];
   __shared__ double2 Fs[kStageM * (kStageM + 1)];
   if (j.pos) set_centroid(j);
-  const int n = min(*count, cap), warp = threadIdx.x >> 5;
+  __shared__ GeoLong co;
+  const int n = min(*count, cap);
   stage_factor(j, Fs);
-  refine_job_warp(j, idx, blockIdx.x * kRefWarps + warp, gridDim.x * kRefWarps, n, out, sh[warp]);
+  refine_job(j, idx, blockIdx.x * kRefWarps, gridDim.x * kRefWarps, n, out, sh, co);
 }
 
 }  // namespace

@@ -290,3 +290,37 @@ def test_refine_single_at_lane_group_sizes(env, M, d):
     for q, k in enumerate(inner):
         (wt, wp), _ = oracle.refine_peak2d(C, pos, 0.0, 2.0, 180, 10.0, 2.0, k)
         assert abs(got[q, 0] - wt) <= 1e-8 and abs(got[q, 1] - wp) <= 1e-8, (k, got[q], wt, wp)
+
+
+@pytest.mark.parametrize("M,d", [(5, 1), (8, 2), (12, 2), (16, 3), (20, 2)])
+def test_refine2d_long_searches_do_not_depend_on_company(env, M, d):
+    """Searches from arbitrary grid points of a planar array (far from a minimum, on maxima and saddles:
+    many steps) give the same angles alone (shared by all warps of a CTA), in pairs and in larger lists
+    (some left open together, the rest finished alone), and end inside the point's cell."""
+    torch, doa = env
+    rng = np.random.default_rng(100 + M)
+    t = 2.0 * np.pi * np.arange(M) / M
+    pos = torch.from_numpy(np.stack([0.5 * np.sin(t), 0.5 * np.cos(t), np.zeros(M)], axis=1)).cuda()
+    La, Le, step = 90, 24, 4.0
+    Q, _ = np.linalg.qr(rng.standard_normal((M, M)) + 1j * rng.standard_normal((M, M)))
+    K = M - d
+    B = torch.from_numpy(np.ascontiguousarray(Q[:, :K].T).reshape(-1)).cuda()
+    geom = doa.geometry(pos, 0.0, step, Le, True)
+    az = doa.grid(0.0, step, La)
+    pts = rng.integers(0, La * Le, 13).astype(np.int32)
+    pts[:4] = [(Le - 1) * La + 3, (Le - 2) * La + 50, 7, (Le - 1) * La + 80]   # near the plane and the pole
+
+    def run(sel):
+        idx = torch.from_numpy(np.ascontiguousarray(sel)).cuda()
+        cnt = torch.tensor([len(sel)], dtype=torch.int32, device="cuda")
+        th = torch.full((len(sel), 2), float("nan"), dtype=torch.float64, device="cuda")
+        doa.doa_refine_peaks2d(B, M, K, az, geom, idx, cnt, th)
+        torch.cuda.synchronize()
+        return th.cpu().numpy()
+
+    alone = np.concatenate([run(pts[i:i + 1]) for i in range(len(pts))])
+    for n in (2, 3, 5, 13):
+        got = np.concatenate([run(pts[i:i + n]) for i in range(0, len(pts), n)])
+        assert np.array_equal(got, alone), n
+    assert np.all(np.abs(alone[:, 0] - step * (pts % La)) <= step * (1 + 1e-12))
+    assert np.all(np.abs(alone[:, 1] - step * (pts // La)) <= step * (1 + 1e-12))
