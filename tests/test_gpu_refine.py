@@ -324,3 +324,69 @@ def test_refine2d_long_searches_do_not_depend_on_company(env, M, d):
         assert np.array_equal(got, alone), n
     assert np.all(np.abs(alone[:, 0] - step * (pts % La)) <= step * (1 + 1e-12))
     assert np.all(np.abs(alone[:, 1] - step * (pts // La)) <= step * (1 + 1e-12))
+
+
+@pytest.mark.parametrize("n", [1, 40])
+def test_refined_and_root_angles_are_done_when_the_solve_is(env, n):
+    """The root form may run inside the refinement's tail: what follows the solve in the stream, directly
+    and in a captured graph, reads both outputs complete (n ULA problems beside a 2-D one whose search
+    in the array plane is long)."""
+    torch, doa = env
+    from paper_2007_14135_gb300.synth import _rng, snapshots_geometry
+    keep, probs = [], []
+    pos = synth.uca_positions(8, 0.5)
+    posd = torch.from_numpy(np.ascontiguousarray(pos)).cuda()
+    Xg = snapshots_geometry(_rng(5), pos, 512, np.array([40.3, 200.7]), np.array([90.0, 90.0]), 20.0)
+    N, M, L = 256, 8, 1801
+    gen = torch.Generator(device="cuda").manual_seed(n)
+    X = torch.view_as_complex(torch.randn(n, M, N, 2, generator=gen, device="cuda"))
+    for i in range(n + 1):
+        geo = i == n
+        npts = 360 * 90 if geo else L
+        t = (torch.from_numpy(Xg).cuda() if geo else X[i], torch.empty(4 * npts, device="cuda"),
+             torch.full((8,), -1, dtype=torch.int32, device="cuda"), torch.zeros(8, device="cuda"),
+             torch.zeros(4, dtype=torch.int32, device="cuda"))
+        keep.append(t)
+        out = torch.full((16 if geo else 8,), float("nan"), dtype=torch.float64, device="cuda")
+        root = None if geo else torch.full((8,), float("nan"), dtype=torch.float64, device="cuda")
+        keep.append((out, root))
+        if geo:
+            probs.append(doa.make_problem(t[0], 2, 0xF, doa.grid(0.0, 1.0, 360), *t[1:5], None,
+                                          geom=doa.geometry(posd, 1.0, 1.0, 90, True), peak_angle=out))
+        else:
+            probs.append(doa.make_problem(t[0], 2, 0xF, doa.grid(-90.0, 0.1, L), *t[1:5], None, peak_angle=out,
+                                          root_angle=root))
+    outs = [o for pair in keep[1::2] for o in pair if o is not None]
+    plan = doa.BatchPlan(probs)
+    ws = doa.workspace(plan)
+    status = torch.full((n + 1,), -1, dtype=torch.int32, device="cuda")
+
+    def solve_and_copy(into):
+        for o in outs:
+            o.fill_(float("nan"))
+        doa.doa_solve_batch(plan, ws, status)
+        for c, o in zip(into, outs):
+            c.copy_(o)
+
+    ref = [torch.empty_like(o) for o in outs]
+    solve_and_copy(ref)
+    torch.cuda.synchronize()
+    want = [o.clone() for o in outs]
+    assert int(status.abs().max()) == 0
+    for r, o in zip(ref, want):
+        assert torch.equal(torch.nan_to_num(r, 1e9), torch.nan_to_num(o, 1e9))
+    s = torch.cuda.Stream()
+    s.wait_stream(torch.cuda.current_stream())
+    with torch.cuda.stream(s):
+        solve_and_copy(ref)
+    torch.cuda.current_stream().wait_stream(s)
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        solve_and_copy(ref)
+    for _ in range(3):
+        for r in ref:
+            r.fill_(0.0)
+        g.replay()
+        torch.cuda.synchronize()
+        for r, o in zip(ref, want):
+            assert torch.equal(torch.nan_to_num(r, 1e9), torch.nan_to_num(o, 1e9))
