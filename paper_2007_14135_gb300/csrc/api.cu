@@ -665,6 +665,13 @@ doa_status doa_batch_plan(const doa_problem *probs, int nprob, const doa_tuning 
     const int64_t gs = std::min<int64_t>(sgsize[b], units / kGeoGroupMinUnits);
     geo_gsize[t] = gs >= geo_group_min(b) ? (int)gs : 0;
   }
+  // points per thread of the geometry problems scanned one by one: the bucket's, if it was asked for
+  int64_t geo_pts[kNumBuckets] = {0, 0, 0, 0};
+  for (int i = 0; i < nprob; ++i)
+    if (probs[i].geom.pos && (steer_of[i] < 0 || geo_gsize[steer_of[i]] == 0))
+      geo_pts[m_bucket(probs[i].M)] += spectrum_points(probs[i]);
+  for (int b = 0; b < kNumBuckets; ++b)
+    h.geo_pt[b] = tuning && tuning->scan_pt[b] != 0 ? tuning->scan_pt[b] : scan_pt_for(b, geo_pts[b]);
   for (int i = 0; i < nprob; ++i) {
     const doa_problem &p = probs[i];
     PlanProblem &q = pp[i];
@@ -712,7 +719,7 @@ doa_status doa_batch_plan(const doa_problem *probs, int nprob, const doa_tuning 
       ++h.geo_jobs[b];
       q.tile_start = 0;
       if (q.geo_steer < 0 || geo_gsize[q.geo_steer] == 0) {
-        const int tp = kScanThreads * pt[b];
+        const int tp = kScanThreads * h.geo_pt[b];
         q.tile_start = h.geo_tiles[b];
         h.geo_tiles[b] += (q.npts + tp - 1) / tp;
         geo[b][h.geo_alone[b]++] = i;

@@ -365,6 +365,7 @@ struct PlanHeader {
   int64_t gg_units[kNumBuckets];
   int64_t off_gg[kNumBuckets];           // PlanScanGroup arrays (grid_id: the shared steering table)
   int64_t off_ggl[kNumBuckets];          // their problem lists
+  int32_t geo_pt[kNumBuckets];           // grid points per thread of the geometry scan
 };
 
 // The Python binding reads these header fields by position (int32 index 22 = scan_pt, 58 = eig_mats,
@@ -392,7 +393,7 @@ static_assert(offsetof(PlanHeader, sg_size) == 464 && offsetof(PlanHeader, sg_un
 static_assert(offsetof(PlanHeader, tcg_groups) == 608 && offsetof(PlanHeader, tcg_units) == 624,
               "PlanHeader layout changed");
 static_assert(offsetof(PlanHeader, geo_alone) == 688 && offsetof(PlanHeader, gg_units) == 704 &&
-                  sizeof(PlanHeader) == 800,
+                  sizeof(PlanHeader) == 816,
               "PlanHeader layout changed");
 
 // Scan tiles: kScanThreads threads, each evaluating PT consecutive grid points (tile shape
@@ -400,6 +401,14 @@ static_assert(offsetof(PlanHeader, geo_alone) == 688 && offsetof(PlanHeader, gg_
 // to {1,2,4} for M <= 16, {1,2} for M <= 32 and 1 for M <= 64.
 constexpr int kScanThreads = 128;
 __host__ __device__ constexpr int scan_pt_default(int bucket) { return bucket <= 1 ? 4 : 1; }
+// Points per thread of scans of npts points in all: the default, or 1 where that leaves SMs without work (a
+// thread's points are then most of the kernel's length). Single scans, 4 points / 1 point per thread: M = 8,
+// 1801 points 6.2 / 5.6 us, 60 001 8.4 / 8.0, 360 x 90 11.1 / 10.0; M = 16, 1801 9.0 / 7.2 us, 18 001
+// 9.0 / 7.3, 60 001 10.9 / 11.1, 360 x 90 15.2 / 12.3.
+constexpr int64_t kScanFewPoints = 304 * 128;
+__host__ __device__ constexpr int scan_pt_for(int bucket, int64_t npts) {
+  return npts < kScanFewPoints * (bucket == 0 ? 2 : 1) ? 1 : scan_pt_default(bucket);
+}
 __host__ __device__ inline bool scan_pt_allowed(int bucket, int pt) {
   return pt == 1 || (pt == 2 && bucket <= 2) || (pt == 4 && bucket <= 1);
 }

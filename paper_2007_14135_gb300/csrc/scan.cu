@@ -43,6 +43,8 @@ __global__ void grid_table_single_kernel(double lo, double step, int k0, int n, 
 }
 
 __global__ void grid_table_batch_kernel(const uint8_t *plan, uint8_t *ws) {
+  // the covariance may start now: it reads none of the tables, and ends after this kernel
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const PlanHeader *h = reinterpret_cast<const PlanHeader *>(plan);
   const PlanGrid g = reinterpret_cast<const PlanGrid *>(plan + h->off_grid)[blockIdx.y];
   uint32_t *S = reinterpret_cast<uint32_t *>(ws + g.S_off);
@@ -503,14 +505,17 @@ cudaError_t launch_grid_tables(const uint8_t *plan_dev, const PlanHeader &h, uin
 cudaError_t launch_scan_single(const double2 *B, int M, int K, int L, double lo, double step, int kofs,
                                const uint32_t *S, float *P, cudaStream_t s) {
   const int b = m_bucket(M);
-  const int tp = kScanThreads * scan_pt_default(b);
+  const int pt = scan_pt_for(b, L), tp = kScanThreads * pt;
   const unsigned grid = (unsigned)((L + tp - 1) / tp);
+#define DOA_SCAN_SINGLE(MP, PT) \
+  scan_single_kernel<MP, PT><<<grid, kScanThreads, 0, s>>>(B, M, K, L, lo, step, kofs, S, P)
   switch (b) {
-    case 0: scan_single_kernel<8, 4><<<grid, kScanThreads, 0, s>>>(B, M, K, L, lo, step, kofs, S, P); break;
-    case 1: scan_single_kernel<16, 4><<<grid, kScanThreads, 0, s>>>(B, M, K, L, lo, step, kofs, S, P); break;
-    case 2: scan_single_kernel<32, 1><<<grid, kScanThreads, 0, s>>>(B, M, K, L, lo, step, kofs, S, P); break;
-    default: scan_single_kernel<64, 1><<<grid, kScanThreads, 0, s>>>(B, M, K, L, lo, step, kofs, S, P); break;
+    case 0: if (pt == 4) DOA_SCAN_SINGLE(8, 4); else DOA_SCAN_SINGLE(8, 1); break;
+    case 1: if (pt == 4) DOA_SCAN_SINGLE(16, 4); else DOA_SCAN_SINGLE(16, 1); break;
+    case 2: DOA_SCAN_SINGLE(32, 1); break;
+    default: DOA_SCAN_SINGLE(64, 1); break;
   }
+#undef DOA_SCAN_SINGLE
   return cudaGetLastError();
 }
 

@@ -54,6 +54,7 @@ struct GeoParams {
 struct GeoShared {
   float4 p32[kMaxM];     // 4 x centred positions in FP32 (x, y, z, 0); rows >= M zero
   double cen[3];         // centroid (FP64)
+  double scale;          // factor of the refinement thresholds
 };
 
 // (sin, cos) table entry e of a grid: e < La the azimuth theta_e, else the elevation angle
@@ -75,12 +76,37 @@ __global__ void geo_table_single_kernel(double az_lo, double az_step, int La, do
 }
 
 __global__ void geo_table_batch_kernel(const uint8_t *plan, uint8_t *ws) {
+  // the covariance may start now: it reads none of the tables, and ends after this kernel
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const PlanHeader *h = reinterpret_cast<const PlanHeader *>(plan);
   const PlanGeoGrid g = reinterpret_cast<const PlanGeoGrid *>(plan + h->off_geo_grid)[blockIdx.y];
   float2 *t32 = reinterpret_cast<float2 *>(ws + g.t32_off);
   double2 *t64 = reinterpret_cast<double2 *>(ws + g.t64_off);
   for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < g.La + g.Le; e += gridDim.x * blockDim.x)
     geo_table_entry(g.az_lo, g.az_step, g.La, g.el_lo, g.el_step, e, t32, t64);
+}
+
+// Centroid of the M positions (FP64, each coordinate summed in order), by one warp: a lane per coordinate,
+// since an FP64 instruction costs the same for one lane as for 32.
+__device__ __forceinline__ void geo_centroid(const double *pos, int M, double (&cen)[3]) {
+  const int lane = threadIdx.x & 31, c = lane < 3 ? lane : 0;
+  double s = 0.0;
+  for (int m = 0; m < M; ++m) s += pos[3 * m + c];
+  s /= M;
+#pragma unroll
+  for (int k = 0; k < 3; ++k) cen[k] = __shfl_sync(0xffffffffu, s, k);
+}
+
+// ((eps_a + 3) / 4)^2, the factor of the refinement thresholds (see the top of the file), by one warp.
+__device__ __forceinline__ double geo_threshold_scale(const double *pos, int M, const double *cen) {
+  double rho = 0.0;
+  for (int m = threadIdx.x & 31; m < M; m += 32)
+    rho = fmax(rho, fabs(pos[3 * m] - cen[0]) + fabs(pos[3 * m + 1] - cen[1]) + fabs(pos[3 * m + 2] - cen[2]));
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) rho = fmax(rho, __shfl_xor_sync(0xffffffffu, rho, off));
+  const double ea = 2.0 * 3.141592653589793 * rho * 7.0 + 3.0;
+  const double sc = (ea + 3.0) / 4.0;
+  return fmax(sc * sc, 1.0);
 }
 
 // FP64 steering source of the refinement and of the shared tables: flat point i -> (u, v, w), then
@@ -109,20 +135,16 @@ struct GeoSource {
 // at a time as (Re, Re, Im, Im) (the operand pairs of the paired contraction), the FP64 phasor of the
 // refinement rounded to FP32; rows m >= M and points i >= npts are zero.
 __global__ void geo_steer_kernel(const uint8_t *plan, uint8_t *ws) {
+  // the covariance may start now: it reads none of the tables, and ends after this kernel
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const PlanHeader *h = reinterpret_cast<const PlanHeader *>(plan);
   const PlanGeoSteer st = reinterpret_cast<const PlanGeoSteer *>(plan + h->off_geo_steer)[blockIdx.y];
   const PlanGeoGrid g = reinterpret_cast<const PlanGeoGrid *>(plan + h->off_geo_grid)[st.geo_grid];
   __shared__ double cen[3];
-  if (threadIdx.x == 0) {
-    double cx = 0.0, cy = 0.0, cz = 0.0;
-    for (int m = 0; m < st.M; ++m) {
-      cx += st.pos[3 * m];
-      cy += st.pos[3 * m + 1];
-      cz += st.pos[3 * m + 2];
-    }
-    cen[0] = cx / st.M;
-    cen[1] = cy / st.M;
-    cen[2] = cz / st.M;
+  if (threadIdx.x < 32) {
+    double c[3];
+    geo_centroid(st.pos, st.M, c);
+    if (threadIdx.x == 0) cen[0] = c[0], cen[1] = c[1], cen[2] = c[2];
   }
   __syncthreads();
   GeoSource src;
@@ -150,34 +172,15 @@ __global__ void geo_steer_kernel(const uint8_t *plan, uint8_t *ws) {
   }
 }
 
-// Centroid of the M positions (FP64, in order).
-__device__ __forceinline__ void geo_centroid(const double *pos, int M, double *cen) {
-  double cx = 0.0, cy = 0.0, cz = 0.0;
-  for (int m = 0; m < M; ++m) {
-    cx += pos[3 * m];
-    cy += pos[3 * m + 1];
-    cz += pos[3 * m + 2];
-  }
-  cen[0] = cx / M;
-  cen[1] = cy / M;
-  cen[2] = cz / M;
-}
-
-// ((eps_a + 3) / 4)^2, the factor of the refinement thresholds (see the top of the file).
-__device__ __forceinline__ double geo_threshold_scale(const double *pos, int M, const double *cen) {
-  double rho = 0.0;
-  for (int m = 0; m < M; ++m)
-    rho = fmax(rho, fabs(pos[3 * m] - cen[0]) + fabs(pos[3 * m + 1] - cen[1]) + fabs(pos[3 * m + 2] - cen[2]));
-  const double ea = 2.0 * 3.141592653589793 * rho * 7.0 + 3.0;
-  const double sc = (ea + 3.0) / 4.0;
-  return fmax(sc * sc, 1.0);
-}
-
 // Per-job constants: centroid, FP32 positions and the scaled thresholds. Every thread of the CTA
 // calls it after load_job; it ends with a barrier.
 template <int MP>
 __device__ void geo_setup(const float2 *Bs, const ScanJob &j, const GeoParams &g, GeoShared &gs, ScanShared &sh) {
-  if (threadIdx.x == 0) geo_centroid(g.pos, j.M, gs.cen);
+  if (threadIdx.x < 32) {
+    double cen[3];
+    geo_centroid(g.pos, j.M, cen);
+    if (threadIdx.x == 0) gs.cen[0] = cen[0], gs.cen[1] = cen[1], gs.cen[2] = cen[2];
+  }
   __syncthreads();
   for (int m = threadIdx.x; m < MP; m += blockDim.x) {
     float4 p = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -187,11 +190,12 @@ __device__ void geo_setup(const float2 *Bs, const ScanJob &j, const GeoParams &g
     gs.p32[m] = p;
   }
   set_threshold<MP>(Bs, j, sh);
-  __syncthreads();
-  if (threadIdx.x == 0) {
+  if (threadIdx.x >= 32 && threadIdx.x < 64) {   // beside it
     const double sc = geo_threshold_scale(g.pos, j.M, gs.cen);
-    for (int r = 0; r < 4; ++r) sh.thr[r] = (float)(sh.thr[r] * sc);
+    if (threadIdx.x == 32) gs.scale = sc;
   }
+  __syncthreads();
+  if (threadIdx.x < 4) sh.thr[threadIdx.x] = (float)(sh.thr[threadIdx.x] * gs.scale);
   __syncthreads();
 }
 
@@ -457,7 +461,11 @@ __global__ void __launch_bounds__(kScanThreads, 3) scan_geometry_shared_kernel(c
     const PlanGeoGrid &gg = geo_grids[st.geo_grid];
     if (gi != cached) {   // the previous unit's drain has ended (barrier at its end)
       for (int i = tid; i < gr.count; i += kScanThreads) jobs[i] = geo_job(probs[list[gr.first + i]], ws);
-      if (tid == 0) geo_centroid(st.pos, st.M, cen);
+      if (tid < 32) {
+        double c[3];
+        geo_centroid(st.pos, st.M, c);
+        if (tid == 0) cen[0] = c[0], cen[1] = c[1], cen[2] = c[2];
+      }
       __syncthreads();
       cached = gi;
     }
@@ -547,15 +555,17 @@ cudaError_t launch_scan_geometry_single(const double2 *B, int M, int K, const do
   geo_table_single_kernel<<<(La + Le + 255) / 256, 256, 0, s>>>(az_lo, az_step, La, el_lo, el_step, Le, t32, t64);
   GeoParams g{pos, t32, t64, La, Le};
   const int b = m_bucket(M);
-  const int pt = scan_pt_default(b);
   const int64_t npts = (int64_t)La * Le;
+  const int pt = scan_pt_for(b, npts);
   const unsigned grid = (unsigned)((npts + kScanThreads * pt - 1) / (kScanThreads * pt));
+#define DOA_GEO_SINGLE(MP, PT) scan_geometry_single_kernel<MP, PT><<<grid, kScanThreads, 0, s>>>(B, M, K, g, P)
   switch (b) {
-    case 0: scan_geometry_single_kernel<8, 4><<<grid, kScanThreads, 0, s>>>(B, M, K, g, P); break;
-    case 1: scan_geometry_single_kernel<16, 4><<<grid, kScanThreads, 0, s>>>(B, M, K, g, P); break;
-    case 2: scan_geometry_single_kernel<32, 1><<<grid, kScanThreads, 0, s>>>(B, M, K, g, P); break;
-    default: scan_geometry_single_kernel<64, 1><<<grid, kScanThreads, 0, s>>>(B, M, K, g, P); break;
+    case 0: if (pt == 4) DOA_GEO_SINGLE(8, 4); else DOA_GEO_SINGLE(8, 1); break;
+    case 1: if (pt == 4) DOA_GEO_SINGLE(16, 4); else DOA_GEO_SINGLE(16, 1); break;
+    case 2: DOA_GEO_SINGLE(32, 1); break;
+    default: DOA_GEO_SINGLE(64, 1); break;
   }
+#undef DOA_GEO_SINGLE
   return cudaGetLastError();
 }
 
@@ -575,19 +585,19 @@ cudaError_t launch_scan_geometry_batch(const uint8_t *plan_dev, const PlanHeader
   if (e != cudaSuccess) return e;
   e = run_geo_shared<16, geo_group_pt(1)>(plan_dev, h, ws, 1, s);
   if (e != cudaSuccess) return e;
-  switch (h.scan_pt[0]) {
+  switch (h.geo_pt[0]) {
     case 1: e = run_geo_batch<8, 1>(plan_dev, h, ws, 0, s); break;
     case 2: e = run_geo_batch<8, 2>(plan_dev, h, ws, 0, s); break;
     default: e = run_geo_batch<8, 4>(plan_dev, h, ws, 0, s); break;
   }
   if (e != cudaSuccess) return e;
-  switch (h.scan_pt[1]) {
+  switch (h.geo_pt[1]) {
     case 1: e = run_geo_batch<16, 1>(plan_dev, h, ws, 1, s); break;
     case 4: e = run_geo_batch<16, 4>(plan_dev, h, ws, 1, s); break;
     default: e = run_geo_batch<16, 2>(plan_dev, h, ws, 1, s); break;
   }
   if (e != cudaSuccess) return e;
-  if (h.scan_pt[2] == 2)
+  if (h.geo_pt[2] == 2)
     e = run_geo_batch<32, 2>(plan_dev, h, ws, 2, s);
   else
     e = run_geo_batch<32, 1>(plan_dev, h, ws, 2, s);

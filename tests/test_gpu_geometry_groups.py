@@ -58,3 +58,44 @@ def test_groups_match_single_problems(env, M, La, Le, B, mask, d):
         out.append((P, idx, val, cnt))
     for a, b in zip(*out):
         assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("M", [5, 8, 13, 16])
+def test_points_per_thread_give_the_same_spectrum(env, M):
+    """A few scans take one point per thread (ULA and geometry, single calls and the batch): bit for bit
+    the spectrum of four points per thread, at sizes on both sides of the rule."""
+    torch, doa = env
+    rng = np.random.default_rng(M)
+    N = 128
+    X = torch.view_as_complex(torch.randn(M, N, 2, generator=torch.Generator(device="cuda").manual_seed(M),
+                                          device="cuda"))
+    t = 2.0 * np.pi * np.arange(M) / M
+    pos = torch.from_numpy(np.stack([0.5 * np.cos(t), 0.5 * np.sin(t), 0.1 * rng.standard_normal(M)], axis=1)).cuda()
+    Q, _ = np.linalg.qr(rng.standard_normal((M, M)) + 1j * rng.standard_normal((M, M)))
+    B = torch.from_numpy(np.ascontiguousarray(Q[:, :M - 2].T).reshape(-1)).cuda()
+    for La, Le in ((1, 1), (97, 13), (360, 90), (361, 333)):
+        out = []
+        for pt in (None, (4, 4, 1, 1), (2, 2, 1, 1), (1, 1, 1, 1)):
+            P = torch.zeros(4 * La * Le, device="cuda")
+            idx = torch.full((8,), -1, dtype=torch.int32, device="cuda")
+            val = torch.zeros(8, device="cuda")
+            cnt = torch.zeros(4, dtype=torch.int32, device="cuda")
+            prob = doa.make_problem(X, 2, 0xF, doa.grid(0.0, 360.0 / La, La), P, idx, val, cnt, None,
+                                    geom=doa.geometry(pos, 2.0, 0.9, Le, True))
+            plan = doa.BatchPlan([prob], scan_pt=pt)
+            status = torch.full((1,), -1, dtype=torch.int32, device="cuda")
+            doa.doa_solve_batch(plan, doa.workspace(plan), status)
+            torch.cuda.synchronize()
+            assert int(status) == 0
+            out.append((P, idx, val, cnt))
+        for o in out[1:]:
+            for a, b in zip(out[0], o):
+                assert torch.equal(a, b)
+    # single ULA scans: a long grid (four points per thread) against its pieces (one point per thread)
+    L, piece = 100003, 7001
+    P = torch.empty(L, device="cuda")
+    doa.doa_scan(B, M, M - 2, doa.grid(-90.0, 180.0 / (L - 1), L), P)
+    short = torch.empty(piece, device="cuda")
+    doa.doa_scan(B, M, M - 2, doa.grid(-90.0, 180.0 / (L - 1), piece), short)
+    torch.cuda.synchronize()
+    assert torch.equal(P[:piece], short)
