@@ -497,6 +497,7 @@ __device__ void cov_tasks(const float2 *__restrict__ X, int M, int ldx, int t0, 
 template <int MB, int kKind>
 __global__ void __launch_bounds__(CovKind<MB, kKind>::kThreads, CovKind<MB, kKind>::kMinBlocks) covariance_tasks_kernel(const uint8_t *plan,
                                                                                         uint8_t *ws, int first) {
+  let_next_start();
   extern __shared__ __align__(16) uint8_t smem[];
   const PlanHeader *h = reinterpret_cast<const PlanHeader *>(plan);
   const PlanCovItem it = reinterpret_cast<const PlanCovItem *>(plan + h->off_cov)[first + blockIdx.x];
@@ -511,10 +512,12 @@ __global__ void __launch_bounds__(CovKind<MB, kKind>::kThreads, CovKind<MB, kKin
     cov_tasks<MB, kKind, true>(X, M, pp.p.ldx, t0, t1, smem, pp.nchunks, inv_n, R64, partial);
   else
     cov_tasks<MB, kKind, false>(X, M, pp.p.ldx, t0, t1, smem, pp.nchunks, inv_n, R64, partial);
+  end_after_previous();
 }
 
 // Batch: one CTA per work item (problem, chunk) of the generic class.
 __global__ void __launch_bounds__(kCovThreads) covariance_batch_kernel(const uint8_t *plan, uint8_t *ws, int first) {
+  let_next_start();
   extern __shared__ __align__(16) uint8_t smem[];
   const PlanHeader *h = reinterpret_cast<const PlanHeader *>(plan);
   const PlanCovItem it = reinterpret_cast<const PlanCovItem *>(plan + h->off_cov)[first + blockIdx.x];
@@ -538,6 +541,7 @@ __global__ void __launch_bounds__(kCovThreads) covariance_batch_kernel(const uin
     else
       partial[row * M + col] = v;
   }
+  end_after_previous();
 }
 
 // Batch reduce: one CTA per multi-chunk problem, chunk partials added in chunk order.
@@ -648,8 +652,7 @@ cudaError_t launch_tasks_kind(const uint8_t *plan_dev, int first, int n, uint8_t
   using K = CovKind<MB, kKind>;
   cudaError_t e = ensure_smem_attr(reinterpret_cast<const void *>(covariance_tasks_kernel<MB, kKind>), K::kSmem);
   if (e != cudaSuccess) return e;
-  covariance_tasks_kernel<MB, kKind><<<n, K::kThreads, K::kSmem, s>>>(plan_dev, ws, first);
-  return cudaGetLastError();
+  return launch_beside(true, covariance_tasks_kernel<MB, kKind>, n, K::kThreads, K::kSmem, s, plan_dev, ws, first);
 }
 
 template <int MB>
@@ -665,16 +668,19 @@ cudaError_t launch_covariance_batch(const uint8_t *plan_dev, const PlanHeader &h
                                     cudaStream_t s) {
   cudaError_t e = ensure_smem_attr(reinterpret_cast<const void *>(covariance_batch_kernel), kSmemBytes);
   if (e != cudaSuccess) return e;
+  // the classes beside each other, and the first beside the phase tables (which always precede it)
   if ((e = launch_tasks<2>(plan_dev, h, ws, s)) != cudaSuccess) return e;
   if ((e = launch_tasks<3>(plan_dev, h, ws, s)) != cudaSuccess) return e;
   if ((e = launch_tasks<4>(plan_dev, h, ws, s)) != cudaSuccess) return e;
   const int ngen = h.cov_first[kCovClasses] - h.cov_first[kCovClasses - 1];
   if (ngen > 0)
-    covariance_batch_kernel<<<ngen, kCovThreads, kSmemBytes, s>>>(plan_dev, ws, h.cov_first[kCovClasses - 1]);
-  if (h.nreduce > 0) covariance_reduce_batch<<<h.nreduce, 256, 0, s>>>(plan_dev, ws);
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    if ((e = launch_beside(true, covariance_batch_kernel, ngen, kCovThreads, kSmemBytes, s, plan_dev, ws,
+                           h.cov_first[kCovClasses - 1])) != cudaSuccess)
+      return e;
   // problems with M <= 16: tensor cores, then the recomputation of any it marked
   if ((e = launch_covariance_tc_batch(plan_dev, h, ws, s)) != cudaSuccess) return e;
+  if (h.nreduce > 0) covariance_reduce_batch<<<h.nreduce, 256, 0, s>>>(plan_dev, ws);
+  if ((e = cudaGetLastError()) != cudaSuccess) return e;
   return launch_covariance_fixup(plan_dev, h, ws, s);
 }
 

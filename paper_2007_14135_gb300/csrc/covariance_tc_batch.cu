@@ -302,6 +302,7 @@ template <int MP>
 __global__ void __launch_bounds__(kCbThreads, 1) covariance_tc_batch_kernel(const uint8_t *plan, uint8_t *ws, int cls) {
   using S = CbShape<MP>;
   using Lay = CbLayout<MP>;
+  let_next_start();
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   uint8_t *sm = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   __shared__ CbShared sh;
@@ -646,8 +647,7 @@ __global__ void __launch_bounds__(kCbThreads, 1) covariance_tc_batch_kernel(cons
   if (*abort && tid == 0)   // every problem of this CTA goes to the fixup kernel
     for (int pi = blockIdx.x; pi < count; pi += gridDim.x) flags[pi] = 2;
   if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512));
-  // launched inside the kernel that writes the phase tables: what follows in the stream finds both done
-  asm volatile("griddepcontrol.wait;" ::: "memory");
+  end_after_previous();
 }
 
 template <int MP>
@@ -657,20 +657,7 @@ cudaError_t launch_class(const uint8_t *plan_dev, const PlanHeader &h, uint8_t *
   cudaError_t e = ensure_smem_attr(reinterpret_cast<const void *>(covariance_tc_batch_kernel<MP>), CbLayout<MP>::kSmem);
   if (e != cudaSuccess) return e;
   const int grid = n < device_sm_count() ? n : device_sm_count();   // one CTA per SM (512 TMEM columns)
-  // The first kernel of the covariance runs beside the phase tables, which it does not read (programmatic
-  // dependent launch): one 360 x 90 estimate loses about 10 of 104 us by it.
-  const bool first = h.cov_first[kCovClasses] == 0 && (cls == 0 || h.ncovtc[0] == 0);
-  cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3((unsigned)grid);
-  cfg.blockDim = dim3(kCbThreads);
-  cfg.dynamicSmemBytes = CbLayout<MP>::kSmem;
-  cfg.stream = s;
-  cudaLaunchAttribute attr{};
-  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr.val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = &attr;
-  cfg.numAttrs = first ? 1 : 0;
-  return cudaLaunchKernelEx(&cfg, covariance_tc_batch_kernel<MP>, plan_dev, ws, cls);
+  return launch_beside(true, covariance_tc_batch_kernel<MP>, grid, kCbThreads, CbLayout<MP>::kSmem, s, plan_dev, ws, cls);
 }
 
 }  // namespace

@@ -881,6 +881,7 @@ __device__ __forceinline__ bool refines_2d(const doa_problem &p) { return p.geom
 template <int NP, int G>
 __global__ void __launch_bounds__(32 * eig_warps<NP>(), eig_min_ctas<NP>()) eig_batch_kernel(const uint8_t *plan, uint8_t *ws, int bucket,
                                                                          int *status) {
+  let_next_start();
   extern __shared__ __align__(16) uint8_t smem[];
   const int grp = threadIdx.x / 32;
   EigSmem<NP> *mats = reinterpret_cast<EigSmem<NP> *>(smem) + grp * G;
@@ -910,12 +911,14 @@ __global__ void __launch_bounds__(32 * eig_warps<NP>(), eig_min_ctas<NP>()) eig_
     if (prob[j] < 0) continue;
     finish_batch<NP, 32>(probs[prob[j]], jobs, mats[j], res[j], ws, status + prob[j]);
   }
+  end_after_previous();
 }
 
 // The CTA form of the batch: a CTA per matrix.
 template <int NP>
 __global__ void __launch_bounds__(cta_threads<NP>()) eig_batch_cta_kernel(const uint8_t *plan, uint8_t *ws, int bucket,
                                                                           int *status) {
+  let_next_start();
   extern __shared__ __align__(16) uint8_t smem[];
   constexpr int T = cta_threads<NP>();
   EigSmem<NP> &s = *reinterpret_cast<EigSmem<NP> *>(smem);
@@ -932,12 +935,14 @@ __global__ void __launch_bounds__(cta_threads<NP>()) eig_batch_cta_kernel(const 
   else
     jacobi_group<ArithDF<NP>, NP, 1, T>(&s, Ms, Rs, both, res);
   finish_batch<NP, T>(pp, jobs, s, res[0], ws, status + prob);
+  end_after_previous();
 }
 
 // Bucket M <= 64 of the batch in double-float: one four-CTA cluster per problem; rank 0 finishes.
 // A problem that asks for the FP64 Jacobi runs it in rank 0 alone (the other CTAs leave at once).
 __global__ void __cluster_dims__(kClRanks, 1, 1) __launch_bounds__(kClThreads, 1)
     eig_cluster_batch_kernel(const uint8_t *plan, uint8_t *ws, int bucket, int *status) {
+  let_next_start();
   extern __shared__ __align__(16) uint8_t smem[];
   EigSmem<64> &s = *reinterpret_cast<EigSmem<64> *>(smem);
   ClusterDF &w = *reinterpret_cast<ClusterDF *>(smem + kClFinBytes);
@@ -964,6 +969,7 @@ __global__ void __cluster_dims__(kClRanks, 1, 1) __launch_bounds__(kClThreads, 1
     if (!rank0) return;
   }
   finish_batch<64, kClThreads>(pp, jobs, s, res, ws, status + prob);
+  end_after_previous();
 }
 
 
@@ -1017,50 +1023,49 @@ int eig_cta_warps() {
 }
 
 template <int NP, int G>
-cudaError_t run_batch_g(const uint8_t *plan, int count, uint8_t *ws, int *status, int bucket, cudaStream_t st) {
+cudaError_t run_batch_g(const uint8_t *plan, int count, uint8_t *ws, int *status, int bucket, bool beside, cudaStream_t st) {
   const int W = eig_cta_warps<NP, G>();
   const int per_cta = W * G;
   const int smem = (int)sizeof(EigSmem<NP>) * per_cta;
   cudaError_t e = ensure_smem_attr(reinterpret_cast<const void *>(eig_batch_kernel<NP, G>), smem);
   if (e != cudaSuccess) return e;
-  eig_batch_kernel<NP, G><<<(count + per_cta - 1) / per_cta, 32 * W, smem, st>>>(plan, ws, bucket, status);
-  return cudaGetLastError();
+  return launch_beside(beside, eig_batch_kernel<NP, G>, (count + per_cta - 1) / per_cta, 32 * W, smem, st, plan, ws, bucket,
+                       status);
 }
 
 template <int NP>
-cudaError_t run_batch_cta(const uint8_t *plan, int count, uint8_t *ws, int *status, int bucket, cudaStream_t st) {
+cudaError_t run_batch_cta(const uint8_t *plan, int count, uint8_t *ws, int *status, int bucket, bool beside, cudaStream_t st) {
   if (count == 0) return cudaSuccess;
   const int smem = (int)sizeof(EigSmem<NP>);
   cudaError_t e = ensure_smem_attr(reinterpret_cast<const void *>(eig_batch_cta_kernel<NP>), smem);
   if (e != cudaSuccess) return e;
-  eig_batch_cta_kernel<NP><<<(unsigned)count, cta_threads<NP>(), smem, st>>>(plan, ws, bucket, status);
-  return cudaGetLastError();
+  return launch_beside(beside, eig_batch_cta_kernel<NP>, count, cta_threads<NP>(), smem, st, plan, ws, bucket, status);
 }
 
 // M <= 16: the CTA form for small batches unless the plan packs matrices (G in {1, 2, 4, 8} up to the
 // bucket's maximum per warp), else the warp form.
 template <int NP>
 cudaError_t run_batch(const uint8_t *plan, const PlanHeader &h, uint8_t *ws, int *status, int bucket,
-                      cudaStream_t st) {
+                      bool beside, cudaStream_t st) {
   const int count = h.eig_count[bucket];
   const int g = h.eig_mats[bucket];
-  if (g == 1 && count <= eig_cta_limit<NP>()) return run_batch_cta<NP>(plan, count, ws, status, bucket, st);
+  if (g == 1 && count <= eig_cta_limit<NP>()) return run_batch_cta<NP>(plan, count, ws, status, bucket, beside, st);
   if (count == 0) return cudaSuccess;
-  if (g >= 8 && mats_per_warp<NP>() >= 8) return run_batch_g<NP, (mats_per_warp<NP>() >= 8 ? 8 : 1)>(plan, count, ws, status, bucket, st);
-  if (g >= 4) return run_batch_g<NP, 4>(plan, count, ws, status, bucket, st);
-  if (g >= 2) return run_batch_g<NP, 2>(plan, count, ws, status, bucket, st);
-  return run_batch_g<NP, 1>(plan, count, ws, status, bucket, st);
+  if (g >= 8 && mats_per_warp<NP>() >= 8) return run_batch_g<NP, (mats_per_warp<NP>() >= 8 ? 8 : 1)>(plan, count, ws, status, bucket, beside, st);
+  if (g >= 4) return run_batch_g<NP, 4>(plan, count, ws, status, bucket, beside, st);
+  if (g >= 2) return run_batch_g<NP, 2>(plan, count, ws, status, bucket, beside, st);
+  return run_batch_g<NP, 1>(plan, count, ws, status, bucket, beside, st);
 }
 
 // Bucket M <= 64: one four-CTA cluster per problem.
 cudaError_t run_batch_cluster(const uint8_t *plan, const PlanHeader &h, uint8_t *ws, int *status, int bucket,
-                              cudaStream_t st) {
+                              bool beside, cudaStream_t st) {
   const int count = h.eig_count[bucket];
   if (count == 0) return cudaSuccess;
   cudaError_t e = ensure_smem_attr(reinterpret_cast<const void *>(eig_cluster_batch_kernel), kClSmemBytes);
   if (e != cudaSuccess) return e;
-  eig_cluster_batch_kernel<<<(unsigned)count * kClRanks, kClThreads, kClSmemBytes, st>>>(plan, ws, bucket, status);
-  return cudaGetLastError();
+  return launch_beside(beside, eig_cluster_batch_kernel, (int64_t)count * kClRanks, kClThreads, kClSmemBytes, st, plan, ws,
+                       bucket, status);
 }
 
 }  // namespace
@@ -1121,10 +1126,15 @@ cudaError_t launch_eig_single(const double2 *R64, int M, int d, int alg, int pre
 cudaError_t launch_eig_batch(const uint8_t *plan_dev, const PlanHeader &h, uint8_t *ws, int *status,
                              cudaStream_t s) {
   cudaError_t e;
-  if ((e = run_batch<8>(plan_dev, h, ws, status, 0, s)) != cudaSuccess) return e;
-  if ((e = run_batch<16>(plan_dev, h, ws, status, 1, s)) != cudaSuccess) return e;
-  if ((e = run_batch_cta<32>(plan_dev, h.eig_count[2], ws, status, 2, s)) != cudaSuccess) return e;
-  return run_batch_cluster(plan_dev, h, ws, status, 3, s);
+  // the buckets beside each other, the largest matrices first: theirs take longest
+  bool beside = false;
+  if ((e = run_batch_cluster(plan_dev, h, ws, status, 3, beside, s)) != cudaSuccess) return e;
+  beside = beside || h.eig_count[3] > 0;
+  if ((e = run_batch_cta<32>(plan_dev, h.eig_count[2], ws, status, 2, beside, s)) != cudaSuccess) return e;
+  beside = beside || h.eig_count[2] > 0;
+  if ((e = run_batch<16>(plan_dev, h, ws, status, 1, beside, s)) != cudaSuccess) return e;
+  beside = beside || h.eig_count[1] > 0;
+  return run_batch<8>(plan_dev, h, ws, status, 0, beside, s);
 }
 
 }  // namespace doa

@@ -700,7 +700,7 @@ __global__ void __launch_bounds__(32 * kRefWarps, 3) refine_batch_kernel(const u
   __shared__ GeoLong co;
   // once every CTA of this grid has started, the next kernel in the stream may use the SMs that the tail of
   // long searches leaves idle (the root form, which waits for this grid's end before it ends itself)
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  let_next_start();
   // the first half of the CTAs takes the 2-D jobs, whose longest searches are the kernel's tail
   const bool geo = blockIdx.x < h->njobs;
   const int job = geo ? blockIdx.x : blockIdx.x - h->njobs;

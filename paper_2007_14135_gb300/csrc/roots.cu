@@ -337,7 +337,7 @@ __device__ __forceinline__ void roots_job(const uint8_t *plan, uint8_t *ws, int 
 __global__ void __launch_bounds__(32 * kRootWarps) roots_batch_kernel(const uint8_t *plan, uint8_t *ws, int *status) {
   __shared__ RootShared sh[kRootWarps];
   roots_job(plan, ws, status, sh);
-  asm volatile("griddepcontrol.wait;" ::: "memory");
+  end_after_previous();
 }
 
 __global__ void __launch_bounds__(32) roots_single_kernel(RootJob j, double *theta, int *info) {
@@ -350,16 +350,8 @@ __global__ void __launch_bounds__(32) roots_single_kernel(RootJob j, double *the
 
 cudaError_t launch_roots_batch(const uint8_t *plan_dev, const PlanHeader &h, uint8_t *ws, int *status, cudaStream_t s) {
   if (h.nroots == 0 || h.njobs == 0) return cudaSuccess;
-  cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3((unsigned)((h.njobs + kRootWarps - 1) / kRootWarps));
-  cfg.blockDim = dim3(32 * kRootWarps);
-  cfg.stream = s;
-  cudaLaunchAttribute attr{};
-  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr.val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = &attr;
-  cfg.numAttrs = h.nrefine > 0 ? 1 : 0;   // only behind the refinement
-  return cudaLaunchKernelEx(&cfg, roots_batch_kernel, plan_dev, ws, status);
+  return launch_beside(h.nrefine > 0, roots_batch_kernel, (h.njobs + kRootWarps - 1) / kRootWarps, 32 * kRootWarps, 0, s,
+                       plan_dev, ws, status);
 }
 
 cudaError_t launch_roots_single(const double2 *B, int M, int K, int d, double *theta, int *info, cudaStream_t s) {

@@ -43,8 +43,7 @@ __global__ void grid_table_single_kernel(double lo, double step, int k0, int n, 
 }
 
 __global__ void grid_table_batch_kernel(const uint8_t *plan, uint8_t *ws) {
-  // the covariance may start now: it reads none of the tables, and ends after this kernel
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  let_next_start();   // the covariance reads none of the tables
   const PlanHeader *h = reinterpret_cast<const PlanHeader *>(plan);
   const PlanGrid g = reinterpret_cast<const PlanGrid *>(plan + h->off_grid)[blockIdx.y];
   uint32_t *S = reinterpret_cast<uint32_t *>(ws + g.S_off);
@@ -113,6 +112,7 @@ constexpr int kRun = 16;   // longest run (large batches); small ones use shorte
 template <int MP, int PT>
 __global__ void __launch_bounds__(kScanThreads) scan_batch_kernel(const uint8_t *plan, uint8_t *ws, int bucket,
                                                                   int run_len) {
+  let_next_start();
   // factor: (bx, bx, by, by) per element for the paired contraction (PT even), else (bx, by)
   constexpr bool kPair = PT % 2 == 0;
   __shared__ __align__(16) float Fsm[(kPair ? 4 : 2) * (MP + 1) * MP];
@@ -167,6 +167,7 @@ __global__ void __launch_bounds__(kScanThreads) scan_batch_kernel(const uint8_t 
     }
     drain_refinements(j, sh);   // once per run: the warps share the FP64 work of its tiles
   }
+  end_after_previous();
 }
 
 // Grid-shared scan (problems of one M bucket that share a grid, in groups of up to
@@ -184,6 +185,7 @@ __global__ void __launch_bounds__(kScanThreads) scan_batch_kernel(const uint8_t 
 // element, w32, thresholds.
 template <int MP>
 __global__ void __launch_bounds__(kScanThreads) scan_prep_kernel(const uint8_t *plan, uint8_t *ws, int bucket) {
+  let_next_start();
   const PlanHeader *h = reinterpret_cast<const PlanHeader *>(plan);
   const int32_t *list = reinterpret_cast<const int32_t *>(plan + h->off_sgl[bucket]);
   const PlanProblem *probs = reinterpret_cast<const PlanProblem *>(plan + h->off_prob);
@@ -210,6 +212,7 @@ __global__ void __launch_bounds__(kScanThreads) scan_prep_kernel(const uint8_t *
   float thr[4] = {0.f, 0.f, 0.f, 0.f};
   job_thresholds2<MP, true>(F32, w32, Kf, Kn, pp.kphd, pp.kmn, thr);
   if (lane < 4) w32[MP + lane] = thr[lane];
+  end_after_previous();
 }
 
 // CTAs per SM the register budget of the grid-shared scan is set for: 4 where the steering of a
@@ -222,6 +225,7 @@ __host__ __device__ constexpr int shared_min_blocks() {
 template <int MP, int PT>
 __global__ void __launch_bounds__(kScanThreads, shared_min_blocks<MP, PT>())
     scan_shared_kernel(const uint8_t *plan, uint8_t *ws, int bucket) {
+  let_next_start();
   constexpr bool kPair = PT % 2 == 0;
   // paired form: two factor buffers; the next problem's factor, EV weights and thresholds are
   // copied asynchronously while the current one is contracted
@@ -326,6 +330,7 @@ __global__ void __launch_bounds__(kScanThreads, shared_min_blocks<MP, PT>())
     }
     drain_tagged<MP>(jobs, tags, sh, [](const ScanJob &j) { return UlaSource{&j}; });
   }
+  end_after_previous();
 }
 
 // Peak polish (DOA_FLAG_POLISH_PEAKS): one CTA per problem (its first warp picks the points, all warps
@@ -472,7 +477,7 @@ __global__ void __launch_bounds__(32 * kPolishWarps) polish_batch_kernel(const u
 
 
 template <int MP, int PT>
-cudaError_t run_batch(const uint8_t *plan, const PlanHeader &h, uint8_t *ws, int bucket, cudaStream_t s) {
+cudaError_t run_batch(const uint8_t *plan, const PlanHeader &h, uint8_t *ws, int bucket, bool &beside, cudaStream_t s) {
   const int64_t tiles = h.scan_tiles[bucket];
   if (tiles == 0) return cudaSuccess;
   int per_sm = 0;
@@ -481,8 +486,9 @@ cudaError_t run_batch(const uint8_t *plan, const PlanHeader &h, uint8_t *ws, int
   const int64_t cap = (int64_t)device_sm_count() * per_sm;
   const int run_len = (int)std::min<int64_t>(kRun, std::max<int64_t>(1, (tiles + cap - 1) / cap));
   const int64_t grid = std::min<int64_t>(cap, (tiles + run_len - 1) / run_len);
-  scan_batch_kernel<MP, PT><<<(unsigned)grid, kScanThreads, 0, s>>>(plan, ws, bucket, run_len);
-  return cudaGetLastError();
+  const cudaError_t e = launch_beside(beside, scan_batch_kernel<MP, PT>, grid, kScanThreads, 0, s, plan, ws, bucket, run_len);
+  beside = true;
+  return e;
 }
 
 }  // namespace
@@ -525,61 +531,78 @@ cudaError_t launch_polish_batch(const uint8_t *plan_dev, const PlanHeader &h, ui
   return cudaGetLastError();
 }
 
-template <int MP, int PT>
-cudaError_t run_shared(const uint8_t *plan, const PlanHeader &h, uint8_t *ws, int bucket, cudaStream_t s) {
+template <int MP>
+cudaError_t run_prep(const uint8_t *plan, const PlanHeader &h, uint8_t *ws, int bucket, bool &beside, cudaStream_t s) {
   if (h.sg_units[bucket] == 0) return cudaSuccess;
-  scan_prep_kernel<MP><<<(h.sg_probs[bucket] + kScanWarps - 1) / kScanWarps, kScanThreads, 0, s>>>(plan, ws, bucket);
+  const cudaError_t e = launch_beside(beside, scan_prep_kernel<MP>, (h.sg_probs[bucket] + kScanWarps - 1) / kScanWarps,
+                                      kScanThreads, 0, s, plan, ws, bucket);
+  beside = true;
+  return e;
+}
+
+template <int MP, int PT>
+cudaError_t run_shared(const uint8_t *plan, const PlanHeader &h, uint8_t *ws, int bucket, bool &beside, cudaStream_t s) {
+  if (h.sg_units[bucket] == 0) return cudaSuccess;
   int per_sm = 0;
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, scan_shared_kernel<MP, PT>, kScanThreads, 0);
   if (per_sm < 1) per_sm = 1;
   const int64_t grid = std::min<int64_t>((int64_t)device_sm_count() * per_sm, h.sg_units[bucket]);
-  scan_shared_kernel<MP, PT><<<(unsigned)grid, kScanThreads, 0, s>>>(plan, ws, bucket);
-  return cudaGetLastError();
+  const cudaError_t e = launch_beside(beside, scan_shared_kernel<MP, PT>, grid, kScanThreads, 0, s, plan, ws, bucket);
+  beside = true;
+  return e;
 }
 
-static cudaError_t launch_scan_shared(const uint8_t *plan_dev, const PlanHeader &h, uint8_t *ws, cudaStream_t s) {
+// The groups of every bucket: all preparations, then the scans, each set beside each other and the scans of
+// the largest arrays first; the per-problem scans (launch_scan_batch) go on beside them.
+static cudaError_t launch_scan_shared(const uint8_t *plan_dev, const PlanHeader &h, uint8_t *ws, bool &beside,
+                                      cudaStream_t s) {
   cudaError_t e;
-  switch (h.scan_pt[0]) {
-    case 1: e = run_shared<8, 1>(plan_dev, h, ws, 0, s); break;
-    case 2: e = run_shared<8, 2>(plan_dev, h, ws, 0, s); break;
-    default: e = run_shared<8, 4>(plan_dev, h, ws, 0, s); break;
-  }
+  bool prep = false;
+  if ((e = run_prep<64>(plan_dev, h, ws, 3, prep, s)) != cudaSuccess) return e;
+  if ((e = run_prep<32>(plan_dev, h, ws, 2, prep, s)) != cudaSuccess) return e;
+  if ((e = run_prep<16>(plan_dev, h, ws, 1, prep, s)) != cudaSuccess) return e;
+  if ((e = run_prep<8>(plan_dev, h, ws, 0, prep, s)) != cudaSuccess) return e;
+  if ((e = run_shared<64, 1>(plan_dev, h, ws, 3, beside, s)) != cudaSuccess) return e;
+  if (h.scan_pt[2] == 2)
+    e = run_shared<32, 2>(plan_dev, h, ws, 2, beside, s);
+  else
+    e = run_shared<32, 1>(plan_dev, h, ws, 2, beside, s);
   if (e != cudaSuccess) return e;
   switch (h.scan_pt[1]) {
-    case 1: e = run_shared<16, 1>(plan_dev, h, ws, 1, s); break;
-    case 4: e = run_shared<16, 4>(plan_dev, h, ws, 1, s); break;
-    default: e = run_shared<16, 2>(plan_dev, h, ws, 1, s); break;
+    case 1: e = run_shared<16, 1>(plan_dev, h, ws, 1, beside, s); break;
+    case 4: e = run_shared<16, 4>(plan_dev, h, ws, 1, beside, s); break;
+    default: e = run_shared<16, 2>(plan_dev, h, ws, 1, beside, s); break;
   }
   if (e != cudaSuccess) return e;
-  if (h.scan_pt[2] == 2)
-    e = run_shared<32, 2>(plan_dev, h, ws, 2, s);
-  else
-    e = run_shared<32, 1>(plan_dev, h, ws, 2, s);
-  if (e != cudaSuccess) return e;
-  return run_shared<64, 1>(plan_dev, h, ws, 3, s);
+  switch (h.scan_pt[0]) {
+    case 1: return run_shared<8, 1>(plan_dev, h, ws, 0, beside, s);
+    case 2: return run_shared<8, 2>(plan_dev, h, ws, 0, beside, s);
+    default: return run_shared<8, 4>(plan_dev, h, ws, 0, beside, s);
+  }
 }
 
 cudaError_t launch_scan_batch(const uint8_t *plan_dev, const PlanHeader &h, uint8_t *ws, cudaStream_t s) {
-  cudaError_t e = launch_scan_shared(plan_dev, h, ws, s);
+  bool beside = false;
+  cudaError_t e = launch_scan_shared(plan_dev, h, ws, beside, s);
   if (e != cudaSuccess) return e;
   switch (h.scan_pt[0]) {
-    case 1: e = run_batch<8, 1>(plan_dev, h, ws, 0, s); break;
-    case 2: e = run_batch<8, 2>(plan_dev, h, ws, 0, s); break;
-    default: e = run_batch<8, 4>(plan_dev, h, ws, 0, s); break;
+    case 1: e = run_batch<8, 1>(plan_dev, h, ws, 0, beside, s); break;
+    case 2: e = run_batch<8, 2>(plan_dev, h, ws, 0, beside, s); break;
+    default: e = run_batch<8, 4>(plan_dev, h, ws, 0, beside, s); break;
   }
   if (e != cudaSuccess) return e;
   switch (h.scan_pt[1]) {
-    case 1: e = run_batch<16, 1>(plan_dev, h, ws, 1, s); break;
-    case 4: e = run_batch<16, 4>(plan_dev, h, ws, 1, s); break;
-    default: e = run_batch<16, 2>(plan_dev, h, ws, 1, s); break;
+    case 1: e = run_batch<16, 1>(plan_dev, h, ws, 1, beside, s); break;
+    case 4: e = run_batch<16, 4>(plan_dev, h, ws, 1, beside, s); break;
+    default: e = run_batch<16, 2>(plan_dev, h, ws, 1, beside, s); break;
   }
   if (e != cudaSuccess) return e;
   if (h.scan_pt[2] == 2)
-    e = run_batch<32, 2>(plan_dev, h, ws, 2, s);
+    e = run_batch<32, 2>(plan_dev, h, ws, 2, beside, s);
   else
-    e = run_batch<32, 1>(plan_dev, h, ws, 2, s);
+    e = run_batch<32, 1>(plan_dev, h, ws, 2, beside, s);
   if (e != cudaSuccess) return e;
-  return run_batch<64, 1>(plan_dev, h, ws, 3, s);
+  return run_batch<64, 1>(plan_dev, h, ws, 3, beside, s);
 }
 
 }  // namespace doa

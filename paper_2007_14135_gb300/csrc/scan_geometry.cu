@@ -76,8 +76,7 @@ __global__ void geo_table_single_kernel(double az_lo, double az_step, int La, do
 }
 
 __global__ void geo_table_batch_kernel(const uint8_t *plan, uint8_t *ws) {
-  // the covariance may start now: it reads none of the tables, and ends after this kernel
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  let_next_start();   // the covariance reads none of the tables
   const PlanHeader *h = reinterpret_cast<const PlanHeader *>(plan);
   const PlanGeoGrid g = reinterpret_cast<const PlanGeoGrid *>(plan + h->off_geo_grid)[blockIdx.y];
   float2 *t32 = reinterpret_cast<float2 *>(ws + g.t32_off);
@@ -135,8 +134,7 @@ struct GeoSource {
 // at a time as (Re, Re, Im, Im) (the operand pairs of the paired contraction), the FP64 phasor of the
 // refinement rounded to FP32; rows m >= M and points i >= npts are zero.
 __global__ void geo_steer_kernel(const uint8_t *plan, uint8_t *ws) {
-  // the covariance may start now: it reads none of the tables, and ends after this kernel
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  let_next_start();   // the covariance reads none of the tables
   const PlanHeader *h = reinterpret_cast<const PlanHeader *>(plan);
   const PlanGeoSteer st = reinterpret_cast<const PlanGeoSteer *>(plan + h->off_geo_steer)[blockIdx.y];
   const PlanGeoGrid g = reinterpret_cast<const PlanGeoGrid *>(plan + h->off_geo_grid)[st.geo_grid];
