@@ -226,6 +226,7 @@ __device__ __forceinline__ void store_r(int M, int row, int col, double2 v, doub
 
 __global__ void __launch_bounds__(kCovThreads) covariance_cluster_kernel(const float2 *X, int M, int N, int ldx,
                                                                          int per_cta, float2 *R, double2 *R64) {
+  let_next_start();
   extern __shared__ __align__(16) uint8_t smem[];
   cg::cluster_group cluster = cg::this_cluster();
   const int rank = (int)cluster.block_rank();
@@ -573,6 +574,8 @@ __global__ void covariance_reduce_batch(const uint8_t *plan, uint8_t *ws) {
 constexpr int kFixupSlots = 160;   // output slots of M <= 16 (10 blocks of 4 x 4)
 
 __global__ void __launch_bounds__(kCovThreads) covariance_fixup_kernel(const uint8_t *plan, uint8_t *ws) {
+  start_after_previous();
+  let_next_start();
   extern __shared__ __align__(16) uint8_t smem[];
   __shared__ double2 acc[kFixupSlots];
   const PlanHeader *h = reinterpret_cast<const PlanHeader *>(plan);
@@ -614,8 +617,7 @@ cudaError_t launch_covariance_fixup(const uint8_t *plan_dev, const PlanHeader &h
   cudaError_t e = ensure_smem_attr(reinterpret_cast<const void *>(covariance_fixup_kernel), kSmemBytes);
   if (e != cudaSuccess) return e;
   const int grid = total < 2 * device_sm_count() ? total : 2 * device_sm_count();
-  covariance_fixup_kernel<<<grid, kCovThreads, kSmemBytes, s>>>(plan_dev, ws);
-  return cudaGetLastError();
+  return launch_chained(covariance_fixup_kernel, grid, kCovThreads, kSmemBytes, s, plan_dev, ws);
 }
 
 cudaError_t launch_covariance_single(const float2 *X, int M, int N, int ldx, float2 *R, double2 *R64,
@@ -652,7 +654,7 @@ cudaError_t launch_tasks_kind(const uint8_t *plan_dev, int first, int n, uint8_t
   using K = CovKind<MB, kKind>;
   cudaError_t e = ensure_smem_attr(reinterpret_cast<const void *>(covariance_tasks_kernel<MB, kKind>), K::kSmem);
   if (e != cudaSuccess) return e;
-  return launch_beside(true, covariance_tasks_kernel<MB, kKind>, n, K::kThreads, K::kSmem, s, plan_dev, ws, first);
+  return launch_beside(covariance_tasks_kernel<MB, kKind>, n, K::kThreads, K::kSmem, s, plan_dev, ws, first);
 }
 
 template <int MB>
@@ -668,15 +670,16 @@ cudaError_t launch_covariance_batch(const uint8_t *plan_dev, const PlanHeader &h
                                     cudaStream_t s) {
   cudaError_t e = ensure_smem_attr(reinterpret_cast<const void *>(covariance_batch_kernel), kSmemBytes);
   if (e != cudaSuccess) return e;
-  // the classes beside each other, and the first beside the phase tables (which always precede it)
+  // the classes beside each other, and the first beside the phase tables (which always precede it);
+  // the longest class first
+  const int ngen = h.cov_first[kCovClasses] - h.cov_first[kCovClasses - 1];
+  if (ngen > 0)
+    if ((e = launch_beside(covariance_batch_kernel, ngen, kCovThreads, kSmemBytes, s, plan_dev, ws,
+                           h.cov_first[kCovClasses - 1])) != cudaSuccess)
+      return e;
   if ((e = launch_tasks<2>(plan_dev, h, ws, s)) != cudaSuccess) return e;
   if ((e = launch_tasks<3>(plan_dev, h, ws, s)) != cudaSuccess) return e;
   if ((e = launch_tasks<4>(plan_dev, h, ws, s)) != cudaSuccess) return e;
-  const int ngen = h.cov_first[kCovClasses] - h.cov_first[kCovClasses - 1];
-  if (ngen > 0)
-    if ((e = launch_beside(true, covariance_batch_kernel, ngen, kCovThreads, kSmemBytes, s, plan_dev, ws,
-                           h.cov_first[kCovClasses - 1])) != cudaSuccess)
-      return e;
   // problems with M <= 16: tensor cores, then the recomputation of any it marked
   if ((e = launch_covariance_tc_batch(plan_dev, h, ws, s)) != cudaSuccess) return e;
   if (h.nreduce > 0) covariance_reduce_batch<<<h.nreduce, 256, 0, s>>>(plan_dev, ws);

@@ -657,7 +657,7 @@ cudaError_t launch_class(const uint8_t *plan_dev, const PlanHeader &h, uint8_t *
   cudaError_t e = ensure_smem_attr(reinterpret_cast<const void *>(covariance_tc_batch_kernel<MP>), CbLayout<MP>::kSmem);
   if (e != cudaSuccess) return e;
   const int grid = n < device_sm_count() ? n : device_sm_count();   // one CTA per SM (512 TMEM columns)
-  return launch_beside(true, covariance_tc_batch_kernel<MP>, grid, kCbThreads, CbLayout<MP>::kSmem, s, plan_dev, ws, cls);
+  return launch_beside(covariance_tc_batch_kernel<MP>, grid, kCbThreads, CbLayout<MP>::kSmem, s, plan_dev, ws, cls);
 }
 
 }  // namespace

@@ -807,6 +807,8 @@ using Arith = std::conditional_t<kDF, ArithDF<NP>, ArithF64<NP>>;
 template <int NP, bool kDF>
 __global__ void __launch_bounds__(cta_threads<NP>()) eig_single_kernel(const double2 *R64, int M, int d, int alg, double *evals,
                                                        double2 *B, int *K_out, int *info) {
+  start_after_previous();
+  let_next_start();
   extern __shared__ __align__(16) uint8_t smem[];
   constexpr int T = cta_threads<NP>();
   EigSmem<NP> *mats = reinterpret_cast<EigSmem<NP> *>(smem);
@@ -822,6 +824,8 @@ __global__ void __launch_bounds__(cta_threads<NP>()) eig_single_kernel(const dou
 __global__ void __cluster_dims__(kClRanks, 1, 1) __launch_bounds__(kClThreads, 1)
     eig_cluster_single_kernel(const double2 *R64, int M, int d, int alg, double *evals, double2 *B, int *K_out,
                               int *info) {
+  start_after_previous();
+  let_next_start();
   extern __shared__ __align__(16) uint8_t smem[];
   EigSmem<64> &s = *reinterpret_cast<EigSmem<64> *>(smem);
   ClusterDF &w = *reinterpret_cast<ClusterDF *>(smem + kClFinBytes);
@@ -880,7 +884,8 @@ __device__ __forceinline__ bool refines_2d(const doa_problem &p) { return p.geom
 
 template <int NP, int G>
 __global__ void __launch_bounds__(32 * eig_warps<NP>(), eig_min_ctas<NP>()) eig_batch_kernel(const uint8_t *plan, uint8_t *ws, int bucket,
-                                                                         int *status) {
+                                                                         int *status, int dep) {
+  if (dep) start_after_previous();
   let_next_start();
   extern __shared__ __align__(16) uint8_t smem[];
   const int grp = threadIdx.x / 32;
@@ -917,7 +922,8 @@ __global__ void __launch_bounds__(32 * eig_warps<NP>(), eig_min_ctas<NP>()) eig_
 // The CTA form of the batch: a CTA per matrix.
 template <int NP>
 __global__ void __launch_bounds__(cta_threads<NP>()) eig_batch_cta_kernel(const uint8_t *plan, uint8_t *ws, int bucket,
-                                                                          int *status) {
+                                                                          int *status, int dep) {
+  if (dep) start_after_previous();
   let_next_start();
   extern __shared__ __align__(16) uint8_t smem[];
   constexpr int T = cta_threads<NP>();
@@ -941,7 +947,8 @@ __global__ void __launch_bounds__(cta_threads<NP>()) eig_batch_cta_kernel(const 
 // Bucket M <= 64 of the batch in double-float: one four-CTA cluster per problem; rank 0 finishes.
 // A problem that asks for the FP64 Jacobi runs it in rank 0 alone (the other CTAs leave at once).
 __global__ void __cluster_dims__(kClRanks, 1, 1) __launch_bounds__(kClThreads, 1)
-    eig_cluster_batch_kernel(const uint8_t *plan, uint8_t *ws, int bucket, int *status) {
+    eig_cluster_batch_kernel(const uint8_t *plan, uint8_t *ws, int bucket, int *status, int dep) {
+  if (dep) start_after_previous();
   let_next_start();
   extern __shared__ __align__(16) uint8_t smem[];
   EigSmem<64> &s = *reinterpret_cast<EigSmem<64> *>(smem);
@@ -979,16 +986,15 @@ cudaError_t run_single_p(const double2 *R64, int M, int d, int alg, double *eval
   const int smem = (int)sizeof(EigSmem<NP>);
   cudaError_t e = ensure_smem_attr((const void *)eig_single_kernel<NP, kDF>, smem);
   if (e != cudaSuccess) return e;
-  eig_single_kernel<NP, kDF><<<1, cta_threads<NP>(), smem, st>>>(R64, M, d, alg, evals, B, K_out, info);
-  return cudaGetLastError();
+  return launch_chained(eig_single_kernel<NP, kDF>, 1, cta_threads<NP>(), smem, st, R64, M, d, alg, evals, B, K_out, info);
 }
 
 cudaError_t run_single_cluster(const double2 *R64, int M, int d, int alg, double *evals, double2 *B, int *K_out,
                                int *info, cudaStream_t st) {
   cudaError_t e = ensure_smem_attr(reinterpret_cast<const void *>(eig_cluster_single_kernel), kClSmemBytes);
   if (e != cudaSuccess) return e;
-  eig_cluster_single_kernel<<<kClRanks, kClThreads, kClSmemBytes, st>>>(R64, M, d, alg, evals, B, K_out, info);
-  return cudaGetLastError();
+  return launch_chained(eig_cluster_single_kernel, kClRanks, kClThreads, kClSmemBytes, st, R64, M, d, alg, evals, B, K_out,
+                          info);
 }
 
 template <int NP>
@@ -1029,8 +1035,9 @@ cudaError_t run_batch_g(const uint8_t *plan, int count, uint8_t *ws, int *status
   const int smem = (int)sizeof(EigSmem<NP>) * per_cta;
   cudaError_t e = ensure_smem_attr(reinterpret_cast<const void *>(eig_batch_kernel<NP, G>), smem);
   if (e != cudaSuccess) return e;
-  return launch_beside(beside, eig_batch_kernel<NP, G>, (count + per_cta - 1) / per_cta, 32 * W, smem, st, plan, ws, bucket,
-                       status);
+  return launch_programmatic(beside || chained_grid((count + per_cta - 1) / per_cta), eig_batch_kernel<NP, G>,
+                             (count + per_cta - 1) / per_cta, 32 * W, smem, st, plan, ws, bucket, status,
+                          (int)!beside);
 }
 
 template <int NP>
@@ -1039,7 +1046,7 @@ cudaError_t run_batch_cta(const uint8_t *plan, int count, uint8_t *ws, int *stat
   const int smem = (int)sizeof(EigSmem<NP>);
   cudaError_t e = ensure_smem_attr(reinterpret_cast<const void *>(eig_batch_cta_kernel<NP>), smem);
   if (e != cudaSuccess) return e;
-  return launch_beside(beside, eig_batch_cta_kernel<NP>, count, cta_threads<NP>(), smem, st, plan, ws, bucket, status);
+  return launch_programmatic(beside || chained_grid(count), eig_batch_cta_kernel<NP>, count, cta_threads<NP>(), smem, st, plan, ws, bucket, status, (int)!beside);
 }
 
 // M <= 16: the CTA form for small batches unless the plan packs matrices (G in {1, 2, 4, 8} up to the
@@ -1064,8 +1071,8 @@ cudaError_t run_batch_cluster(const uint8_t *plan, const PlanHeader &h, uint8_t 
   if (count == 0) return cudaSuccess;
   cudaError_t e = ensure_smem_attr(reinterpret_cast<const void *>(eig_cluster_batch_kernel), kClSmemBytes);
   if (e != cudaSuccess) return e;
-  return launch_beside(beside, eig_cluster_batch_kernel, (int64_t)count * kClRanks, kClThreads, kClSmemBytes, st, plan, ws,
-                       bucket, status);
+  return launch_programmatic(beside || chained_grid((int64_t)count * kClRanks), eig_cluster_batch_kernel, (int64_t)count * kClRanks, kClThreads, kClSmemBytes, st, plan, ws, bucket,
+                          status, (int)!beside);
 }
 
 }  // namespace

@@ -132,12 +132,16 @@ __device__ void peaks2d_block(const float *__restrict__ P, int La, int Le, bool 
 template <int kCs>
 __global__ void __launch_bounds__(kPeakThreads) peaks2d_single_kernel(const float *P, int La, int Le, int wrap, int d,
                                                                       int *idx, float *val, int *count) {
+  start_after_previous();
+  let_next_start();
   peaks2d_block<kCs>(P, La, Le, wrap != 0, d, idx, val, count);
 }
 
 template <int kCs>
 __global__ void __launch_bounds__(kPeakThreads) peaks_single_kernel(const float *P, int L, int d, int *idx, float *val,
                                                                     int *count) {
+  start_after_previous();
+  let_next_start();
   peaks_block<kCs, kPeakThreads>(P, L, d, idx, val, count);
 }
 
@@ -156,6 +160,8 @@ constexpr int kSmallThreads = 64, kSmallPoints = 65536;
 // repick: the pick after the peak polish, only for the jobs the polish marked (NaN next value).
 template <int kCs, int T>
 __global__ void __launch_bounds__(T, kBatchThreads / T) peaks_batch_kernel(const uint8_t *plan, uint8_t *ws, int repick) {
+  start_after_previous();
+  let_next_start();
   const int job = blockIdx.x / kCs;
   const PlanHeader *h = reinterpret_cast<const PlanHeader *>(plan);
   const PlanJob &jb = reinterpret_cast<const PlanJob *>(plan + h->off_job)[job];
@@ -174,6 +180,8 @@ __global__ void __launch_bounds__(T, kBatchThreads / T) peaks_batch_kernel(const
 
 template <int kCs>
 __global__ void __launch_bounds__(kPeakThreads, 4) peaks2d_batch_kernel(const uint8_t *plan) {
+  start_after_previous();
+  let_next_start();
   const PlanHeader *h = reinterpret_cast<const PlanHeader *>(plan);
   const PlanJob &jb = reinterpret_cast<const PlanJob *>(plan + h->off_job)[blockIdx.x / kCs];
   const PlanProblem &pp = reinterpret_cast<const PlanProblem *>(plan + h->off_prob)[jb.prob];
@@ -287,12 +295,15 @@ cudaError_t launch_jobs(void (*kernel)(Args...), int jobs, cudaStream_t s, Args.
   cfg.gridDim = dim3((unsigned)jobs * kCs);
   cfg.blockDim = dim3(T);
   cfg.stream = s;
-  cudaLaunchAttribute attr{};
-  attr.id = cudaLaunchAttributeClusterDimension;
-  attr.val.clusterDim.x = kCs;
-  attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
-  cfg.attrs = &attr;
-  cfg.numAttrs = kCs > 1 ? 1 : 0;
+  cudaLaunchAttribute attr[2] = {};
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = kCs;
+  attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
+  const bool chained = chained_grid((int64_t)jobs * kCs);
+  cfg.attrs = chained ? attr : attr + 1;
+  cfg.numAttrs = (chained ? 1 : 0) + (kCs > 1 ? 1 : 0);
   return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 

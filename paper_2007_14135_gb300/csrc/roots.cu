@@ -350,8 +350,10 @@ __global__ void __launch_bounds__(32) roots_single_kernel(RootJob j, double *the
 
 cudaError_t launch_roots_batch(const uint8_t *plan_dev, const PlanHeader &h, uint8_t *ws, int *status, cudaStream_t s) {
   if (h.nroots == 0 || h.njobs == 0) return cudaSuccess;
-  return launch_beside(h.nrefine > 0, roots_batch_kernel, (h.njobs + kRootWarps - 1) / kRootWarps, 32 * kRootWarps, 0, s,
-                       plan_dev, ws, status);
+  const int grid = (h.njobs + kRootWarps - 1) / kRootWarps, block = 32 * kRootWarps;
+  if (h.nrefine > 0) return launch_beside(roots_batch_kernel, grid, block, 0, s, plan_dev, ws, status);
+  roots_batch_kernel<<<grid, block, 0, s>>>(plan_dev, ws, status);
+  return cudaGetLastError();
 }
 
 cudaError_t launch_roots_single(const double2 *B, int M, int K, int d, double *theta, int *info, cudaStream_t s) {

@@ -38,6 +38,8 @@ namespace {
 using namespace scanc;
 
 __global__ void grid_table_single_kernel(double lo, double step, int k0, int n, uint32_t *S) {
+  start_after_previous();   // an earlier scan may still read the table
+  let_next_start();
   int k = blockIdx.x * blockDim.x + threadIdx.x;
   if (k < n) S[k] = grid_phase_step(lo, step, k0 + k);
 }
@@ -60,6 +62,8 @@ template <int MP, int PT>
 __global__ void __launch_bounds__(kScanThreads) scan_single_kernel(const double2 *B, int M, int K, int L, double lo,
                                                                    double step, int kofs, const uint32_t *S,
                                                                    float *P) {
+  start_after_previous();
+  let_next_start();
   __shared__ __align__(16) float2 Bs[MP * MP];
   __shared__ ScanShared sh;
   ScanJob j{};
@@ -111,7 +115,8 @@ constexpr int kRun = 16;   // longest run (large batches); small ones use shorte
 
 template <int MP, int PT>
 __global__ void __launch_bounds__(kScanThreads) scan_batch_kernel(const uint8_t *plan, uint8_t *ws, int bucket,
-                                                                  int run_len) {
+                                                                  int run_len, int dep) {
+  if (dep) start_after_previous();
   let_next_start();
   // factor: (bx, bx, by, by) per element for the paired contraction (PT even), else (bx, by)
   constexpr bool kPair = PT % 2 == 0;
@@ -184,7 +189,8 @@ __global__ void __launch_bounds__(kScanThreads) scan_batch_kernel(const uint8_t 
 // FP32 copy of each grouped problem's factor (one warp per problem): F32 as (bx, bx, by, by) per
 // element, w32, thresholds.
 template <int MP>
-__global__ void __launch_bounds__(kScanThreads) scan_prep_kernel(const uint8_t *plan, uint8_t *ws, int bucket) {
+__global__ void __launch_bounds__(kScanThreads) scan_prep_kernel(const uint8_t *plan, uint8_t *ws, int bucket, int dep) {
+  if (dep) start_after_previous();
   let_next_start();
   const PlanHeader *h = reinterpret_cast<const PlanHeader *>(plan);
   const int32_t *list = reinterpret_cast<const int32_t *>(plan + h->off_sgl[bucket]);
@@ -224,7 +230,8 @@ __host__ __device__ constexpr int shared_min_blocks() {
 
 template <int MP, int PT>
 __global__ void __launch_bounds__(kScanThreads, shared_min_blocks<MP, PT>())
-    scan_shared_kernel(const uint8_t *plan, uint8_t *ws, int bucket) {
+    scan_shared_kernel(const uint8_t *plan, uint8_t *ws, int bucket, int dep) {
+  if (dep) start_after_previous();
   let_next_start();
   constexpr bool kPair = PT % 2 == 0;
   // paired form: two factor buffers; the next problem's factor, EV weights and thresholds are
@@ -486,7 +493,7 @@ cudaError_t run_batch(const uint8_t *plan, const PlanHeader &h, uint8_t *ws, int
   const int64_t cap = (int64_t)device_sm_count() * per_sm;
   const int run_len = (int)std::min<int64_t>(kRun, std::max<int64_t>(1, (tiles + cap - 1) / cap));
   const int64_t grid = std::min<int64_t>(cap, (tiles + run_len - 1) / run_len);
-  const cudaError_t e = launch_beside(beside, scan_batch_kernel<MP, PT>, grid, kScanThreads, 0, s, plan, ws, bucket, run_len);
+  const cudaError_t e = launch_programmatic(beside || chained_grid(grid), scan_batch_kernel<MP, PT>, grid, kScanThreads, 0, s, plan, ws, bucket, run_len, (int)!beside);
   beside = true;
   return e;
 }
@@ -494,8 +501,7 @@ cudaError_t run_batch(const uint8_t *plan, const PlanHeader &h, uint8_t *ws, int
 }  // namespace
 
 cudaError_t launch_grid_table_single(double lo, double step, int k0, int n, uint32_t *S, cudaStream_t s) {
-  grid_table_single_kernel<<<(n + 255) / 256, 256, 0, s>>>(lo, step, k0, n, S);
-  return cudaGetLastError();
+  return launch_chained(grid_table_single_kernel, (n + 255) / 256, 256, 0, s, lo, step, k0, n, S);
 }
 
 cudaError_t launch_grid_tables(const uint8_t *plan_dev, const PlanHeader &h, uint8_t *ws, cudaStream_t s) {
@@ -514,15 +520,14 @@ cudaError_t launch_scan_single(const double2 *B, int M, int K, int L, double lo,
   const int pt = scan_pt_for(b, L), tp = kScanThreads * pt;
   const unsigned grid = (unsigned)((L + tp - 1) / tp);
 #define DOA_SCAN_SINGLE(MP, PT) \
-  scan_single_kernel<MP, PT><<<grid, kScanThreads, 0, s>>>(B, M, K, L, lo, step, kofs, S, P)
+  launch_chained(scan_single_kernel<MP, PT>, grid, kScanThreads, 0, s, B, M, K, L, lo, step, kofs, S, P)
   switch (b) {
-    case 0: if (pt == 4) DOA_SCAN_SINGLE(8, 4); else DOA_SCAN_SINGLE(8, 1); break;
-    case 1: if (pt == 4) DOA_SCAN_SINGLE(16, 4); else DOA_SCAN_SINGLE(16, 1); break;
-    case 2: DOA_SCAN_SINGLE(32, 1); break;
-    default: DOA_SCAN_SINGLE(64, 1); break;
+    case 0: return pt == 4 ? DOA_SCAN_SINGLE(8, 4) : DOA_SCAN_SINGLE(8, 1);
+    case 1: return pt == 4 ? DOA_SCAN_SINGLE(16, 4) : DOA_SCAN_SINGLE(16, 1);
+    case 2: return DOA_SCAN_SINGLE(32, 1);
+    default: return DOA_SCAN_SINGLE(64, 1);
   }
 #undef DOA_SCAN_SINGLE
-  return cudaGetLastError();
 }
 
 cudaError_t launch_polish_batch(const uint8_t *plan_dev, const PlanHeader &h, uint8_t *ws, cudaStream_t s) {
@@ -534,8 +539,9 @@ cudaError_t launch_polish_batch(const uint8_t *plan_dev, const PlanHeader &h, ui
 template <int MP>
 cudaError_t run_prep(const uint8_t *plan, const PlanHeader &h, uint8_t *ws, int bucket, bool &beside, cudaStream_t s) {
   if (h.sg_units[bucket] == 0) return cudaSuccess;
-  const cudaError_t e = launch_beside(beside, scan_prep_kernel<MP>, (h.sg_probs[bucket] + kScanWarps - 1) / kScanWarps,
-                                      kScanThreads, 0, s, plan, ws, bucket);
+  const int64_t grid = (h.sg_probs[bucket] + kScanWarps - 1) / kScanWarps;
+  const cudaError_t e = launch_programmatic(beside || chained_grid(grid), scan_prep_kernel<MP>, grid,
+                                            kScanThreads, 0, s, plan, ws, bucket, (int)!beside);
   beside = true;
   return e;
 }
@@ -547,7 +553,8 @@ cudaError_t run_shared(const uint8_t *plan, const PlanHeader &h, uint8_t *ws, in
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, scan_shared_kernel<MP, PT>, kScanThreads, 0);
   if (per_sm < 1) per_sm = 1;
   const int64_t grid = std::min<int64_t>((int64_t)device_sm_count() * per_sm, h.sg_units[bucket]);
-  const cudaError_t e = launch_beside(beside, scan_shared_kernel<MP, PT>, grid, kScanThreads, 0, s, plan, ws, bucket);
+  const cudaError_t e = launch_programmatic(beside || chained_grid(grid), scan_shared_kernel<MP, PT>, grid,
+                                            kScanThreads, 0, s, plan, ws, bucket, (int)!beside);
   beside = true;
   return e;
 }

@@ -315,6 +315,8 @@ constexpr int kRun = 16;   // longest run (large batches); small ones use shorte
 template <int MP, int PT>
 __global__ void __launch_bounds__(kScanThreads) scan_geometry_batch_kernel(const uint8_t *plan, uint8_t *ws,
                                                                            int bucket, int run_len) {
+  start_after_previous();
+  let_next_start();
   __shared__ __align__(16) float2 Bs[(MP + 1) * MP];
   __shared__ ScanShared sh;
   __shared__ GeoShared gs;
@@ -539,8 +541,7 @@ cudaError_t run_geo_batch(const uint8_t *plan, const PlanHeader &h, uint8_t *ws,
   const int64_t cap = (int64_t)device_sm_count() * per_sm;
   const int run_len = (int)std::min<int64_t>(kRun, std::max<int64_t>(1, (tiles + cap - 1) / cap));
   const int64_t grid = std::min<int64_t>(cap, (tiles + run_len - 1) / run_len);
-  scan_geometry_batch_kernel<MP, PT><<<(unsigned)grid, kScanThreads, 0, s>>>(plan, ws, bucket, run_len);
-  return cudaGetLastError();
+  return launch_chained(scan_geometry_batch_kernel<MP, PT>, grid, kScanThreads, 0, s, plan, ws, bucket, run_len);
 }
 
 }  // namespace
