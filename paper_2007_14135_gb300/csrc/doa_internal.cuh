@@ -458,10 +458,10 @@ __device__ __forceinline__ void start_after_previous() { asm volatile("griddepco
 // Only small grids: the blocks of a large one come onto the SMs while the kernel before still sets their split of
 // L1 and shared memory, which cost the peak picker of 4096 problems 0.08 ms.
 template <class... P, class... A>
-cudaError_t launch_programmatic(bool on, void (*kernel)(P...), int64_t grid, int block, size_t smem, cudaStream_t s,
+cudaError_t launch_programmatic(bool on, void (*kernel)(P...), dim3 grid, int block, size_t smem, cudaStream_t s,
                                 A... args) {
   cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3((unsigned)grid);
+  cfg.gridDim = grid;
   cfg.blockDim = dim3((unsigned)block);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
@@ -474,14 +474,14 @@ cudaError_t launch_programmatic(bool on, void (*kernel)(P...), int64_t grid, int
 }
 // Launches a kernel beside the one before it in the stream, which it does not depend on.
 template <class... P, class... A>
-cudaError_t launch_beside(void (*kernel)(P...), int64_t grid, int block, size_t smem, cudaStream_t s, A... args) {
+cudaError_t launch_beside(void (*kernel)(P...), dim3 grid, int block, size_t smem, cudaStream_t s, A... args) {
   return launch_programmatic(true, kernel, grid, block, smem, s, args...);
 }
 // Launches a kernel that begins with start_after_previous.
 inline bool chained_grid(int64_t grid) { return grid <= 2 * device_sm_count(); }
 template <class... P, class... A>
-cudaError_t launch_chained(void (*kernel)(P...), int64_t grid, int block, size_t smem, cudaStream_t s, A... args) {
-  return launch_programmatic(chained_grid(grid), kernel, grid, block, smem, s, args...);
+cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, int block, size_t smem, cudaStream_t s, A... args) {
+  return launch_programmatic(chained_grid((int64_t)grid.x * grid.y * grid.z), kernel, grid, block, smem, s, args...);
 }
 #endif
 // The first bytes of a batch workspace hold per-solve counters (uint32, zeroed at the start of

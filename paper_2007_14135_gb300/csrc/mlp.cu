@@ -59,6 +59,8 @@ struct NetPtrs {
 
 // Adam on the FP32 masters, then the BF16 copies (row-major and transposed); grid.y = layer.
 __global__ void adam_kernel(const __grid_constant__ NetPtrs net, float lr, float b1, float b2, float eps, float c1, float c2, int update) {
+  start_after_previous();
+  let_next_start();
   const LayerPtrs &p = net.l[blockIdx.y];
   const int nW = p.out * p.in;
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < nW + p.out; i += gridDim.x * blockDim.x) {
@@ -112,8 +114,7 @@ cudaError_t adam(const doa_mlp *net, float lr, float b1, float b2, float eps, fl
                  cudaStream_t s) {
   NetPtrs n;
   for (int l = 0; l < 4; ++l) n.l[l] = layer(net, l);
-  adam_kernel<<<dim3(256, 4), 256, 0, s>>>(n, lr, b1, b2, eps, c1, c2, update);
-  return cudaGetLastError();
+  return launch_programmatic(true, adam_kernel, dim3(256, 4), 256, 0, s, n, lr, b1, b2, eps, c1, c2, update);
 }
 
 bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; }

@@ -148,6 +148,8 @@ __device__ __forceinline__ RowPass row_pass(int p) {
 template <bool kTrain>
 __global__ void __launch_bounds__(kRowsThreads, 1) mlp_rows_kernel(const __grid_constant__ MlpMaps maps,
                                                                    const __grid_constant__ MlpRowArgs g) {
+  start_after_previous();
+  let_next_start();
   constexpr int kPasses = kTrain ? 7 : 4;
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   uint8_t *sm = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -493,6 +495,8 @@ static_assert(kMlpDwTiles == 10 + 3 * 8, "tiles of the four layers");
 
 __global__ void __launch_bounds__(kDwThreads) mlp_dw_kernel(const __grid_constant__ MlpDwMaps maps, int B, int splits,
                                                                float *part, int *err) {
+  start_after_previous();
+  let_next_start();
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   uint8_t *sm = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   __shared__ __align__(8) uint64_t full_bar[kDwStages], empty_bar[kDwStages], done_bar;
@@ -580,6 +584,8 @@ __global__ void __launch_bounds__(kDwThreads) mlp_dw_kernel(const __grid_constan
 // fastest as in the partial layout); then the bias gradients (32 columns a block) and the loss.
 __global__ void __launch_bounds__(256) mlp_reduce_kernel(const float *part, int splits, int tiles, const float *gb_part,
                                                          const float *loss_part, MlpGrads o) {
+  start_after_previous();
+  let_next_start();
   constexpr int kGwBlocks = kMlpDwTiles * 8;
   const int tid = threadIdx.x;
   if (blockIdx.x < kGwBlocks) {
@@ -686,11 +692,8 @@ cudaError_t launch_mlp_rows(const doa_mlp *net, const MlpRowArgs &g, bool train,
   const void *k = train ? (const void *)mlp_rows_kernel<true> : (const void *)mlp_rows_kernel<false>;
   if ((e = ensure_smem_attr(k, kRowsSmem)) != cudaSuccess) return e;
   const int tiles = (g.B + kTcRows - 1) / kTcRows, ctas = std::min(tiles, device_sm_count());
-  if (train)
-    mlp_rows_kernel<true><<<ctas, kRowsThreads, kRowsSmem, s>>>(maps, g);
-  else
-    mlp_rows_kernel<false><<<ctas, kRowsThreads, kRowsSmem, s>>>(maps, g);
-  return cudaGetLastError();
+  return train ? launch_chained(mlp_rows_kernel<true>, ctas, kRowsThreads, kRowsSmem, s, maps, g)
+               : launch_chained(mlp_rows_kernel<false>, ctas, kRowsThreads, kRowsSmem, s, maps, g);
 }
 
 cudaError_t launch_mlp_dw(const MlpRowArgs &g, float *part, const MlpGrads &o, cudaStream_t s) {
@@ -703,9 +706,12 @@ cudaError_t launch_mlp_dw(const MlpRowArgs &g, float *part, const MlpGrads &o, c
   }
   if ((e = ensure_smem_attr((const void *)mlp_dw_kernel, kDwSmem)) != cudaSuccess) return e;
   const int splits = mlp_dw_splits(g.B), tiles = (g.B + kTcRows - 1) / kTcRows;
-  mlp_dw_kernel<<<dim3(kMlpDwTiles, splits), kDwThreads, kDwSmem, s>>>(maps, g.B, splits, part, g.err);
-  mlp_reduce_kernel<<<kMlpDwTiles * 8 + kMlpGbCols / 32 + 1, 256, 0, s>>>(part, splits, tiles, g.gb_part, g.loss_part, o);
-  return cudaGetLastError();
+  // the step's kernels and Adam queue behind each other: a step of 4096 rows 75.5 -> 70.5 us
+  if ((e = launch_chained(mlp_dw_kernel, dim3(kMlpDwTiles, splits), kDwThreads, kDwSmem, s, maps, g.B, splits, part, g.err)) !=
+      cudaSuccess)
+    return e;
+  return launch_programmatic(true, mlp_reduce_kernel, kMlpDwTiles * 8 + kMlpGbCols / 32 + 1, 256, 0, s, part, splits, tiles,
+                             g.gb_part, g.loss_part, o);
 }
 
 }  // namespace doa
