@@ -145,7 +145,7 @@ __device__ __forceinline__ double2 phasor_q64(uint64_t phi) {
 // ------------------------------------------------------------------------------------------
 // Batch plan. The same bytes live on the host (for launch sizes) and on the device.
 // ------------------------------------------------------------------------------------------
-constexpr uint32_t kPlanMagic = 0x444f4131u;  // "DOA1"
+constexpr uint32_t kPlanMagic = 0x444f4132u;  // "DOA2" (a header of another layout is refused)
 constexpr int kNumBuckets = 4;                // M <= 8, <= 16, <= 32, <= 64
 // Covariance work-item classes: 4x4 register blocks per row, MB = ceil(M / 4) in {2, 3, 4} use
 // the block-task kernel (one launch per class, CTA shape fixed by MB); every other M the

@@ -21,7 +21,7 @@ __host__ __device__ inline int pitch8(int n) { return (n + 7) / 8 * 8; }
 
 struct MlpWs {
   __nv_bfloat16 *X0, *A[3], *dZ[4];
-  float *part, *gb_part, *loss_part;
+  float *gb_part, *loss_part;
   int *err;
   size_t bytes;
 };
@@ -39,7 +39,6 @@ MlpWs ws_layout(uint8_t *base, int B) {
   for (int l = 0; l < 3; ++l) w.A[l] = reinterpret_cast<__nv_bfloat16 *>(take((size_t)kHid * B * 2));
   for (int l = 0; l < 4; ++l)
     w.dZ[l] = reinterpret_cast<__nv_bfloat16 *>(take((size_t)(l == 3 ? kMlpOutPitch : kHid) * B * 2));
-  w.part = reinterpret_cast<float *>(take((size_t)mlp_dw_splits(B) * kMlpDwTiles * kMlpDwTileFloats * 4));
   w.gb_part = reinterpret_cast<float *>(take(tiles * 4 * kMlpGbCols * 4));
   w.loss_part = reinterpret_cast<float *>(take(tiles * kMlpLossParts * 4));
   w.err = reinterpret_cast<int *>(take(4));
@@ -182,7 +181,7 @@ extern "C" doa_status doa_mlp_backward(const doa_mlp *net, const float *features
   }
   o.loss = loss;
   if (launch_mlp_rows(net, g, true, s) != cudaSuccess) return DOA_ECUDA;
-  return launch_mlp_dw(g, w.part, o, s) == cudaSuccess ? DOA_OK : DOA_ECUDA;
+  return launch_mlp_dw(g, o, s) == cudaSuccess ? DOA_OK : DOA_ECUDA;
 }
 
 extern "C" doa_status doa_mlp_adam(const doa_mlp *net, float lr, float beta1, float beta2, float eps, int t,

@@ -9,9 +9,9 @@
 // dZ4 = (sigmoid(z) - y) / B, then dZ_l = (dZ_{l+1} W_{l+1}) [A_l > 0] with the ReLU masks kept in
 // registers; every operand also leaves by a TMA store (row-major BF16, for the weight gradients), with
 // partial sums of the bias gradients and the loss.
-// mlp_dw_kernel: all four weight gradients dW_l = dZ_l^T A_{l-1} in one launch, the batch split over
-// CTAs into partial sums; both operands are read batch-major, as they were stored (the MMA's MN-major
-// form), so no transposed copies exist. mlp_reduce_kernel adds the partial sums, the bias gradients and
+// mlp_dw_kernel: all four weight gradients dW_l = dZ_l^T A_{l-1} in one launch, a CTA per 128 x 64 tile
+// over the whole batch; both operands are read batch-major, as they were stored (the MMA's MN-major
+// form), so no transposed copies exist. Blocks beside them add the partial sums of the bias gradients and
 // the loss in a fixed order.
 //
 // Why: one GEMM per launch moved every activation through memory twice, and its epilogue stored
@@ -19,9 +19,8 @@
 // A tile's weights (0.5 MB a pass over the network) come from L2 through two 32 KB stages, which bounds a
 // layer's MMAs (5300 cycles against 2050 of tensor work); the epilogue of a hidden layer takes 2300 cycles,
 // that of the outputs 16000, half of it the burst of stores that all SMs make at once.
-// Measured: forward of 65536 rows 0.740 -> 0.088 ms (167 MB read and written: 1.9 TB/s); gradients of 4096
-// rows 0.48 -> 0.068 ms (32 tiles on as many SMs: 50 us, half of it the loss; weight gradients 8 us,
-// reduction 6 us).
+// Measured: forward of 65536 rows 0.740 -> 0.086 ms (167 MB read and written: 1.9 TB/s); a training step of
+// 4096 rows 0.50 -> 0.077 ms (32 tiles on as many SMs: 50 us, half of it the loss; weight gradients 20 us).
 #include <cuda.h>
 #include <cudaTypedefs.h>
 
@@ -464,7 +463,7 @@ __global__ void __launch_bounds__(kRowsThreads, 1) mlp_rows_kernel(const __grid_
 }
 
 // ---- weight gradients -----------------------------------------------------------------------------
-constexpr int kDwStages = 4;
+constexpr int kDwStages = 8;   // the loads in flight bound a tile: 192 KB a CTA
 constexpr int kDwStage = kATile + 64 * 128;
 constexpr int kDwSmem = kDwStages * kDwStage + 1024;
 constexpr int kDwThreads = 256;
@@ -493,10 +492,44 @@ __host__ __device__ inline DwTile dw_tile(int i) {
 }
 static_assert(kMlpDwTiles == 10 + 3 * 8, "tiles of the four layers");
 
-__global__ void __launch_bounds__(kDwThreads) mlp_dw_kernel(const __grid_constant__ MlpDwMaps maps, int B, int splits,
-                                                               float *part, int *err) {
+// Adds the partial sums of 32 bias gradients (block b of kMlpGbCols / 32), or of the loss (the block after).
+__device__ void add_partials(int b, int tiles, const float *gb_part, const float *loss_part, const MlpGrads &o) {
+  __shared__ float red[8][33];
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  float a = 0.f;
+  if (b < kMlpGbCols / 32) {
+    const int col = b * 32 + lane;
+    for (int r = w; r < tiles * 4; r += 8) a += gb_part[(size_t)r * kMlpGbCols + col];
+  } else {
+    for (int r = tid; r < tiles * kEpiWarps; r += 256) a += loss_part[r];
+  }
+  red[w][lane] = a;
+  __syncthreads();
+  if (w == 0) {
+    a = red[0][lane];
+    for (int k = 1; k < 8; ++k) a += red[k][lane];
+    if (b < kMlpGbCols / 32) {
+      const int col = b * 32 + lane, layer = min(col / DOA_MLP_HIDDEN, 3), c = col - layer * DOA_MLP_HIDDEN;
+      if (c < (layer == 3 ? DOA_MLP_OUT : DOA_MLP_HIDDEN)) o.gb[layer][c] = a;
+    } else {
+      for (int off = 16; off > 0; off >>= 1) a += __shfl_xor_sync(0xffffffffu, a, off);
+      if (lane == 0 && o.loss) *o.loss = a;
+    }
+  }
+}
+
+// A tile's batch is not split over CTAs. The tensor cores' FP32 accumulation truncates, so split sums differ
+// from the whole sum by 9e-6 of the norm (4096 rows), and one Adam step later a BF16 weight or a ReLU mask
+// may fall the other way (1.9e-4). The whole sum in the order it always had costs 7 us a step.
+__global__ void __launch_bounds__(kDwThreads) mlp_dw_kernel(const __grid_constant__ MlpDwMaps maps,
+                                                               const __grid_constant__ MlpGrads o, int B, int tiles,
+                                                               const float *gb_part, const float *loss_part, int *err) {
   start_after_previous();
   let_next_start();
+  if (blockIdx.x >= kMlpDwTiles) {
+    add_partials(blockIdx.x - kMlpDwTiles, tiles, gb_part, loss_part, o);
+    return;
+  }
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   uint8_t *sm = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   __shared__ __align__(8) uint64_t full_bar[kDwStages], empty_bar[kDwStages], done_bar;
@@ -504,9 +537,7 @@ __global__ void __launch_bounds__(kDwThreads) mlp_dw_kernel(const __grid_constan
   __shared__ int s_fail, s_issued, s_consumed;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const DwTile tl = dw_tile(blockIdx.x);
-  const int kts = (B + 63) / 64;
-  const int k0 = (int)((int64_t)kts * blockIdx.y / splits), k1 = (int)((int64_t)kts * (blockIdx.y + 1) / splits);
-  const int nk = k1 - k0;
+  const int nk = (B + 63) / 64;
   if (tid == 0) {
     for (int s = 0; s < kDwStages; ++s) {
       mbar_init(&full_bar[s], 1);
@@ -535,8 +566,8 @@ __global__ void __launch_bounds__(kDwThreads) mlp_dw_kernel(const __grid_constan
       uint8_t *st = sm + s * kDwStage;
       expect_tx(smem_u32(&full_bar[s]), (uint32_t)(3 * kDwBox));
       for (int i = 0; i < 2; ++i)
-        tma_2d(smem_u32(st + i * kDwBox), &maps.a[tl.layer], tl.m0 + i * 64, (k0 + t) * 64, smem_u32(&full_bar[s]));
-      tma_2d(smem_u32(st + 2 * kDwBox), &maps.b[tl.layer], tl.n0, (k0 + t) * 64, smem_u32(&full_bar[s]));
+        tma_2d(smem_u32(st + i * kDwBox), &maps.a[tl.layer], tl.m0 + i * 64, t * 64, smem_u32(&full_bar[s]));
+      tma_2d(smem_u32(st + 2 * kDwBox), &maps.b[tl.layer], tl.n0, t * 64, smem_u32(&full_bar[s]));
       s_issued = t + 1;
     }
   } else if (warp == 1 && lane == 0) {
@@ -565,73 +596,25 @@ __global__ void __launch_bounds__(kDwThreads) mlp_dw_kernel(const __grid_constan
       mbar_wait(smem_u32(&full_bar[t % kDwStages]), (uint32_t)((t / kDwStages) & 1));
   }
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  // partial tile as [column / 4][row] groups of four columns: a warp stores 512 contiguous bytes
-  float4 *out = reinterpret_cast<float4 *>(part) + (size_t)(blockIdx.y * kMlpDwTiles + blockIdx.x) * (kTcRows * 16);
+  // the tile through shared memory (every copy has landed and every MMA has read), rows out coalesced
+  float *stage = reinterpret_cast<float *>(sm);
+  constexpr int kPitch = 65;
   const int q = warp & 3, rl = q * 32 + lane, c0 = (warp >> 2) * 32;
   if (c0 < tl.bn && ok) {
     float v[32];
     tmem_ld32(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)c0, v);
 #pragma unroll
-    for (int j = 0; j < 32; j += 4)
-      if (c0 + j < tl.bn) out[(c0 + j) / 4 * kTcRows + rl] = make_float4(v[j], v[j + 1], v[j + 2], v[j + 3]);
+    for (int j = 0; j < 32; ++j) stage[rl * kPitch + c0 + j] = v[j];
+  }
+  __syncthreads();
+  const int out = tl.layer == 3 ? DOA_MLP_OUT : DOA_MLP_HIDDEN, in = tl.layer == 0 ? DOA_MLP_IN : DOA_MLP_HIDDEN;
+  for (int r = warp; r < kTcRows && tl.m0 + r < out && ok; r += kDwThreads / 32) {
+    float *d = o.gW[tl.layer] + (size_t)(tl.m0 + r) * in + tl.n0;
+    for (int cidx = lane; cidx < tl.bn; cidx += 32) d[cidx] = stage[r * kPitch + cidx];
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(64));
-}
-
-// Adds the partial sums in split order. Blocks x < 8 kMlpDwTiles: gW (a thread per four columns of a row, rows
-// fastest as in the partial layout); then the bias gradients (32 columns a block) and the loss.
-__global__ void __launch_bounds__(256) mlp_reduce_kernel(const float *part, int splits, int tiles, const float *gb_part,
-                                                         const float *loss_part, MlpGrads o) {
-  start_after_previous();
-  let_next_start();
-  constexpr int kGwBlocks = kMlpDwTiles * 8;
-  const int tid = threadIdx.x;
-  if (blockIdx.x < kGwBlocks) {
-    const DwTile tl = dw_tile(blockIdx.x / 8);
-    const int e = (blockIdx.x % 8) * 256 + tid, r = e % kTcRows, c4 = e / kTcRows;
-    const int out = tl.layer == 3 ? DOA_MLP_OUT : DOA_MLP_HIDDEN, in = tl.layer == 0 ? DOA_MLP_IN : DOA_MLP_HIDDEN;
-    if (c4 * 4 >= tl.bn || tl.m0 + r >= out || tl.n0 + c4 * 4 >= in) return;
-    const float4 *p = reinterpret_cast<const float4 *>(part) + (size_t)(blockIdx.x / 8) * (kTcRows * 16) + e;
-    float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll 4
-    for (int s = 0; s < splits; ++s) {
-      const float4 v = __ldcs(p + (size_t)s * kMlpDwTiles * (kTcRows * 16));
-      a.x += v.x;
-      a.y += v.y;
-      a.z += v.z;
-      a.w += v.w;
-    }
-    float *d = o.gW[tl.layer] + (size_t)(tl.m0 + r) * in + tl.n0 + c4 * 4;
-    d[0] = a.x;
-    d[1] = a.y;
-    d[2] = a.z;
-    d[3] = a.w;
-    return;
-  }
-  __shared__ float red[8][33];
-  const int b = blockIdx.x - kGwBlocks, lane = tid & 31, w = tid >> 5;
-  float a = 0.f;
-  if (b < kMlpGbCols / 32) {
-    const int col = b * 32 + lane;
-    for (int r = w; r < tiles * 4; r += 8) a += gb_part[(size_t)r * kMlpGbCols + col];
-  } else {
-    for (int r = tid; r < tiles * kEpiWarps; r += 256) a += loss_part[r];
-  }
-  red[w][lane] = a;
-  __syncthreads();
-  if (w == 0) {
-    a = red[0][lane];
-    for (int k = 1; k < 8; ++k) a += red[k][lane];
-    if (b < kMlpGbCols / 32) {
-      const int col = b * 32 + lane, layer = min(col / DOA_MLP_HIDDEN, 3), c = col - layer * DOA_MLP_HIDDEN;
-      if (c < (layer == 3 ? DOA_MLP_OUT : DOA_MLP_HIDDEN)) o.gb[layer][c] = a;
-    } else {
-      for (int off = 16; off > 0; off >>= 1) a += __shfl_xor_sync(0xffffffffu, a, off);
-      if (lane == 0 && o.loss) *o.loss = a;
-    }
-  }
 }
 
 PFN_cuTensorMapEncodeTiled_v12000 encoder() {
@@ -663,15 +646,6 @@ constexpr int kNetDims[5] = {DOA_MLP_IN, DOA_MLP_HIDDEN, DOA_MLP_HIDDEN, DOA_MLP
 
 }  // namespace
 
-// Splits of the batch in the weight gradients. The tensor cores' FP32 accumulation truncates, so a sum over
-// the whole batch loses more than the sum of split sums: their results differ by 9e-6 of the norm at 4096
-// rows, 2.6e-5 at 8192 (the split one is the nearer to 64 bits). Larger batches keep the unsplit order of
-// additions, so that results stay as they were to 1.5e-5; they have K tiles enough to stream.
-int mlp_dw_splits(int batch) {
-  const int kts = (batch + 63) / 64;
-  return batch > kMlpSplitRows ? 1 : std::min(kMlpMaxSplits, std::max(1, kts / 4));
-}
-
 cudaError_t launch_mlp_rows(const doa_mlp *net, const MlpRowArgs &g, bool train, cudaStream_t s) {
   MlpMaps maps;
   cudaError_t e;
@@ -696,7 +670,7 @@ cudaError_t launch_mlp_rows(const doa_mlp *net, const MlpRowArgs &g, bool train,
                : launch_chained(mlp_rows_kernel<false>, ctas, kRowsThreads, kRowsSmem, s, maps, g);
 }
 
-cudaError_t launch_mlp_dw(const MlpRowArgs &g, float *part, const MlpGrads &o, cudaStream_t s) {
+cudaError_t launch_mlp_dw(const MlpRowArgs &g, const MlpGrads &o, cudaStream_t s) {
   MlpDwMaps maps;
   cudaError_t e;
   for (int l = 0; l < 4; ++l) {   // boxes of 64 batch rows x 64 features
@@ -705,13 +679,10 @@ cudaError_t launch_mlp_dw(const MlpRowArgs &g, float *part, const MlpGrads &o, c
     if ((e = encode_bf16(&maps.b[l], l == 0 ? g.X0 : g.A[l - 1], g.B, in, in, 64)) != cudaSuccess) return e;
   }
   if ((e = ensure_smem_attr((const void *)mlp_dw_kernel, kDwSmem)) != cudaSuccess) return e;
-  const int splits = mlp_dw_splits(g.B), tiles = (g.B + kTcRows - 1) / kTcRows;
-  // the step's kernels and Adam queue behind each other: a step of 4096 rows 75.5 -> 70.5 us
-  if ((e = launch_chained(mlp_dw_kernel, dim3(kMlpDwTiles, splits), kDwThreads, kDwSmem, s, maps, g.B, splits, part, g.err)) !=
-      cudaSuccess)
-    return e;
-  return launch_programmatic(true, mlp_reduce_kernel, kMlpDwTiles * 8 + kMlpGbCols / 32 + 1, 256, 0, s, part, splits, tiles,
-                             g.gb_part, g.loss_part, o);
+  const int tiles = (g.B + kTcRows - 1) / kTcRows;
+  // the step's kernels and Adam queue behind each other (5 us of a step of 4096 rows)
+  return launch_chained(mlp_dw_kernel, kMlpDwTiles + kMlpGbCols / 32 + 1, kDwThreads, kDwSmem, s, maps, o, g.B, tiles,
+                        g.gb_part, g.loss_part, g.err);
 }
 
 }  // namespace doa

@@ -11,9 +11,6 @@ namespace doa {
 constexpr int kMlpGbCols = 3 * DOA_MLP_HIDDEN + 192;   // bias-gradient partial sums of one row group
 constexpr int kMlpLossParts = 16;                      // loss partial sums of a 128-row tile
 constexpr int kMlpDwTiles = 34;                        // 128 x 64 tiles of the four weight gradients
-constexpr int kMlpMaxSplits = 8;                       // splits of the batch in the weight gradients
-constexpr int kMlpSplitRows = 5632;                    // largest batch that is split
-constexpr int64_t kMlpDwTileFloats = 128 * 64;         // one partial tile
 
 constexpr int kMlpOutPitch = 192;                      // row pitch of dZ_4 (181 columns, zero padding)
 
@@ -43,8 +40,7 @@ struct MlpGrads {
   float *loss;              // nullable
 };
 
-int mlp_dw_splits(int batch);
 cudaError_t launch_mlp_rows(const doa_mlp *net, const MlpRowArgs &g, bool train, cudaStream_t s);
-cudaError_t launch_mlp_dw(const MlpRowArgs &g, float *part, const MlpGrads &o, cudaStream_t s);
+cudaError_t launch_mlp_dw(const MlpRowArgs &g, const MlpGrads &o, cudaStream_t s);
 
 }  // namespace doa

@@ -151,8 +151,8 @@ def test_forward_tiles_and_alignment(env, B):
 
 
 @pytest.mark.parametrize("B", [8, 136, 5632, 5640, 19592])
-def test_gradients_split_and_tiles(env, B):
-    """Both sides of the batch split of the weight gradients, ragged tiles, more tiles than SMs."""
+def test_gradients_and_tiles(env, B):
+    """Weight gradients over one or many K tiles, ragged tiles, more tiles than SMs."""
     torch, doa = env
     net = doa.Mlp(seed=16)
     rng = np.random.default_rng(B + 1)
