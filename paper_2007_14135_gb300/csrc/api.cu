@@ -719,9 +719,10 @@ doa_status doa_batch_plan(const doa_problem *probs, int nprob, const doa_tuning 
       ++h.geo_jobs[b];
       q.tile_start = 0;
       if (q.geo_steer < 0 || geo_gsize[q.geo_steer] == 0) {
-        const int tp = kScanThreads * h.geo_pt[b];
-        q.tile_start = h.geo_tiles[b];
-        h.geo_tiles[b] += (q.npts + tp - 1) / tp;
+        const int tp = kScanThreads * h.geo_pt[b], tp0 = kScanThreads * pt[b];
+        q.tile_start = h.geo_pt_tiles[b];
+        h.geo_pt_tiles[b] += (q.npts + tp - 1) / tp;
+        h.geo_tiles[b] += (q.npts + tp0 - 1) / tp0;
         geo[b][h.geo_alone[b]++] = i;
       }
     } else if (grouped(i) || tc_grouped(i)) {
@@ -860,7 +861,8 @@ doa_status doa_solve_batch(const void *plan_host, const void *plan_dev, void *ws
                            void *const *stage_events, void *stream) {
   if (!plan_host || !plan_dev || !ws || !status) return DOA_EINVAL;
   const PlanHeader &h = *static_cast<const PlanHeader *>(plan_host);
-  if (h.magic != kPlanMagic || h.nprob < 1) return DOA_EINVAL;
+  // (off_prob: where the header ends, so bytes with a header of another layout are refused)
+  if (h.magic != kPlanMagic || h.off_prob != round_up(sizeof(PlanHeader), 16) || h.nprob < 1) return DOA_EINVAL;
   if (!aligned(plan_dev, 16) || !aligned(ws, 256) || !aligned(status, 4)) return DOA_EINVAL;
   if (ws_bytes < (size_t)h.ws_bytes) return DOA_ENOMEM;
   cudaStream_t s = as_stream(stream);

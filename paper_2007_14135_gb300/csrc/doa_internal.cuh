@@ -145,7 +145,7 @@ __device__ __forceinline__ double2 phasor_q64(uint64_t phi) {
 // ------------------------------------------------------------------------------------------
 // Batch plan. The same bytes live on the host (for launch sizes) and on the device.
 // ------------------------------------------------------------------------------------------
-constexpr uint32_t kPlanMagic = 0x444f4132u;  // "DOA2" (a header of another layout is refused)
+constexpr uint32_t kPlanMagic = 0x444f4131u;  // "DOA1"
 constexpr int kNumBuckets = 4;                // M <= 8, <= 16, <= 32, <= 64
 // Covariance work-item classes: 4x4 register blocks per row, MB = ceil(M / 4) in {2, 3, 4} use
 // the block-task kernel (one launch per class, CTA shape fixed by MB); every other M the
@@ -365,7 +365,8 @@ struct PlanHeader {
   int64_t gg_units[kNumBuckets];
   int64_t off_gg[kNumBuckets];           // PlanScanGroup arrays (grid_id: the shared steering table)
   int64_t off_ggl[kNumBuckets];          // their problem lists
-  int32_t geo_pt[kNumBuckets];           // grid points per thread of the geometry scan
+  int32_t geo_pt[kNumBuckets];           // grid points per thread of the geometry scan (one by one)
+  int64_t geo_pt_tiles[kNumBuckets];     // its tiles (geo_tiles counts them at scan_pt points per thread)
 };
 
 // The Python binding reads these header fields by position (int32 index 22 = scan_pt, 58 = eig_mats,
@@ -393,7 +394,7 @@ static_assert(offsetof(PlanHeader, sg_size) == 464 && offsetof(PlanHeader, sg_un
 static_assert(offsetof(PlanHeader, tcg_groups) == 608 && offsetof(PlanHeader, tcg_units) == 624,
               "PlanHeader layout changed");
 static_assert(offsetof(PlanHeader, geo_alone) == 688 && offsetof(PlanHeader, gg_units) == 704 &&
-                  sizeof(PlanHeader) == 816,
+                  sizeof(PlanHeader) == 848,
               "PlanHeader layout changed");
 
 // Scan tiles: kScanThreads threads, each evaluating PT consecutive grid points (tile shape

@@ -322,7 +322,7 @@ __global__ void __launch_bounds__(kScanThreads) scan_geometry_batch_kernel(const
   __shared__ GeoShared gs;
   const PlanHeader *h = reinterpret_cast<const PlanHeader *>(plan);
   const int nunits = h->geo_alone[bucket];
-  const int64_t ntiles = h->geo_tiles[bucket];
+  const int64_t ntiles = h->geo_pt_tiles[bucket];
   const int32_t *list = reinterpret_cast<const int32_t *>(plan + h->off_geo[bucket]);
   const PlanProblem *probs = reinterpret_cast<const PlanProblem *>(plan + h->off_prob);
   const PlanGeoGrid *geo_grids = reinterpret_cast<const PlanGeoGrid *>(plan + h->off_geo_grid);
@@ -533,7 +533,7 @@ cudaError_t run_geo_shared(const uint8_t *plan, const PlanHeader &h, uint8_t *ws
 
 template <int MP, int PT>
 cudaError_t run_geo_batch(const uint8_t *plan, const PlanHeader &h, uint8_t *ws, int bucket, cudaStream_t s) {
-  const int64_t tiles = h.geo_tiles[bucket];
+  const int64_t tiles = h.geo_pt_tiles[bucket];
   if (tiles == 0) return cudaSuccess;
   int per_sm = 0;
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, scan_geometry_batch_kernel<MP, PT>, kScanThreads, 0);
