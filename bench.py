@@ -1144,6 +1144,9 @@ def run_uca(args, emit=True):
                               unit="TFLOP/s", peak=round(FP32_PEAK_TFLOPS, 2))
     stage_info["scan"]["frac"] = round(stage_info["scan"]["achieved"] / FP32_PEAK_TFLOPS, 4)
     dom = max(range(doa.BATCH_STAGES), key=lambda i: stage_ms[i])
+    # problems that share their array are scanned in groups (header int32 164: groups of the bucket M <= 8)
+    grouped = int(bt["plan"].host[:1024].view(np.int32)[164]) > 0
+    scan_kernel = "scan_geometry_shared_kernel<8,4>" if grouped else f"scan_geometry_batch_kernel<8,{bt['plan'].scan_pt[0]}>"
     result = {
         "metric": METRIC, "value": points / (ms / 1e3), "unit": "points/s", "n_gpus": world, "steps": args.steps,
         "warmup": args.warmup, "ms_per_step": ms, "higher_is_better": True, "scaling": "weak", "vs_baseline": None,
@@ -1162,9 +1165,8 @@ def run_uca(args, emit=True):
         "dominant_stage": doa.STAGE_NAMES[dom],
         "roofline": {"bound": "alu", "achieved": stage_info["scan"]["achieved"], "peak": round(FP32_PEAK_TFLOPS, 2),
                      "unit": "TFLOP/s", "frac": stage_info["scan"]["frac"],
-                     "traffic": (TRAFFIC_BYTES.get(f"scan_geometry_batch_kernel<8,{bt['plan'].scan_pt[0]}>") or 0) * B / 4096
-                     or None,
-                     "kernel": f"scan_geometry_batch_kernel<8,{bt['plan'].scan_pt[0]}>",
+                     "traffic": (TRAFFIC_BYTES.get(scan_kernel) or 0) * B / 4096 or None,
+                     "kernel": scan_kernel,
                      "peak_source": "derived: 152 SMs x 128 FP32 lanes x 2 flop x 2.07 GHz"},
         "single_solve": single,
         "table10": table10,
