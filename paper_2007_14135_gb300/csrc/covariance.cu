@@ -21,9 +21,9 @@
 // Batched form: one CTA per work item (problem, chunk of kCovChunk snapshots); multi-chunk
 // problems add their chunk partials in chunk order in FP64 (covariance_reduce_batch), so the
 // result is deterministic. Problems that request PHD use the compensated mode.
-// Single-problem form: clusters of up to 8 CTAs, each cluster on some of the blocks, split the
-// snapshots (always compensated); CTA rank 0 adds the other CTAs' partials through distributed shared
-// memory.
+// Single-problem form: a thread-block cluster of up to 8 CTAs splits the snapshots (always
+// compensated), the blocks are dealt over such clusters and the entries of a block over threads; CTA
+// rank 0 adds the other CTAs' partials through distributed shared memory.
 #include <cooperative_groups.h>
 
 #include <algorithm>
@@ -43,28 +43,15 @@ constexpr int kSmemBytes = 65536;
 constexpr int kMaxCluster = 8;
 
 struct CovLayout {
-  int M, MB, nb, groups, b0;
-  uint32_t rows;        // row blocks that the CTA's blocks read
-  __device__ CovLayout(int M_) : CovLayout(M_, 0, (M_ + kRB - 1) / kRB * ((M_ + kRB - 1) / kRB + 1) / 2) {}
-  // blocks first .. last - 1 of the upper triangle only
-  __device__ CovLayout(int M_, int first, int last) : M(M_), b0(first) {
+  int M, MB, nb, groups;
+  __host__ __device__ CovLayout(int M_) : M(M_) {
     MB = (M + kRB - 1) / kRB;
-    nb = last - first;
-    groups = max(1, kCovThreads / nb);
-    rows = 0u;
-    if (nb == MB * (MB + 1) / 2) {
-      rows = 0xffffffffu;
-    } else {
-      for (int b = 0; b < nb; ++b) {
-        int bi, bj;
-        block_of(b, bi, bj);
-        rows |= (1u << bi) | (1u << bj);
-      }
-    }
+    nb = MB * (MB + 1) / 2;
+    groups = kCovThreads / nb > 1 ? kCovThreads / nb : 1;
   }
-  // block (bi, bj), bi <= bj, of the CTA's block b
+  // block (bi, bj), bi <= bj, of the linear upper-triangle block index b
   __device__ void block_of(int b, int &bi, int &bj) const {
-    int i = 0, rem = b0 + b;
+    int i = 0, rem = b;
     while (rem >= MB - i) { rem -= MB - i; ++i; }
     bi = i;
     bj = i + rem;
@@ -140,7 +127,6 @@ __device__ float4 *cov_accumulate(const float2 *__restrict__ X, int ldx, int t0,
     __syncthreads();
     for (int e = tid; e < MP * kTS; e += kCovThreads) {
       int r = e / kTS, t = e % kTS;
-      if (!((lay.rows >> (r / kRB)) & 1u)) continue;
       float2 v = make_float2(0.f, 0.f);
       if (r < lay.M && t < cnt) v = X[(size_t)r * ldx + ts + t];
       tile[r * kTS + t] = v;
@@ -224,27 +210,147 @@ __device__ __forceinline__ void store_r(int M, int row, int col, double2 v, doub
   }
 }
 
-__global__ void __launch_bounds__(kCovThreads) covariance_cluster_kernel(const float2 *X, int M, int N, int ldx,
-                                                                         int per_cta, float2 *R, double2 *R64) {
+// Single problem. Every entry of R is the sum of chains of compensated additions whose order depends on M
+// and N alone: a chain per cluster rank (per_cta snapshots) and snapshot group (lay.groups of the whole
+// triangle; group g takes snapshots g, g + groups, ... of each tile), groups added in order in
+// double-float, ranks in FP64. Noise eigenvectors follow the last digits of R (a relative change of
+// 1e-14 moves one by 1e-6 where their eigenvalues nearly meet), so only where a chain is computed may be
+// chosen: the blocks are dealt over the clusters, and a thread takes kE x kE entries of its block.
+// Bound by FP32 issue (ten instructions a multiply-add) and, for small problems, by the loads' latency:
+// a CTA keeps only the rows that its blocks read, as many tiles at once as fit. Against one cluster for the
+// whole triangle, a block a thread (events around one call): M = 8, N = 1024 38 -> 25 us; M = 16,
+// N = 16384 117 -> 39; M = 32, N = 16384 324 -> 69; M = 64, N = 16384 1826 -> 157.
+constexpr int kTSP = kTS + 1;                  // row pitch of a staged tile: rows on different banks
+constexpr int kSingleSmem = 69632;             // 16 tiles of two row blocks; the staged group sums fit too
+
+template <int kE>
+__global__ void __launch_bounds__(kCovThreads) covariance_cluster_kernel(const float2 *__restrict__ X, int M, int N,
+                                                                         int ldx, int per_cta, float2 *R, double2 *R64) {
   let_next_start();
   extern __shared__ __align__(16) uint8_t smem[];
+  constexpr int kParts = (kRB / kE) * (kRB / kE);
   cg::cluster_group cluster = cg::this_cluster();
   const int rank = (int)cluster.block_rank();
   const int nranks = (int)cluster.num_blocks();
-  const int MB = (M + kRB - 1) / kRB, nb = MB * (MB + 1) / 2, nsplit = gridDim.x / nranks, split = blockIdx.x / nranks;
-  const CovLayout lay(M, nb * split / nsplit, nb * (split + 1) / nsplit);
-  const int t0 = rank * per_cta;
-  const int t1 = min(N, t0 + per_cta);
-  float4 *part = cov_accumulate<true>(X, ldx, t0, max(t0, t1), lay, smem);
+  const CovLayout lay(M);
+  const int nsplit = gridDim.x / nranks, split = blockIdx.x / nranks;
+  const int b0 = lay.nb * split / nsplit, nbc = lay.nb * (split + 1) / nsplit - b0;   // this cluster's blocks
+  const int groups = min(lay.groups, kTS);     // those beyond a tile's snapshots stay empty
+  const int t0 = rank * per_cta, len = max(0, min(per_cta, N - t0));   // this CTA's snapshots
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  __shared__ int row_block[kMaxM / kRB];
+  uint32_t rows = 0u;                          // row blocks in use; they are staged packed
+  for (int b = 0; b < nbc; ++b) {
+    int bi, bj;
+    lay.block_of(b0 + b, bi, bj);
+    rows |= (1u << bi) | (1u << bj);
+  }
+  const int nrows = __popc(rows) * kRB;
+  auto slot_of = [&](int rb) { return __popc(rows & ((1u << rb) - 1u)) * kRB; };
+  if (tid < kMaxM / kRB && ((rows >> tid) & 1u)) row_block[slot_of(tid) / kRB] = tid;
+  const int grp = tid % groups, part = tid / groups % kParts, blk = tid / (groups * kParts);
+  const bool active = blk < nbc;
+  const int oi = part / (kRB / kE) * kE, oj = part % (kRB / kE) * kE;
+  int bi = 0, bj = 0;
+  if (active) lay.block_of(b0 + blk, bi, bj);
+  float2 *tile = reinterpret_cast<float2 *>(smem);
+  const int arow = (slot_of(bi) + oi) * kTSP, brow = (slot_of(bj) + oj) * kTSP;
+
+  float rh[kE][kE], rl[kE][kE], ih[kE][kE], il[kE][kE];
+#pragma unroll
+  for (int i = 0; i < kE; ++i)
+#pragma unroll
+    for (int j = 0; j < kE; ++j) rh[i][j] = rl[i][j] = ih[i][j] = il[i][j] = 0.f;
+
+  const int fit = kSingleSmem / (nrows * kTSP * (int)sizeof(float2));   // tiles staged at once (64 rows: two)
+  for (int ts = 0; ts < len; ts += fit * kTS) {
+    const int nt = min(fit, (len - ts + kTS - 1) / kTS);
+    __syncthreads();
+    // a warp per (tile, row): four of them, eight loads a lane, in flight
+    for (int e0 = warp; e0 < nt * nrows; e0 += 4 * (kCovThreads / 32)) {
+      float2 v[4][2];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int e = e0 + u * (kCovThreads / 32), w = e / nrows, sr = e - w * nrows;
+        const bool in = e < nt * nrows;
+        const int r = in ? row_block[sr / kRB] * kRB + sr % kRB : M;
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+          const int t = ts + w * kTS + lane + 32 * k;
+          v[u][k] = r < M && t < len ? X[(size_t)r * ldx + t0 + t] : make_float2(0.f, 0.f);
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int e = e0 + u * (kCovThreads / 32);
+        if (e < nt * nrows) {
+          tile[e * kTSP + lane] = v[u][0];
+          tile[e * kTSP + lane + 32] = v[u][1];
+        }
+      }
+    }
+    __syncthreads();
+    if (active) {
+      for (int w = 0; w < nt; ++w) {
+        const int cnt = min(kTS, len - ts - w * kTS);
+        const float2 *ta = tile + w * nrows * kTSP + arow, *tb = tile + w * nrows * kTSP + brow;
+#pragma unroll 4
+        for (int t = grp; t < cnt; t += groups) {
+          float2 xa[kE], xb[kE];
+#pragma unroll
+          for (int i = 0; i < kE; ++i) {
+            xa[i] = ta[i * kTSP + t];
+            xb[i] = tb[i * kTSP + t];
+          }
+#pragma unroll
+          for (int i = 0; i < kE; ++i)
+#pragma unroll
+            for (int j = 0; j < kE; ++j) {
+              mac<true>(rh[i][j], rl[i][j], xa[i].x, xb[j].x);
+              mac<true>(rh[i][j], rl[i][j], xa[i].y, xb[j].y);
+              mac<true>(ih[i][j], il[i][j], xa[i].y, xb[j].x);
+              mac<true>(ih[i][j], il[i][j], -xa[i].x, xb[j].y);
+            }
+        }
+      }
+    }
+  }
+  __syncthreads();
+  float4 *part_sum = reinterpret_cast<float4 *>(smem);   // groups x nout
+  const int nout = nbc * kRB * kRB;
+  if (active) {
+#pragma unroll
+    for (int i = 0; i < kE; ++i)
+#pragma unroll
+      for (int j = 0; j < kE; ++j)
+        part_sum[grp * nout + (blk * kRB + oi + i) * kRB + oj + j] = make_float4(rh[i][j], rl[i][j], ih[i][j], il[i][j]);
+  }
+  __syncthreads();
+  for (int e = tid; e < nout; e += kCovThreads) {        // the slot's only reader (see cov_accumulate)
+    float4 s = part_sum[e];
+    for (int g = 1; g < groups; ++g) {
+      const float4 v = part_sum[g * nout + e];
+      df_add(s.x, s.y, v.x, v.y);
+      df_add(s.z, s.w, v.z, v.w);
+    }
+    // the empty groups' zeros renormalise the sum until it stays as it is
+    for (int g = groups; g < lay.groups; ++g) {
+      const float4 v = s;
+      df_add(s.x, s.y, 0.f, 0.f);
+      df_add(s.z, s.w, 0.f, 0.f);
+      if (s.x == v.x && s.y == v.y && s.z == v.z && s.w == v.w) break;
+    }
+    part_sum[e] = s;
+  }
   cluster.sync();
   if (rank == 0) {
     const double inv_n = 1.0 / (double)N;
-    for (int e = threadIdx.x; e < lay.nout(); e += kCovThreads) {
+    for (int e = tid; e < nout; e += kCovThreads) {
       int row, col;
-      if (!slot_rc(lay, e, row, col)) continue;
+      if (!slot_rc(lay, b0 * kRB * kRB + e, row, col)) continue;
       double2 s = make_double2(0.0, 0.0);
       for (int r = 0; r < nranks; ++r) {
-        const float4 *rp = cluster.map_shared_rank(part, r);
+        const float4 *rp = cluster.map_shared_rank(part_sum, r);
         double2 v = slot_value(rp[e]);
         s.x += v.x;
         s.y += v.y;
@@ -620,33 +726,38 @@ cudaError_t launch_covariance_fixup(const uint8_t *plan_dev, const PlanHeader &h
   return launch_chained(covariance_fixup_kernel, grid, kCovThreads, kSmemBytes, s, plan_dev, ws);
 }
 
-cudaError_t launch_covariance_single(const float2 *X, int M, int N, int ldx, float2 *R, double2 *R64,
-                                     cudaStream_t s) {
-  cudaError_t e = ensure_smem_attr(reinterpret_cast<const void *>(covariance_cluster_kernel), kSmemBytes);
+template <int kE>
+cudaError_t run_covariance_single(int nc, int ns, const float2 *X, int M, int N, int ldx, int per, float2 *R, double2 *R64,
+                                  cudaStream_t s) {
+  cudaError_t e = ensure_smem_attr(reinterpret_cast<const void *>(covariance_cluster_kernel<kE>), kSingleSmem);
   if (e != cudaSuccess) return e;
-  // Snapshots over a cluster, at least two tiles a CTA; the blocks of the triangle over clusters, as many
-  // as the SMs hold, while a thread still has eight snapshots or more to add (a CTA has 256 / nb groups
-  // of threads for its nb blocks). One cluster that took 1024 snapshots a CTA needed 29 us for M = 8,
-  // N = 1024 (one CTA) and 1.8 ms for M = 64, N = 16384; now 15 and 170 us.
-  const int tiles = (N + kTS - 1) / kTS;
-  const int nc = std::max(1, std::min(kMaxCluster, tiles / 2));
-  const int per = (N + nc - 1) / nc;
-  const int MB = (M + kRB - 1) / kRB, nb = MB * (MB + 1) / 2;
-  int ns = std::min(nb, std::max(1, device_sm_count() / nc));
-  while (ns > 1 && (int64_t)per * ((nb + ns - 1) / ns) < 8 * kCovThreads) --ns;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(nc * ns);
   cfg.blockDim = dim3(kCovThreads);
-  cfg.dynamicSmemBytes = kSmemBytes;
+  cfg.dynamicSmemBytes = kSingleSmem;
   cfg.stream = s;
-  cudaLaunchAttribute attr_[1];
-  attr_[0].id = cudaLaunchAttributeClusterDimension;
-  attr_[0].val.clusterDim.x = nc;
-  attr_[0].val.clusterDim.y = 1;
-  attr_[0].val.clusterDim.z = 1;
-  cfg.attrs = attr_;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = nc;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, covariance_cluster_kernel, X, M, N, ldx, per, R, R64);
+  return cudaLaunchKernelEx(&cfg, covariance_cluster_kernel<kE>, X, M, N, ldx, per, R, R64);
+}
+
+// The cluster's split of the snapshots fixes the order of the sums. The blocks go to as many clusters as the
+// SMs hold, or as leave a thread for each 2 x 2 entries of every chain of a CTA; a thread takes one entry
+// where there are enough.
+cudaError_t launch_covariance_single(const float2 *X, int M, int N, int ldx, float2 *R, double2 *R64,
+                                     cudaStream_t s) {
+  const int nc = std::min(kMaxCluster, (N - 1) / kCovChunk + 1), per = (N - 1) / nc + 1;
+  const CovLayout lay(M);
+  const int groups = std::min(lay.groups, kTS), most = kCovThreads / (4 * groups);   // blocks a CTA can take
+  const int ns = std::max(std::min(lay.nb, std::max(1, device_sm_count() / nc)), (lay.nb + most - 1) / most);
+  const int nbc = (lay.nb + ns - 1) / ns;
+  return 16 * nbc * groups <= kCovThreads ? run_covariance_single<1>(nc, ns, X, M, N, ldx, per, R, R64, s)
+                                          : run_covariance_single<2>(nc, ns, X, M, N, ldx, per, R, R64, s);
 }
 
 template <int MB, int kKind>
