@@ -7,8 +7,8 @@
 // for a pair (p, q) with a_pq = |a_pq| e^{j phi}, tau = (a_qq - a_pp) / (2 |a_pq|),
 // t = sgn(tau) / (|tau| + sqrt(1 + tau^2)), c = 1/sqrt(1 + t^2), s = t c, sigma = s e^{j phi};
 // J = [[c, sigma], [-conj(sigma), c]] on coordinates (p, q) zeroes (J^H A J)_pq.
-// Each rotation's parameters use reciprocal square roots and one reciprocal (no divisions,
-// hypot or sqrt), so c^2 + |sigma|^2 = 1 holds to FP64 rounding.
+// The parameters use reciprocal square roots (no hypot or sqrt; in FP64 no tau or t either, see
+// rotation_of), so c^2 + |sigma|^2 = 1 holds to rounding.
 //
 // Parallel ordering: n/2 disjoint rotations per round (round-robin "circle" ordering over
 // n = M rounded up to even; a pair that touches the padding index is not rotated). A pair is
@@ -16,17 +16,20 @@
 // nothing. A round updates A block by block: the 2 x 2 block of the rows of pair a and the columns of
 // pair b >= a takes four lanes, one element each -- the row mix A <- J^H A of the lane's element,
 // exchanged with the lane of the other column, then the column mix A <- A J -- and is written to its
-// mirror image as well, so only half of A is computed; V <- V J takes a lane per pair and row. Matrices
-// of M <= 8 (where half the blocks take as many warp steps as all of them) and those whose eigenvectors
-// go into a 2-D refinement compute both halves: where a minimum of the planar array's spectrum meets its
-// mirror image at the array plane, the refined angle moves by the square root of a rounding error.
+// mirror image as well, so only half of A is computed; V <- V J takes a lane per pair and row. Both halves
+// are computed, each element by the row mix and then the column mix, for matrices of M <= 8 (where half the
+// blocks take as many warp steps as all of them), for geometry problems (where a minimum of the planar
+// array's spectrum meets its mirror image at the array plane, the refined angle moves by the square root of a
+// rounding error) and in double-float: it rotates down to 1e-12 only, so noise eigenvectors whose eigenvalues
+// nearly meet keep 1e-7 to 1e-6 of whatever is added in another order.
 //
 // Two shapes, with the same arithmetic and results. A warp per matrix (or G packed matrices, every
 // lane owning one pair's rotation) keeps the most matrices resident and suits large batches of M <= 16.
 // A CTA per matrix (3, 5 or 17 warps at M <= 8, 16, 32) suits single calls, small batches and M <= 32,
 // which otherwise wait for one warp's chain of instructions: one FP64 matrix of M = 8 in 78 instead of
-// 141 us, 254 double-float matrices of M = 32 in 0.8 instead of 3.2 ms. Half of A: 4096 matrices of
-// M = 16 in 1.10 instead of 1.27 ms.
+// 141 us, 256 double-float matrices of M = 32 in 0.96 instead of 2.84 ms. Half of A: one FP64 matrix of M = 64
+// in 6.8 instead of 9.6 ms. The warp form in double-float takes two lanes a block, a column each, which
+// share the indices and rotations of two elements: 4096 matrices of M = 16 in 1.10 ms (1.21 with four).
 // M <= 64 gets a 512-thread CTA in FP64, or in double-float a cluster of four CTAs that split its
 // rows (jacobi_cluster_df).
 #include <cooperative_groups.h>
@@ -60,15 +63,15 @@ struct EigSmem {
 };
 
 // Threads per matrix of the CTA form: a round's warp steps (blocks of A, then rows of V) are 2 + 1 at
-// M = 8, 5 + 4 at M = 16, 17 + 16 at M = 32, taken in one, two and two turns. At M = 16 nine warps take
-// them in one turn but let fewer matrices reside: 0.13 against 0.14 ms for one matrix, 0.41 against
-// 0.34 ms for 1024.
+// M = 8, 5 + 4 (both halves: 8 + 4) at M = 16, 17 + 16 (32 + 16) at M = 32, taken in one, two (three) and
+// two (three) turns. Six and 24 warps take the larger numbers in two turns but let fewer matrices reside
+// (double-float): 0.125 against 0.14 ms for one matrix of M = 16, 0.44 against 0.38 for 1024; 0.48 against
+// 0.50 ms for one of M = 32, 1.20 against 0.96 for 256.
 template <int NP>
 __host__ __device__ constexpr int cta_threads() { return NP <= 8 ? 96 : (NP <= 16 ? 160 : (NP <= 32 ? 544 : 512)); }
 // Largest batch that takes the CTA form (the eig stage, warp form against CTA form): at M <= 8, 63 / 47
-// us for 1 matrix, 82 / 74 for 1024, 112 / 131 for 2048; at M <= 16, 0.32 / 0.14 ms for 1, 0.53 / 0.23
-// for 512, 0.77 / 0.64 for 2048, 1.06 / 1.20 for 4096; at M <= 32 always (2.3 / 0.53 ms for 1, 4.7 / 2.7
-// for 1024).
+// us for 1 matrix, 82 / 74 for 1024, 112 / 131 for 2048; at M <= 16, 0.32 / 0.14 ms for 1, 0.55 / 0.38
+// for 1024, 0.80 / 0.71 for 2048; at M <= 32 always (1.9 / 0.50 ms for 1, 5.3 / 3.1 for 1024).
 template <int NP>
 __host__ constexpr int eig_cta_limit() { return NP <= 8 ? 1024 : 2048; }
 template <int NP>
@@ -230,6 +233,7 @@ struct ArithF64 {
   static __device__ __forceinline__ El conj(El x) { return make_double2(x.x, neg(x.y)); }
   static __device__ __forceinline__ El real(El x) { return make_double2(x.x, 0.0); }
   static constexpr bool kZeroes = true;   // the annihilated entry is set to zero
+  static constexpr bool kBoth = false;    // half of A, unless asked for
 };
 
 template <int NP>
@@ -252,6 +256,7 @@ struct ArithDF {
   static __device__ __forceinline__ El conj(El x) { return make_float4(x.x, x.y, -x.z, -x.w); }
   static __device__ __forceinline__ El real(El x) { return make_float4(x.x, x.y, 0.f, 0.f); }
   static constexpr bool kZeroes = false;  // it keeps its computed residual for the next sweep
+  static constexpr bool kBoth = true;     // both halves of A
 };
 
 __device__ __forceinline__ double2 shfl_xor1(double2 x) {
@@ -264,11 +269,12 @@ __device__ __forceinline__ float4 shfl_xor1(float4 x) {
 
 // Runs Jacobi on the G matrices of a group of T threads (matrix j has size Ms[j] <= NP, 0 = unused),
 // all loaded from Rs[j] (upper triangle). T = 32: a warp; otherwise the whole CTA on one matrix.
-// both[j]: compute both halves of A (always at M <= 8). res[j] receives sweeps (> 0) or -status; on return A (its diagonal) and V hold FP64.
+// both[j]: compute both halves of A (always at M <= 8 and in double-float). res[j] receives sweeps (> 0) or -status; on return A (its diagonal) and V hold FP64.
 template <class Ar, int NP, int G, int T>
 __device__ void jacobi_group(EigSmem<NP> *mats, const int *Ms, const double2 *const *Rs, const bool *both, int *res) {
   static_assert(T == 32 || G == 1, "a CTA works on one matrix");
   constexpr int HP = NP / 2, W = T / 32;
+  constexpr bool kColumns = T == 32 && Ar::kBoth;   // a lane per column of a block, not per element
   using g = Grp<T>;
   using El = typename Ar::El;
   __shared__ unsigned smask[2];   // the round's rotations, by round parity (CTA form)
@@ -340,12 +346,50 @@ __device__ void jacobi_group(EigSmem<NP> *mats, const int *Ms, const double2 *co
         rotated |= 1u << j;
         EigSmem<NP> &s = mats[j];
         const int M = Ms[j], m = (M + 1) >> 1;
-        const bool full = NP <= 8 || both[j];
-        const int na = ((full ? 4 * m * m : 2 * m * (m + 1)) + 31) >> 5, nv = (m * M + 31) >> 5;   // warp steps: blocks of A, V
+        const bool full = NP <= 8 || Ar::kBoth || both[j];
+        const int na = ((kColumns ? 2 * m * m : full ? 4 * m * m : 2 * m * (m + 1)) + 31) >> 5, nv = (m * M + 31) >> 5;   // warp steps: blocks of A, V
         const int wid = full ? m : m + ((m & 1) ^ 1);   // the square of blocks, or the triangle of blocks a <= b, folded into rows of equal length
         const float inv_w = __fdividef(1.f, (float)wid), inv_m = __fdividef(1.f, (float)M);
         for (int st = wp; st < na + nv; st += W) {
-          if (st < na) {
+          if (kColumns && st < na) {
+            const int blk = (st << 4) + (lane >> 1);
+            const int a = (int)(((float)blk + 0.5f) * inv_w), b = blk - a * m;
+            const bool in = blk < m * m, lo_col = (lane & 1) == 0;
+            const bool acta = in && ((seg >> a) & 1u), actb = in && ((seg >> b) & 1u);
+            int2 pa = make_int2(0, 0);
+            int col = 0;
+            El xp{}, xq{};
+            if (acta || actb) {
+              pa = s.pq[a];
+              const int2 pb = s.pq[b];
+              col = lo_col ? pb.x : pb.y;
+              xp = Ar::a(s, pa.x, col);
+              xq = Ar::a(s, pa.y, col);
+              if (acta) {
+                const typename Ar::Ro ro = Ar::rot(s)[a];
+                const El np = Ar::mix(ro.c, Ar::neg(ro.sr), ro.si, xp, xq);
+                xq = Ar::mix(ro.c, ro.sr, ro.si, xq, xp);
+                xp = np;
+              }
+            }
+            const El yp = shfl_xor1(xp), yq = shfl_xor1(xq);   // the block's other column, same rows
+            if (acta || actb) {
+              if (actb) {
+                const typename Ar::Ro ro = Ar::rot(s)[b];
+                const auto sr = lo_col ? Ar::neg(ro.sr) : ro.sr;
+                xp = Ar::mix(ro.c, sr, Ar::neg(ro.si), xp, yp);
+                xq = Ar::mix(ro.c, sr, Ar::neg(ro.si), xq, yq);
+              }
+              if (a == b) {              // the diagonal of a Hermitian matrix is real
+                if (lo_col)
+                  xp = Ar::real(xp);
+                else
+                  xq = Ar::real(xq);
+              }
+              Ar::a(s, pa.x, col) = xp;
+              Ar::a(s, pa.y, col) = xq;
+            }
+          } else if (st < na) {
             const int blk = (st << 3) + (lane >> 2);
             const int i = (int)(((float)blk + 0.5f) * inv_w), jj = blk - i * wid;
             const bool head = full || jj < m - i;
@@ -880,8 +924,6 @@ __device__ void finish_batch(const PlanProblem &pp, const PlanJob *jobs, EigSmem
   Grp<T>::sync();
 }
 
-__device__ __forceinline__ bool refines_2d(const doa_problem &p) { return p.geom.pos && p.peak_angle; }
-
 template <int NP, int G>
 __global__ void __launch_bounds__(32 * eig_warps<NP>(), eig_min_ctas<NP>()) eig_batch_kernel(const uint8_t *plan, uint8_t *ws, int bucket,
                                                                          int *status, int dep) {
@@ -906,7 +948,7 @@ __global__ void __launch_bounds__(32 * eig_warps<NP>(), eig_min_ctas<NP>()) eig_
   }
   bool fp64 = false;   // a group runs FP64 when any of its problems asks for it
   bool both[G];
-  for (int j = 0; j < G; ++j) both[j] = prob[j] >= 0 && refines_2d(probs[prob[j]].p);
+  for (int j = 0; j < G; ++j) both[j] = prob[j] >= 0 && probs[prob[j]].p.geom.pos != nullptr;
   for (int j = 0; j < G; ++j) fp64 = fp64 || (prob[j] >= 0 && probs[prob[j]].p.eig_prec == DOA_EIG_FP64);
   if (fp64)
     jacobi_group<ArithF64<NP>, NP, G, 32>(mats, Ms, Rs, both, res);
@@ -934,7 +976,7 @@ __global__ void __launch_bounds__(cta_threads<NP>()) eig_batch_cta_kernel(const 
   const PlanJob *jobs = reinterpret_cast<const PlanJob *>(plan + h->off_job);
   const int Ms[1] = {pp.p.M};
   const double2 *Rs[1] = {reinterpret_cast<const double2 *>(ws + pp.r64_off)};
-  const bool both[1] = {refines_2d(pp.p)};
+  const bool both[1] = {pp.p.geom.pos != nullptr};
   int res[1];
   if (pp.p.eig_prec == DOA_EIG_FP64)
     jacobi_group<ArithF64<NP>, NP, 1, T>(&s, Ms, Rs, both, res);
@@ -968,7 +1010,7 @@ __global__ void __cluster_dims__(kClRanks, 1, 1) __launch_bounds__(kClThreads, 1
     if (!rank0) return;
     int Ms[1] = {pp.p.M}, r1[1];
     const double2 *Rs[1] = {R};
-    const bool both[1] = {refines_2d(pp.p)};
+    const bool both[1] = {pp.p.geom.pos != nullptr};
     jacobi_group<ArithF64<64>, 64, 1, kClThreads>(&s, Ms, Rs, both, r1);
     res = r1[0];
   } else {

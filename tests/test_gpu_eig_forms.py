@@ -63,3 +63,37 @@ def test_single_calls_at_odd_sizes(M, prec):
     F = B.cpu().numpy()[:(M - d) * M].reshape(M - d, M).T
     E = V[:, :M - d]
     assert np.abs(F @ F.conj().T - E @ E.conj().T).max() <= 100 * tol
+
+
+@pytest.mark.parametrize("M", [5, 9, 12, 16, 17, 31, 33])
+@pytest.mark.parametrize("prec", [0, 1])
+def test_digits_do_not_depend_on_the_outputs_asked_for(M, prec):
+    """A geometry problem with and without peak_angle, in a CTA per matrix and packed: eigenvalues, factor and
+    spectrum bit for bit (both halves of A are computed for either)."""
+    torch, doa = require_gpu()
+    rng = np.random.default_rng(900 + M)
+    a = 2.0 * np.pi * np.arange(M) / M
+    pos = np.stack([0.6 * np.cos(a), 0.6 * np.sin(a), np.zeros(M)], axis=1)
+    X = torch.from_numpy((rng.standard_normal((M, 300)) + 1j * rng.standard_normal((M, 300))).astype(np.complex64)).cuda()
+    posd, geom_grid = torch.from_numpy(pos).cuda(), doa.grid(0.0, 4.0, 90)
+    geom = doa.geometry(posd, 2.0, 4.0, 20, True)
+    results = []
+    for refine, mats in ((False, None), (True, None), (True, [2, 2, 0, 0])):
+        P = torch.zeros(90 * 20, dtype=torch.float32, device="cuda")
+        idx = torch.full((2,), -1, dtype=torch.int32, device="cuda")
+        val = torch.zeros(2, dtype=torch.float32, device="cuda")
+        cnt = torch.zeros(1, dtype=torch.int32, device="cuda")
+        ev = torch.zeros(M, dtype=torch.float64, device="cuda")
+        B = torch.zeros(M * M, dtype=torch.complex128, device="cuda")
+        ang = torch.zeros(4, dtype=torch.float64, device="cuda")
+        plan = doa.BatchPlan([doa.make_problem(X, 2, 1 << doa.MUSIC, geom_grid, P, idx, val, cnt, evals=ev, B_out=B, geom=geom,
+                                               eig_prec=prec, peak_angle=ang if refine else None)],
+                             eig_mats=mats)
+        status = torch.full((1,), -1, dtype=torch.int32, device="cuda")
+        doa.doa_solve_batch(plan, doa.workspace(plan), status)
+        torch.cuda.synchronize()
+        assert status.item() == 0
+        results.append((ev.cpu().numpy(), B.cpu().numpy(), P.cpu().numpy()))
+    for r in results[1:]:
+        for x, y in zip(results[0], r):
+            np.testing.assert_array_equal(x, y)
