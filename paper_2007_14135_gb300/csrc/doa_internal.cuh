@@ -457,7 +457,10 @@ __device__ __forceinline__ void end_after_previous() {
 // 92 -> 85 us.
 __device__ __forceinline__ void start_after_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 // Only small grids: the blocks of a large one come onto the SMs while the kernel before still sets their split of
-// L1 and shared memory, which cost the peak picker of 4096 problems 0.08 ms.
+// L1 and shared memory, which cost the peak picker of 4096 problems 0.08 ms. A kernel of long blocks (the
+// batch's decompositions and scans, single scans of M > 32) only with up to eight: started early, the blocks
+// go several to an SM, onto the first ones with room, where a normal launch deals them one to an SM. The
+// grid-shared scan of 1024 problems on 181 points (32 blocks): 0.34 ms chained, 0.11 launched normally.
 template <class... P, class... A>
 cudaError_t launch_programmatic(bool on, void (*kernel)(P...), dim3 grid, int block, size_t smem, cudaStream_t s,
                                 A... args) {
@@ -479,7 +482,9 @@ cudaError_t launch_beside(void (*kernel)(P...), dim3 grid, int block, size_t sme
   return launch_programmatic(true, kernel, grid, block, smem, s, args...);
 }
 // Launches a kernel that begins with start_after_previous.
-inline bool chained_grid(int64_t grid) { return grid <= 2 * device_sm_count(); }
+inline bool chained_grid(int64_t grid, bool long_blocks = false) {
+  return grid <= (long_blocks ? 8 : 2 * device_sm_count());
+}
 template <class... P, class... A>
 cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, int block, size_t smem, cudaStream_t s, A... args) {
   return launch_programmatic(chained_grid((int64_t)grid.x * grid.y * grid.z), kernel, grid, block, smem, s, args...);

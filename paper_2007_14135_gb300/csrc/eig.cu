@@ -1077,7 +1077,7 @@ cudaError_t run_batch_g(const uint8_t *plan, int count, uint8_t *ws, int *status
   const int smem = (int)sizeof(EigSmem<NP>) * per_cta;
   cudaError_t e = ensure_smem_attr(reinterpret_cast<const void *>(eig_batch_kernel<NP, G>), smem);
   if (e != cudaSuccess) return e;
-  return launch_programmatic(beside || chained_grid((count + per_cta - 1) / per_cta), eig_batch_kernel<NP, G>,
+  return launch_programmatic(beside || chained_grid((count + per_cta - 1) / per_cta, true), eig_batch_kernel<NP, G>,
                              (count + per_cta - 1) / per_cta, 32 * W, smem, st, plan, ws, bucket, status,
                           (int)!beside);
 }
@@ -1088,7 +1088,7 @@ cudaError_t run_batch_cta(const uint8_t *plan, int count, uint8_t *ws, int *stat
   const int smem = (int)sizeof(EigSmem<NP>);
   cudaError_t e = ensure_smem_attr(reinterpret_cast<const void *>(eig_batch_cta_kernel<NP>), smem);
   if (e != cudaSuccess) return e;
-  return launch_programmatic(beside || chained_grid(count), eig_batch_cta_kernel<NP>, count, cta_threads<NP>(), smem, st, plan, ws, bucket, status, (int)!beside);
+  return launch_programmatic(beside || chained_grid(count, true), eig_batch_cta_kernel<NP>, count, cta_threads<NP>(), smem, st, plan, ws, bucket, status, (int)!beside);
 }
 
 // M <= 16: the CTA form for small batches unless the plan packs matrices (G in {1, 2, 4, 8} up to the
@@ -1113,7 +1113,7 @@ cudaError_t run_batch_cluster(const uint8_t *plan, const PlanHeader &h, uint8_t 
   if (count == 0) return cudaSuccess;
   cudaError_t e = ensure_smem_attr(reinterpret_cast<const void *>(eig_cluster_batch_kernel), kClSmemBytes);
   if (e != cudaSuccess) return e;
-  return launch_programmatic(beside || chained_grid((int64_t)count * kClRanks), eig_cluster_batch_kernel, (int64_t)count * kClRanks, kClThreads, kClSmemBytes, st, plan, ws, bucket,
+  return launch_programmatic(beside || chained_grid((int64_t)count * kClRanks, true), eig_cluster_batch_kernel, (int64_t)count * kClRanks, kClThreads, kClSmemBytes, st, plan, ws, bucket,
                           status, (int)!beside);
 }
 

@@ -493,7 +493,7 @@ cudaError_t run_batch(const uint8_t *plan, const PlanHeader &h, uint8_t *ws, int
   const int64_t cap = (int64_t)device_sm_count() * per_sm;
   const int run_len = (int)std::min<int64_t>(kRun, std::max<int64_t>(1, (tiles + cap - 1) / cap));
   const int64_t grid = std::min<int64_t>(cap, (tiles + run_len - 1) / run_len);
-  const cudaError_t e = launch_programmatic(beside || chained_grid(grid), scan_batch_kernel<MP, PT>, grid, kScanThreads, 0, s, plan, ws, bucket, run_len, (int)!beside);
+  const cudaError_t e = launch_programmatic(beside || chained_grid(grid, true), scan_batch_kernel<MP, PT>, grid, kScanThreads, 0, s, plan, ws, bucket, run_len, (int)!beside);
   beside = true;
   return e;
 }
@@ -520,7 +520,7 @@ cudaError_t launch_scan_single(const double2 *B, int M, int K, int L, double lo,
   const int pt = scan_pt_for(b, L), tp = kScanThreads * pt;
   const unsigned grid = (unsigned)((L + tp - 1) / tp);
 #define DOA_SCAN_SINGLE(MP, PT) \
-  launch_chained(scan_single_kernel<MP, PT>, grid, kScanThreads, 0, s, B, M, K, L, lo, step, kofs, S, P)
+  launch_programmatic(chained_grid(grid, MP > 32), scan_single_kernel<MP, PT>, grid, kScanThreads, 0, s, B, M, K, L, lo, step, kofs, S, P)
   switch (b) {
     case 0: return pt == 4 ? DOA_SCAN_SINGLE(8, 4) : DOA_SCAN_SINGLE(8, 1);
     case 1: return pt == 4 ? DOA_SCAN_SINGLE(16, 4) : DOA_SCAN_SINGLE(16, 1);
@@ -540,7 +540,7 @@ template <int MP>
 cudaError_t run_prep(const uint8_t *plan, const PlanHeader &h, uint8_t *ws, int bucket, bool &beside, cudaStream_t s) {
   if (h.sg_units[bucket] == 0) return cudaSuccess;
   const int64_t grid = (h.sg_probs[bucket] + kScanWarps - 1) / kScanWarps;
-  const cudaError_t e = launch_programmatic(beside || chained_grid(grid), scan_prep_kernel<MP>, grid,
+  const cudaError_t e = launch_programmatic(beside || chained_grid(grid, true), scan_prep_kernel<MP>, grid,
                                             kScanThreads, 0, s, plan, ws, bucket, (int)!beside);
   beside = true;
   return e;
@@ -553,7 +553,7 @@ cudaError_t run_shared(const uint8_t *plan, const PlanHeader &h, uint8_t *ws, in
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, scan_shared_kernel<MP, PT>, kScanThreads, 0);
   if (per_sm < 1) per_sm = 1;
   const int64_t grid = std::min<int64_t>((int64_t)device_sm_count() * per_sm, h.sg_units[bucket]);
-  const cudaError_t e = launch_programmatic(beside || chained_grid(grid), scan_shared_kernel<MP, PT>, grid,
+  const cudaError_t e = launch_programmatic(beside || chained_grid(grid, true), scan_shared_kernel<MP, PT>, grid,
                                             kScanThreads, 0, s, plan, ws, bucket, (int)!beside);
   beside = true;
   return e;
