@@ -148,12 +148,16 @@ __global__ void windows_kernel(const float *probs, const int32_t *d, int batch, 
   }
 }
 
-// Windowed scan: block = (row slot, window, run of `run` tiles of 128 x PT points). PT = 4 points a thread
+// Windowed scan: block = (row slot, window, run of `run` tiles of 128 x PT points). PT = 2 points a thread
 // in the paired form of the batch scan (the same operations, so the same bits as every other tile shape);
 // the factor and its thresholds are prepared once per run and the flagged points re-evaluated at its end (or when the queue fills).
-// A block per 256 points, which prepared them for two points a thread, took 1.96 ms for 12288 windows of
-// 4001 points; now 1.45 ms, 0.7 of the FP32 issue rate.
-constexpr int kWinPT = 4, kWinRun = 16;
+// A run is also what one block re-evaluates alone (0.4 us a point: 0.1 ms for a tile that is flagged
+// throughout, in a window between close sources), so it grows only where the whole launch is long against
+// it. Of the time of unpaired tiles of 256 points, one to a block: runs of 1 take 0.82-1.01 over 64..2048
+// rows, of 2 0.76-1.29, of 4 0.75-1.51, tiles of 512 points in runs of up to 16 0.75-1.77; the lower ends from 1200
+// rows on. 2048 rows of 4001 points: 2.19 -> 1.67 ms.
+constexpr int kWinPT = 2, kWinRun = 4;
+constexpr int kWinTilesPerSm = 320;   // tiles per SM of the launch for each tile of a run
 
 template <int MP>
 __global__ void __launch_bounds__(kScanThreads) scan_windows_kernel(const double2 *B, int M, const int32_t *K,
@@ -200,15 +204,15 @@ __global__ void __launch_bounds__(kScanThreads) scan_windows_kernel(const double
   }
 }
 
-// Launches the scan of nrows x nw windows of len points (or whole rows); false: too many blocks.
+// Launches the scan of nrows x nw windows of len points (or whole rows) in runs of at least `least` tiles; false:
+// too many blocks.
 bool launch_scan_windows(const double *B, int M, const int32_t *K, const int32_t *rows, int nrows, int nw, int dmax,
                          const doa_grid &fine, const int32_t *win_first, int width, int full, const uint32_t *S,
-                         float *P, cudaStream_t s) {
+                         float *P, int least, cudaStream_t s) {
   const int tp = kScanThreads * kWinPT;
   const int tiles = ((full ? fine.L : width) + tp - 1) / tp;
-  // runs as long as leave eight blocks per SM
-  const long long want = (long long)nrows * nw * tiles / (8 * device_sm_count());
-  const int run = (int)std::max(1ll, std::min<long long>(std::min(kWinRun, tiles), want));
+  const long long want = (long long)nrows * nw * tiles / (kWinTilesPerSm * device_sm_count());
+  const int run = (int)std::min<long long>(tiles, std::max<long long>(least, std::min<long long>(kWinRun, want)));
   const int runs = (tiles + run - 1) / run;
   const long long blocks = (long long)nrows * nw * runs;
   if (blocks > INT_MAX) return false;
@@ -484,7 +488,7 @@ extern "C" doa_status doa_scan_windows(const double *B, int M, const int32_t *K,
   const int tp = kScanThreads * 2;
   if ((long long)nrows * (full ? 1 : dmax) * (((full ? fine.L : width) + tp - 1) / tp) > INT_MAX) return DOA_EINVAL;
   phase_table_kernel<<<(fine.L + 255) / 256, 256, 0, s>>>(fine.lo_deg, fine.step_deg, fine.L, S);
-  if (!launch_scan_windows(B, M, K, rows, nrows, full ? 1 : dmax, dmax, fine, win_first, width, full, S, Pwin, s))
+  if (!launch_scan_windows(B, M, K, rows, nrows, full ? 1 : dmax, dmax, fine, win_first, width, full, S, Pwin, 1, s))
     return DOA_EINVAL;
   window_peaks_kernel<<<nrows, pk::kPeakThreads, 0, s>>>(Pwin, rows, d, dmax, fine.L, win_first, width, full, idx, val,
                                                    count, fallback);
@@ -510,7 +514,8 @@ extern "C" doa_status doa_proposal_judge(const double *B, int M, const int32_t *
       jwidth, batch, judge_first, fallback);
   if (launch_beside(phase_table_kernel, (fine.L + 255) / 256, 256, 0, s, fine.lo_deg, fine.step_deg, fine.L, S) != cudaSuccess)
     return DOA_ECUDA;
-  if (!launch_scan_windows(B, M, K, nullptr, batch, kJudgeMax, kJudgeMax, fine, judge_first, jwidth, 0, S, Pjudge, s))
+  // away from the peaks hardly a point is flagged
+  if (!launch_scan_windows(B, M, K, nullptr, batch, kJudgeMax, kJudgeMax, fine, judge_first, jwidth, 0, S, Pjudge, 2, s))
     return DOA_EINVAL;
   judge_compare_kernel<<<batch, 256, 0, s>>>(Pjudge, judge_first, jwidth, fine.L, val, count, d, dmax, fallback);
   return cudaGetLastError() == cudaSuccess ? DOA_OK : DOA_ECUDA;
