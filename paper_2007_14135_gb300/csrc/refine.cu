@@ -80,7 +80,10 @@ __device__ __forceinline__ double vertex_offset(float pa, float pb, float pc) {
   return fmin(fmax(0.5 * (da - dc) / curv, -0.9), 0.9);
 }
 
-constexpr int kChainCols = 32;   // columns up to which a lane takes one real recurrence
+// Columns up to which a lane takes one real recurrence: 6 Kf of them in up to three turns. More turns cost more
+// than a column per lane (one ULA peak: M = 18, Kf = 14 0.33 instead of 0.42 ms, but M = 24, Kf = 18 0.066 instead
+// of 0.062, M = 32, Kf = 24 0.80 instead of 0.62).
+constexpr int kChainCols = 16;
 struct RefShared {
   double2 v[6][kMaxM];   // a and its derivatives (1-D: a, a', a''; 2-D: a, a_t, a_p, a_tt, a_tp, a_pp)
   double y[12][kChainCols + 1];   // F^H v: real and imaginary parts per column
