@@ -18,11 +18,15 @@
 // circle p is evaluated as z^n q(1/z) with the reversed coefficients, so powers never overflow: with
 // plain Horner a root beyond 20 or so (a small leading coefficient) put infinities into the FP32 phase,
 // which then ran to its cap and left the FP64 phase to start from the circle.
+// The coefficients are divided by the power of two of the largest one (the roots are the same), so the
+// FP32 phase and the squares below stay in range whatever the factor's scale or the EV weights.
 // One warp per (problem, algorithm) job: lanes own coefficients, then roots, then selected roots.
 //
 // Bound by FP64 issue (an FP64 warp instruction holds its sub-partition for 64 cycles), so the FP64
-// iteration keeps only the two Horner recurrences in FP64 -- the repulsion sum and the rounding bound
-// steer the step and its stop, and FP32 serves them -- and the selection works in parallel lanes.
+// iteration keeps the two Horner recurrences and what decides its stop in FP64, while the repulsion sum,
+// which only steers the step, is taken in FP32 from the roots' leading parts and remainders (in FP64
+// where that leaves its range: far roots, or two iterates that meet); the selection works in parallel
+// lanes.
 // Measured (2048 jobs of degree 30): 5.1 -> 0.58 ms.
 #include <math_constants.h>
 
@@ -39,10 +43,11 @@ constexpr int kRootMaxIterF = 64;    // FP32 phase
 
 struct RootShared {
   float2 af[kMaxDeg + 1];   // the coefficients rounded to FP32 (first phase)
-  float amf[kMaxDeg + 1];   // |a_t| (for the rounding bound of the Horner evaluation)
+  float amf[kMaxDeg + 1];
   float2 zf[kMaxDeg];       // FP32 roots; in the second phase the FP64 roots' leading parts
   float2 wf[kMaxDeg];       // FP32 corrections; in the second phase the FP64 roots' remainders
   double2 a[kMaxDeg + 1];   // polynomial coefficients, a[t] multiplies z^t
+  double am[kMaxDeg + 1];   // |a_t| (for the rounding bound of the Horner evaluation)
   double2 z[kMaxDeg];       // current roots
   double2 w[kMaxDeg];       // corrections of this iteration
   int conv[kMaxDeg];        // root converged (its correction is no longer computed)
@@ -83,12 +88,38 @@ __device__ __forceinline__ double root_weight(const RootJob &j, int c) {
   }
 }
 
+// sum_{k != i} 1 / (z_i - z_k): in FP32 from the roots' leading parts and remainders; in FP64 when that is
+// not finite (two iterates within 2^-48, or one beyond FP32's range) or was not asked for. An iterate
+// equal to z_i adds nothing.
+__device__ __forceinline__ double2 repulsion(const RootShared &sh, int i, int n, bool fp32) {
+  if (fp32) {
+    const float2 zh = sh.zf[i], zl = sh.wf[i];
+    float2 rep = make_float2(0.f, 0.f);
+    for (int k = 0; k < n; ++k) {
+      if (k == i) continue;
+      const float2 kh = sh.zf[k], kl = sh.wf[k];
+      const float2 d = make_float2((zh.x - kh.x) + (zl.x - kl.x), (zh.y - kh.y) + (zl.y - kl.y));
+      rep = fcadd(rep, fcdiv(make_float2(1.f, 0.f), d));
+    }
+    if (isfinite(rep.x) && isfinite(rep.y)) return make_double2((double)rep.x, (double)rep.y);
+  }
+  double2 rep = make_double2(0.0, 0.0);
+  for (int k = 0; k < n; ++k) {
+    const double2 d = csub(sh.z[i], sh.z[k]);
+    if (k == i || (d.x == 0.0 && d.y == 0.0)) continue;
+    const double2 r = crcp(d);
+    rep = make_double2(rep.x + r.x, rep.y + r.y);
+  }
+  return rep;
+}
+
 // Writes the d angles (degrees, ascending) of one job to out; returns 0 or DOA_ENOCONV.
 __device__ int root_music_warp(const RootJob &j, RootShared &sh, double *out) {
   const int lane = threadIdx.x & 31;
   const int M = j.M, n = 2 * M - 2;
   // coefficients: a[t] = c_{t - (M-1)}, c_{-l} = conj(c_l); lanes pair up on an l >= 0, each taking every
   // other column
+  int top = 0;
   for (int l0 = 0; l0 < M; l0 += 16) {
     const int l = l0 + (lane >> 1);
     double cr = 0.0, ci = 0.0;
@@ -111,9 +142,19 @@ __device__ int root_music_warp(const RootJob &j, RootShared &sh, double *out) {
       const int t = (lane & 1) ? M - 1 - l : M - 1 + l;
       const double im = (lane & 1) ? -ci : (l == 0 ? 0.0 : ci);
       sh.a[t] = make_double2(cr, im);
-      sh.af[t] = make_float2((float)cr, (float)im);
-      sh.amf[t] = (float)sqrt(cr * cr + ci * ci);
+      top = max(top, max(__double2hiint(cr) & 0x7fffffff, __double2hiint(im) & 0x7fffffff));
     }
+  }
+  top = __reduce_max_sync(0xffffffffu, top) >> 20;    // the largest coefficient's exponent field
+  const int ex = top == 0 || top == 0x7ff ? 0 : 1023 - top;   // (zero or not finite: left as it is)
+  __syncwarp();
+  for (int t = lane; t <= n; t += 32) {
+    const double2 c = make_double2(scalbn(sh.a[t].x, ex), scalbn(sh.a[t].y, ex));
+    const double m = sqrt(c.x * c.x + c.y * c.y);
+    sh.a[t] = c;
+    sh.am[t] = m;
+    sh.af[t] = make_float2((float)c.x, (float)c.y);
+    sh.amf[t] = (float)m;
   }
   for (int i = lane; i < n; i += 32) {
     float s, c;
@@ -195,37 +236,32 @@ __device__ int root_music_warp(const RootJob &j, RootShared &sh, double *out) {
       for (int i = lane; i < n; i += 32) {
         if (sh.conv[i]) continue;                    // converged: no more correction
         const double2 zi = sh.z[i];
-        const float2 zh = sh.zf[i], zl = sh.wf[i];
-        const float zm = hypotf(zh.x, zh.y);
-        const bool outer = zm > 1.f;
-        const double2 x = outer ? crcp(zi) : zi;
-        const float xm = outer ? 1.f / zm : zm;
+        const double r2 = zi.x * zi.x + zi.y * zi.y, zm = sqrt(r2);
+        const bool outer = zm > 1.0;
+        const double inv = outer ? __drcp_rn(r2) : 1.0;
+        const double2 x = outer ? make_double2(zi.x * inv, -zi.y * inv) : zi;
+        const double xm = zm * inv;
         int t = outer ? 0 : n;
         const int dt = outer ? 1 : -1;
         double2 p = sh.a[t], dp = make_double2(0.0, 0.0);
-        float pe = sh.amf[t];
+        double pe = sh.am[t];
         for (int k = 0; k < n; ++k) {                // Horner for p, p' and the bound sum |a_t| |x|^t
           t += dt;
           const double2 at = sh.a[t];
           dp = make_double2(fma(dp.x, x.x, fma(-dp.y, x.y, p.x)), fma(dp.x, x.y, fma(dp.y, x.x, p.y)));
           p = make_double2(fma(p.x, x.x, fma(-p.y, x.y, at.x)), fma(p.x, x.y, fma(p.y, x.x, at.y)));
-          pe = fmaf(pe, xm, sh.amf[t]);
+          pe = fma(pe, xm, sh.am[t]);
         }
-        float2 rep = make_float2(0.f, 0.f);          // sum_{k != i} 1 / (z_i - z_k)
-        for (int k = 0; k < n; ++k) {
-          if (k == i) continue;
-          const float2 kh = sh.zf[k], kl = sh.wf[k];
-          const float2 d = make_float2((zh.x - kh.x) + (zl.x - kl.x), (zh.y - kh.y) + (zl.y - kl.y));
-          rep = fcadd(rep, fcdiv(make_float2(1.f, 0.f), d));
-        }
-        if (outer) dp = cmul(x, csub(make_double2(n * p.x, n * p.y), cmul(x, dp)));
-        const double2 ratio = cdiv(p, dp);
-        const double2 den = csub(make_double2(1.0, 0.0), cmul(ratio, make_double2((double)rep.x, (double)rep.y)));
+        const double2 rep = repulsion(sh, i, n, zm < 1e15);
+        // Newton ratio p / p': outside it is z q / (n q - x q')
+        if (outer) dp = csub(make_double2(n * p.x, n * p.y), cmul(x, dp));
+        const double2 pdp = cdiv(p, dp), ratio = outer ? cmul(zi, pdp) : pdp;
+        const double2 den = csub(make_double2(1.0, 0.0), cmul(ratio, rep));
         const double2 wi = cdiv(ratio, den);
         sh.w[i] = wi;
         const double mag = sqrt(wi.x * wi.x + wi.y * wi.y);
         const double res = sqrt(p.x * p.x + p.y * p.y);
-        const bool ok = isfinite(mag) && (mag <= 1e-14 * (double)fmaxf(1.f, zm) || res <= 8.0 * n * 1.1102230246251565e-16 * (double)pe);
+        const bool ok = isfinite(mag) && isfinite(zm) && (mag <= 1e-14 * fmax(1.0, zm) || res <= 8.0 * n * 1.1102230246251565e-16 * pe);
         small = small && ok;
         if (ok) sh.conv[i] = 1;
       }
