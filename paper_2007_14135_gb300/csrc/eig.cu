@@ -84,6 +84,10 @@ __host__ __device__ constexpr int eig_warps() { return NP <= 8 ? 4 : 9; }
 template <int NP>
 __host__ __device__ constexpr int eig_min_ctas() { return NP <= 8 ? 8 : 3; }
 
+// FP64 matrices whose largest element is outside 2^-400 .. 2^400 are brought to the nearer end by a power of two
+// (exactly) for the Jacobi, whose rotations square differences and elements.
+constexpr int kEigSafeExp = 400;
+
 template <int T>
 struct Grp {
   __device__ static int id() { return (int)(threadIdx.x % T); }
@@ -267,6 +271,26 @@ __device__ __forceinline__ float4 shfl_xor1(float4 x) {
                      __shfl_xor_sync(0xffffffffu, x.z, 1), __shfl_xor_sync(0xffffffffu, x.w, 1));
 }
 
+// Brings the n x n matrix in s.A into that range; ex: the exponent of this thread's largest element. Returns
+// the exponent of the power of two that it was divided by.
+template <int T, int NP>
+__device__ __noinline__ int scale_to_safe(EigSmem<NP> &s, int n, int ex) {
+  __shared__ int warp_top[T / 32];
+  int top = __reduce_max_sync(0xffffffffu, ex);
+  if (T > 32) {
+    if ((threadIdx.x & 31) == 0) warp_top[threadIdx.x >> 5] = top;
+    __syncthreads();
+    for (int w = 0; w < T / 32; ++w) top = max(top, warp_top[w]);
+  }
+  top -= top > 0 ? kEigSafeExp : -kEigSafeExp;
+  for (int e = Grp<T>::id(); e < n * n; e += T) {   // the elements this thread wrote
+    double2 &v = s.a(e / n, e % n);
+    v = make_double2(scalbn(v.x, -top), scalbn(v.y, -top));
+  }
+  Grp<T>::sync();
+  return top;
+}
+
 // Runs Jacobi on the G matrices of a group of T threads (matrix j has size Ms[j] <= NP, 0 = unused),
 // all loaded from Rs[j] (upper triangle). T = 32: a warp; otherwise the whole CTA on one matrix.
 // both[j]: compute both halves of A (always at M <= 8 and in double-float). res[j] receives sweeps (> 0) or -status; on return A (its diagonal) and V hold FP64.
@@ -280,13 +304,15 @@ __device__ void jacobi_group(EigSmem<NP> *mats, const int *Ms, const double2 *co
   __shared__ unsigned smask[2];   // the round's rotations, by round parity (CTA form)
   const int tid = g::id(), lane = tid & 31, wp = tid >> 5;
   unsigned live = 0u;  // matrices still iterating
+  int scaled[G];       // the exponent of the power of two it was divided by
   for (int j = 0; j < G; ++j) {
     const int M = Ms[j], n = (M + 1) & ~1;
-    res[j] = 0;
+    res[j] = scaled[j] = 0;
     if (M <= 0) continue;
     EigSmem<NP> &s = mats[j];
     const double2 *R = Rs[j];
     bool finite = true;
+    int top = 0;       // high word of the largest |re|, |im|
     for (int e = tid; e < n * n; e += T) {
       const int i = e / n, k = e - i * n;
       double2 v = make_double2(0.0, 0.0);   // an odd M is padded with a zero row and column
@@ -296,6 +322,7 @@ __device__ void jacobi_group(EigSmem<NP> *mats, const int *Ms, const double2 *co
         if (i == k) v.y = 0.0;
       }
       finite = finite && isfinite(v.x) && isfinite(v.y);
+      top = max(top, max(__double2hiint(v.x) & 0x7fffffff, __double2hiint(v.y) & 0x7fffffff));
       Ar::a(s, i, k) = Ar::from(v);
       Ar::v(s, i, k) = Ar::from(make_double2(i == k ? 1.0 : 0.0, 0.0));
     }
@@ -303,6 +330,11 @@ __device__ void jacobi_group(EigSmem<NP> *mats, const int *Ms, const double2 *co
       live |= 1u << j;
     else
       res[j] = -DOA_ENONFINITE;
+    if constexpr (Ar::kZeroes) {
+      const int ex = (top >> 20) - 1023;
+      if (((live >> j) & 1u) && (g::any(ex > kEigSafeExp) || !g::any(ex >= -kEigSafeExp)))
+        scaled[j] = scale_to_safe<T>(s, n, ex);
+    }
   }
   g::sync();
   int maxn = 0;
@@ -450,7 +482,13 @@ __device__ void jacobi_group(EigSmem<NP> *mats, const int *Ms, const double2 *co
   }
   for (int j = 0; j < G; ++j)
     if ((live >> j) & 1u) res[j] = -DOA_ENOCONV;
-  if constexpr (!Ar::kZeroes) {
+  if constexpr (Ar::kZeroes) {
+    for (int j = 0; j < G; ++j)
+      if (scaled[j] != 0) {
+        for (int e = tid; e < Ms[j]; e += T) mats[j].a(e, e).x = scalbn(mats[j].a(e, e).x, scaled[j]);
+        g::sync();
+      }
+  } else {
     // double-float -> FP64 in place (same bytes per element; every element has one owner lane)
     for (int j = 0; j < G; ++j) {
       const int M = Ms[j];
