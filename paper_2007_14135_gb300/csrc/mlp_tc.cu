@@ -128,6 +128,17 @@ __device__ __forceinline__ float column_sums(float (&v)[N]) {
   return v[0];
 }
 
+// Barrier 1 of the epilogue warps: true if p holds in all of their threads (a wait that ran out ends their loop
+// over the tiles for all of them or for none, since they meet at barriers in it).
+__device__ __forceinline__ bool all_ok(bool p) {
+  uint32_t r;
+  asm volatile("{\n.reg .pred p, q;\nsetp.ne.u32 p, %1, 0;\nbarrier.cta.red.and.pred q, 1, %2, p;\nselp.b32 %0, 1, 0, q;\n}\n"
+               : "=r"(r)
+               : "r"((uint32_t)p), "r"(kEpiThreads)
+               : "memory");
+  return r != 0;
+}
+
 // One layer pass of the row kernel: its weights' tensor map, MMA N and K steps of 16.
 struct RowPass {
   int map, n, k16;
@@ -278,7 +289,7 @@ __global__ void __launch_bounds__(kRowsThreads, 1) mlp_rows_kernel(const __grid_
       mbar_arrive(smem_u32(&a_bar));
     };
     auto wait_acc = [&]() {
-      ok = ok && mbar_wait(smem_u32(&acc_bar), (uint32_t)(na & 1));
+      ok = __all_sync(0xffffffffu, ok && mbar_wait(smem_u32(&acc_bar), (uint32_t)(na & 1)));
       ++na;
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     };
@@ -384,7 +395,7 @@ __global__ void __launch_bounds__(kRowsThreads, 1) mlp_rows_kernel(const __grid_
             }
           }
           // the staged rows are read before they (or the buffer's next input) are written again
-          asm volatile("bar.sync 1, %0;" ::"r"(kEpiThreads) : "memory");
+          ok = all_ok(ok);
         }
       } else {
         const float invB = 1.f / (float)g.B;
@@ -445,7 +456,10 @@ __global__ void __launch_bounds__(kRowsThreads, 1) mlp_rows_kernel(const __grid_
           publish();
         }
         wait_acc();                          // dZ_1 is stored
-        if (next < tiles) load(next, nbuf);
+        if (next < tiles) {
+          load(next, nbuf);
+          ok = all_ok(ok);
+        }
       }
       abuf = nbuf;
     }
