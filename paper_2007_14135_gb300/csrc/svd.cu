@@ -27,6 +27,8 @@
 // kernels per sweep with one rotation after the other. A level at M = 16 takes about 4600 cycles: 1900
 // for the rotations' FP64 chain, 400 for the diagonal, 2000 for the element updates; at M = 64 the
 // element updates are bound by one SM's FP64 rate (8200 of 11100 cycles).
+#include <cuda.h>
+#include <cudaTypedefs.h>
 #include <cuda_runtime.h>
 #include <math_constants.h>
 
@@ -522,6 +524,28 @@ __global__ void __launch_bounds__(kSvdThreads, 1) svd_kernel(const void *X, int 
   if (!ok && blockIdx.x == 0 && tid == 0) *info = -(int)DOA_ETIMEOUT;
 }
 
+// SMs that kernels of a stream may use: the device's, or those of the stream's green context. The CTAs of the
+// grid wait for one another, so a launch of more of them than can be resident is refused.
+int stream_sm_count(cudaStream_t s) {
+  auto entry = [](const char *name, unsigned version) {
+    cudaDriverEntryPointQueryResult q;
+    void *fn = nullptr;
+    const cudaError_t e = cudaGetDriverEntryPointByVersion(name, &fn, version, cudaEnableDefault, &q);
+    return e == cudaSuccess && q == cudaDriverEntryPointSuccess ? fn : nullptr;
+  };
+  static const auto stream_ctx = reinterpret_cast<PFN_cuStreamGetCtx_v12050>(entry("cuStreamGetCtx", 12050));
+  static const auto ctx_res = reinterpret_cast<PFN_cuCtxGetDevResource_v12040>(entry("cuCtxGetDevResource", 12040));
+  static const auto green_res =
+      reinterpret_cast<PFN_cuGreenCtxGetDevResource_v12040>(entry("cuGreenCtxGetDevResource", 12040));
+  const int all = device_sm_count();
+  CUcontext ctx = nullptr;
+  CUgreenCtx green = nullptr;
+  CUdevResource r{};
+  if (!stream_ctx || !ctx_res || !green_res || stream_ctx(s, &ctx, &green) != CUDA_SUCCESS) return all;
+  const CUresult got = green ? green_res(green, &r, CU_DEV_RESOURCE_TYPE_SM) : ctx_res(ctx, &r, CU_DEV_RESOURCE_TYPE_SM);
+  return got == CUDA_SUCCESS && r.sm.smCount > 0 ? std::min(all, (int)r.sm.smCount) : all;
+}
+
 }  // namespace
 }  // namespace doa
 
@@ -546,7 +570,7 @@ doa_status doa_svd_data(const void *X, int x_c128, int M, int N, int ldx, double
   if (ws_bytes < (size_t)lay.bytes) return DOA_ENOMEM;
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   const int nchunks = (N + kSvdT - 1) / kSvdT;
-  const int nblk = std::min(std::min(nchunks, kSvdMaxBlocks), device_sm_count());
+  const int nblk = std::min(std::min(nchunks, kSvdMaxBlocks), stream_sm_count(s));
   const int smem = (int)((size_t)(2 * M * kSvdT + M * M) * sizeof(double2));
   if (ensure_smem_attr((const void *)svd_kernel, smem) != cudaSuccess) return DOA_ECUDA;
   uint8_t *w = static_cast<uint8_t *>(ws);
