@@ -92,7 +92,7 @@ inline __device__ bool fill(const float *__restrict__ P, int L, int t0, int stri
     float lf[U], rt[U];
     const float *p = P + (4 * q - off);
     const int i0 = 4 * q - off;
-    if (i0 >= 1 && i0 + 4 * (U - 1) * stride + 4 <= L - 1) {   // inside, with a point to spare at either end
+    if (i0 >= 1 && i0 <= L - 5 - 4 * (U - 1) * stride) {   // inside, with a point to spare at either end
 #pragma unroll
       for (int u = 0; u < U; ++u) {
         v[u] = *reinterpret_cast<const float4 *>(p + 4 * u * stride);
@@ -102,8 +102,8 @@ inline __device__ bool fill(const float *__restrict__ P, int L, int t0, int stri
     } else {
 #pragma unroll
       for (int u = 0; u < U; ++u) {
-        const int iu = i0 + 4 * u * stride;
-        const bool in = q + u * stride < nq;
+        const bool in = q + u * stride < nq;   // (beyond it the index may leave the range of int)
+        const int iu = in ? i0 + 4 * u * stride : 0;
         v[u] = in ? load_quad(P, L, iu) : make_float4(0.f, 0.f, 0.f, 0.f);
         lf[u] = in && iu >= 1 ? P[iu - 1] : 0.f;
         rt[u] = in && iu + 4 <= L - 1 ? P[iu + 4] : 0.f;
@@ -356,12 +356,6 @@ inline __device__ bool fill2d(const float *__restrict__ P, int La, int Le, bool 
     }
   }
   return more;
-}
-
-__device__ __forceinline__ int select_top2d(const float *__restrict__ P, int La, int Le, bool wrap, int d, Cand *sel) {
-  return select_rounds(d, sel, [&](const Cand &thr, Cand (&cache)[kCache], int &n) {
-    return fill2d(P, La, Le, wrap, (int)threadIdx.x, kPeakThreads, thr, cache, n);
-  });
 }
 
 }  // namespace pk

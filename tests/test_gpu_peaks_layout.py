@@ -168,3 +168,30 @@ def test_many_spectra_match_the_single_picker(env, L, d):
             n = int(c1)
             assert int(cnt[i, a]) == n
             assert torch.equal(idx[i, a * d:a * d + n], i1[:n]) and torch.equal(val[i, a * d:a * d + n], v1[:n])
+
+
+@pytest.mark.parametrize("L,off,d", [(4095, 1, 5), (4096, 0, 9), (4101, 3, 63), (8191, 2, 1)])
+def test_peaks_around_the_shortest_cluster(env, L, off, d):
+    test_peaks_cluster_matches_oracle(env, L, off, d)
+
+
+def test_peaks_of_the_longest_spectra(env):
+    """2^31 - 64 points, where an index four quads ahead of a spectrum's last ones is beyond an int: peaks at
+    both ends and around the last steps, found exactly."""
+    torch, doa = env
+    L = 2 ** 31 - 64
+    free, _ = torch.cuda.mem_get_info()
+    if free < 6 * L:
+        pytest.skip("needs 12 GB")
+    P = torch.zeros(L, dtype=torch.float32, device="cuda")
+    at = [1, 4097, L // 2 + 3, L - 70001, L - 24581, L - 24577, L - 8190, L - 5, L - 2]
+    for k, i in enumerate(at):
+        P[i] = float(k + 1)
+    idx = torch.full((16,), -1, dtype=torch.int32, device="cuda")
+    val = torch.zeros(16, dtype=torch.float32, device="cuda")
+    cnt = torch.zeros(1, dtype=torch.int32, device="cuda")
+    doa.doa_peaks(P, 16, idx, val, cnt)
+    torch.cuda.synchronize()
+    assert cnt.item() == len(at)
+    assert idx.cpu().tolist()[:len(at)] == at
+    assert val.cpu().tolist()[:len(at)] == [float(k + 1) for k in range(len(at))]
