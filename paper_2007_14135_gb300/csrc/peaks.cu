@@ -48,7 +48,9 @@ __device__ void write_sel(Cand *sel, int nsel, int *idx, float *val, int *count)
 
 namespace cg = cooperative_groups;
 constexpr int kPeakCluster = 8;
-constexpr int kClusterPoints = 16384;      // points from which a spectrum takes a cluster
+// Points from which a spectrum takes a cluster, one CTA / cluster: smooth spectra the same from here to 16384
+// (13 us); rough ones (a peak in most quads) 20 / 12 us at 4096, 24 / 7 at 8192, 35 / 8 at 16383.
+constexpr int kClusterPoints = 4096;
 
 // This CTA's share of a spectrum's quads: rank of kCs CTAs of T threads.
 template <int kCs, int T>
