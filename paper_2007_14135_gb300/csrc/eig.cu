@@ -25,11 +25,11 @@
 //
 // Two shapes, with the same arithmetic and results. A warp per matrix (or G packed matrices, every
 // lane owning one pair's rotation) keeps the most matrices resident and suits large batches of M <= 16.
-// A CTA per matrix (3, 5 or 17 warps at M <= 8, 16, 32) suits single calls, small batches and M <= 32,
+// A CTA per matrix (3, 4 or 5, 16 or 17 warps at M <= 8, 16, 32) suits single calls, small batches and M <= 32,
 // which otherwise wait for one warp's chain of instructions: one FP64 matrix of M = 8 in 78 instead of
-// 141 us, 256 double-float matrices of M = 32 in 0.96 instead of 2.84 ms. Half of A: one FP64 matrix of M = 64
-// in 6.8 instead of 9.6 ms. The warp form in double-float takes two lanes a block, a column each, which
-// share the indices and rotations of two elements: 4096 matrices of M = 16 in 1.10 ms (1.21 with four).
+// 141 us, 256 double-float matrices of M = 32 in 0.81 instead of 2.84 ms. Half of A: one FP64 matrix of M = 64
+// in 6.8 instead of 9.6 ms. Double-float takes two lanes a block, a column each, which share the indices and
+// rotations of two elements: 4096 matrices of M = 16 (warp form) in 1.09 ms, 1.21 with four.
 // M <= 64 gets a 512-thread CTA in FP64, or in double-float a cluster of four CTAs that split its
 // rows (jacobi_cluster_df).
 #include <cooperative_groups.h>
@@ -62,16 +62,18 @@ struct EigSmem {
   static_assert(sizeof(Rot) * (NP / 2) >= NP * (sizeof(double) + sizeof(int)), "lam and order fit in rot");
 };
 
-// Threads per matrix of the CTA form: a round's warp steps (blocks of A, then rows of V) are 2 + 1 at
-// M = 8, 5 + 4 (both halves: 8 + 4) at M = 16, 17 + 16 (32 + 16) at M = 32, taken in one, two (three) and
-// two (three) turns. Six and 24 warps take the larger numbers in two turns but let fewer matrices reside
-// (double-float): 0.125 against 0.14 ms for one matrix of M = 16, 0.44 against 0.38 for 1024; 0.48 against
-// 0.50 ms for one of M = 32, 1.20 against 0.96 for 256.
-template <int NP>
-__host__ __device__ constexpr int cta_threads() { return NP <= 8 ? 96 : (NP <= 16 ? 160 : (NP <= 32 ? 544 : 512)); }
+// Threads per matrix of the CTA form. A round's warp steps (blocks of A, then rows of V) are 2 + 1 at M = 8; in
+// double-float 4 + 4 at M = 16 and 16 + 16 at M = 32, two turns of four and 16 warps; in FP64 with half of A
+// 5 + 4 and 17 + 16, which suits five and 17. Batches take the first numbers for either, as
+// more matrices reside (double-float, five / four warps: 1024 matrices of M = 16 0.36 / 0.32 ms; FP64 256 of
+// M = 16 0.37 / 0.43, 1024 0.90 / 0.89); single calls their own (one FP64 matrix of M = 16 0.23 / 0.28).
+template <int NP, bool kDF = true>
+__host__ __device__ constexpr int cta_threads() {
+  return NP <= 8 ? 96 : NP <= 16 ? (kDF ? 128 : 160) : NP <= 32 ? (kDF ? 512 : 544) : 512;
+}
 // Largest batch that takes the CTA form (the eig stage, warp form against CTA form): at M <= 8, 63 / 47
-// us for 1 matrix, 82 / 74 for 1024, 112 / 131 for 2048; at M <= 16, 0.32 / 0.14 ms for 1, 0.55 / 0.38
-// for 1024, 0.80 / 0.71 for 2048; at M <= 32 always (1.9 / 0.50 ms for 1, 5.3 / 3.1 for 1024).
+// us for 1 matrix, 82 / 74 for 1024, 112 / 131 for 2048; at M <= 16, 0.32 / 0.14 ms for 1, 0.55 / 0.32
+// for 1024, 0.80 / 0.59 for 2048; at M <= 32 always (1.9 / 0.41 ms for 1, 5.3 / 2.6 for 1024).
 template <int NP>
 __host__ constexpr int eig_cta_limit() { return NP <= 8 ? 1024 : 2048; }
 template <int NP>
@@ -298,7 +300,8 @@ template <class Ar, int NP, int G, int T>
 __device__ void jacobi_group(EigSmem<NP> *mats, const int *Ms, const double2 *const *Rs, const bool *both, int *res) {
   static_assert(T == 32 || G == 1, "a CTA works on one matrix");
   constexpr int HP = NP / 2, W = T / 32;
-  constexpr bool kColumns = T == 32 && Ar::kBoth;   // a lane per column of a block, not per element
+  // a lane per column of a block, not per element (a CTA of M <= 8 has a warp for each element step)
+  constexpr bool kColumns = Ar::kBoth && (T == 32 || NP > 8);
   using g = Grp<T>;
   using El = typename Ar::El;
   __shared__ unsigned smask[2];   // the round's rotations, by round parity (CTA form)
@@ -887,12 +890,12 @@ template <int NP, bool kDF>
 using Arith = std::conditional_t<kDF, ArithDF<NP>, ArithF64<NP>>;
 
 template <int NP, bool kDF>
-__global__ void __launch_bounds__(cta_threads<NP>()) eig_single_kernel(const double2 *R64, int M, int d, int alg, double *evals,
+__global__ void __launch_bounds__(cta_threads<NP, kDF>()) eig_single_kernel(const double2 *R64, int M, int d, int alg, double *evals,
                                                        double2 *B, int *K_out, int *info) {
   start_after_previous();
   let_next_start();
   extern __shared__ __align__(16) uint8_t smem[];
-  constexpr int T = cta_threads<NP>();
+  constexpr int T = cta_threads<NP, kDF>();
   EigSmem<NP> *mats = reinterpret_cast<EigSmem<NP> *>(smem);
   const int Ms[1] = {M};
   const double2 *Rs[1] = {R64};
@@ -1066,7 +1069,7 @@ cudaError_t run_single_p(const double2 *R64, int M, int d, int alg, double *eval
   const int smem = (int)sizeof(EigSmem<NP>);
   cudaError_t e = ensure_smem_attr((const void *)eig_single_kernel<NP, kDF>, smem);
   if (e != cudaSuccess) return e;
-  return launch_chained(eig_single_kernel<NP, kDF>, 1, cta_threads<NP>(), smem, st, R64, M, d, alg, evals, B, K_out, info);
+  return launch_chained(eig_single_kernel<NP, kDF>, 1, cta_threads<NP, kDF>(), smem, st, R64, M, d, alg, evals, B, K_out, info);
 }
 
 cudaError_t run_single_cluster(const double2 *R64, int M, int d, int alg, double *evals, double2 *B, int *K_out,
