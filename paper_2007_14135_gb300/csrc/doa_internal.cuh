@@ -289,6 +289,8 @@ constexpr int kScanGroupDefault = 32;
 // 725 / 695, 256 (groups of 13) 297 / 294, 64 (groups of 3) 174 / 188; M = 16, 1024 problems
 // 2400 / 2158, 64 (groups of 6) 506 / 426; M = 12, 64 (6) 346 / 326, 32 (3) 277 / 290.
 __host__ __device__ constexpr int geo_group_pt(int bucket) { return bucket == 0 ? 4 : bucket == 1 ? 2 : 0; }
+// (1216: eight per SM of the 152 these kernels are written for. A plan is made on the host, perhaps without a
+// device, and its bytes do not depend on one.)
 constexpr int64_t kGeoGroupMinUnits = 1216;
 __host__ __device__ constexpr int geo_group_min(int bucket) { return bucket == 0 ? 16 : 4; }
 __host__ __device__ inline bool scan_group_allowed(int g) { return g >= 1 && g <= kScanGroupMax && (g & (g - 1)) == 0; }
@@ -406,6 +408,7 @@ __host__ __device__ constexpr int scan_pt_default(int bucket) { return bucket <=
 // thread's points are then most of the kernel's length). Single scans, 4 points / 1 point per thread: M = 8,
 // 1801 points 6.2 / 5.6 us, 60 001 8.4 / 8.0, 360 x 90 11.1 / 10.0; M = 16, 1801 9.0 / 7.2 us, 18 001
 // 9.0 / 7.3, 60 001 10.9 / 11.1, 360 x 90 15.2 / 12.3.
+// (Two blocks per SM of 152, a constant for the reason given at kGeoGroupMinUnits.)
 constexpr int64_t kScanFewPoints = 304 * 128;
 __host__ __device__ constexpr int scan_pt_for(int bucket, int64_t npts) {
   return npts < kScanFewPoints * (bucket == 0 ? 2 : 1) ? 1 : scan_pt_default(bucket);
@@ -443,7 +446,11 @@ int device_sm_count();
 // programmatic dependents: each starts once every block of the one before it has started
 // (let_next_start), in the room that one leaves, and ends after it (end_after_previous: block 0 waits
 // before it exits, and a grid is complete when its last block is), so that a normal launch after
-// them finds all of them done. 1024 mixed problems (M of 8, 12, 16 and 32): covariance 1.20 -> 0.96 ms,
+// them finds all of them done. What such a set reads of earlier stages (covariances, factors, tables) its
+// first kernel vouches for, in order and in visibility: it is launched normally, or waits
+// (start_after_previous) before it lets the next one start, so the earlier grids are complete and their
+// writes flushed before any block of the set's other kernels begins; those never wait before they read.
+// Where a set begins with a kernel that may be absent, the next one takes its part (dep, beside). 1024 mixed problems (M of 8, 12, 16 and 32): covariance 1.20 -> 0.96 ms,
 // decompositions 1.17 -> 0.89, scans 2.32 -> 2.10, the solve 5.17 -> 4.33 ms.
 #ifdef __CUDACC__
 __device__ __forceinline__ void let_next_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
