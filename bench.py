@@ -44,15 +44,13 @@ def workload_name(batch):
             f"grid -90:{STEP}:90 deg (L={grid_L()}), PHD+MUSIC+EV+MN on each")
 
 
-# DRAM bytes (read + write) per launch of the dominant kernels, from ncu: the paper-density kernels
-# captured at the bench's 4096 problems (one pass, profiles/paper_density_batch_launches.md), the
-# circular array from a smaller case scaled to the bench's batch by the problem count (every problem
-# is an independent, equal unit; profiles/paper_uca_geometry_scan_ncu.md). Reset an entry to None
-# when its kernel changes.
+# DRAM bytes (read + write) per launch of the dominant kernels, from ncu, one pass at the bench's 4096
+# problems (profiles/paper_density_batch_launches.md, profiles/paper_uca_geometry_scan_ncu.md). Reset an
+# entry to None when its kernel changes.
 TRAFFIC_BYTES = {
-    "scan_shared_kernel<16,4>": 35197696 + 1122881024,        # read + written, 4096-problem launch
-    "covariance_tc_batch_kernel<16>": 2148942336 + 15538176,
-    "scan_geometry_batch_kernel<8,4>": 2 * (4493312 + 206536704),   # 2048-problem capture x 2
+    "scan_shared_kernel<16,4>": 36733696 + 1120996608,        # read + written, 4096-problem launch
+    "covariance_tc_batch_kernel<16>": 2148950016 + 18747904,
+    "scan_geometry_shared_kernel<8,4>": 10754816 + 472654080,
     "scan_geometry_batch_kernel<8,2>": None,
 }
 

@@ -161,6 +161,9 @@ doa_status doa_covariance_noalloc(const float *X, int M, int N, int ldx, float *
 doa_status doa_noise_subspace(const double *R64, int M, int d, int alg, double *evals, double *B,
                               int *K_out, int *info, void *stream);
 
+/* Single columns of B are fixed by R's last digits only where noise eigenvalues nearly meet (a change of
+ * 1e-14 of R may move one by 1e-6 of its norm); B B^H and the eigenvalues are not. */
+
 /* doa_noise_subspace with the Jacobi's arithmetic chosen (doa_eig_prec): doa_noise_subspace is
  * this call with DOA_EIG_FP64. With DOA_EIG_DOUBLE_FLOAT the rotations run until no pair has
  * |a_pq| > 1e-12 sqrt(|a_pp a_qq|), the converged A and V are rounded to FP64 and sorted, and the
@@ -245,7 +248,8 @@ doa_status doa_model_order(const double *evals, int M, int N, int *mdl, int *aic
  * iteration stops after the first sweep that rotates nothing. Then X = U S V^H, and the eigenvalues of R are
  * S_k^2 / N with eigenvectors the columns of U. Small singular values keep their relative
  * accuracy (R's eigenvalues below ~1e-16 of the largest do not).
- * GPU form: one cooperative kernel (its CTAs, one per SM at most, wait for one another). The rows
+ * GPU form: one cooperative kernel (its CTAs, at most one per SM that the stream's context has, wait
+ * for one another). The rows
  * live in an FP64 copy Y of X in ws; a pass over Y on all SMs applies the rotations found so far and
  * forms the Gram matrix Y Y^H in FP64, and the sweep's rotations run on that Gram matrix in one CTA
  * (its pair entries are the rotated Gram entries). While off-diagonal entries above 1e-4
