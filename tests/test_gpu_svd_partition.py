@@ -18,7 +18,7 @@ class Resource(ctypes.Structure):
 
 
 def partition_stream(cu, sms):
-    """A stream of a green context of `sms` SMs or a few more, and their number; None where the driver has none."""
+    """A stream of a green context of `sms` SMs or a few more, and their number; None where there are none."""
     p = ctypes.c_void_p
     whole, part, rest, n = Resource(), Resource(), Resource(), ctypes.c_uint(1)
     desc, green, stream = p(), p(), p()
