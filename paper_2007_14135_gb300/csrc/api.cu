@@ -682,6 +682,7 @@ doa_status doa_batch_plan(const doa_problem *probs, int nprob, const doa_tuning 
     ws = round_up(ws + mm, 256);
     q.npts = (int32_t)spectrum_points(p);
     h.max_points = std::max(h.max_points, q.npts);
+    if (p.eig_prec == DOA_EIG_FP64) h.eig_fp64 |= 1 << b;
     q.part_off = ws;
     if (cov_tc_ok(p)) {
       q.nchunks = 0;

@@ -356,7 +356,7 @@ struct PlanHeader {
   int32_t tcg_groups;
   int32_t tcg_chunks;                    // runs of up to kTcgChunk groups of one grid and key
   int32_t tcg_probs;
-  int32_t tcg_pad;
+  int32_t eig_fp64;                      // bit b: some problem of bucket b asks for the FP64 Jacobi
   int64_t tcg_units;                     // (tile, chunk) units
   int64_t off_tcg, off_tcc, off_tcgl;    // PlanTcGroup, PlanTcChunk arrays and the problem list
   // shared-steering geometry scan, per M bucket (the problems of these groups are counted in geo_jobs

@@ -64,9 +64,8 @@ struct EigSmem {
 
 // Threads per matrix of the CTA form. A round's warp steps (blocks of A, then rows of V) are 2 + 1 at M = 8; in
 // double-float 4 + 4 at M = 16 and 16 + 16 at M = 32, two turns of four and 16 warps; in FP64 with half of A
-// 5 + 4 and 17 + 16, which suits five and 17. Batches take the first numbers for either, as
-// more matrices reside (double-float, five / four warps: 1024 matrices of M = 16 0.36 / 0.32 ms; FP64 256 of
-// M = 16 0.37 / 0.43, 1024 0.90 / 0.89); single calls their own (one FP64 matrix of M = 16 0.23 / 0.28).
+// 5 + 4 and 17 + 16, which suits five and 17 (double-float, five / four warps: 1024 matrices of M = 16 0.36 /
+// 0.32 ms; FP64 one 0.23 / 0.28, 256 0.37 / 0.43, 1024 0.90 / 0.89). A bucket with both takes FP64's.
 template <int NP, bool kDF = true>
 __host__ __device__ constexpr int cta_threads() {
   return NP <= 8 ? 96 : NP <= 16 ? (kDF ? 128 : 160) : NP <= 32 ? (kDF ? 512 : 544) : 512;
@@ -1002,14 +1001,13 @@ __global__ void __launch_bounds__(32 * eig_warps<NP>(), eig_min_ctas<NP>()) eig_
   end_after_previous();
 }
 
-// The CTA form of the batch: a CTA per matrix.
-template <int NP>
-__global__ void __launch_bounds__(cta_threads<NP>()) eig_batch_cta_kernel(const uint8_t *plan, uint8_t *ws, int bucket,
-                                                                          int *status, int dep) {
+// The CTA form of the batch: a CTA of T threads per matrix.
+template <int NP, int T>
+__global__ void __launch_bounds__(T) eig_batch_cta_kernel(const uint8_t *plan, uint8_t *ws, int bucket, int *status,
+                                                          int dep) {
   if (dep) start_after_previous();
   let_next_start();
   extern __shared__ __align__(16) uint8_t smem[];
-  constexpr int T = cta_threads<NP>();
   EigSmem<NP> &s = *reinterpret_cast<EigSmem<NP> *>(smem);
   const PlanHeader *h = reinterpret_cast<const PlanHeader *>(plan);
   const int prob = reinterpret_cast<const int32_t *>(plan + h->off_eig[bucket])[blockIdx.x];
@@ -1123,13 +1121,22 @@ cudaError_t run_batch_g(const uint8_t *plan, int count, uint8_t *ws, int *status
                           (int)!beside);
 }
 
-template <int NP>
-cudaError_t run_batch_cta(const uint8_t *plan, int count, uint8_t *ws, int *status, int bucket, bool beside, cudaStream_t st) {
-  if (count == 0) return cudaSuccess;
+template <int NP, int T>
+cudaError_t run_batch_cta_t(const uint8_t *plan, int count, uint8_t *ws, int *status, int bucket, bool beside, cudaStream_t st) {
   const int smem = (int)sizeof(EigSmem<NP>);
-  cudaError_t e = ensure_smem_attr(reinterpret_cast<const void *>(eig_batch_cta_kernel<NP>), smem);
+  cudaError_t e = ensure_smem_attr(reinterpret_cast<const void *>(eig_batch_cta_kernel<NP, T>), smem);
   if (e != cudaSuccess) return e;
-  return launch_programmatic(beside || chained_grid(count, true), eig_batch_cta_kernel<NP>, count, cta_threads<NP>(), smem, st, plan, ws, bucket, status, (int)!beside);
+  return launch_programmatic(beside || chained_grid(count, true), eig_batch_cta_kernel<NP, T>, count, T, smem, st, plan,
+                             ws, bucket, status, (int)!beside);
+}
+
+template <int NP>
+cudaError_t run_batch_cta(const uint8_t *plan, const PlanHeader &h, uint8_t *ws, int *status, int bucket, bool beside, cudaStream_t st) {
+  const int count = h.eig_count[bucket];
+  if (count == 0) return cudaSuccess;
+  return (h.eig_fp64 >> bucket) & 1
+             ? run_batch_cta_t<NP, cta_threads<NP, false>()>(plan, count, ws, status, bucket, beside, st)
+             : run_batch_cta_t<NP, cta_threads<NP>()>(plan, count, ws, status, bucket, beside, st);
 }
 
 // M <= 16: the CTA form for small batches unless the plan packs matrices (G in {1, 2, 4, 8} up to the
@@ -1139,7 +1146,7 @@ cudaError_t run_batch(const uint8_t *plan, const PlanHeader &h, uint8_t *ws, int
                       bool beside, cudaStream_t st) {
   const int count = h.eig_count[bucket];
   const int g = h.eig_mats[bucket];
-  if (g == 1 && count <= eig_cta_limit<NP>()) return run_batch_cta<NP>(plan, count, ws, status, bucket, beside, st);
+  if (g == 1 && count <= eig_cta_limit<NP>()) return run_batch_cta<NP>(plan, h, ws, status, bucket, beside, st);
   if (count == 0) return cudaSuccess;
   if (g >= 8 && mats_per_warp<NP>() >= 8) return run_batch_g<NP, (mats_per_warp<NP>() >= 8 ? 8 : 1)>(plan, count, ws, status, bucket, beside, st);
   if (g >= 4) return run_batch_g<NP, 4>(plan, count, ws, status, bucket, beside, st);
@@ -1220,7 +1227,7 @@ cudaError_t launch_eig_batch(const uint8_t *plan_dev, const PlanHeader &h, uint8
   bool beside = false;
   if ((e = run_batch_cluster(plan_dev, h, ws, status, 3, beside, s)) != cudaSuccess) return e;
   beside = beside || h.eig_count[3] > 0;
-  if ((e = run_batch_cta<32>(plan_dev, h.eig_count[2], ws, status, 2, beside, s)) != cudaSuccess) return e;
+  if ((e = run_batch_cta<32>(plan_dev, h, ws, status, 2, beside, s)) != cudaSuccess) return e;
   beside = beside || h.eig_count[2] > 0;
   if ((e = run_batch<16>(plan_dev, h, ws, status, 1, beside, s)) != cudaSuccess) return e;
   beside = beside || h.eig_count[1] > 0;

@@ -97,3 +97,36 @@ def test_digits_do_not_depend_on_the_outputs_asked_for(M, prec):
     for r in results[1:]:
         for x, y in zip(results[0], r):
             np.testing.assert_array_equal(x, y)
+
+
+@pytest.mark.parametrize("M", [7, 13, 16, 24, 32])
+def test_digits_do_not_depend_on_the_neighbours_arithmetic(M):
+    """A bucket with an FP64 problem takes FP64's CTA size: the double-float problems' outputs, and the FP64 one's,
+    are those of buckets of one arithmetic."""
+    torch, doa = require_gpu()
+    insts = [synth.custom(M, max(1, M // 4), 200, None, 10.0, 1.0, seed=960 + M + i) for i in range(3)]
+
+    def solve(precs):
+        outs, probs = [], []
+        for inst, prec in zip(insts, precs):
+            X = torch.from_numpy(inst.X).cuda()
+            P = torch.empty(inst.L, dtype=torch.float32, device="cuda")
+            pk = [torch.zeros(inst.d, dtype=t, device="cuda") for t in (torch.int32, torch.float32)]
+            cnt = torch.zeros(1, dtype=torch.int32, device="cuda")
+            ev = torch.zeros(M, dtype=torch.float64, device="cuda")
+            B = torch.zeros(M * M, dtype=torch.complex128, device="cuda")
+            probs.append(doa.make_problem(X, inst.d, 1 << doa.MUSIC, doa.grid(inst.lo, inst.step, inst.L), P, *pk, cnt,
+                                          evals=ev, B_out=B, eig_prec=prec))
+            outs.append((X, P, ev, B, pk, cnt))
+        status = torch.full((len(insts),), -1, dtype=torch.int32, device="cuda")
+        plan = doa.BatchPlan(probs)
+        doa.doa_solve_batch(plan, doa.workspace(plan), status)
+        torch.cuda.synchronize()
+        assert status.cpu().tolist() == [0] * len(insts)
+        return [[t.cpu().numpy() for t in o[1:4]] for o in outs]
+
+    df, f64 = doa.EIG_DOUBLE_FLOAT, doa.EIG_FP64
+    mixed, alone, wide = solve([df, f64, df]), solve([df, df, df]), solve([f64, f64, f64])
+    for got, want in zip(mixed, (alone[0], wide[1], alone[2])):
+        for x, y in zip(got, want):
+            np.testing.assert_array_equal(x, y)
